@@ -46,7 +46,7 @@
  * Environment (read once per process; results do not depend on them):
  *            PC_APPLY_KERNEL = legacy | tma | split | row forces one stencil-
  *            kernel family for A/B comparisons (default: the plane-pipelined
- *            kernel for complex64 parity blocks, the two-pass kernels for
+ *            kernel for complex64 parity blocks, the integer-pipe kernel for
  *            complex128, or the autotuner's choice); PC_PCG_GRAPHS = 0 turns off CUDA-graph replay of PCG
  *            iterations; PC_TUNE_CACHE names the autotuner's cache file
  *            (pc_autotune); PC_WAIT_LIMIT = n sets how many polls a kernel's
@@ -81,7 +81,7 @@ extern "C" {
 
 /* ---- element types ----------------------------------------------------- */
 #define PC_C64 1   /* complex64: FP32 storage and FP32 arithmetic */
-#define PC_C128 2  /* complex128: FP64 storage and FP64 arithmetic */
+#define PC_C128 2  /* complex128: FP64 storage; arithmetic of at least FP64 accuracy */
 
 /* ---- precision of pc_eigs ---------------------------------------------- */
 #define PC_PREC_FP64 0   /* FP64 operator, inner PCG iterates, Krylov recurrences and residuals; the
@@ -164,7 +164,7 @@ int pc_grid_create(int N, const pc_material* m, pc_grid** out);
  * Voigt stiffness in row order ([11,22,33,23,13,12], engineering shear, Pa); rho: host [N^3],
  * kg/m^3, positive; a_lat as in pc_material.  Both arrays are copied (caller keeps ownership).
  * The device holds 22 FP64 values per node in each layout (about 0.35 KB per node in all).
- * Supported paths: complex128 applies (two-pass kernels), PC_PREC_FP64 eigen-solves, PCG,
+ * Supported paths: complex128 applies (integer-pipe or two-pass kernels), PC_PREC_FP64 eigen-solves, PCG,
  * mass, gradients (pc_eig_grad); complex64 applies and PC_PREC_MIXED return PC_EINVAL.  The
  * preconditioner's reference medium and the default shift use the nodes' volume averages and
  * largest entries.  PC_EINVAL for a non-finite entry or a non-positive density. */
@@ -313,7 +313,7 @@ int pc_apply_batch(pc_grid* g, int dtype, int count, const int* blocks, const vo
 int pc_set_k_multi(pc_grid* g, int nk, const double* kappas);
 
 /* pc_apply_batch with item i at the Bloch vector of slot kslots[i] (host; NULL = all slot 0):
- * y_i = (A_hat(kappa_{kslots[i]}) - shift_i M_hat) x_i.  The two-pass complex128 kernels and the
+ * y_i = (A_hat(kappa_{kslots[i]}) - shift_i M_hat) x_i.  The complex128 kernels and the
  * plane-pipelined complex64 kernel serve all slots in one launch; other launch shapes run once
  * per run of equal slots. */
 int pc_apply_batch_k(pc_grid* g, int dtype, int count, const int* blocks, const int* kslots,
@@ -392,8 +392,9 @@ int pc_eigs_batch(pc_batch_job* jobs, int njobs, const pc_options* opt, int work
 int pc_autotune(pc_grid* g, int dtype, int layout, int nitems, void* stream);
 
 /* The launch configuration the library will use for a batch of `nitems` vectors of `dtype` in
- * layout 0 (blocks) or 1 (full): kind 0 = register-staged, 1 = TMA tile, 2 = row tile, 3 = two-pass
- * (fluxes once per node, then gather; the default for complex128), 4 = plane-pipelined (producer
+ * layout 0 (blocks) or 1 (full): kind 0 = fused tile (shapes 0-3 register-staged; shape 8 the
+ * integer-pipe kernel, the default for complex128), 1 = TMA tile, 2 = row tile, 3 = two-pass
+ * (fluxes once per node, then gather), 4 = plane-pipelined (producer
  * warp + consumer warps; the default for complex64 parity blocks); tile shape code; planes per CTA
  * (tz; row and plane-pipelined kernels: least planes per CTA); CTAs of the launch (two-pass: of
  * its gather). */

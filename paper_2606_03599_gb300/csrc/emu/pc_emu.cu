@@ -13,6 +13,7 @@
 #include "../pc_apply_row.cuh"
 #include "../pc_apply_pipe.cuh"
 #include "../pc_apply_split.cuh"
+#include "../pc_apply_int.cuh"
 #include "../pc_small_dft.cuh"
 
 using namespace pc;
@@ -354,6 +355,99 @@ static void emu_run_split(const StencilParams<R>& P, int block, const void* x, v
         T::gather_node(P, G, p12, p13, fe.data(), xv, static_cast<C*>(y), mat, (R)shift, t, true);
 }
 
+// Same step sequence as fix_apply (tz planes per CTA; tx, ty > 0 force the tile extents); shared
+// memory poisoned first.
+template <bool CUBIC, int MATK>
+static int emu_run_fix(const StencilParams<double>& P, int block, const void* x, void* y, const void* mat,
+                       double shift, int tz, int tx, int ty) {
+    using T = FixApply<CUBIC, MATK>;
+    FixGeom G;
+    make_fix_geom(G, P.N, block < 0);
+    if (tx > 0) {
+        G.TX = tx < G.X ? tx : G.X;
+        G.TY = ty < G.Y ? ty : G.Y;
+        G.ntx = (G.X + G.TX - 1) / G.TX;
+        G.nty = (G.Y + G.TY - 1) / G.TY;
+        G.ncell = (G.TX + 1) * (G.TY + 2);
+    }
+    G.tz = tz > 0 && tz < G.Z ? tz : G.Z;
+    G.nch = (G.Z + G.tz - 1) / G.tz;
+    FixParams F;
+    if (!make_fix_params(F, P, CUBIC, MATK)) return -2;
+    const int n = G.ncell;
+    std::vector<unsigned char> mem(T::shared_bytes(G) + 64);
+    std::vector<typename T::Regs> regs(n);
+    for (int sub = 0; sub < (G.full ? 4 : 1); ++sub)
+        for (int blk = 0; blk < G.ntx * G.nty * G.nch; ++blk) {
+            std::memset(mem.data(), 0x7B, mem.size());
+            unsigned char* base = mem.data();
+            while ((uintptr_t)base & 15) ++base;
+            typename T::Shared sh;
+            T::carve(sh, base, G);
+            typename T::Ctx c;
+            c.F = &F;
+            c.G = &G;
+            c.kph = P.ph;
+            c.x = static_cast<const double2*>(x);
+            c.y = static_cast<double2*>(y);
+            c.mat = mat;
+            c.shift = shift;
+            c.dot = true;
+            const int tiles = G.ntx * G.nty, tile = blk % tiles;
+            c.a0 = (tile % G.ntx) * G.TX;
+            c.b0 = (tile / G.ntx) * G.TY;
+            c.k0 = (blk / tiles) * G.tz;
+            c.tz = G.tz < G.Z - c.k0 ? G.tz : G.Z - c.k0;
+            const int pb = G.full ? sub : block;
+            c.p12 = pb >> 1;
+            c.p13 = pb & 1;
+            for (int t = 0; t < n; ++t) T::load_tables(c, sh, t, n);
+            for (int t = 0; t < n; ++t) T::init(c, t, regs[t]);
+            for (int i = 0; i < 3; ++i)
+                for (int t = 0; t < n; ++t) {
+                    T::stage(c, sh, regs[t], t, c.k0 - 2 + i);
+                    T::convert(c, sh, regs[t], t, c.k0 - 2 + i, i);
+                }
+            const int klast = c.k0 + c.tz + 1;
+            for (int t = 0; t < n; ++t) {
+                T::stage(c, sh, regs[t], t, c.k0 + 1);
+                regs[t].mcur = T::read_mat(c, regs[t], c.k0 - 1);
+            }
+            int sm = 0, sc = 1, sp = 2;
+            for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; ++kf) {
+                for (int t = 0; t < n; ++t) {
+                    if (kf < c.k0 + c.tz) regs[t].mnext = T::read_mat(c, regs[t], kf + 1);
+                    T::flux(c, sh, regs[t], t, kf, sm, sc, sp);
+                    T::load_own(c, regs[t], kf);
+                }
+                for (int t = 0; t < n; ++t) {
+                    T::gather(c, sh, regs[t], kf);
+                    if (kf + 2 <= klast) T::convert(c, sh, regs[t], t, kf + 2, sm);
+                    if (kf + 3 <= klast) T::stage(c, sh, regs[t], t, kf + 3);
+                    T::next_mat(regs[t]);
+                }
+                const int t = sm;
+                sm = sc;
+                sc = sp;
+                sp = t;
+            }
+            for (int t = 0; t < n; ++t)
+                if (regs[t].ks < c.k0 + c.tz) T::slow_column(c, regs[t].ks, regs[t].off[0], regs[t].off[1]);
+        }
+    return 0;
+}
+
+static int emu_fix(bool cubic, int matkind, const StencilParams<double>& P, int block, const void* x, void* y,
+                   const void* mat, double shift, int tz, int tx, int ty) {
+    if (cubic)
+        return matkind == 2 ? emu_run_fix<true, 2>(P, block, x, y, mat, shift, tz, tx, ty)
+               : matkind    ? emu_run_fix<true, 1>(P, block, x, y, mat, shift, tz, tx, ty)
+                            : emu_run_fix<true, 0>(P, block, x, y, mat, shift, tz, tx, ty);
+    return matkind == 2 ? emu_run_fix<false, 2>(P, block, x, y, mat, shift, tz, tx, ty)
+           : matkind    ? emu_run_fix<false, 1>(P, block, x, y, mat, shift, tz, tx, ty)
+                        : emu_run_fix<false, 0>(P, block, x, y, mat, shift, tz, tx, ty);
+}
+
 template <typename R, bool FULL, bool CUBIC, int MATK>
 static int emu_shape(int shape, const StencilParams<R>& P, int block, const void* x, void* y, const void* mat,
                      double shift, int tz) {
@@ -426,6 +520,9 @@ extern "C" int pc_emu_apply(int N, int block, int dtype, int shape, int tz, cons
     }
     StencilParams<double> P;
     make_stencil_params(P, Chat, rhohat2, ainv9, cubic != 0, N, phi3, X, Y, Z);
+    if (shape == 60) return emu_fix(cubic != 0, matkind, P, block, x, y, mat, shift, tz, 0, 0);  // integer-pipe kernel
+    if (shape > 6000)  // the same with tiles of (shape / 10 % 100) x (shape % 10) columns
+        return emu_fix(cubic != 0, matkind, P, block, x, y, mat, shift, tz, shape / 10 % 100, shape % 10);
     if (matkind == 2) {  // nodewise material: the two-pass kernels only ([22][m] FP64 in mat)
         if (shape != 30) return -1;
         if (full) cubic ? emu_run_split<double, true, true, 2>(P, block, x, y, mat, shift)

@@ -82,8 +82,17 @@ int device_sm_count() {
     return n;
 }
 
-ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks, int matkind, bool scratch_ok) {
+ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks, int matkind, bool scratch_ok,
+                                bool int_ok) {
     ApplyConfig c;
+    if (int_ok && dtype == PC_C128 && apply_kernel_mode() == 0) {
+        // the FP64 pipe of GB300 (2 lanes per clock and SM) is left to the integer units; see
+        // pc_apply_int.cuh
+        c.fix = true;
+        c.shape = kFixShape;
+        c.ctas = fix_apply_ctas(Z, !blocks, nitems, 0, &c.tz);
+        return c;
+    }
     if (scratch_ok && ((dtype == PC_C128 && (apply_kernel_mode() == 0 || matkind == 2)) || apply_kernel_mode() == 3)) {
         // complex128 is bound by GB300's FP64 pipe: fluxes once per node (two-pass kernels)
         c.split = true;
@@ -196,6 +205,7 @@ void slot_phases(const pc_grid* g, int slot, double ph[3][2]) {
 static void fill_params(pc_grid* g) {
     make_stencil_params(g->P64, g->Chat, g->rhohat, g->Ainv, g->cubic, g->N, g->k.phi, g->X, g->Y, g->Z);
     make_stencil_params(g->P32, g->Chat, g->rhohat, g->Ainv, g->cubic, g->N, g->k.phi, g->X, g->Y, g->Z);
+    g->int_ok = fix_apply_ok(g->P64, g->cubic, g->matkind);
 }
 
 namespace pc {
@@ -494,6 +504,9 @@ static int apply_launch(pc_grid* g, int dtype, bool full, const ApplyConfig& cfg
                         const double* item_ph, int nitems, int slot, double* dot_partials, int dot_stride,
                         cudaStream_t s) {
     const int X = full ? g->N : g->X, Y = full ? g->N : g->Y, Z = g->Z;
+    if (cfg.fix)
+        return launch_apply_fix(full, g->cubic, g->matkind, params_at(g, g->P64, X, Y, Z, slot), items, item_ph, nitems,
+                                cfg.tz, dot_partials, dot_stride, s);
     if (cfg.split) {
         const size_t need = split_scratch_bytes(X, Y, Z, nitems, dtype);
         if (g->split_bytes < need) {
@@ -542,8 +555,8 @@ int grid_apply(pc_grid* g, int dtype, bool full, const ApplyItem* items, int nit
                int dot_stride, cudaStream_t s, const ApplyConfig* cfg_in) {
     const int X = full ? g->N : g->X, Y = full ? g->N : g->Y, Z = g->Z;
     ApplyConfig cfg = cfg_in ? *cfg_in : apply_config_for(g, full, nitems, dtype);
-    if (g->matkind == 2 && !(dtype == PC_C128 && cfg.split))
-        return fail(PC_EINVAL, "apply: a nodewise material is applied by the complex128 two-pass kernels only");
+    if (g->matkind == 2 && !(dtype == PC_C128 && (cfg.split || cfg.fix)))
+        return fail(PC_EINVAL, "apply: a nodewise material is applied in complex128 only");
     bool uniform = true;
     std::vector<double> iph((size_t)6 * std::max(nitems, 1));
     for (int i = 0; i < nitems; ++i) {
@@ -554,7 +567,7 @@ int grid_apply(pc_grid* g, int dtype, bool full, const ApplyItem* items, int nit
     }
     void* th = timing_enabled() ? timing_begin(s) : nullptr;
     int rc = PC_OK;
-    const bool per_item = cfg.split || (dtype == PC_C64 && cfg.pipe);
+    const bool per_item = cfg.split || cfg.fix || (dtype == PC_C64 && cfg.pipe);
     if (uniform || per_item) {
         rc = apply_launch(g, dtype, full, cfg, items, iph.data(), nitems, nitems ? items[0].kslot : 0, dot_partials,
                           dot_stride, s);

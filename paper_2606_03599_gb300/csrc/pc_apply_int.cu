@@ -1,0 +1,198 @@
+// Integer-pipe complex128 stencil apply (see pc_apply_int.cuh): kernel and launcher.
+#include <algorithm>
+
+#include "pc_apply_int.cuh"
+
+namespace pc {
+
+namespace {
+
+constexpr int kFixMaxItems = 64;
+
+struct FixBatch {
+    ApplyItem it[kFixMaxItems];
+    double ph[kFixMaxItems][3][2];  // (cos, sin) of each item's Bloch phases
+    int n;
+};
+
+// blockIdx.x = (tile, chunk of planes), blockIdx.y = item (full space: item * 4 + parity block).
+template <bool CUBIC, int MATK>
+__global__ void __launch_bounds__(kFixCells, 2)
+    fix_apply(const __grid_constant__ FixParams F, const __grid_constant__ FixBatch B, const __grid_constant__ FixGeom G,
+              double* __restrict__ dot_partials, int dot_stride) {
+    using T = FixApply<CUBIC, MATK>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int item = G.full ? (int)blockIdx.y >> 2 : (int)blockIdx.y;
+    const ApplyItem& it = B.it[item];
+    if (it.skip != nullptr && *it.skip) return;
+    typename T::Shared sh;
+    T::carve(sh, smem_raw, G);
+    const int tid = threadIdx.x, n = G.ncell;
+    const bool live = tid < n;
+    typename T::Ctx c;
+    c.F = &F;
+    c.G = &G;
+    c.kph = B.ph[item];
+    c.x = static_cast<const double2*>(it.x);
+    c.y = static_cast<double2*>(it.y);
+    c.mat = it.mat;
+    c.shift = it.shift;
+    c.dot = dot_partials != nullptr && it.dot_slot >= 0;
+    const int tiles = G.ntx * G.nty;
+    const int tile = (int)blockIdx.x % tiles, ch = (int)blockIdx.x / tiles;
+    c.a0 = (tile % G.ntx) * G.TX;
+    c.b0 = (tile / G.ntx) * G.TY;
+    c.k0 = ch * G.tz;
+    c.tz = min(G.tz, G.Z - c.k0);
+    const int blk = G.full ? (int)(blockIdx.y & 3) : it.block;
+    c.p12 = blk >> 1;
+    c.p13 = blk & 1;
+    typename T::Regs r;
+    T::load_tables(c, sh, tid, blockDim.x);
+    T::init(c, min(tid, n - 1), r);
+    if (!live) r.flags = 0;
+    const int klast = c.k0 + c.tz + 1;  // last plane of x
+    if (live) {
+        // the first three planes go through the flux cells, which nothing uses yet
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            typename T::Shared t = sh;
+            t.raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * n;
+            T::stage(c, t, r, tid, c.k0 - 2 + i);
+        }
+        T::stage(c, sh, r, tid, c.k0 + 1);
+        r.mcur = T::read_mat(c, r, c.k0 - 1);
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // phase table
+    if (live) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            typename T::Shared t = sh;
+            t.raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * n;
+            T::convert(c, t, r, tid, c.k0 - 2 + i, i);
+        }
+    }
+    __syncthreads();
+    int sm = 0, sc = 1, sp = 2;
+    for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; ++kf) {
+        if (live) {
+            if (kf < c.k0 + c.tz) r.mnext = T::read_mat(c, r, kf + 1);
+            T::flux(c, sh, r, tid, kf, sm, sc, sp);
+            T::load_own(c, r, kf);
+        }
+        __syncthreads();
+        T::gather(c, sh, r, kf);
+        if (kf + 2 <= klast && live) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            T::convert(c, sh, r, tid, kf + 2, sm);
+            if (kf + 3 <= klast) T::stage(c, sh, r, tid, kf + 3);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+        T::next_mat(r);
+        __syncthreads();
+        const int t = sm;
+        sm = sc;
+        sc = sp;
+        sp = t;
+    }
+    if (r.ks < c.k0 + c.tz) r.dot += T::slow_column(c, r.ks, r.off[0], r.off[1]);
+    if (c.dot) {
+        double v = r.dot;
+        double* red = reinterpret_cast<double*>(sh.fs);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((tid & 31) == 0) red[tid >> 5] = v;
+        __syncthreads();
+        if (tid == 0) {
+            double s = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+            const int sub = G.full ? (int)(blockIdx.y & 3) * (int)gridDim.x : 0;
+            dot_partials[(int64_t)it.dot_slot * dot_stride + sub + blockIdx.x] = s;
+        }
+    }
+}
+
+template <bool CUBIC, int MATK>
+int launch_fix_t(const FixParams& F, const FixBatch& B, const FixGeom& G, double* dp, int ds, cudaStream_t s) {
+    using T = FixApply<CUBIC, MATK>;
+    auto kern = fix_apply<CUBIC, MATK>;
+    const size_t smem = T::shared_bytes(G);
+    // the largest tile's need, set on every launch: an attribute of the kernel on the current device
+    PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 << 10));
+    const dim3 grid(G.ntx * G.nty * G.nch, B.n * (G.full ? 4 : 1));
+    kern<<<grid, (G.ncell + 31) / 32 * 32, smem, s>>>(F, B, G, dp, ds);
+    note_launch();
+    note_apply_launch();
+    PC_CUDA_TRY(cudaGetLastError());
+    return PC_OK;
+}
+
+// Chunks of planes per tile.  A chunk repeats two flux planes and loads three more of x, so few
+// chunks are best once every SM has work; below that more CTAs shorten the march.
+void fix_chunks(FixGeom& G, int nitems) {
+    const long base = (long)G.ntx * G.nty * (G.full ? 4 : 1) * std::max(nitems, 1);
+    const int sm = device_sm_count();
+    double best = -1;
+    for (int nch = 1; nch <= std::max(1, G.Z / 2); ++nch) {
+        const int tz = (G.Z + nch - 1) / nch;
+        if ((G.Z + tz - 1) / tz != nch) continue;
+        const long per = (base * nch + sm - 1) / sm;  // CTAs of the fullest SM
+        const double cost = (per == 1 ? 1.0 : 0.75 * per) * (tz + 4);
+        if (best < 0 || cost < best) {
+            best = cost;
+            G.tz = tz;
+            G.nch = nch;
+        }
+    }
+}
+
+}  // namespace
+
+int fix_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz) {
+    FixGeom G;
+    make_fix_geom(G, N, full);
+    if (tz_in > 0) {
+        G.tz = std::min(tz_in, G.Z);
+        G.nch = (G.Z + G.tz - 1) / G.tz;
+    } else {
+        fix_chunks(G, std::min(nitems, kFixMaxItems));
+    }
+    if (tz) *tz = G.tz;
+    return G.ntx * G.nty * G.nch * (full ? 4 : 1);
+}
+
+bool fix_apply_ok(const StencilParams<double>& P, bool cubic, int matkind) {
+    FixParams F;
+    return make_fix_params(F, P, cubic, matkind);
+}
+
+int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<double>& P, const ApplyItem* items,
+                     const double* item_ph, int nitems, int tz, double* dp, int ds, cudaStream_t s) {
+    FixGeom G;
+    make_fix_geom(G, P.N, full);
+    G.tz = std::max(1, std::min(tz, G.Z));
+    G.nch = (G.Z + G.tz - 1) / G.tz;
+    if (dp != nullptr && G.ntx * G.nty * G.nch * (full ? 4 : 1) > ds)
+        return fail(PC_EINVAL, "apply: launch has more CTAs than partial-sum slots");
+    FixParams F;
+    if (!make_fix_params(F, P, cubic, matkind)) return fail(PC_EINVAL, "apply: material scale outside the integer kernel's range");
+    for (int base = 0; base < nitems; base += kFixMaxItems) {
+        FixBatch B;
+        B.n = std::min(nitems - base, kFixMaxItems);
+        for (int i = 0; i < B.n; ++i) {
+            B.it[i] = items[base + i];
+            for (int e = 0; e < 6; ++e) B.ph[i][e / 2][e % 2] = item_ph[(size_t)6 * (base + i) + e];
+        }
+        int rc;
+        if (cubic) rc = matkind == 2 ? launch_fix_t<true, 2>(F, B, G, dp, ds, s)
+                        : matkind    ? launch_fix_t<true, 1>(F, B, G, dp, ds, s)
+                                     : launch_fix_t<true, 0>(F, B, G, dp, ds, s);
+        else rc = matkind == 2 ? launch_fix_t<false, 2>(F, B, G, dp, ds, s)
+                  : matkind    ? launch_fix_t<false, 1>(F, B, G, dp, ds, s)
+                               : launch_fix_t<false, 0>(F, B, G, dp, ds, s);
+        PC_TRY(rc);
+    }
+    return PC_OK;
+}
+
+}  // namespace pc

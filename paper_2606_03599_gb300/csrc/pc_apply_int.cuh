@@ -1,0 +1,889 @@
+// Complex128 stencil apply on the integer pipe: y = (A - shift M) x with every FP64 operand of the
+// stencil held as a 64-bit integer and one binary exponent per node.
+//
+// GB300 issues 2 FP64 lanes per clock and SM, but 64 lanes of 64-bit integer addition and 64 of
+// 32 x 32 + 64 bit multiply-add (measured: add.s64 63.9, mad.wide.s32 63.7, fma.f64 2.0).  The
+// stencil is additions and products with constants, so it is done in block floating point: a node's
+// six reals are integers below 2^56 in units of 2^(E - 1078), E the largest biased exponent among
+// them (FP64 values with an exponent within 3 of E keep every bit).  Sums are exact; a product with
+// a stiffness entry is 3 multiply-adds of 32-bit halves (the low x low part, below 2^-2 units, is
+// left out) and rounds once per output.  The rounding of a flux is a few units of 2^-57 of the
+// largest strain its node's values allow, where FP64 rounds the same sums at 2^-53 of them.
+//
+// Bounds (units of the node's exponent): x < 2^56, the sums H < 2^59 and strain < 2^60, stiffness
+// rows sum to less than 2^62 so that a stress is below 2^58 after the division by 2^64 (general
+// lattice: mixed sums < 2^59, stresses < 2^60 and their mixing < 0.98 2^59), fluxes < 2^59.6 and an output
+// below 2^62.2 (2^60.6 and 0.98 2^63).  Accumulated products: high parts < 2^58, middle parts < 2^62.4.
+//
+// The operator, the layouts and the flux regions are those of pc_apply_tile.cuh.  A full-space
+// vector is treated as its four parity blocks with strided addresses (the blocks do not couple), so
+// one geometry serves both layouts.
+//
+// Tile.  A CTA owns TX x TY columns of the quarter grid and marches through tz planes.  Thread
+// cells: the TX x TY output columns first, then the column at a0 + TX or a0 - 1 (by the plane's
+// parity), the row b0 + TY and the row b0 - 1.  Each cell is one thread: it stages x of its column
+// (asynchronous copy, Bloch phase if wrapped, conversion), forms the fluxes of its column when the
+// plane's parity needs them, and the first TX x TY finish the outputs.  Whatever wraps around the
+// cell sits in the last warps, so the FP64 phase products are not spread over all of them.
+//
+// Measured (one GB300, N = 48, 64 block vectors, shift on): 0.205 ms against 0.667 ms of the two-pass
+// FP64 kernels; N = 60 FCC sub-pixel material, four blocks: 0.084 against 0.195 ms; N = 64 nodewise
+// material, full space: 0.102 against 0.146 ms.  Bound by the instruction stream (half the issue slots
+// at 16 warps per SM); DRAM moves 143 MB per launch at N = 48, close to the 170 MB of x and y.
+//
+// Values outside the exponent range (infinities, NaN, below 2^-823 or above 2^877) mark their node;
+// a column is handed to FP64 (slow_column) from the first output that depends on a marked node.
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#include "pc_apply_tile.cuh"  // PC_IDX
+#include "pc_complex.cuh"
+#include "pc_internal.h"
+
+#if defined(__CUDACC__)
+#define PC_FIX_COLD __noinline__
+#else
+#define PC_FIX_COLD
+#endif
+
+namespace pc {
+
+constexpr int kFixCells = 256;       // most cells (threads) of a CTA
+constexpr int kFixSpecial = 1 << 14;  // exponent of a node that FP64 has to handle
+constexpr int kFixLow = 200, kFixHigh = 1900;  // biased exponents the integer path takes
+
+struct FixGeom {
+    int X, Y, Z;   // quarter-grid extents (N/2, N/2, N)
+    int N, full;   // full-space layout: addresses of the full grid
+    int TX, TY, ntx, nty, ncell;
+    int tz, nch;
+    int plane, vstr;  // nodes per plane and per component of the vector layout (N <= 1024: below 2^31)
+};
+
+struct FixHalf {
+    int hi, lo;  // c = hi 2^32 + lo, lo signed
+};
+
+struct FixParams {
+    StencilParams<double> P;  // FP64 tables: density, slow_column
+    FixHalf c[2][21];         // phase tables; MATK 1: C_0 and C_1 - C_0
+    FixHalf mix[9];           // lattice mixing (general lattices)
+    int coff[2];              // exponent a product with c[p] adds
+    int moff;                 // and the two lattice mixings together
+    int nthr;
+};
+
+PC_HD FixHalf fix_split(int64_t v) {
+    FixHalf h;
+    h.hi = (int)((v + 0x80000000LL) >> 32);
+    h.lo = (int)(uint32_t)v;
+    return h;
+}
+PC_HD int fix_upper(int p, int r) { return p <= r ? p * 6 - p * (p - 1) / 2 + (r - p) : r * 6 - r * (r - 1) / 2 + (p - r); }
+
+// Tables of one launch; false when a scale is out of the exponent range the kernel allows for.
+inline bool make_fix_params(FixParams& F, const StencilParams<double>& P, bool cubic, int matkind) {
+    F.P = P;
+    memset(F.c, 0, sizeof(F.c));
+    memset(F.mix, 0, sizeof(F.mix));
+    F.coff[0] = F.coff[1] = F.moff = 0;
+    if (matkind != 2) {
+        double rs[2];
+        for (int p = 0; p < 2; ++p) {
+            rs[p] = 0.0;
+            for (int i = 0; i < 6; ++i) {
+                double s = 0.0;
+                for (int j = 0; j < 6; ++j) s += fabs(P.C[p][i * 6 + j]);
+                rs[p] = fmax(rs[p], s);
+            }
+        }
+        if (matkind == 1) rs[0] = rs[1] = fmax(rs[0], rs[1]);
+        int k[2];
+        for (int p = 0; p < 2; ++p) {
+            int ex = 0;
+            if (!isfinite(rs[p])) return false;
+            if (rs[p] > 0) frexp(rs[p], &ex);
+            k[p] = (matkind == 1 ? 61 : 62) - ex;  // row sums of |c| below 2^62 (2^61: C_1 - C_0)
+            F.coff[p] = 64 - k[p];
+        }
+        for (int i = 0; i < 6; ++i)
+            for (int j = i; j < 6; ++j) {
+                const int64_t a = llrint(ldexp(P.C[0][i * 6 + j], k[0]));
+                const int64_t b = llrint(ldexp(P.C[1][i * 6 + j], k[1]));
+                F.c[0][fix_upper(i, j)] = fix_split(a);
+                F.c[1][fix_upper(i, j)] = fix_split(matkind == 1 ? b - a : b);
+            }
+    }
+    if (!cubic) {
+        double ms = 0.0;
+        for (int i = 0; i < 3; ++i) {
+            ms = fmax(ms, fabs(P.Mmix[i]) + fabs(P.Mmix[3 + i]) + fabs(P.Mmix[6 + i]));
+            ms = fmax(ms, fabs(P.Mmix[3 * i]) + fabs(P.Mmix[3 * i + 1]) + fabs(P.Mmix[3 * i + 2]));
+        }
+        int ex = 0;
+        if (!isfinite(ms)) return false;
+        // sums below 0.98 2^62: the outputs, below 16 x 0.98 2^59, stay clear of the sign bit
+        if (ms > 0 && frexp(ms, &ex) > 0.98) ++ex;
+        F.moff = 2 * (64 - (62 - ex)) - 5;  // both mixings, less the bits their shifts keep
+        for (int e = 0; e < 9; ++e) F.mix[e] = fix_split(llrint(ldexp(P.Mmix[e], 62 - ex)));
+    }
+    for (int p = 0; p < 2; ++p)
+        if (F.coff[p] + F.moff > 100 || F.coff[p] + F.moff < -100) return false;
+    return true;
+}
+
+// Tile extents: least warps over the whole plane with at most kFixCells cells per CTA (ties: the
+// larger tile).  CTAs and planes per CTA: see fix_chunks.
+inline void make_fix_geom(FixGeom& G, int N, bool full) {
+    G.N = N;
+    G.full = full ? 1 : 0;
+    G.X = N / 2;
+    G.Y = N / 2;
+    G.Z = N;
+    G.plane = full ? N * N : G.X * G.Y;
+    G.vstr = G.plane * N;
+    long best = -1;
+    for (int nx = 1; nx <= G.X; ++nx) {
+        const int tx = (G.X + nx - 1) / nx, most = kFixCells / (tx + 1) - 2;
+        if (most < 1) continue;
+        const int ny0 = (G.Y + most - 1) / most;
+        for (int ny = ny0; ny <= G.Y && ny < ny0 + 3; ++ny) {
+            const int ty = (G.Y + ny - 1) / ny;
+            const int cells = (tx + 1) * (ty + 2);
+            const long cost = (long)nx * ny * ((cells + 31) / 32);
+            if (best < 0 || cost < best) {
+                best = cost;
+                G.TX = tx;
+                G.TY = ty;
+                G.ntx = (G.X + tx - 1) / tx;
+                G.nty = (G.Y + ty - 1) / ty;
+                G.ncell = cells;
+            }
+        }
+    }
+    G.tz = G.Z;
+    G.nch = 1;
+}
+
+PC_HD longlong2 fix_ashr2(longlong2 v, int s) {
+    longlong2 r;
+    r.x = v.x >> s;
+    r.y = v.y >> s;
+    return r;
+}
+PC_HD int imax(int a, int b) { return a > b ? a : b; }
+PC_HD int imin(int a, int b) { return a < b ? a : b; }
+
+PC_HD int64_t fix_bits(double v) {
+#if defined(__CUDA_ARCH__)
+    return __double_as_longlong(v);
+#else
+    int64_t b;
+    memcpy(&b, &v, 8);
+    return b;
+#endif
+}
+PC_HD double fix_from_bits(int64_t b) {
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double(b);
+#else
+    double v;
+    memcpy(&v, &b, 8);
+    return v;
+#endif
+}
+PC_HD int fix_clz64(uint64_t v) {
+#if defined(__CUDA_ARCH__)
+    return __clzll((long long)v);
+#else
+    return __builtin_clzll(v);
+#endif
+}
+
+// v as an integer below 2^up (up in 53..63) in units of 2^(E - 1022 - up); base = E, or 64 for E = 0
+// (all values of the node zero).  Bits below the unit are dropped.
+PC_HD int64_t fix_from_double(double v, int base, int lead) {
+    const int64_t b = fix_bits(v);
+    const int hi = (int)(b >> 32);
+    const int e = (hi >> 20) & 0x7ff;
+    const uint64_t m = (((uint64_t)b & 0xfffffffffffffULL) | 0x10000000000000ULL) << lead;
+    const int64_t s = hi >> 31;
+    return ((int64_t)(m >> imin(base - e, 63)) ^ s) - s;
+}
+// largest |high word| of a complex number
+PC_HD int fix_high(double2 v, int m) {
+    m = imax(m, (int)(fix_bits(v.x) >> 32) & 0x7fffffff);
+    return imax(m, (int)(fix_bits(v.y) >> 32) & 0x7fffffff);
+}
+// v 2^(E - 1078), rounded to nearest
+PC_HD double fix_to_double(int64_t v, int E) {
+#if defined(__CUDA_ARCH__)
+    // one conversion on the FP64 pipe, which has room, instead of twenty integer instructions; the
+    // scale goes into the exponent field
+    const double d = __ll2double_rn(v);
+    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (E - 1078) * (1 << 20), __double2loint(d));
+#else
+    const int64_t s = v >> 63;
+    const uint64_t mag = (uint64_t)((v ^ s) - s);
+    if (mag == 0) return 0.0;
+    const int lz = fix_clz64(mag);
+    const uint64_t n = mag << lz;
+    const uint64_t r = (n >> 11) + ((n >> 10) & 1);
+    const uint64_t bits = ((uint64_t)(E + 7 - lz) << 52) + r;
+    return fix_from_bits((int64_t)(bits | ((uint64_t)s & 0x8000000000000000ULL)));
+#endif
+}
+
+// acc + a b.  In PTX on the device: written in C++ the compiler loses sight of the operands being
+// 32 bits wide and multiplies 64 x 64.
+PC_HD void fix_mad(int64_t& acc, int a, int b) {
+#if defined(__CUDA_ARCH__)
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+#else
+    acc += (int64_t)a * b;
+#endif
+}
+// hi 2^64 + mid 2^32 accumulates e c for signed halves
+PC_HD void fix_mac(int64_t& hi, int64_t& mid, FixHalf e, FixHalf c) {
+    fix_mad(hi, e.hi, c.hi);
+    fix_mad(mid, e.hi, c.lo);
+    fix_mad(mid, e.lo, c.hi);
+}
+// the accumulated product over 2^(64 - s), rounded (s in 0..8)
+PC_HD int64_t fix_sum(int64_t hi, int64_t mid, int s) { return (hi << s) + ((mid + (0x80000000LL >> s)) >> (32 - s)); }
+
+// theta in [0, 1] as an integer in units of 2^-62
+PC_HD int64_t fix_theta(float t) {
+#if defined(__CUDA_ARCH__)
+    const uint32_t b = __float_as_uint(t);
+#else
+    uint32_t b;
+    memcpy(&b, &t, 4);
+#endif
+    const int e = (int)(b >> 23);
+    if (e == 0) return 0;
+    const uint64_t m = (uint64_t)((b & 0x7fffffu) | 0x800000u) << 39;
+    return (int64_t)(m >> imin(127 - e, 63));
+}
+
+// MATK: 0 = phase ids, 1 = inclusion fraction, 2 = nodewise material (as SplitApply).
+template <bool CUBIC, int MATK>
+struct FixApply {
+    struct Shared {
+        longlong2* xs;  // [3 slots][3][ncell]
+        longlong2* fs;  // [12][ncell]: F_l of component c at l * 3 + c
+        double2* raw;   // [3][ncell]: the next plane of x, as read
+        double2* ph;    // [27] Bloch phases of the wraps (wa, wb, wk)
+        FixHalf* c;     // [2][21]
+        int* xe;        // [3][ncell]
+        int* fe;        // [ncell]
+    };
+    static inline size_t shared_bytes(const FixGeom& G) {
+        return (size_t)G.ncell * (16 * (9 + 12 + 3) + 4 * 4) + 16 * 27 + sizeof(FixHalf) * 42;
+    }
+    static PC_HD void carve(Shared& sh, unsigned char* p, const FixGeom& G) {
+        const int n = G.ncell;
+        sh.xs = reinterpret_cast<longlong2*>(p);
+        sh.fs = sh.xs + 9 * n;
+        sh.raw = reinterpret_cast<double2*>(sh.fs + 12 * n);
+        sh.ph = sh.raw + 3 * n;
+        sh.c = reinterpret_cast<FixHalf*>(sh.ph + 27);
+        sh.xe = reinterpret_cast<int*>(sh.c + 42);
+        sh.fe = sh.xe + 3 * n;
+    }
+
+    struct Ctx {
+        const FixParams* F;
+        const FixGeom* G;
+        const double (*kph)[2];
+        const double2* x;
+        double2* y;
+        const void* mat;
+        double shift;
+        bool dot;
+        int a0, b0, k0, tz, p12, p13;
+    };
+    struct Regs {
+        int off[2];  // in-plane offset of the cell's node, by plane parity
+        int wab[2];  // (wa + 1) + 3 (wb + 1) of that node
+        int nb[2];   // backward neighbour cells, s2 = +1 low half, -1 high half (flux)
+        int gn[2];   // forward flux cells, s2 = +1 low half, -1 high half (gather)
+        int flags;   // bit 0, 1: flux on even, odd planes; bit 2: output
+        int mprev, mcur, mnext;  // material of planes kf - 1, kf, kf + 1 (id, or the float's bits)
+        longlong2 pv[3], cv[3];  // y(kf - 1) and y(kf) so far
+        int pe, ce;
+        int ks;  // first output plane left to slow_column
+        double2 xo[3];
+        double dot;
+    };
+
+    static PC_HD int wrap1(int v, int n, int& w) {
+        w = v < 0 ? -1 : (v >= n ? 1 : 0);
+        return v - w * n;
+    }
+    // cell of tile coordinates (cx in [0, TX], row r in [-1, TY])
+    static PC_HD int cell_of(const FixGeom& G, int cx, int r) {
+        const int main = G.TX * G.TY;
+        if (r >= 0 && r < G.TY) return cx < G.TX ? r * G.TX + cx : main + r;
+        return main + G.TY + (r < 0 ? G.TX + 1 : 0) + cx;
+    }
+
+    static PC_HD void init(const Ctx& c, int tid, Regs& r) {
+        const FixGeom& G = *c.G;
+        const int main = G.TX * G.TY;
+        int cx, row;
+        if (tid < main) {
+            row = tid / G.TX;
+            cx = tid - row * G.TX;
+        } else if (tid < main + G.TY) {
+            cx = G.TX;
+            row = tid - main;
+        } else {
+            const int e = tid - main - G.TY;
+            row = e > G.TX ? -1 : G.TY;
+            cx = e > G.TX ? e - (G.TX + 1) : e;
+        }
+        r.flags = 0;
+        if (tid < main && c.a0 + cx < G.X && c.b0 + row < G.Y) r.flags |= 4;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i0 = (q + c.p13) & 1, j0 = (q + c.p12 + c.p13) & 1;
+            int wa, wb;
+            const int a = wrap1(c.a0 + ((cx == G.TX && i0) ? -1 : cx), G.X, wa);
+            const int b = wrap1(c.b0 + row, G.Y, wb);
+            r.off[q] = G.full ? (2 * a + i0) + G.N * (2 * b + j0) : a + G.X * b;
+            r.wab[q] = (wa + 1) + 3 * (wb + 1);
+            // fluxes: columns a0 .. a0 + TX - i0, rows b0 - j0 .. b0 + TY - j0
+            const bool f = (cx < G.TX || !i0) && row >= -j0 && row <= G.TY - j0;
+            if (f) r.flags |= 1 << q;
+            r.nb[q] = 0;
+            if (f) {
+                const int ncx = i0 ? cx : (cx > 0 ? cx - 1 : G.TX);
+                r.nb[q] = cell_of(G, ncx, row + j0 - 1) | (cell_of(G, ncx, row + j0) << 16);
+            }
+            r.gn[q] = 0;
+            if (tid < main) r.gn[q] = cell_of(G, cx + i0, row + j0) | (cell_of(G, cx + i0, row + j0 - 1) << 16);
+        }
+        r.pe = r.ce = 0;
+        r.ks = 1 << 30;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            r.pv[a].x = r.pv[a].y = r.cv[a].x = r.cv[a].y = 0;
+            r.xo[a] = czero(0.0);
+        }
+        r.dot = 0.0;
+        r.mprev = r.mcur = r.mnext = 0;
+    }
+
+    static PC_HD void load_tables(const Ctx& c, Shared& sh, int tid, int nthr) {
+        for (int i = tid; i < 42; i += nthr) sh.c[i] = c.F->c[i / 21][i % 21];
+        for (int i = tid; i < 27; i += nthr) {
+            const int w[3] = {i % 3 - 1, (i / 3) % 3 - 1, i / 9 - 1};
+            double2 e = cmk(1.0, 0.0);
+            for (int l = 0; l < 3; ++l)
+                if (w[l] != 0) e = cmul(e, cmk(c.kph[l][0], w[l] < 0 ? -c.kph[l][1] : c.kph[l][1]));
+            sh.ph[i] = e;
+        }
+    }
+
+    // Start the copy of plane kp of x into the staging cells (a cell is read by its own thread only).
+    static PC_HD void stage(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp) {
+        const FixGeom& G = *c.G;
+        int wk;
+        const int k = wrap1(kp, G.Z, wk);
+        const int at = k * G.plane + ((kp & 1) ? r.off[1] : r.off[0]);
+        PC_IDX(at, G.vstr);
+        PC_IDX(tid, G.ncell);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double2* d = sh.raw + a * G.ncell + tid;
+            const double2* s = c.x + at + (int64_t)a * G.vstr;
+#if defined(__CUDA_ARCH__)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(s)
+                         : "memory");
+#else
+            *d = *s;
+#endif
+        }
+    }
+
+    // Plane kp from the staging cells into slot sl: phase, exponent, integers.
+    static PC_HD void convert(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp, int sl) {
+        const FixGeom& G = *c.G;
+        int wk;
+        wrap1(kp, G.Z, wk);
+        const int w = ((kp & 1) ? r.wab[1] : r.wab[0]) + 9 * (wk + 1);
+        double2 v[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a] = sh.raw[a * G.ncell + tid];
+        if (w != 13) {
+            const double2 ph = sh.ph[w];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) v[a] = cmul(v[a], ph);
+        }
+        const int top = fix_high(v[2], fix_high(v[1], fix_high(v[0], 0)));
+        int E = top >> 20, base = E;
+        if (E < kFixLow || E > kFixHigh) {
+            int64_t any = 0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) any |= (fix_bits(v[a].x) | fix_bits(v[a].y)) & 0x7fffffffffffffffLL;
+            base = 64;
+            E = any ? kFixSpecial : 0;
+        }
+        longlong2* xs = sh.xs + (int64_t)sl * 3 * G.ncell + tid;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            longlong2 o;
+            o.x = E == 0 ? 0 : fix_from_double(v[a].x, base, 3);
+            o.y = E == 0 ? 0 : fix_from_double(v[a].y, base, 3);
+            xs[a * G.ncell] = o;
+        }
+        sh.xe[sl * G.ncell + tid] = E;
+    }
+
+    static PC_HD int read_mat(const Ctx& c, const Regs& r, int kp) {
+        if (MATK == 2) return 0;
+        const FixGeom& G = *c.G;
+        int wk;
+        const int k = wrap1(kp, G.Z, wk);
+        const int at = k * G.plane + ((kp & 1) ? r.off[1] : r.off[0]);
+        PC_IDX(at, G.vstr);
+        if (MATK == 0) return static_cast<const uint8_t*>(c.mat)[at];
+#if defined(__CUDA_ARCH__)
+        return __float_as_int(static_cast<const float*>(c.mat)[at]);
+#else
+        int b;
+        memcpy(&b, static_cast<const float*>(c.mat) + at, 4);
+        return b;
+#endif
+    }
+    static PC_HD float mat_theta(int b) {
+#if defined(__CUDA_ARCH__)
+        return __int_as_float(b);
+#else
+        float f;
+        memcpy(&f, &b, 4);
+        return f;
+#endif
+    }
+
+    template <bool ORTHO>
+    static PC_HD void stress(const FixHalf* C, const FixHalf* ex, const FixHalf* ey, longlong2* t) {
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+            int64_t hx = 0, hy = 0, mx = 0, my = 0;
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                if (ORTHO && !((p < 3 && u < 3) || p == u)) continue;
+                const FixHalf cc = C[fix_upper(p, u)];
+                fix_mac(hx, mx, ex[u], cc);
+                fix_mac(hy, my, ey[u], cc);
+            }
+            t[p].x = fix_sum(hx, mx, CUBIC ? 0 : 2);
+            t[p].y = fix_sum(hy, my, CUBIC ? 0 : 2);
+        }
+    }
+
+    // Fluxes of plane kf at the thread's column; -4 P_0 into y(kf).  sm, sc, sp: slots of planes
+    // kf - 1, kf, kf + 1.
+    static PC_HD void flux(const Ctx& c, Shared& sh, Regs& r, int tid, int kf, int sm, int sc, int sp) {
+        const FixGeom& G = *c.G;
+        const int q = kf & 1, n = G.ncell;
+        if (!((r.flags >> q) & 1)) return;
+        const int nb = q ? r.nb[1] : r.nb[0];
+        const int n0 = nb & 0xffff, n1 = nb >> 16;
+        PC_IDX(n0, n);
+        PC_IDX(n1, n);
+        const int eo = sh.xe[sc * n + tid];
+        const int e0 = sh.xe[sm * n + n0], e1 = sh.xe[sp * n + n0], e2 = sh.xe[sm * n + n1], e3 = sh.xe[sp * n + n1];
+        const int E = imax(imax(imax(e0, e1), imax(e2, e3)), eo);
+        if (E >= kFixSpecial) {
+            sh.fe[tid] = kFixSpecial;
+            r.ce = kFixSpecial;
+            return;
+        }
+        const int s0 = imin(E - e0, 63), s1 = imin(E - e1, 63), s2 = imin(E - e2, 63), s3 = imin(E - e3, 63),
+                  so = imin(E - eo, 63);
+        longlong2 H[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const longlong2 v0 = fix_ashr2(sh.xs[(sm * 3 + a) * n + n0], s0), v1 = fix_ashr2(sh.xs[(sp * 3 + a) * n + n0], s1);
+            const longlong2 v2 = fix_ashr2(sh.xs[(sm * 3 + a) * n + n1], s2), v3 = fix_ashr2(sh.xs[(sp * 3 + a) * n + n1], s3);
+            const longlong2 vo = fix_ashr2(sh.xs[(sc * 3 + a) * n + tid], so);
+            const int64_t ux = v0.x + v1.x, uy = v0.y + v1.y, vx = v2.x + v3.x, vy = v2.y + v3.y;
+            H[0][a].x = ux + vx - 4 * vo.x;
+            H[0][a].y = uy + vy - 4 * vo.y;
+            H[1][a].x = ux - vx;
+            H[1][a].y = uy - vy;
+            H[2][a].x = (v0.x - v1.x) + (v2.x - v3.x);
+            H[2][a].y = (v0.y - v1.y) + (v2.y - v3.y);
+        }
+        int up = 0;
+        if (!CUBIC || MATK != 0) {
+            // more roundings follow than in the plain case: scale the sums up to their bound first
+            int top = 0;
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    top |= (int)((H[m][a].x ^ (H[m][a].x >> 63)) >> 32) | (int)((H[m][a].y ^ (H[m][a].y >> 63)) >> 32);
+            up = fix_clz64((uint64_t)(uint32_t)top | 1) - 32 - 5;
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    H[m][a].x <<= up;
+                    H[m][a].y <<= up;
+                }
+        }
+        if (!CUBIC) mix3(c, H, false);
+        // strain halves: xx, yy, zz, yz, xz, xy (real and imaginary parts)
+        FixHalf ex[6], ey[6];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            ex[p] = fix_split(H[p][p].x);
+            ey[p] = fix_split(H[p][p].y);
+            const int u = p == 0 ? 1 : 0, v = p == 2 ? 1 : 2;
+            ex[3 + p] = fix_split(H[v][u].x + H[u][v].x);
+            ey[3 + p] = fix_split(H[v][u].y + H[u][v].y);
+        }
+        longlong2 t[6];
+        int fe = E - up + c.F->moff;
+        if (MATK == 0) {
+            const int ph = r.mcur != 0 ? 1 : 0;
+            const FixHalf* C = sh.c + 21 * ph;
+            fe += ph ? c.F->coff[1] : c.F->coff[0];
+            // every node of the warp orthotropic: normal block and shear diagonal only
+            if (warp_all(c.F->P.ortho[ph] != 0)) stress<true>(C, ex, ey, t);
+            else stress<false>(C, ex, ey, t);
+        } else {
+            int64_t hx[6], hy[6], mx[6], my[6];
+#pragma unroll
+            for (int p = 0; p < 6; ++p) {
+                hx[p] = hy[p] = 0;
+                mx[p] = my[p] = 0;
+            }
+            int row[6] = {0, 0, 0, 0, 0, 0};  // row sums of |c| / 2^32
+            FixHalf th = {0, 0};
+            const double* md = nullptr;
+            int base = 64;
+            if (MATK == 1) {
+                th = fix_split(fix_theta(mat_theta(r.mcur)));
+                fe += c.F->coff[0];
+            } else {
+                int wk;
+                const int at = wrap1(kf, G.Z, wk) * G.plane + (q ? r.off[1] : r.off[0]);
+                md = static_cast<const double*>(c.mat) + at;
+                int top = 0;
+#pragma unroll
+                for (int u = 0; u < 21; ++u) top = imax(top, (int)(fix_bits(md[(int64_t)u * G.vstr]) >> 32) & 0x7fffffff);
+                base = top >> 20;  // entries below 2^59: row sums below 2^62
+                fe += base - 1017;
+                if (base < 950 || base > 1100) {  // tables far outside hat units
+                    sh.fe[tid] = kFixSpecial;
+                    r.ce = kFixSpecial;
+                    return;
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < 6; ++p)
+#pragma unroll
+                for (int u = p; u < 6; ++u) {
+                    FixHalf cc;
+                    if (MATK == 1) {  // c = C_0 + theta (C_1 - C_0)
+                        int64_t h = 0, m = 1LL << 29;
+                        const FixHalf d = sh.c[21 + fix_upper(p, u)], z = sh.c[fix_upper(p, u)];
+                        fix_mac(h, m, th, d);
+                        cc = fix_split((int64_t)z.hi * 0x100000000LL + z.lo + h * 4 + (m >> 30));
+                    } else {
+                        cc = fix_split(fix_from_double(md[(int64_t)fix_upper(p, u) * G.vstr], base, 6));
+                    }
+                    const int ab = cc.hi < 0 ? -cc.hi : cc.hi;
+                    row[p] += ab;
+                    fix_mac(hx[p], mx[p], ex[u], cc);
+                    fix_mac(hy[p], my[p], ey[u], cc);
+                    if (u != p) {
+                        row[u] += ab;
+                        fix_mac(hx[u], mx[u], ex[p], cc);
+                        fix_mac(hy[u], my[u], ey[p], cc);
+                    }
+                }
+            // the node's own row sums are below the bound the scale allows for: keep that many more bits
+            const int top = imax(imax(imax(row[0], row[1]), imax(row[2], row[3])), imax(row[4], row[5])) + 6;
+            int sh2 = (top < (1 << 24) ? 6 : top < (1 << 25) ? 5 : top < (1 << 26) ? 4 : top < (1 << 27) ? 3
+                       : top < (1 << 28) ? 2 : top < (1 << 29) ? 1 : 0);
+            fe -= sh2;
+            sh2 += CUBIC ? 0 : 2;
+#pragma unroll
+            for (int p = 0; p < 6; ++p) {
+                t[p].x = fix_sum(hx[p], mx[p], sh2);
+                t[p].y = fix_sum(hy[p], my[p], sh2);
+            }
+        }
+        if (E == 0) fe = 0;  // zero fluxes
+        sh.fe[tid] = fe;
+        // P_s (s, component)
+        longlong2 Q[3][3];
+        Q[0][0] = t[0];
+        Q[1][1] = t[1];
+        Q[2][2] = t[2];
+        Q[0][1] = Q[1][0] = t[5];
+        Q[0][2] = Q[2][0] = t[4];
+        Q[1][2] = Q[2][1] = t[3];
+        if (!CUBIC) mix3(c, Q, true);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            longlong2 f;
+            const int64_t ux = Q[0][a].x + Q[1][a].x, uy = Q[0][a].y + Q[1][a].y;
+            const int64_t vx = Q[0][a].x - Q[1][a].x, vy = Q[0][a].y - Q[1][a].y;
+            f.x = ux + Q[2][a].x;
+            f.y = uy + Q[2][a].y;
+            sh.fs[(0 + a) * n + tid] = f;
+            f.x = ux - Q[2][a].x;
+            f.y = uy - Q[2][a].y;
+            sh.fs[(3 + a) * n + tid] = f;
+            f.x = vx + Q[2][a].x;
+            f.y = vy + Q[2][a].y;
+            sh.fs[(6 + a) * n + tid] = f;
+            f.x = vx - Q[2][a].x;
+            f.y = vy - Q[2][a].y;
+            sh.fs[(9 + a) * n + tid] = f;
+        }
+        if (r.flags & 4) {
+            const int m = imax(r.ce, fe);
+            const int sa = imin(m - r.ce, 63), sf = imin(m - fe, 63);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                r.cv[a].x = (r.cv[a].x >> sa) - 4 * (Q[0][a].x >> sf);
+                r.cv[a].y = (r.cv[a].y >> sa) - 4 * (Q[0][a].y >> sf);
+            }
+            r.ce = m;
+        }
+    }
+
+    // Rows of a 3 x 3 complex table through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or
+    // (transposed) out[s] = sum_m Mmix[s][m] in[m].
+    static PC_HD void mix3(const Ctx& c, longlong2 (*V)[3], bool rows) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            FixHalf vx[3], vy[3];
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                vx[s] = fix_split(V[s][a].x);
+                vy[s] = fix_split(V[s][a].y);
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                int64_t hx = 0, hy = 0, mx = 0, my = 0;
+#pragma unroll
+                for (int s = 0; s < 3; ++s) {
+                    const FixHalf w = c.F->mix[rows ? m * 3 + s : s * 3 + m];
+                    fix_mac(hx, mx, vx[s], w);
+                    fix_mac(hy, my, vy[s], w);
+                }
+                V[m][a].x = fix_sum(hx, mx, rows ? 1 : 2);
+                V[m][a].y = fix_sum(hy, my, rows ? 1 : 2);
+            }
+        }
+    }
+
+    // The node's own x of plane kf - 1, for the shift term and the inner product.
+    static PC_HD void load_own(const Ctx& c, Regs& r, int kf) {
+        const int k = kf - 1;
+        if (!(r.flags & 4) || k < c.k0) return;
+        const int at = k * c.G->plane + ((k & 1) ? r.off[1] : r.off[0]);
+        PC_IDX(at, c.G->vstr);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r.xo[a] = (c.x + at)[(int64_t)a * c.G->vstr];
+    }
+
+    // Outputs y(kf - 1); y(kf) moves on; y(kf + 1) starts with F_1, F_3 of plane kf.
+    static PC_HD void gather(const Ctx& c, Shared& sh, Regs& r, int kf) {
+        const FixGeom& G = *c.G;
+        if (!(r.flags & 4)) return;
+        const int n = G.ncell, k = kf - 1, q = k & 1;  // planes kf - 1 and kf + 1 share the offsets
+        const int gn = q ? r.gn[1] : r.gn[0];
+        const int c0 = gn & 0xffff, c1 = gn >> 16;
+        PC_IDX(c0, n);
+        PC_IDX(c1, n);
+        const int f0 = sh.fe[c0], f1 = sh.fe[c1];
+        if (k >= c.k0) {
+            const int at = k * G.plane + (q ? r.off[1] : r.off[0]);
+            const int E = imax(r.pe, imax(f0, f1));
+            if (E >= kFixSpecial && r.ks > k) r.ks = k;
+            if (k < r.ks) {
+                const double sr = c.shift * density(c, r.mprev, at);
+                const int sa = imin(E - r.pe, 63), s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const longlong2 g0 = sh.fs[a * n + c0], g1 = sh.fs[(6 + a) * n + c1];
+                    double2 w;
+                    w.x = fix_to_double((r.pv[a].x >> sa) + (g0.x >> s0) + (g1.x >> s1), E);
+                    w.y = fix_to_double((r.pv[a].y >> sa) + (g0.y >> s0) + (g1.y >> s1), E);
+                    w = cfma(-sr, r.xo[a], w);
+                    (c.y + at)[(int64_t)a * G.vstr] = w;
+                    if (c.dot) r.dot = cdotre(r.xo[a], w, r.dot);
+                }
+            }
+        }
+        const int E = imax(f0, f1);
+        r.pe = r.ce;
+        r.ce = E;
+        const int s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            r.pv[a] = r.cv[a];
+            const longlong2 g0 = sh.fs[(3 + a) * n + c0], g1 = sh.fs[(9 + a) * n + c1];
+            r.cv[a].x = (g0.x >> s0) + (g1.x >> s1);
+            r.cv[a].y = (g0.y >> s0) + (g1.y >> s1);
+        }
+    }
+
+    static PC_HD double density(const Ctx& c, int m, int at) {
+        const StencilParams<double>& P = c.F->P;
+        if (MATK == 0) return P.rho[m != 0 ? 1 : 0];
+        if (MATK == 1) return P.rho[0] + (double)mat_theta(m) * (P.rho[1] - P.rho[0]);
+        return static_cast<const double*>(c.mat)[21LL * c.G->vstr + at];
+    }
+
+    static PC_HD void next_mat(Regs& r) {
+        r.mprev = r.mcur;
+        r.mcur = r.mnext;
+    }
+
+    // Fluxes at node (a, b, k) of the block in FP64 (coordinates inside the grid).
+    static __host__ __device__ void slow_flux(const Ctx& c, int a, int b, int k, double2 (*Fo)[3]) {
+        const FixGeom& G = *c.G;
+        const StencilParams<double>& P = c.F->P;
+        auto addr = [&](int aa, int bb, int kk) -> int64_t {
+            const int i0 = (kk + c.p13) & 1, j0 = (kk + c.p12 + c.p13) & 1;
+            return (int64_t)kk * G.plane + (G.full ? (2 * aa + i0) + (int64_t)G.N * (2 * bb + j0) : aa + (int64_t)G.X * bb);
+        };
+        const int64_t at = addr(a, b, k);
+        const int i0 = (k + c.p13) & 1, j0 = (k + c.p12 + c.p13) & 1;
+        double2 H[3][3];
+        for (int al = 0; al < 3; ++al) {
+            double2 nv[4];
+            for (int l = 0; l < 4; ++l) {
+                const int s2 = (l < 2) ? 1 : -1, s3 = (l & 1) ? -1 : 1;
+                int w[3];
+                const int na = wrap1(a + i0 - 1, G.X, w[0]), nbb = wrap1(b + j0 - ((s2 + 1) >> 1), G.Y, w[1]),
+                          nk = wrap1(k - s3, G.Z, w[2]);
+                nv[l] = c.x[(int64_t)al * G.vstr + addr(na, nbb, nk)];
+                if (w[0] | w[1] | w[2]) {
+                    double2 ph = cmk(1.0, 0.0);
+                    for (int d = 0; d < 3; ++d)
+                        if (w[d] != 0) ph = cmul(ph, cmk(c.kph[d][0], w[d] < 0 ? -c.kph[d][1] : c.kph[d][1]));
+                    nv[l] = cmul(nv[l], ph);
+                }
+            }
+            const double2 u = cadd(nv[0], nv[1]), v = cadd(nv[2], nv[3]);
+            H[0][al] = cfma(-4.0, c.x[(int64_t)al * G.vstr + at], cadd(u, v));
+            H[1][al] = csub(u, v);
+            H[2][al] = cadd(csub(nv[0], nv[1]), csub(nv[2], nv[3]));
+        }
+        double2 Gm[3][3];
+        for (int m = 0; m < 3; ++m)
+            for (int al = 0; al < 3; ++al) {
+                if (CUBIC) {
+                    Gm[m][al] = H[m][al];
+                } else {
+                    double2 acc = cscale(P.Mmix[m], H[0][al]);
+                    acc = cfma(P.Mmix[3 + m], H[1][al], acc);
+                    Gm[m][al] = cfma(P.Mmix[6 + m], H[2][al], acc);
+                }
+            }
+        const double2 e[6] = {Gm[0][0], Gm[1][1], Gm[2][2], cadd(Gm[2][1], Gm[1][2]), cadd(Gm[2][0], Gm[0][2]),
+                              cadd(Gm[1][0], Gm[0][1])};
+        double2 t[6];
+        int ph = 0;
+        double th = 0.0;
+        if (MATK == 0) ph = static_cast<const uint8_t*>(c.mat)[at] != 0 ? 1 : 0;
+        if (MATK == 1) th = (double)static_cast<const float*>(c.mat)[at];
+        for (int p = 0; p < 6; ++p) {
+            double2 acc = czero(0.0);
+            bool first = true;
+            for (int u = 0; u < 6; ++u) {
+                double cc;
+                if (MATK == 0) {
+                    if (P.ortho[ph] && !((p < 3 && u < 3) || p == u)) continue;  // structural zeros
+                    cc = P.C[ph][p * 6 + u];
+                } else if (MATK == 1) {
+                    cc = P.C[0][p * 6 + u] + th * (P.C[1][p * 6 + u] - P.C[0][p * 6 + u]);
+                } else {
+                    cc = static_cast<const double*>(c.mat)[(int64_t)fix_upper(p, u) * G.vstr + at];
+                }
+                acc = first ? cscale(cc, e[u]) : cfma(cc, e[u], acc);
+                first = false;
+            }
+            t[p] = acc;
+        }
+        const double2 S[3][3] = {{t[0], t[5], t[4]}, {t[5], t[1], t[3]}, {t[4], t[3], t[2]}};
+        for (int al = 0; al < 3; ++al) {
+            double2 Pm[3];
+            for (int s = 0; s < 3; ++s) {
+                if (CUBIC) {
+                    Pm[s] = S[al][s];
+                } else {
+                    double2 acc = cscale(P.Mmix[s * 3], S[al][0]);
+                    acc = cfma(P.Mmix[s * 3 + 1], S[al][1], acc);
+                    Pm[s] = cfma(P.Mmix[s * 3 + 2], S[al][2], acc);
+                }
+            }
+            const double2 u = cadd(Pm[0], Pm[1]), v = csub(Pm[0], Pm[1]);
+            Fo[0][al] = cadd(u, Pm[2]);
+            Fo[1][al] = csub(u, Pm[2]);
+            Fo[2][al] = cadd(v, Pm[2]);
+            Fo[3][al] = csub(v, Pm[2]);
+            Fo[4][al] = Pm[0];
+        }
+    }
+
+    // Outputs of the thread's column from plane k to the end of the chunk in FP64, from x itself:
+    // the first node whose values leave the integer path's range hands its column over.  Rare, so
+    // its speed does not matter; after the march and not inlined, so that it costs the march no
+    // registers.  Returns the column's part of Re<x, y>.
+    static __host__ __device__ PC_FIX_COLD double slow_column(const Ctx& c, int k, int off0, int off1) {
+        const FixGeom& G = *c.G;
+        double dot = 0.0;
+        for (; k < c.k0 + c.tz; ++k) {
+            const int off = (k & 1) ? off1 : off0;
+            const int i0 = (k + c.p13) & 1, j0 = (k + c.p12 + c.p13) & 1;
+            const int a = G.full ? (off % G.N - i0) >> 1 : off % G.X, b = G.full ? (off / G.N - j0) >> 1 : off / G.X;
+            const int64_t at = (int64_t)k * G.plane + off;
+            PC_IDX(at, G.vstr);
+            double2 F[5][3], own[3], g[4][3];
+            slow_flux(c, a, b, k, F);
+            for (int al = 0; al < 3; ++al) own[al] = F[4][al];
+            for (int l = 0; l < 4; ++l) {
+                const int s2 = (l < 2) ? 1 : -1, s3 = (l & 1) ? -1 : 1;
+                int w[3];
+                const int na = wrap1(a + i0, G.X, w[0]), nb = wrap1(b + j0 + ((s2 - 1) >> 1), G.Y, w[1]),
+                          nk = wrap1(k + s3, G.Z, w[2]);
+                slow_flux(c, na, nb, nk, F);
+                double2 ph = cmk(1.0, 0.0);
+                for (int d = 0; d < 3; ++d)
+                    if (w[d] != 0) ph = cmul(ph, cmk(c.kph[d][0], w[d] < 0 ? -c.kph[d][1] : c.kph[d][1]));
+                for (int al = 0; al < 3; ++al) g[l][al] = (w[0] | w[1] | w[2]) ? cmul(F[l][al], ph) : F[l][al];
+            }
+            double rho;
+            if (MATK == 0) rho = c.F->P.rho[static_cast<const uint8_t*>(c.mat)[at] != 0 ? 1 : 0];
+            else if (MATK == 1)
+                rho = c.F->P.rho[0] + (double)static_cast<const float*>(c.mat)[at] * (c.F->P.rho[1] - c.F->P.rho[0]);
+            else rho = static_cast<const double*>(c.mat)[21LL * G.vstr + at];
+            for (int al = 0; al < 3; ++al) {
+                const double2 xv = c.x[(int64_t)al * G.vstr + at];
+                double2 w = cfma(-4.0, own[al], cadd(cadd(g[0][al], g[1][al]), cadd(g[2][al], g[3][al])));
+                w = cfma(-(c.shift * rho), xv, w);
+                c.y[(int64_t)al * G.vstr + at] = w;
+                dot = cdotre(xv, w, dot);
+            }
+        }
+        return dot;
+    }
+};
+
+}  // namespace pc

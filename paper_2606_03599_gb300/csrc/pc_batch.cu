@@ -43,6 +43,7 @@ extern "C" int pc_grid_clone(const pc_grid* src, pc_grid** out) {
     std::memcpy(g->Ainv, src->Ainv, sizeof(g->Ainv));
     g->cubic = src->cubic;
     g->matkind = src->matkind;
+    g->int_ok = src->int_ok;
     g->mean_theta = src->mean_theta;
     g->sigma_cmax = src->sigma_cmax;
     g->sigma_rmax = src->sigma_rmax;

@@ -94,6 +94,13 @@ int launch_apply_split_f64(bool full, bool cubic, int matkind, const StencilPara
 int launch_apply_split_f32(bool full, bool cubic, int matkind, const StencilParams<float>& P, const ApplyItem* items,
                            const double* item_ph, int nitems, void* scratch, size_t scratch_bytes, double* dp, int ds,
                            cudaStream_t s);
+// Integer-pipe complex128 apply (block floating point, no scratch; every item its own Bloch phases):
+// tz planes per CTA; fix_apply_ctas gives the CTAs per item of the default chunking (tz_in 0) or of
+// tz_in planes, and the planes in *tz.  fix_apply_ok: the material's scale is within its range.
+int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<double>& P, const ApplyItem* items,
+                     const double* item_ph, int nitems, int tz, double* dp, int ds, cudaStream_t s);
+int fix_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz);
+bool fix_apply_ok(const StencilParams<double>& P, bool cubic, int matkind);
 size_t split_scratch_bytes(int X, int Y, int Z, int nitems, int dtype);
 int split_apply_ctas(int64_t m);
 
@@ -105,14 +112,17 @@ struct ApplyConfig {
     bool row = false;  // row-tile kernel (complex64 parity blocks, X even)
     bool split = false;  // two-pass complex128 kernels (flux, then gather)
     bool pipe = false;   // plane-pipelined kernel (complex64 parity blocks, even X)
+    bool fix = false;    // integer-pipe complex128 kernel (shape code kFixShape)
 };
+constexpr int kFixShape = 8;
 // Kind code of a configuration as pc_tuned_config reports it.
 inline int config_kind(const ApplyConfig& c) {
     return c.pipe ? 4 : (c.split ? 3 : (c.row ? 2 : (c.tma ? 1 : 0)));
 }
-// scratch_ok = false: only kernels that need no scratch memory of their own (no two-pass apply).
+// scratch_ok = false: only kernels that need no scratch memory of their own (no two-pass apply);
+// int_ok: the integer-pipe complex128 kernel may be chosen.
 ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks = false, int matkind = 0,
-                                bool scratch_ok = true);
+                                bool scratch_ok = true, bool int_ok = false);
 // Launch configuration for a grid layout: the autotuned one when present, else the heuristic.
 ApplyConfig apply_config_for(const pc_grid* g, bool full, int nitems, int dtype);
 bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool cubic, int nitems, ApplyConfig* out);
@@ -219,6 +229,7 @@ struct pc_grid {
     double rhohat[2];
     double Ainv[9];  // (A_hat^-1)_{s m}, row-major s*3+m
     bool cubic = true;
+    bool int_ok = false;  // the integer-pipe complex128 apply can take this material
     int matkind = 0;  // 0 = uint8 phase ids, 1 = float theta, 2 = nodewise ([22][m] FP64)
     double sigma_cmax = 0.0, sigma_rmax = 0.0;  // largest |C| entry and density (hat units): default shift
     double mean_theta = 0.0;  // volume fraction of phase 1

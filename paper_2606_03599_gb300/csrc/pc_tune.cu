@@ -77,6 +77,7 @@ void load_locked() {
         c.row = kind == 2;
         c.split = kind == 3;
         c.pipe = kind == 4;
+        c.fix = kind == 0 && shape == kFixShape;
         g_tuned[key] = c;
     }
 }
@@ -99,7 +100,9 @@ bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool c
     if (it == g_tuned.end()) return false;
     *out = it->second;
     // a tuned chunking for a bucket is reused for every batch size in it: recount the CTAs
-    if (out->split) {
+    if (out->fix) {
+        out->ctas = fix_apply_ctas(Z, full, nitems, out->tz, nullptr);
+    } else if (out->split) {
         out->ctas = split_apply_ctas((int64_t)X * Y * Z);
     } else if (out->pipe) {
         out->ctas = pipe_apply_ctas(X, Y, Z, matkind, nitems, out->tz);
@@ -116,8 +119,9 @@ bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool c
 ApplyConfig apply_config_for(const pc_grid* g, bool full, int nitems, int dtype) {
     const int X = full ? g->N : g->X, Y = full ? g->N : g->Y, Z = g->Z;
     ApplyConfig c;
-    if (tuned_config(X, Y, Z, dtype, full, g->matkind, g->cubic, nitems, &c)) return c;
-    return choose_apply_config(X, Y, Z, nitems, dtype, !full, g->matkind);
+    if (tuned_config(X, Y, Z, dtype, full, g->matkind, g->cubic, nitems, &c) && !(c.fix && !g->int_ok)) return c;
+    c = ApplyConfig();
+    return choose_apply_config(X, Y, Z, nitems, dtype, !full, g->matkind, true, g->int_ok);
 }
 
 // Time one candidate on scratch vectors: after two warm-up launches, the best of three
@@ -141,8 +145,16 @@ static int time_candidate(pc_grid* g, int dtype, bool full, std::vector<ApplyIte
     return PC_OK;
 }
 
-static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool full, int matkind, int nitems) {
+static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool full, int matkind, int nitems,
+                                           bool int_ok) {
     std::vector<ApplyConfig> out;
+    if (int_ok && dtype == PC_C128) {  // integer-pipe kernel: the default chunking
+        ApplyConfig c;
+        c.fix = true;
+        c.shape = kFixShape;
+        c.ctas = fix_apply_ctas(Z, full, nitems, 0, &c.tz);
+        out.push_back(c);
+    }
     const int sm = device_sm_count();
     // two-pass kernels: the default for complex128; for complex64 a candidate while the batch's
     // scratch (15 complex64 flux arrays per extended cell plus x's ghost cells) fits in L2
@@ -175,7 +187,7 @@ static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool 
         base.tz = (int)((Z + nch - 1) / nch);
         base.ctas = tiles * ((Z + base.tz - 1) / base.tz);
         for (auto& o : out)
-            if (!o.pipe && o.row == base.row && o.tma == base.tma && o.shape == base.shape && o.tz == base.tz) return;
+            if (!o.pipe && !o.fix && o.row == base.row && o.tma == base.tma && o.shape == base.shape && o.tz == base.tz) return;
         out.push_back(base);
     };
     if (!full && dtype == PC_C64 && pipe_geom_ok(X, Y, Z, matkind)) {
@@ -261,13 +273,13 @@ int autotune_layout(pc_grid* g, int dtype, bool full, int nitems, cudaStream_t s
     int rc = PC_OK;
     const bool was_timing = timing_enabled();
     if (was_timing) pc_stats_timing(0);  // candidate launches stay out of the apply statistics
-    for (const ApplyConfig& c : candidates(X, Y, Z, dtype, full, g->matkind, n)) {
+    for (const ApplyConfig& c : candidates(X, Y, Z, dtype, full, g->matkind, n, g->int_ok)) {
         double us = 0;
         rc = time_candidate(g, dtype, full, items, c, s, e0, e1, &us);
         if (rc != PC_OK) break;
         if (verbose)
             std::fprintf(stderr, "[pcband tune] %s kind=%s shape=%d tz=%d ctas=%d: %.1f us\n", key.c_str(),
-                         c.pipe ? "pipe" : (c.split ? "split" : (c.row ? "row" : (c.tma ? "tma" : "regs"))), c.shape,
+                         c.fix ? "int" : c.pipe ? "pipe" : (c.split ? "split" : (c.row ? "row" : (c.tma ? "tma" : "regs"))), c.shape,
                          c.tz, c.ctas, us);
         if (us < best_us) {
             best_us = us;

@@ -1,0 +1,123 @@
+"""The integer-pipe complex128 apply (host emulation of its per-thread functions) against the
+two-pass FP64 apply, over the forms both accept (CPU only).
+
+Tolerance: both sides round at most about 60 times in a chain, and a unit roundoff is 2^-53, so
+two correct results differ by at most 2 * 60 * 2^-53 = 1.4e-14 of the output's norm on broad-band
+vectors.
+"""
+
+import ctypes
+import importlib.util
+import os
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from workloads import complex_gaussian, two_phase_sphere
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+TOL = 1.4e-14
+TWO_PASS, INT = 30, 60
+LATTICES = {"cubic": np.eye(3), "fcc": 0.5 * (np.ones((3, 3)) - np.eye(3)),
+            "skew": np.array([[1.0, 0.2, -0.1], [0.0, 0.9, 0.3], [0.1, 0.0, 1.2]])}
+
+
+@pytest.fixture(scope="module")
+def emu():
+    spec = importlib.util.spec_from_file_location(
+        "pcband_build", os.path.join(ROOT, "paper_2606_03599_gb300", "build.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    lib = ctypes.CDLL(mod.build_emulator())
+    dp = ctypes.POINTER(ctypes.c_double)
+    lib.pc_emu_apply.argtypes = [ctypes.c_int] * 5 + [dp, dp, dp, ctypes.c_int, dp, ctypes.c_void_p,
+                                                      ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
+                                                      ctypes.c_double]
+    lib.pc_emu_apply.restype = ctypes.c_int
+    return lib
+
+
+def both(lib, N, block, lattice, matkind, x, tilings, kappa=(0.21, -0.33, 0.4), shift=0.7):
+    """The two-pass result and the integer kernel's for each (shape, tz) of `tilings`."""
+    rng = np.random.default_rng(N + matkind)
+    n = N ** 3
+    cell = two_phase_sphere(N, 0.35, 3)
+    A = LATTICES[lattice]
+    ainv = np.ascontiguousarray(np.linalg.inv(A / abs(np.linalg.det(A)) ** (1 / 3)))
+    idx = np.arange(n) if block < 0 else O.block_index((N,) * 3, block)
+    C, rho = cell.C / 1e9, cell.rho / 1e3
+    if matkind == 2:
+        iu = np.triu_indices(6)
+        G = rng.standard_normal((n, 6, 6))
+        Cn = C[cell.phase.astype(int)] + 0.1 * (G + np.transpose(G, (0, 2, 1)))
+        q2 = (N / 4.0) ** 2 if lattice == "cubic" else 1.0
+        lay = np.concatenate([Cn[:, iu[0], iu[1]].T * q2, rng.uniform(1, 8, (1, n))], axis=0)
+        mat = np.ascontiguousarray(lay[:, idx])
+    elif matkind == 1:
+        mat = rng.uniform(0, 1, n).astype(np.float32)
+        mat[:2] = [0.0, 1.0]
+        mat = np.ascontiguousarray(mat[idx])
+    else:
+        mat = np.ascontiguousarray(cell.phase[idx])
+    dp = ctypes.POINTER(ctypes.c_double)
+    C72 = np.ascontiguousarray(C.reshape(72))
+    phi = np.ascontiguousarray(2 * np.pi * (np.asarray(kappa) - np.floor(kappa)))
+    x = np.ascontiguousarray(x[:, idx])
+    out = []
+    for shape, tz in [(TWO_PASS, 0)] + list(tilings):
+        y = np.full_like(x, np.nan)
+        assert lib.pc_emu_apply(N, block, 2, shape, tz, C72.ctypes.data_as(dp), rho.ctypes.data_as(dp),
+                                ainv.ctypes.data_as(dp), int(lattice == "cubic"), phi.ctypes.data_as(dp),
+                                mat.ctypes.data, matkind, x.ctypes.data, y.ctypes.data, shift) == 0
+        out.append(y)
+    return out
+
+
+# (shape, planes per CTA): the default tile whole and cut, and tiles that leave ragged edges
+TILINGS = [(INT, 0), (INT, 3), (6033, 2), (6052, 5), (6119, 4), (6219, 1)]
+
+
+@pytest.mark.parametrize("N", [4, 6, 8, 14, 34])
+@pytest.mark.parametrize("lattice", list(LATTICES))
+@pytest.mark.parametrize("matkind", [0, 1, 2])
+@pytest.mark.parametrize("block", [-1, 1, 2])
+def test_integer_apply_equals_two_pass(emu, N, lattice, matkind, block):
+    if N == 34 and (block != 2 or lattice == "skew"):
+        pytest.skip("one block and two lattices at the largest size")
+    ref, *got = both(emu, N, block, lattice, matkind, complex_gaussian((3, N ** 3), 7), TILINGS)
+    for y in got:
+        assert np.linalg.norm(y - ref) <= TOL * np.linalg.norm(ref)
+        assert np.array_equal(y, got[0])  # a node's arithmetic does not depend on the tile
+
+
+@pytest.mark.parametrize("lattice,matkind", [("cubic", 0), ("fcc", 1), ("cubic", 2)])
+@pytest.mark.parametrize("value", [0.0, 5e-324, 1e-300, 1e-200, 1e250, 1e300, np.inf, np.nan])
+def test_integer_apply_takes_every_double(emu, lattice, matkind, value):
+    """Nodes outside the exponent range go through FP64: infinities and NaN spread as they do there,
+    and huge or tiny values keep their relative accuracy."""
+    N, block = 8, 3
+    x = complex_gaussian((3, N ** 3), 9)
+    if value == 0.0:
+        x[:] = 0.0
+    elif np.isfinite(value):
+        x *= value
+    else:
+        x[1, O.block_index((N,) * 3, block)[37]] = value
+    ref, y, cut = both(emu, N, block, lattice, matkind, x, [(INT, 0), (6023, 3)])
+    fine = np.isfinite(ref)
+    for v in (y, cut):
+        assert np.array_equal(fine, np.isfinite(v))
+        scale = np.abs(ref[fine]).max(initial=0.0)
+        assert np.abs(v[fine] - ref[fine]).max(initial=0.0) <= max(TOL * 4 * scale, 1e-320)
+
+
+def test_integer_apply_keeps_each_nodes_own_scale(emu):
+    """A vector whose size falls by 1e-60 across the cell: every node's output is accurate relative
+    to the values around it, not to the vector's largest."""
+    N, block = 16, 0
+    l = np.arange(N ** 3)
+    x = complex_gaussian((3, N ** 3), 4) * 10.0 ** (-4.0 * (l // (N * N)))
+    ref, y = both(emu, N, block, "cubic", 0, x, [(INT, 5)], kappa=(0.2, 0.1, 0.3))
+    scale = np.abs(ref).reshape(3, N, -1).max(axis=(0, 2))[None, :, None]
+    assert (np.abs(y - ref).reshape(3, N, -1) <= 4 * TOL * scale).all()
