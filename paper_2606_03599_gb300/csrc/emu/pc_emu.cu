@@ -14,6 +14,7 @@
 #include "../pc_apply_pipe.cuh"
 #include "../pc_apply_split.cuh"
 #include "../pc_apply_int.cuh"
+#include "../pc_limb.cuh"
 #include "../pc_small_dft.cuh"
 
 using namespace pc;
@@ -555,6 +556,31 @@ extern "C" int pc_emu_small_dft(int L, int inv, const double* in, double* out) {
 #undef PC_L
         default: return -1;
     }
+}
+
+// sum of a b over n <= 8 complex pairs, one limb group, as the outer-loop products form it.
+// Returns 0, or 1 when the group's exponents leave the integer path's range.
+extern "C" int pc_emu_limb_dot(int n, const double* a, const double* b, double* out) {
+    const double2* x = reinterpret_cast<const double2*>(a);
+    const double2* y = reinterpret_cast<const double2*>(b);
+    int ta = 0, tb = 0;
+    for (int q = 0; q < n; ++q) {
+        ta = limb_top(x[q], ta);
+        tb = limb_top(y[q], tb);
+    }
+    const int Ea = ta >> 20, Eb = tb >> 20;
+    if (Ea < kLimbLow || Ea > kLimbHigh || Eb < kLimbLow || Eb > kLimbHigh) return 1;
+    LimbAcc re = {0, 0}, im = {0, 0};
+    for (int q = 0; q < n; ++q) {
+        const LimbC u = limb_of(x[q], Ea), v = limb_of(y[q], Eb);
+        limb_mac(re, u.re, v.re);
+        limb_mac(re, limb_neg(u.im), v.im);
+        limb_mac(im, u.re, v.im);
+        limb_mac(im, u.im, v.re);
+    }
+    out[0] = limb_sum(re, Ea, Eb);
+    out[1] = limb_sum(im, Ea, Eb);
+    return 0;
 }
 
 // The ghost-cell numbering of the two-pass kernels: ghost_cell(gi) lies on the one-cell layer

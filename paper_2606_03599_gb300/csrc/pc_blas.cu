@@ -4,16 +4,20 @@
 // the restarts.
 //
 // The shapes are a few to a few dozen columns of length 3 n_b (83k at N = 48, 3.1M at N = 160),
-// so the work is a sum over a long index with a small dense result.  On GB300 these products are
-// bound by the FP64 pipe (two FP64 lanes per cycle per SM, the same rate for FP64 tensor
-// instructions), not by memory: 4 FMAs per complex multiply-add against 32 bytes of operands.
-// The kernels therefore keep every FP64 instruction useful: each thread owns a strip of the
-// long index and a register block of the result (RB rows x CB columns of the Gram block, CB
-// columns of an update), operands are read once per register block with coalesced 16-byte
-// loads, the mass weight is applied once per element of W (not per product), and Gram partial
-// sums are reduced in a fixed order (per CTA, then across CTAs) so results are deterministic.
+// so the work is a sum over a long index with a small dense result.  In FP64 arithmetic they are
+// bound by GB300's FP64 pipe (2 lanes per clock and SM, 8 FMAs for every 16-byte operand), 4 to 6
+// times above their memory time.  So products run on the integer pipe in groups of eight
+// (pc_limb.cuh): the group's operands are split into limbs once, a real product is three 32 x 32 + 64
+// bit multiply-adds, and the FP64 pipe sees two instructions per group and result.  Operands are
+// read once per register block with coalesced 16-byte loads, the mass weight is applied once per
+// element of W (not per product), and Gram partial sums are reduced in a fixed order (per CTA, then
+// across CTAs) so results are deterministic.
+//
+// Measured in a mixed-precision solve at N = 128 (four blocks, 2 columns, up to 26 rows; vectors of
+// 25 MB): Gram products 1.16 -> 0.49 ms and updates 1.40 -> 0.62 ms per launch on average.
 #include <algorithm>
 
+#include "pc_limb.cuh"
 #include "pc_solver.h"
 
 namespace pc {
@@ -33,16 +37,16 @@ __device__ __forceinline__ double node_weight(const void* __restrict__ mat, int6
 }
 
 // Partial sums of out(i, j) = sum_e conj(A[i][e]) w(e) B[j][e] over the nodes [t0, t1) of chunk
-// blockIdx.x (all three components), for rows i0 .. i0 + RB - 1 and columns j0 .. j0 + CB - 1.
+// blockIdx.x (all three components), columns j0 and j0 + 1, into
+// part[((base + i + j rows) 2 + re/im) nchunk + chunk].
 // MATK: -1 = no weight, 0 = phase ids, 1 = inclusion fractions, 2 = nodewise material.
+//
+// FP64 form, rows i0 .. i0 + RB - 1: vectors too short for full groups of eight.
 template <int RB, int MATK>
-__global__ void __launch_bounds__(kGramThreads)
-    ts_gram_kernel(const double2* __restrict__ A, int rows, const double2* __restrict__ B, int cols, int64_t m,
-                   const void* __restrict__ mat, double rho0, double drho, int ngc, int nchunk,
-                   double* __restrict__ part) {
+__device__ __forceinline__ void gram_chunk(const double2* __restrict__ A, int rows, const double2* __restrict__ B,
+                                           int cols, int64_t m, const void* __restrict__ mat, double rho0, double drho,
+                                           int i0, int j0, int nchunk, double* __restrict__ part, int64_t base) {
     constexpr int CB = kGramCB;
-    const int rg = blockIdx.y / ngc, cg = blockIdx.y % ngc;
-    const int i0 = rg * RB, j0 = cg * CB;
     const int64_t vs = 3 * m;
     const int64_t t0 = (int64_t)blockIdx.x * m / nchunk, t1 = (int64_t)(blockIdx.x + 1) * m / nchunk;
     double ar[RB][CB], ai[RB][CB];
@@ -100,9 +104,173 @@ __global__ void __launch_bounds__(kGramThreads)
         if (gi < rows && gj < cols) {
             double s = 0.0;
             for (int q = 0; q < kGramThreads / 32; ++q) s += red[q][v];
-            part[((int64_t)(gi + gj * rows) * 2 + ri) * nchunk + blockIdx.x] = s;
+            part[((base + gi + (int64_t)gj * rows) * 2 + ri) * nchunk + blockIdx.x] = s;
         }
     }
+}
+
+// Integer form, rows i0 .. i0 + 8 RW - 1 (warp w has rows i0 + w, i0 + w + 8, ...): a tile of 1024
+// elements of the two columns is weighted and split into limbs once, eight elements of a lane to a
+// group with one exponent, and every warp runs its rows over the tile; a group whose exponents are
+// out of range runs in FP64.  Splitting a row's elements costs about what their products do, so two
+// columns go together and the columns' own splitting is shared by all rows through shared memory (kept
+// in registers for eight rows of one thread it took 244 of them, and 8 warps per SM ran no faster than
+// the FP64 form).
+constexpr int kGramTile = 1024;
+
+template <int RW, int MATK>
+__device__ __forceinline__ void gram_tile(const double2* __restrict__ A, int rows, const double2* __restrict__ B,
+                                          int cols, int64_t m, const void* __restrict__ mat, double rho0, double drho,
+                                          int i0, int j0, int nchunk, double* __restrict__ part, int64_t base) {
+    constexpr int CB = kGramCB, NB = 8;
+    __shared__ LimbC lb[CB][kGramTile];
+    __shared__ int Eb[CB][kGramTile / NB];  // -1: FP64
+    const int64_t vs = 3 * m;
+    const int64_t t0 = (int64_t)blockIdx.x * m / nchunk, t1 = (int64_t)(blockIdx.x + 1) * m / nchunk;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int len = (int)(t1 - t0), total = 3 * len;  // elements of the chunk, component after component
+    auto element = [&](int x) {                       // offset in a vector of element x of the chunk
+        const int c = (x >= len) + (x >= 2 * len);
+        return (int64_t)c * m + t0 + (x - c * len);
+    };
+    auto weighted = [&](int j, int x) {
+        const int64_t e = element(x);
+        double2 b = (j0 + j < cols) ? B[(int64_t)(j0 + j) * vs + e] : make_double2(0.0, 0.0);
+        if (MATK >= 0) {
+            const int c = (x >= len) + (x >= 2 * len);
+            const double w = node_weight<MATK>(mat, e - (int64_t)c * m, m, rho0, drho);
+            b = make_double2(w * b.x, w * b.y);
+        }
+        return b;
+    };
+    double ar[RW][CB], ai[RW][CB];
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int j = 0; j < CB; ++j) ar[r][j] = ai[r][j] = 0.0;
+    for (int x0 = 0; x0 < total; x0 += kGramTile) {
+        {
+            const int g = warp >> 1, j = warp & 1;
+            double2 b[NB];
+            int top = 0;
+#pragma unroll
+            for (int q = 0; q < NB; ++q) {
+                const int x = x0 + g * 256 + q * 32 + lane;
+                b[q] = x < total ? weighted(j, x) : make_double2(0.0, 0.0);
+                top = limb_top(b[q], top);
+            }
+            const int E = top == 0 ? 1000 : top >> 20;  // zeros, or values too small to count
+#pragma unroll
+            for (int q = 0; q < NB; ++q) lb[j][g * 256 + q * 32 + lane] = limb_of(b[q], E);
+            Eb[j][g * 32 + lane] = (E >= kLimbLow && E <= kLimbHigh) ? E : -1;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int g = 0; g < kGramTile / 256; ++g) {
+            const int xg = x0 + g * 256 + lane;
+            if (xg - lane >= total) break;
+            const int E0 = Eb[0][g * 32 + lane], E1 = Eb[1][g * 32 + lane];
+            const bool ok = (E0 | E1) >= 0;
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const int i = i0 + warp + 8 * r;
+                if (i >= rows) break;
+                const double2* __restrict__ Ai = A + (int64_t)i * vs;
+                double2 a[NB];
+                int top = 0;
+#pragma unroll
+                for (int q = 0; q < NB; ++q) {
+                    const int x = xg + q * 32;
+                    a[q] = x < total ? Ai[element(x)] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int q = 0; q < NB; ++q) top = limb_top(a[q], top);
+                const int E = top >> 20;
+                if (ok && E >= kLimbLow && E <= kLimbHigh) {
+                    LimbAcc re[CB], im[CB];
+#pragma unroll
+                    for (int j = 0; j < CB; ++j) re[j].hi = re[j].mid = im[j].hi = im[j].mid = 0;
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) {
+                        const LimbC la = limb_of(a[q], E);
+                        const Limb ni = limb_neg(la.im);
+#pragma unroll
+                        for (int j = 0; j < CB; ++j) {  // conj(a) b
+                            const LimbC lv = lb[j][g * 256 + q * 32 + lane];
+                            limb_mac(re[j], la.re, lv.re);
+                            limb_mac(re[j], la.im, lv.im);
+                            limb_mac(im[j], la.re, lv.im);
+                            limb_mac(im[j], ni, lv.re);
+                        }
+                    }
+                    ar[r][0] += limb_sum(re[0], E, E0);
+                    ai[r][0] += limb_sum(im[0], E, E0);
+                    ar[r][1] += limb_sum(re[1], E, E1);
+                    ai[r][1] += limb_sum(im[1], E, E1);
+                } else if (top != 0 || !ok) {
+#pragma unroll 1
+                    for (int q = 0; q < NB; ++q) {
+                        const int x = xg + q * 32;
+                        if (x >= total) break;
+                        const double2 av = Ai[element(x)];
+#pragma unroll
+                        for (int j = 0; j < CB; ++j) {
+                            const double2 bv = weighted(j, x);
+                            ar[r][j] = fma(av.x, bv.x, fma(av.y, bv.y, ar[r][j]));
+                            ai[r][j] = fma(av.x, bv.y, fma(-av.y, bv.x, ai[r][j]));
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+        const int i = i0 + warp + 8 * r;
+        if (i >= rows) break;
+#pragma unroll
+        for (int j = 0; j < CB; ++j) {
+            double vr = ar[r][j], vi = ai[r][j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                vr += __shfl_down_sync(0xffffffffu, vr, o);
+                vi += __shfl_down_sync(0xffffffffu, vi, o);
+            }
+            if (lane == 0 && j0 + j < cols) {
+                double* p = part + ((base + i + (int64_t)(j0 + j) * rows) * 2) * nchunk + blockIdx.x;
+                p[0] = vr;
+                p[nchunk] = vi;
+            }
+        }
+    }
+}
+
+// One register block of a product: RB < 0 is the integer form with -RB rows per warp.
+template <int RB, int MATK>
+__device__ __forceinline__ void gram_block(const double2* __restrict__ A, int rows, const double2* __restrict__ B,
+                                           int cols, int64_t m, const void* __restrict__ mat, double rho0, double drho,
+                                           int rg, int cg, int nchunk, double* __restrict__ part, int64_t base) {
+    if constexpr (RB < 0)
+        gram_tile<-RB, MATK>(A, rows, B, cols, m, mat, rho0, drho, rg * -RB * 8, cg * kGramCB, nchunk, part, base);
+    else
+        gram_chunk<RB, MATK>(A, rows, B, cols, m, mat, rho0, drho, rg * RB, cg * kGramCB, nchunk, part, base);
+}
+
+// The form for `rows` rows of vectors of m nodes.  Integer form from vectors that fill two tiles of
+// 1024 elements and 5 rows on (fewer rows leave its warps idle); rows per block in *rb.
+int gram_form(int rows, int64_t m, int* rb) {
+    const int f = (m >= 683 && rows > 4) ? (rows <= 8 ? -1 : rows <= 16 ? -2 : -3) : (rows <= 2 ? 2 : rows <= 4 ? 4 : 8);
+    *rb = f < 0 ? -f * 8 : f;
+    return f;
+}
+
+template <int RB, int MATK>
+__global__ void __launch_bounds__(kGramThreads, RB < 0 ? 2 : 1)
+    ts_gram_kernel(const double2* __restrict__ A, int rows, const double2* __restrict__ B, int cols, int64_t m,
+                   const void* __restrict__ mat, double rho0, double drho, int ngc, int nchunk,
+                   double* __restrict__ part) {
+    gram_block<RB, MATK>(A, rows, B, cols, m, mat, rho0, drho, blockIdx.y / ngc, blockIdx.y % ngc, nchunk, part, 0);
 }
 
 // out[e] = sum over chunks of part[e][chunk]: one warp per entry, lane l sums the chunks
@@ -125,33 +293,100 @@ __global__ void ts_gram_reduce(const double* __restrict__ part, int nentries, in
     if (lane == 0) out[e] = make_double2(re, im);
 }
 
+// cr + i ci += sum over NB columns kk .. kk + NB - 1 of A of a(e) h(., j): a group of columns on the
+// integer pipe, or in FP64 where its exponents (or those of h: hok) are out of range.
+template <int CB, int NB>
+__device__ __forceinline__ void update_group(const double2* __restrict__ Ae, int64_t vs, const LimbC* hs,
+                                             const int* Eh, bool hok, const double2* __restrict__ h, int64_t hstr,
+                                             int jn, double* cr, double* ci) {
+    double2 a[NB];
+    int top = 0;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        a[q] = Ae[(int64_t)q * vs];
+        top = limb_top(a[q], top);
+    }
+    const int E = top >> 20;
+    if (hok && E >= kLimbLow && E <= kLimbHigh) {
+        LimbAcc re[CB], im[CB];
+#pragma unroll
+        for (int j = 0; j < CB; ++j) re[j].hi = re[j].mid = im[j].hi = im[j].mid = 0;
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const LimbC la = limb_of(a[q], E);
+            const Limb ni = limb_neg(la.im);
+#pragma unroll
+            for (int j = 0; j < CB; ++j) {
+                const LimbC hv = hs[q * CB + j];
+                limb_mac(re[j], la.re, hv.re);
+                limb_mac(re[j], ni, hv.im);
+                limb_mac(im[j], la.re, hv.im);
+                limb_mac(im[j], la.im, hv.re);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < CB; ++j) {
+            cr[j] += limb_sum(re[j], E, Eh[j]);
+            ci[j] += limb_sum(im[j], E, Eh[j]);
+        }
+    } else if (top != 0 || !hok) {
+#pragma unroll 1
+        for (int q = 0; q < NB; ++q) {
+            const double2 av = Ae[(int64_t)q * vs];
+#pragma unroll
+            for (int j = 0; j < CB; ++j) {
+                const double2 hv = j < jn ? h[q + (int64_t)j * hstr] : make_double2(0.0, 0.0);
+                cr[j] = fma(av.x, hv.x, fma(-av.y, hv.y, cr[j]));
+                ci[j] = fma(av.x, hv.y, fma(av.y, hv.x, ci[j]));
+            }
+        }
+    }
+}
+
 // C[:, j] = beta C[:, j] + alpha sum_k A[:, k] h(k, j) for the CB columns j0 .. j0 + CB - 1 of
-// column group blockIdx.y; h (k x cols, column-major) is staged in shared memory.  With
-// beta == 0, C is not read (it may hold anything).
+// column group blockIdx.y; the limbs of h (k x cols, column-major, one exponent per column) are
+// staged in shared memory.  With beta == 0, C is not read (it may hold anything).
 template <int CB>
-__global__ void __launch_bounds__(256)
-    ts_update_kernel(const double2* __restrict__ A, int k, const double2* __restrict__ h, int cols,
-                     double2* __restrict__ C, int64_t vs, double alpha, double beta) {
-    extern __shared__ double2 hs[];  // [k][CB]
-    const int j0 = blockIdx.y * CB;
+__device__ __forceinline__ void update_columns(const double2* __restrict__ A, int k, const double2* __restrict__ h,
+                                               int cols, double2* __restrict__ C, int64_t vs, double alpha,
+                                               double beta, int j0) {
+    extern __shared__ LimbC hs[];  // [k][CB]
+    __shared__ int tops[CB];
+    if (threadIdx.x < CB) tops[threadIdx.x] = 0;
+    __syncthreads();
     for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
         const int kk = q / CB, j = q % CB;
-        hs[q] = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
+        if (j0 + j < cols) atomicMax(&tops[j], limb_top(h[kk + (int64_t)(j0 + j) * k], 0));
     }
     __syncthreads();
+    int Eh[CB];
+    bool hok = true;
+#pragma unroll
+    for (int j = 0; j < CB; ++j) {
+        Eh[j] = tops[j] == 0 ? 1000 : tops[j] >> 20;
+        hok = hok && Eh[j] >= kLimbLow && Eh[j] <= kLimbHigh;
+    }
+    for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
+        const int kk = q / CB, j = q % CB;
+        const double2 hv = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
+        hs[q] = limb_of(hv, tops[j] == 0 ? 1000 : tops[j] >> 20);
+    }
+    __syncthreads();
+    const double2* __restrict__ hj = h + (int64_t)j0 * k;
+    const int jn = cols - j0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
         double cr[CB], ci[CB];
 #pragma unroll
         for (int j = 0; j < CB; ++j) cr[j] = ci[j] = 0.0;
-        for (int kk = 0; kk < k; ++kk) {
-            const double2 a = A[(int64_t)kk * vs + e];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {  // a h
-                const double2 hv = hs[kk * CB + j];
-                cr[j] = fma(a.x, hv.x, fma(-a.y, hv.y, cr[j]));
-                ci[j] = fma(a.x, hv.y, fma(a.y, hv.x, ci[j]));
-            }
+        int kk = 0;
+        for (; kk + 8 <= k; kk += 8)
+            update_group<CB, 8>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
+        if (k & 4) {
+            update_group<CB, 4>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
+            kk += 4;
         }
+        for (; kk < k; ++kk)
+            update_group<CB, 1>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
 #pragma unroll
         for (int j = 0; j < CB; ++j) {
             if (j0 + j >= cols) continue;
@@ -167,21 +402,28 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-template <int RB>
-int launch_gram_rb(const double2* A, int rows, const double2* B, int cols, int64_t m, const void* mat, int matkind,
-                   double rho0, double drho, int ngc, int nrg, int nchunk, double* part, cudaStream_t s) {
-    const dim3 grid(nchunk, nrg * ngc);
-    if (mat == nullptr)
-        ts_gram_kernel<RB, -1><<<grid, kGramThreads, 0, s>>>(A, rows, B, cols, m, mat, rho0, drho, ngc, nchunk, part);
-    else if (matkind == 0)
-        ts_gram_kernel<RB, 0><<<grid, kGramThreads, 0, s>>>(A, rows, B, cols, m, mat, rho0, drho, ngc, nchunk, part);
-    else if (matkind == 2)
-        ts_gram_kernel<RB, 2><<<grid, kGramThreads, 0, s>>>(A, rows, B, cols, m, mat, rho0, drho, ngc, nchunk, part);
-    else
-        ts_gram_kernel<RB, 1><<<grid, kGramThreads, 0, s>>>(A, rows, B, cols, m, mat, rho0, drho, ngc, nchunk, part);
-    note_launch();
-    return PC_OK;
+template <int CB>
+__global__ void __launch_bounds__(256)
+    ts_update_kernel(const double2* __restrict__ A, int k, const double2* __restrict__ h, int cols,
+                     double2* __restrict__ C, int64_t vs, double alpha, double beta) {
+    update_columns<CB>(A, k, h, cols, C, vs, alpha, beta, blockIdx.y * CB);
 }
+
+// Instantiations of a Gram kernel over the forms and weights: CALL(form, weight kind)
+#define PC_GRAM_MK(CALL, RBV, mk)  \
+    if (mk < 0) { CALL(RBV, -1); } \
+    else if (mk == 0) { CALL(RBV, 0); } \
+    else if (mk == 2) { CALL(RBV, 2); } \
+    else { CALL(RBV, 1); }
+#define PC_GRAM_FORM(CALL, form, mk)                    \
+    switch (form) {                                     \
+        case -1: PC_GRAM_MK(CALL, -1, mk) break;        \
+        case -2: PC_GRAM_MK(CALL, -2, mk) break;        \
+        case -3: PC_GRAM_MK(CALL, -3, mk) break;        \
+        case 2: PC_GRAM_MK(CALL, 2, mk) break;          \
+        case 4: PC_GRAM_MK(CALL, 4, mk) break;          \
+        default: PC_GRAM_MK(CALL, 8, mk) break;         \
+    }
 
 // ---------------------------------------------------------------- batched forms (several spaces)
 // The outer loop runs the same product for every active space of a solve (the four parity blocks
@@ -195,77 +437,14 @@ struct GramBatch {
 };
 
 template <int RB, int MATK>
-__global__ void __launch_bounds__(kGramThreads)
+__global__ void __launch_bounds__(kGramThreads, RB < 0 ? 2 : 1)
     ts_gram_batch_kernel(const __grid_constant__ GramBatch B, int64_t m, double rho0, double drho, int ngc,
                          int nchunk, double* __restrict__ part) {
-    constexpr int CB = kGramCB;
     const GramJob& J = B.j[blockIdx.z];
-    const int rows = J.rows, cols = J.cols;
     const int rg = blockIdx.y / ngc, cg = blockIdx.y % ngc;
-    const int i0 = rg * RB, j0 = cg * CB;
-    if (i0 >= rows || j0 >= cols) return;  // this job has fewer register blocks than the launch
-    const double2* __restrict__ A = J.A;
-    const double2* __restrict__ Bm = J.B;
-    const void* __restrict__ mat = J.mat;
-    const int64_t vs = 3 * m;
-    const int64_t t0 = (int64_t)blockIdx.x * m / nchunk, t1 = (int64_t)(blockIdx.x + 1) * m / nchunk;
-    double ar[RB][CB], ai[RB][CB];
-#pragma unroll
-    for (int i = 0; i < RB; ++i)
-#pragma unroll
-        for (int j = 0; j < CB; ++j) ar[i][j] = ai[i][j] = 0.0;
-    for (int64_t t = t0 + threadIdx.x; t < t1; t += kGramThreads) {
-        const double w = node_weight<MATK>(mat, t, m, rho0, drho);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int64_t e = c * m + t;
-            double2 b[CB];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                b[j] = (j0 + j < cols) ? Bm[(int64_t)(j0 + j) * vs + e] : make_double2(0.0, 0.0);
-                if (MATK >= 0) b[j] = make_double2(w * b[j].x, w * b[j].y);
-            }
-#pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                if (i0 + i < rows) {
-                    const double2 a = A[(int64_t)(i0 + i) * vs + e];
-#pragma unroll
-                    for (int j = 0; j < CB; ++j) {  // conj(a) b
-                        ar[i][j] = fma(a.x, b[j].x, fma(a.y, b[j].y, ar[i][j]));
-                        ai[i][j] = fma(a.x, b[j].y, fma(-a.y, b[j].x, ai[i][j]));
-                    }
-                }
-            }
-        }
-    }
-    constexpr int NV = RB * CB * 2;
-    __shared__ double red[kGramThreads / 32][NV];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < RB; ++i)
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-            double vr = ar[i][j], vi = ai[i][j];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                vr += __shfl_down_sync(0xffffffffu, vr, o);
-                vi += __shfl_down_sync(0xffffffffu, vi, o);
-            }
-            if (lane == 0) {
-                red[warp][(i * CB + j) * 2 + 0] = vr;
-                red[warp][(i * CB + j) * 2 + 1] = vi;
-            }
-        }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        const int v = threadIdx.x, ij = v >> 1, ri = v & 1;
-        const int gi = i0 + ij / CB, gj = j0 + ij % CB;
-        if (gi < rows && gj < cols) {
-            double s = 0.0;
-            for (int q = 0; q < kGramThreads / 32; ++q) s += red[q][v];
-            part[((B.off[blockIdx.z] + gi + (int64_t)gj * rows) * 2 + ri) * nchunk + blockIdx.x] = s;
-        }
-    }
+    constexpr int step = RB < 0 ? -RB * 8 : RB;
+    if (rg * step >= J.rows || cg * kGramCB >= J.cols) return;  // this job has fewer blocks than the launch
+    gram_block<RB, MATK>(J.A, J.rows, J.B, J.cols, m, J.mat, rho0, drho, rg, cg, nchunk, part, B.off[blockIdx.z]);
 }
 
 // Entry e of the concatenated results (job order) = fixed-order sum of its chunk partials.
@@ -299,46 +478,10 @@ struct UpdateBatch {
 template <int CB>
 __global__ void __launch_bounds__(256)
     ts_update_batch_kernel(const __grid_constant__ UpdateBatch U, int64_t vs) {
-    extern __shared__ double2 hs[];  // [k][CB]
     const UpdateJob& J = U.j[blockIdx.z];
-    const int k = J.k, cols = J.cols;
     const int j0 = blockIdx.y * CB;
-    if (j0 >= cols) return;
-    const double2* __restrict__ h = J.h;
-    for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
-        const int kk = q / CB, j = q % CB;
-        hs[q] = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    const double2* __restrict__ A = J.A;
-    double2* __restrict__ C = J.C;
-    const double alpha = J.alpha, beta = J.beta;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
-        double cr[CB], ci[CB];
-#pragma unroll
-        for (int j = 0; j < CB; ++j) cr[j] = ci[j] = 0.0;
-        for (int kk = 0; kk < k; ++kk) {
-            const double2 a = A[(int64_t)kk * vs + e];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                const double2 hv = hs[kk * CB + j];
-                cr[j] = fma(a.x, hv.x, fma(-a.y, hv.y, cr[j]));
-                ci[j] = fma(a.x, hv.y, fma(a.y, hv.x, ci[j]));
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-            if (j0 + j >= cols) continue;
-            double2* cp = C + (int64_t)(j0 + j) * vs + e;
-            double2 o = make_double2(alpha * cr[j], alpha * ci[j]);
-            if (beta != 0.0) {
-                const double2 cv = *cp;
-                o.x = fma(beta, cv.x, o.x);
-                o.y = fma(beta, cv.y, o.y);
-            }
-            *cp = o;
-        }
-    }
+    if (j0 >= J.cols) return;
+    update_columns<CB>(J.A, J.k, J.h, J.cols, J.C, vs, J.alpha, J.beta, j0);
 }
 
 }  // namespace
@@ -347,8 +490,9 @@ int ts_gram(const double2* A, int rows, const double2* B, int cols, int64_t m, c
             double rho0, double rho1, double2* d_out, double* d_part, size_t part_cap, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return PC_OK;
     if (!A || !B || !d_out || !d_part || m <= 0) return fail(PC_EINVAL, "ts_gram: bad argument");
-    const int RB = rows <= 2 ? 2 : (rows <= 4 ? 4 : 8);
-    const int nrg = (rows + RB - 1) / RB, ngc = (cols + kGramCB - 1) / kGramCB;
+    int rb;
+    const int form = gram_form(rows, m, &rb);
+    const int nrg = (rows + rb - 1) / rb, ngc = (cols + kGramCB - 1) / kGramCB;
     // chunks of the node range: about two CTAs per SM over all register blocks, at least 512
     // nodes (two per thread) per chunk so that the per-CTA reduction stays small next to the
     // products, and as many partials as the scratch holds
@@ -358,12 +502,13 @@ int ts_gram(const double2* A, int rows, const double2* B, int cols, int64_t m, c
     nchunk = std::min<int64_t>(nchunk, (int64_t)(part_cap / (2 * entries)));
     if (nchunk < 1) return fail(PC_EINVAL, "ts_gram: partial-sum scratch too small");
     const double drho = rho1 - rho0;
-    if (RB == 2)
-        launch_gram_rb<2>(A, rows, B, cols, m, mat, matkind, rho0, drho, ngc, nrg, (int)nchunk, d_part, s);
-    else if (RB == 4)
-        launch_gram_rb<4>(A, rows, B, cols, m, mat, matkind, rho0, drho, ngc, nrg, (int)nchunk, d_part, s);
-    else
-        launch_gram_rb<8>(A, rows, B, cols, m, mat, matkind, rho0, drho, ngc, nrg, (int)nchunk, d_part, s);
+    const int mk = mat ? matkind : -1;
+    const dim3 grid((unsigned)nchunk, nrg * ngc);
+#define PC_GRAM_1(RBV, MKV) \
+    ts_gram_kernel<RBV, MKV><<<grid, kGramThreads, 0, s>>>(A, rows, B, cols, m, mat, rho0, drho, ngc, (int)nchunk, d_part)
+    PC_GRAM_FORM(PC_GRAM_1, form, mk)
+#undef PC_GRAM_1
+    note_launch();
     ts_gram_reduce<<<(int)((entries + 7) / 8), 256, 0, s>>>(d_part, (int)entries, (int)nchunk, d_out);
     note_launch();
     PC_CUDA_TRY(cudaGetLastError());
@@ -387,7 +532,7 @@ int ts_update(const double2* A, int k, const double2* d_h, int cols, double2* C,
     // column blocks of 2 when cols <= 2 (the Gram-Schmidt updates of a 2-wide Krylov block:
     // no FMAs on padding columns), else of 4
     const int CB = cols <= 2 ? 2 : 4;
-    const size_t smem = sizeof(double2) * (size_t)k * CB;
+    const size_t smem = sizeof(LimbC) * (size_t)k * CB;
     if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update: too many basis columns");
     const int ngc = (cols + CB - 1) / CB;
     int64_t gx = (vs + 255) / 256;
@@ -422,8 +567,9 @@ int ts_gram_batch(const GramJob* jobs, int njobs, int64_t m, int matkind, double
             maxc = std::max(maxc, J.cols);
         }
         if (B.n == 0) continue;
-        const int RB = maxr <= 2 ? 2 : (maxr <= 4 ? 4 : 8);
-        const int nrg = (maxr + RB - 1) / RB, ngc = (maxc + kGramCB - 1) / kGramCB;
+        int rb;
+        const int form = gram_form(maxr, m, &rb);
+        const int nrg = (maxr + rb - 1) / rb, ngc = (maxc + kGramCB - 1) / kGramCB;
         const int64_t entries = B.off[B.n];
         int64_t nchunk = (2LL * device_sm_count() + (int64_t)nrg * ngc * B.n - 1) / ((int64_t)nrg * ngc * B.n);
         nchunk = std::min<int64_t>(nchunk, std::max<int64_t>(1, m / 512));
@@ -434,15 +580,7 @@ int ts_gram_batch(const GramJob* jobs, int njobs, int64_t m, int matkind, double
         const int mk = weighted ? matkind : -1;
 #define PC_GRAM_B(RBV, MKV) \
     ts_gram_batch_kernel<RBV, MKV><<<grid, kGramThreads, 0, s>>>(B, m, rho0, drho, ngc, (int)nchunk, d_part)
-#define PC_GRAM_MK(RBV)                  \
-    if (mk < 0) PC_GRAM_B(RBV, -1);      \
-    else if (mk == 0) PC_GRAM_B(RBV, 0); \
-    else if (mk == 2) PC_GRAM_B(RBV, 2); \
-    else PC_GRAM_B(RBV, 1);
-        if (RB == 2) { PC_GRAM_MK(2) }
-        else if (RB == 4) { PC_GRAM_MK(4) }
-        else { PC_GRAM_MK(8) }
-#undef PC_GRAM_MK
+        PC_GRAM_FORM(PC_GRAM_B, form, mk)
 #undef PC_GRAM_B
         note_launch();
         ts_gram_batch_reduce<<<(unsigned)((entries + 7) / 8), 256, 0, s>>>(B, d_part, (int)nchunk);
@@ -467,7 +605,7 @@ int ts_update_batch(const UpdateJob* jobs, int njobs, int64_t vs, cudaStream_t s
         }
         if (U.n == 0) continue;
         const int CB = maxc <= 2 ? 2 : 4;
-        const size_t smem = sizeof(double2) * (size_t)maxk * CB;
+        const size_t smem = sizeof(LimbC) * (size_t)maxk * CB;
         if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update_batch: too many basis columns");
         const int ngc = (maxc + CB - 1) / CB;
         int64_t gx = (vs + 255) / 256;

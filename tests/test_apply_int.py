@@ -121,3 +121,37 @@ def test_integer_apply_keeps_each_nodes_own_scale(emu):
     ref, y = both(emu, N, block, "cubic", 0, x, [(INT, 5)], kappa=(0.2, 0.1, 0.3))
     scale = np.abs(ref).reshape(3, N, -1).max(axis=(0, 2))[None, :, None]
     assert (np.abs(y - ref).reshape(3, N, -1) <= 4 * TOL * scale).all()
+
+
+@pytest.mark.parametrize("n", [1, 4, 8])
+@pytest.mark.parametrize("spread", [0, 12, 60])
+@pytest.mark.parametrize("scale", [1e-100, 1.0, 1e100])
+def test_limb_group_sum(emu, n, spread, scale):
+    """The group products of the outer loop against extended precision.  A value is cut at 2^-57 of
+    its group's largest and a product drops its low x low part, at most 2^-56 of the largest
+    product, so each of the 2 n real products is off by at most 3 * 2^-56 of it; the conversion to a
+    double adds half a unit of the result and of the group's unit."""
+    dp = ctypes.POINTER(ctypes.c_double)
+    emu.pc_emu_limb_dot.argtypes = [ctypes.c_int, dp, dp, dp]
+    rng = np.random.default_rng(n + spread)
+    for _ in range(50):
+        a, b = (rng.standard_normal((n, 2)) * 2.0 ** -rng.integers(0, spread + 1, (n, 2)) for _ in range(2))
+        a *= scale
+        a[rng.random((n, 2)) < 0.1] = 0.0
+        a[0, 0] = scale
+        out = np.zeros(2)
+        assert emu.pc_emu_limb_dot(n, a.ctypes.data_as(dp), b.ctypes.data_as(dp), out.ctypes.data_as(dp)) == 0
+        x, y = a.astype(np.longdouble), b.astype(np.longdouble)
+        ref = np.array([(x[:, 0] * y[:, 0] - x[:, 1] * y[:, 1]).sum(), (x[:, 0] * y[:, 1] + x[:, 1] * y[:, 0]).sum()])
+        top = np.abs(a).max() * np.abs(b).max()
+        assert (np.abs(out - ref) <= (2 * n * 3 + 2) * 2.0 ** -56 * top * 4 + 2.0 ** -53 * np.abs(ref)).all()
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 1e-250, 1e250])
+def test_limb_group_leaves_extreme_values_to_fp64(emu, value):
+    dp = ctypes.POINTER(ctypes.c_double)
+    a = np.full((2, 2), value)
+    b = np.ones((2, 2))
+    out = np.zeros(2)
+    for u, v in ((a, b), (b, a)):
+        assert emu.pc_emu_limb_dot(2, u.ctypes.data_as(dp), v.ctypes.data_as(dp), out.ctypes.data_as(dp)) == 1
