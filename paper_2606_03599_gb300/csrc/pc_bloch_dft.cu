@@ -31,6 +31,7 @@
 #include <mutex>
 #include <vector>
 
+#include "pc_bloch_fused.cuh"
 #include "pc_complex.cuh"
 #include "pc_fourier.h"
 #include "pc_internal.h"
@@ -560,12 +561,14 @@ static int own_precond_t(int n, int nsys, const V* r, V* z, C* W, const C* wn, c
                          double shift_rho, double scale, double* part, cudaStream_t s) {
     int n1, n2;
     if (!bloch_dft_supported(n, &n1, &n2)) return fail(PC_EINVAL, "block DFT: unsupported size");
+    if constexpr (sizeof(C) == sizeof(double2)) {  // the complex64 forms of these sizes are the fused kernels
 #define PC_DFT_CASE(A, B)                                                                                   \
     if (n1 == A && n2 == B)                                                                                 \
         return precond_launch<A, B>(n, n1, n2, nsys, r, z, W, wn, twa, twb, twk, ea, eb, eg, Aref, sys_block, \
                                     sys_k, tab_stride, skip, shift_rho, scale, part, s);
-    PC_DFT_SIZES(PC_DFT_CASE)
+        PC_DFT_SIZES(PC_DFT_CASE)
 #undef PC_DFT_CASE
+    }
     return precond_launch<0, 0>(n, n1, n2, nsys, r, z, W, wn, twa, twb, twk, ea, eb, eg, Aref, sys_block, sys_k,
                                 tab_stride, skip, shift_rho, scale, part, s);
 }
@@ -574,6 +577,35 @@ int own_precond(int n, int wdt, int vdt, int nsys, const void* r, void* z, void*
                 const int* sys_block, const int* sys_k, const int* skip, double shift_rho, double scale,
                 double* part, cudaStream_t s) {
     const int64_t ts = P->tab_len;
+    if (wdt == PC_C64 && P->fused) {
+        fused::Args a;
+        a.r = r;
+        a.z = z;
+        a.W = static_cast<float2*>(W);
+        a.wn = P->wn32;
+        a.twa = P->twa32;
+        a.twb = P->twb32;
+        a.twk = P->twk32;
+        a.ea = P->ea32;
+        a.eb = P->eb32;
+        a.eg = P->egh32;
+        a.A = P->d_Aref32;
+        a.sys_block = sys_block;
+        a.sys_k = sys_k;
+        a.skip = skip;
+        a.tab_stride = ts;
+        a.shift_rho = (float)shift_rho;
+        a.scale = (float)scale;
+        a.part = part;
+        a.npart = bloch_dft_partials(n);
+        a.nsys = nsys;
+        bool found = false;
+        for (auto f : {fused::launch_a, fused::launch_b, fused::launch_c, fused::launch_d}) {
+            PC_TRY(f(n, vdt == PC_C128, a, s, &found));
+            if (found) return PC_OK;
+        }
+        return fail(PC_EINVAL, "block DFT: no fused kernels for this size");
+    }
     if (wdt == PC_C64 && vdt == PC_C64)
         return own_precond_t<float2, float2, float2>(n, nsys, (const float2*)r, (float2*)z, (float2*)W, P->wn32,
                                                      P->twa32, P->twb32, P->twk32, P->ea32, P->eb32, P->egh32,

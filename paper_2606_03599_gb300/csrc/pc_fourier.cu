@@ -26,6 +26,7 @@
 #include <cstring>
 #include <vector>
 
+#include "pc_bloch_fused.cuh"
 #include "pc_complex.cuh"
 #include "pc_fourier.h"
 #include "pc_internal.h"
@@ -250,6 +251,18 @@ __global__ void table_to_f32(const double* __restrict__ a, float* __restrict__ b
         b[i] = (float)a[i];
 }
 
+// The table of one slot for the fused kernels: entry-major, both plane axes in position order
+// (position k1 n2 + k2 holds mode k1 + n1 k2).
+__global__ void table_to_positions(const double* __restrict__ a, float* __restrict__ b, int n, int n1, int n2) {
+    const int64_t nn = (int64_t)n * n, nb = 2 * n * nn;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(i / nn), c = (int)(i - r * nn), qp = c / n, pp = c - qp * n;
+        const int q = qp / n2 + n1 * (qp % n2), p = pp / n2 + n1 * (pp % n2);
+        const double* src = a + 9 * (r * nn + (int64_t)q * n + p);
+        for (int e = 0; e < 9; ++e) b[e * nb + i] = (float)src[e];
+    }
+}
+
 // Reference symbol A_ref(m) = B_hat(m) C_ref B_hat(m)^H for every mode (p, q, r), r < Z, and
 // the zero-derivative flag ||eta(m)|| == 0 (B_hat(m) = 0: rank-0 symbol, Sec. 6.2).
 __global__ void symbol_table(double* __restrict__ Aref, int* __restrict__ nnull, int* __restrict__ null_modes,
@@ -364,6 +377,7 @@ Precond::~Precond() {
     cudaFree(d_wn);
     cudaFree(d_wn32);
     cudaFree(d_blockids);
+    cudaFree(d_part);
 }
 
 namespace pc {
@@ -378,6 +392,8 @@ int precond_create(pc_grid* g) {
     P->tab_len = X + Y + Z / 2 + Z + X + Y + Z / 2;
     // roots of the own quarter-grid DFT (Bloch-independent) and the block ids
     P->own_dft = g->X == g->Y && g->Z == 2 * g->X && bloch_dft_supported(g->X, nullptr, nullptr);
+    P->fused = P->own_dft && fused::supported(g->X);
+    PC_CUDA_TRY(cudaMalloc(&P->d_part, sizeof(double) * 4 * precond_partials(g)));
     {
         const int n = g->X;
         std::vector<double2> w(n);
@@ -481,7 +497,14 @@ static int precond_fill_slot(pc_grid* g, int slot) {
     PC_CUDA_TRY(cudaMemset(dn, 0, sizeof(int) * 65));
     symbol_table<<<nblocks_for(g->nb), 256>>>(aref, dn, dn + 1, P->ea + to, P->eb + to, P->egf + to, sp);
     note_launch();
-    table_to_f32<<<nblocks_for(9 * g->nb), 256>>>(aref, P->d_Aref32 + (size_t)slot * 9 * g->nb, 9 * g->nb);
+    float* aref32 = P->d_Aref32 + (size_t)slot * 9 * g->nb;
+    if (P->fused) {
+        int n1, n2;
+        bloch_dft_supported(X, &n1, &n2);
+        table_to_positions<<<nblocks_for(g->nb), 256>>>(aref, aref32, X, n1, n2);
+    } else {
+        table_to_f32<<<nblocks_for(9 * g->nb), 256>>>(aref, aref32, 9 * g->nb);
+    }
     note_launch();
     PC_CUDA_TRY(cudaGetLastError());
     int hn[65];

@@ -38,7 +38,8 @@ struct Precond {
     const float2 *ea32 = nullptr, *eb32 = nullptr, *egh32 = nullptr;
     const float2 *twa32 = nullptr, *twb32 = nullptr, *twk32 = nullptr;
     double* d_Aref = nullptr;  // 9 reals per mode (Hermitian 3x3 reference symbol)
-    float* d_Aref32 = nullptr; // the same table rounded to FP32 (complex64 preconditioning)
+    float* d_Aref32 = nullptr; // the same table rounded to FP32 (complex64 preconditioning); with `fused`
+                               // [9][r][position q][position p] (pc_bloch_fused.cuh)
     int* d_null = nullptr;     // per slot: [0] = count, [1..64] = modes with a vanishing symbol
     std::vector<int> null_modes;                 // slot 0
     std::vector<std::vector<int>> null_slot;     // every slot
@@ -55,6 +56,8 @@ struct Precond {
     const float2* wn32 = nullptr;
     int* d_blockids = nullptr;
     bool own_dft = false;  // the own kernels handle this grid's size
+    bool fused = false;    // complex64 preconditioner in the fused kernels (d_Aref32 in their order)
+    double* d_part = nullptr;  // partial sums of pc_block_precond (not returned)
 };
 
 namespace pc {
