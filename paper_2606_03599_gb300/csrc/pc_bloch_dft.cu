@@ -49,9 +49,14 @@ constexpr int kPencilThreads = 256;
 // shared memory per CTA, so few CTAs fit on an SM; more threads per CTA keep the SM's warps up.
 template <int N1, int N2>
 constexpr int plane_nt() { return N1 > 0 && N1 * N2 >= 40 ? 512 : kPlaneThreads; }
-template <int N1, int N2>
-constexpr int pencil_nt() { return N1 > 0 && N1 * N2 >= 40 ? 512 : kPencilThreads; }
-constexpr int kPencilTileMax = 16;  // p positions per pencil CTA: the largest divisor of n up to this
+template <int N1, int N2, typename C>
+constexpr int pencil_nt() {
+    return sizeof(C) == 16 ? 128 : N1 > 0 && N1 * N2 >= 40 ? 512 : kPencilThreads;
+}
+// p positions per pencil CTA: the largest divisor of n up to this.  complex64: 128-byte rows.  complex128
+// is bound by the FP64 pipe, so it takes small tiles (64-byte rows) that reach every SM also for one
+// system: N = 48, one system, 144 CTAs instead of 48.
+template <typename C> constexpr int pencil_tile_max() { return sizeof(C) == 16 ? 4 : 16; }
 
 template <typename C> struct RTy;
 template <> struct RTy<float2> { using R = float; };
@@ -165,10 +170,11 @@ __device__ __forceinline__ void dft_inv(C* buf, const Lines ln, int n1, int n2, 
 // Planes per CTA of the plane kernels (one: many small CTAs keep every SM busy at the solver's sizes).
 __host__ __device__ __forceinline__ int planes_per_cta(int) { return 1; }
 
-// p positions per pencil CTA: the largest divisor of n that is at most kPencilTileMax (no ragged tile).
+// p positions per pencil CTA: the largest divisor of n that is at most the precision's bound (no ragged tile).
+template <typename C>
 __host__ __device__ constexpr int pencil_tile(int n) {
     int t = 1;
-    for (int d = 1; d <= kPencilTileMax && d <= n; ++d)
+    for (int d = 1; d <= pencil_tile_max<C>() && d <= n; ++d)
         if (n % d == 0) t = d;
     return t;
 }
@@ -314,7 +320,7 @@ __global__ void __launch_bounds__(plane_nt<N1, N2>())
 // mode order [comp][r < 2n][q][p]); 2 = inverse block transform (reads `out`'s layout from W, inverse
 // butterfly, inverse DFT over k', written to W).
 template <int N1, int N2, typename C, typename R, typename TT>
-__global__ void __launch_bounds__(pencil_nt<N1, N2>())
+__global__ void __launch_bounds__(pencil_nt<N1, N2, C>())
     bdft_pencil(C* __restrict__ W, C* __restrict__ out, const C* __restrict__ wn_g, const R* __restrict__ Aref,
                 const TT* __restrict__ ea, const TT* __restrict__ eb, const TT* __restrict__ eg,
                 const int* __restrict__ sys_block, const int* __restrict__ skip, int n_rt, int n1, int n2,
@@ -326,8 +332,8 @@ __global__ void __launch_bounds__(pencil_nt<N1, N2>())
         n2 = N2;
     }
     extern __shared__ __align__(16) unsigned char smem_bdft[];
-    constexpr int PTc = N1 > 0 ? pencil_tile(N1 * N2) : 1;
-    const int PT = N1 > 0 ? PTc : pencil_tile(n);
+    constexpr int PTc = N1 > 0 ? pencil_tile<C>(N1 * N2) : 1;
+    const int PT = N1 > 0 ? PTc : pencil_tile<C>(n);
     C* buf = reinterpret_cast<C*>(smem_bdft);  // [pencil = comp * 2 + par][k'][pl]
     C* wn = buf + 6 * n * PT;
     const int tiles = n / PT;
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(pencil_nt<N1, N2>())
 template <typename C>
 size_t plane_smem(int n) { return sizeof(C) * ((size_t)planes_per_cta(n) * n * n + n); }
 template <typename C>
-size_t pencil_smem(int n) { return sizeof(C) * ((size_t)6 * n * pencil_tile(n) + n); }
+size_t pencil_smem(int n) { return sizeof(C) * ((size_t)6 * n * pencil_tile<C>(n) + n); }
 
 // Dynamic shared memory beyond 48 KB is granted once per kernel (the largest size asked so far).
 template <typename K>
@@ -490,8 +496,8 @@ static int precond_launch(int n, int n1, int n2, int nsys, const V* r, V* z, C* 
     bdft_plane_fwd<N1, N2, C, V><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(r, W, wn, twa, twb, twk, n, n1, n2, planes, vs, vs,
                                                                skip, 0, sys_k, tab_stride);
     note_launch();
-    const int tiles = n / pencil_tile(n);
-    bdft_pencil<N1, N2, C, R, TT><<<nsys * n * tiles, (pencil_nt<N1, N2>()), sq, s>>>(
+    const int tiles = n / pencil_tile<C>(n);
+    bdft_pencil<N1, N2, C, R, TT><<<nsys * n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
         W, nullptr, wn, Aref, ea, eb, eg, sys_block, skip, n, n1, n2, vs, shift_rho, scale, 0, sys_k, tab_stride,
         aref_stride);
     note_launch();
@@ -514,16 +520,16 @@ static int fourier_launch(int n, int n1, int n2, int inverse, const C* in, C* ou
     PC_TRY(allow_smem(bdft_pencil<N1, N2, C, R, C>, sq));
     PC_TRY(allow_smem(bdft_plane_inv<N1, N2, C, C>, sp));
     const int planes = 6 * n, pctas = (planes + planes_per_cta(n) - 1) / planes_per_cta(n);
-    const int tiles = n / pencil_tile(n);
+    const int tiles = n / pencil_tile<C>(n);
     if (!inverse) {
         bdft_plane_fwd<N1, N2, C, C><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(in, W, wn, twa, twb, twk, n, n1, n2, planes, vs,
                                                                    vs, nullptr, 0, nullptr, 0);
         note_launch();
-        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2>()), sq, s>>>(
+        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
             W, out, wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, vs, 0.0, scale, 1, nullptr, 0, 0);
         note_launch();
     } else {
-        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2>()), sq, s>>>(
+        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
             W, const_cast<C*>(in), wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, vs, 0.0, 1.0, 2, nullptr, 0, 0);
         note_launch();
         bdft_plane_inv<N1, N2, C, C><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(W, out, nullptr, wn, twa, twb, twk, n, n1, n2,

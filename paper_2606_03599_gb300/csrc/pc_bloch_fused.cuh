@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(pencil_threads<N1, N2>()) pencil(const __grid_
     const int64_t nb = (int64_t)2 * n * nn;
     float2* __restrict__ Ws = P.W + (int64_t)sys * 3 * nb + c0;
     __syncthreads();
-#pragma unroll 2
+#pragma unroll 3
     for (int g = threadIdx.x; g < 6 * N2 * PT; g += T) {
         const int pl = g % PT, i2 = (g / PT) % N2, pen = g / (PT * N2);
         const float2* __restrict__ src = Ws + (pen >> 1) * nb + (pen & 1) * (nb / 2) + pl;
