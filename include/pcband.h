@@ -44,10 +44,10 @@
  * Threads:   a pc_grid handle must not be used by two threads at once; any
  *            number of handles may coexist.
  * Environment (read once per process; results do not depend on them):
- *            PC_APPLY_KERNEL = legacy | tma | split | row forces one stencil-
- *            kernel family for A/B comparisons (default: the plane-pipelined
- *            kernel for complex64 parity blocks, the integer-pipe kernel for
- *            complex128, or the autotuner's choice); PC_PCG_GRAPHS = 0 turns off CUDA-graph replay of PCG
+ *            PC_APPLY_KERNEL = legacy | tma | split | row | pipe forces one
+ *            stencil-kernel family for A/B comparisons (default: the cell kernel
+ *            for complex64, the integer-pipe kernel for complex128, or the
+ *            autotuner's choice); PC_PCG_GRAPHS = 0 turns off CUDA-graph replay of PCG
  *            iterations; PC_TUNE_CACHE names the autotuner's cache file
  *            (pc_autotune); PC_WAIT_LIMIT = n sets how many polls a kernel's
  *            wait on its own shared-memory copies makes before it gives up
@@ -314,7 +314,7 @@ int pc_set_k_multi(pc_grid* g, int nk, const double* kappas);
 
 /* pc_apply_batch with item i at the Bloch vector of slot kslots[i] (host; NULL = all slot 0):
  * y_i = (A_hat(kappa_{kslots[i]}) - shift_i M_hat) x_i.  The complex128 kernels and the
- * plane-pipelined complex64 kernel serve all slots in one launch; other launch shapes run once
+ * cell and plane-pipelined complex64 kernels serve all slots in one launch; other launch shapes run once
  * per run of equal slots. */
 int pc_apply_batch_k(pc_grid* g, int dtype, int count, const int* blocks, const int* kslots,
                      const void* const* x, void* const* y, const double* shifts, void* stream);
@@ -393,9 +393,10 @@ int pc_autotune(pc_grid* g, int dtype, int layout, int nitems, void* stream);
 
 /* The launch configuration the library will use for a batch of `nitems` vectors of `dtype` in
  * layout 0 (blocks) or 1 (full): kind 0 = fused tile (shapes 0-3 register-staged; shape 8 the
- * integer-pipe kernel, the default for complex128), 1 = TMA tile, 2 = row tile, 3 = two-pass
+ * integer-pipe kernel, the default for complex128; shape 9 the cell kernel, the default for
+ * complex64), 1 = TMA tile, 2 = row tile, 3 = two-pass
  * (fluxes once per node, then gather), 4 = plane-pipelined (producer
- * warp + consumer warps; the default for complex64 parity blocks); tile shape code; planes per CTA
+ * warp + consumer warps); tile shape code; planes per CTA
  * (tz; row and plane-pipelined kernels: least planes per CTA); CTAs of the launch (two-pass: of
  * its gather). */
 int pc_tuned_config(const pc_grid* g, int dtype, int layout, int nitems, int* kind, int* shape, int* tz, int* ctas);

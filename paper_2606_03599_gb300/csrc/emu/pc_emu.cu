@@ -14,6 +14,7 @@
 #include "../pc_apply_pipe.cuh"
 #include "../pc_apply_split.cuh"
 #include "../pc_apply_int.cuh"
+#include "../pc_apply_cell.cuh"
 #include "../pc_limb.cuh"
 #include "../pc_small_dft.cuh"
 
@@ -362,8 +363,8 @@ template <bool CUBIC, int MATK>
 static int emu_run_fix(const StencilParams<double>& P, int block, const void* x, void* y, const void* mat,
                        double shift, int tz, int tx, int ty) {
     using T = FixApply<CUBIC, MATK>;
-    FixGeom G;
-    make_fix_geom(G, P.N, block < 0);
+    CellGeom G;
+    make_cell_geom(G, P.N, block < 0, false);
     if (tx > 0) {
         G.TX = tx < G.X ? tx : G.X;
         G.TY = ty < G.Y ? ty : G.Y;
@@ -371,12 +372,11 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
         G.nty = (G.Y + G.TY - 1) / G.TY;
         G.ncell = (G.TX + 1) * (G.TY + 2);
     }
-    G.tz = tz > 0 && tz < G.Z ? tz : G.Z;
-    G.nch = (G.Z + G.tz - 1) / G.tz;
+    cell_planes(G, tz > 0 ? tz : G.Z);
     FixParams F;
     if (!make_fix_params(F, P, CUBIC, MATK)) return -2;
     const int n = G.ncell;
-    std::vector<unsigned char> mem(T::shared_bytes(G) + 64);
+    std::vector<unsigned char> mem(T::shared_bytes() + 64);
     std::vector<typename T::Regs> regs(n);
     for (int sub = 0; sub < (G.full ? 4 : 1); ++sub)
         for (int blk = 0; blk < G.ntx * G.nty * G.nch; ++blk) {
@@ -384,7 +384,7 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
             unsigned char* base = mem.data();
             while ((uintptr_t)base & 15) ++base;
             typename T::Shared sh;
-            T::carve(sh, base, G);
+            T::carve(sh, base);
             typename T::Ctx c;
             c.F = &F;
             c.G = &G;
@@ -404,38 +404,130 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
             c.p13 = pb & 1;
             for (int t = 0; t < n; ++t) T::load_tables(c, sh, t, n);
             for (int t = 0; t < n; ++t) T::init(c, t, regs[t]);
-            for (int i = 0; i < 3; ++i)
-                for (int t = 0; t < n; ++t) {
-                    T::stage(c, sh, regs[t], t, c.k0 - 2 + i);
-                    T::convert(c, sh, regs[t], t, c.k0 - 2 + i, i);
-                }
-            const int klast = c.k0 + c.tz + 1;
             for (int t = 0; t < n; ++t) {
-                T::stage(c, sh, regs[t], t, c.k0 + 1);
-                regs[t].mcur = T::read_mat(c, regs[t], c.k0 - 1);
+                auto& r = regs[t];
+                T::template stage<0>(c, sh, r, t, c.k0 - 2);
+                T::template convert<0>(c, sh, r, t, c.k0 - 2, 0);
+                T::template stage<1>(c, sh, r, t, c.k0 - 1);
+                T::template convert<1>(c, sh, r, t, c.k0 - 1, 1);
+                T::template stage<0>(c, sh, r, t, c.k0);
+                T::template convert<0>(c, sh, r, t, c.k0, 2);
+                T::template stage<1>(c, sh, r, t, c.k0 + 1);
+                r.mcur = T::template read_mat<1>(c, r, c.k0 - 1);
             }
+            const int klast = c.k0 + c.tz + 1;
             int sm = 0, sc = 1, sp = 2;
-            for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; ++kf) {
+            auto step = [&](auto parity, int kf) {
+                constexpr int Q = decltype(parity)::value;
                 for (int t = 0; t < n; ++t) {
-                    if (kf < c.k0 + c.tz) regs[t].mnext = T::read_mat(c, regs[t], kf + 1);
-                    T::flux(c, sh, regs[t], t, kf, sm, sc, sp);
-                    T::load_own(c, regs[t], kf);
+                    if (kf < c.k0 + c.tz) regs[t].mnext = T::template read_mat<1 - Q>(c, regs[t], kf + 1);
+                    T::template flux<Q>(c, sh, regs[t], kf, sm, sc, sp);
+                    T::template load_own<Q>(c, regs[t], kf);
                 }
                 for (int t = 0; t < n; ++t) {
-                    T::gather(c, sh, regs[t], kf);
-                    if (kf + 2 <= klast) T::convert(c, sh, regs[t], t, kf + 2, sm);
-                    if (kf + 3 <= klast) T::stage(c, sh, regs[t], t, kf + 3);
+                    T::template gather<Q>(c, sh, regs[t], kf);
+                    if (kf + 2 <= klast) T::template convert<Q>(c, sh, regs[t], t, kf + 2, sm);
+                    if (kf + 3 <= klast) T::template stage<1 - Q>(c, sh, regs[t], t, kf + 3);
                     T::next_mat(regs[t]);
                 }
                 const int t = sm;
                 sm = sc;
                 sc = sp;
                 sp = t;
+            };
+            for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; kf += 2) {
+                step(std::integral_constant<int, 1>(), kf);
+                step(std::integral_constant<int, 0>(), kf + 1);
             }
             for (int t = 0; t < n; ++t)
                 if (regs[t].ks < c.k0 + c.tz) T::slow_column(c, regs[t].ks, regs[t].off[0], regs[t].off[1]);
         }
     return 0;
+}
+
+// Same step sequence as cell_apply; shared memory poisoned with NaN first.
+template <bool CUBIC, int MATK>
+static int emu_run_cell(const StencilParams<float>& P, int block, const void* x, void* y, const void* mat,
+                        double shift, int tz, int tx, int ty) {
+    using T = CellApply<CUBIC, MATK>;
+    CellGeom G;
+    make_cell_geom(G, P.N, block < 0, true);
+    if (tx > 0) {
+        G.TX = tx < G.X ? tx : G.X;
+        G.TY = ty < G.Y ? ty : G.Y;
+        G.ntx = (G.X + G.TX - 1) / G.TX;
+        G.nty = (G.Y + G.TY - 1) / G.TY;
+        G.ncell = (G.TX + 1) * (G.TY + 2);
+    }
+    cell_planes(G, tz > 0 ? tz : G.Z);
+    const int n = G.ncell;
+    std::vector<float4> mem(T::shared_bytes() / sizeof(float4));
+    std::vector<typename T::Regs> regs(n);
+    for (int sub = 0; sub < (G.full ? 4 : 1); ++sub)
+        for (int blk = 0; blk < G.ntx * G.nty * G.nch; ++blk) {
+            std::memset((void*)mem.data(), 0xFF, sizeof(float4) * mem.size());
+            typename T::Shared sh;
+            T::carve(sh, mem.data());
+            typename T::Ctx c;
+            c.P = &P;
+            c.G = &G;
+            c.kph = P.ph;
+            c.x = static_cast<const float2*>(x);
+            c.y = static_cast<float2*>(y);
+            c.mat = mat;
+            c.shift = (float)shift;
+            c.dot = true;
+            const int tiles = G.ntx * G.nty, tile = blk % tiles;
+            c.a0 = (tile % G.ntx) * G.TX;
+            c.b0 = (tile / G.ntx) * G.TY;
+            c.k0 = (blk / tiles) * G.tz;
+            c.tz = G.tz < G.Z - c.k0 ? G.tz : G.Z - c.k0;
+            const int pb = G.full ? sub : block;
+            c.p12 = pb >> 1;
+            c.p13 = pb & 1;
+            const int kfirst = c.k0 - 2, klast = c.k0 + c.tz + 1;
+            for (int t = 0; t < n; ++t) T::load_tables(c, sh, t, n);
+            for (int t = 0; t < n; ++t) T::init(c, t, regs[t]);
+            for (int t = 0; t < n; ++t) {
+                auto& r = regs[t];
+                T::template stage<0>(c, sh, r, kfirst, 0);
+                T::template stage<1>(c, sh, r, kfirst + 1, 1);
+                T::template stage<0>(c, sh, r, kfirst + 2, 2);
+                T::template stage<1>(c, sh, r, kfirst + 3, 3);
+                T::template settle<0>(c, sh, r, kfirst, 0);
+                T::template settle<1>(c, sh, r, kfirst + 1, 1);
+                T::template settle<0>(c, sh, r, kfirst + 2, 2);
+                r.mcur = T::template read_mat<1>(c, r, c.k0 - 1);
+            }
+            auto step = [&](auto parity, int kf, int j) {
+                constexpr int Q = decltype(parity)::value;
+                const int sm = j & 3, sn = (j + 3) & 3;
+                for (int t = 0; t < n; ++t) {
+                    if (kf < c.k0 + c.tz) regs[t].mnext = T::template read_mat<1 - Q>(c, regs[t], kf + 1);
+                    T::template flux<Q>(c, sh, regs[t], sm, (j + 1) & 3, (j + 2) & 3);
+                }
+                for (int t = 0; t < n; ++t) {
+                    T::template gather<Q>(c, sh, regs[t], kf, sm);
+                    if (kf + 3 <= klast) T::template stage<1 - Q>(c, sh, regs[t], kf + 3, sm);
+                    if (kf + 2 <= klast) T::template settle<Q>(c, sh, regs[t], kf + 2, sn);
+                    regs[t].mcur = regs[t].mnext;
+                }
+            };
+            for (int kf = c.k0 - 1, j = 0; kf <= c.k0 + c.tz; kf += 2, j += 2) {
+                step(std::integral_constant<int, 1>(), kf, j);
+                step(std::integral_constant<int, 0>(), kf + 1, j + 1);
+            }
+        }
+    return 0;
+}
+
+static int emu_cell(bool cubic, int matkind, const StencilParams<float>& P, int block, const void* x, void* y,
+                    const void* mat, double shift, int tz, int tx, int ty) {
+    if (cubic)
+        return matkind ? emu_run_cell<true, 1>(P, block, x, y, mat, shift, tz, tx, ty)
+                       : emu_run_cell<true, 0>(P, block, x, y, mat, shift, tz, tx, ty);
+    return matkind ? emu_run_cell<false, 1>(P, block, x, y, mat, shift, tz, tx, ty)
+                   : emu_run_cell<false, 0>(P, block, x, y, mat, shift, tz, tx, ty);
 }
 
 static int emu_fix(bool cubic, int matkind, const StencilParams<double>& P, int block, const void* x, void* y,
@@ -490,6 +582,9 @@ extern "C" int pc_emu_apply(int N, int block, int dtype, int shape, int tz, cons
     if (dtype == PC_C64) {
         StencilParams<float> P;
         make_stencil_params(P, Chat, rhohat2, ainv9, cubic != 0, N, phi3, X, Y, Z);
+        if (shape == 60 || shape > 6000)  // cell kernel (tiles as the integer-pipe kernel's codes)
+            return emu_cell(cubic != 0, matkind, P, block, x, y, mat, shift, tz, shape > 6000 ? shape / 10 % 100 : 0,
+                            shape > 6000 ? shape % 10 : 0);
         if (shape == 20 || shape == 21) {  // row-tile kernel (21: compile-time width), tz = persistent CTAs
             if (full) return -1;
             const bool ct = shape == 21;

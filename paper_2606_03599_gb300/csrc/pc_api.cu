@@ -32,12 +32,12 @@ int tile_ty(int shape) { return shape <= 2 ? 8 : 4; }
 static int apply_kernel_mode() {
     // PC_APPLY_KERNEL=legacy selects the register-staged kernel everywhere, =tma the TMA tile
     // kernel in place of the plane-pipelined kernel, =split the two-pass kernels for both
-    // precisions, =row the row-tile kernel (A/B comparisons)
+    // precisions, =row the row-tile and =pipe the plane-pipelined kernel (A/B comparisons)
     static int mode = -1;
     if (mode < 0) {
         const char* v = std::getenv("PC_APPLY_KERNEL");
         const std::string m = v ? v : "";
-        mode = m == "legacy" ? 1 : (m == "tma" ? 2 : (m == "split" ? 3 : (m == "row" ? 4 : 0)));
+        mode = m == "legacy" ? 1 : (m == "tma" ? 2 : (m == "split" ? 3 : (m == "row" ? 4 : (m == "pipe" ? 5 : 0))));
     }
     return mode;
 }
@@ -83,9 +83,9 @@ int device_sm_count() {
 }
 
 ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks, int matkind, bool scratch_ok,
-                                bool int_ok) {
+                                bool int_ok, bool cubic) {
     ApplyConfig c;
-    if (int_ok && dtype == PC_C128 && apply_kernel_mode() == 0) {
+    if (int_ok && dtype == PC_C128 && (apply_kernel_mode() == 0 || apply_kernel_mode() == 5)) {
         // the FP64 pipe of GB300 (2 lanes per clock and SM) is left to the integer units; see
         // pc_apply_int.cuh
         c.fix = true;
@@ -93,7 +93,7 @@ ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool
         c.ctas = fix_apply_ctas(Z, !blocks, nitems, 0, &c.tz);
         return c;
     }
-    if (scratch_ok && ((dtype == PC_C128 && (apply_kernel_mode() == 0 || matkind == 2)) || apply_kernel_mode() == 3)) {
+    if (scratch_ok && ((dtype == PC_C128 && (apply_kernel_mode() == 0 || apply_kernel_mode() == 5 || matkind == 2)) || apply_kernel_mode() == 3)) {
         // complex128 is bound by GB300's FP64 pipe: fluxes once per node (two-pass kernels)
         c.split = true;
         c.shape = 0;
@@ -101,7 +101,19 @@ ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool
         c.ctas = split_apply_ctas((int64_t)X * Y * Z);
         return c;
     }
-    if (apply_kernel_mode() == 0 && blocks && dtype == PC_C64 && pipe_geom_ok(X, Y, Z, matkind)) {
+    // complex64: the cell kernel, except for several block vectors at the widest width that the plane-
+    // pipelined kernel has compiled in (N = 160, 4 items: 103 us against 107 us, 2 items 56.6 against 57.5;
+    // one item: 35.8 against 32.9; N = 128, 4 items: 60.5 against 56.4; sizes without a compiled width take
+    // it 1.6 to 5 times as long, e.g. N = 60, 64 items: 203 against 120 us)
+    const bool pipe_width = blocks && cubic && matkind == 0 && X == 80 && nitems >= 2 && pipe_geom_ok(X, Y, Z, matkind);
+    if (apply_kernel_mode() == 0 && scratch_ok && dtype == PC_C64 && matkind != 2 && !pipe_width) {
+        c.cell = true;
+        c.shape = kCellShape;
+        c.ctas = cell_apply_ctas(Z, !blocks, nitems, 0, &c.tz);
+        return c;
+    }
+    if ((apply_kernel_mode() == 0 || apply_kernel_mode() == 5) && blocks && dtype == PC_C64 &&
+        pipe_geom_ok(X, Y, Z, matkind)) {
         // plane-pipelined kernel: persistent, whole rows per tile, producer warp + consumer warps
         c.pipe = true;
         c.shape = 0;
@@ -507,6 +519,9 @@ static int apply_launch(pc_grid* g, int dtype, bool full, const ApplyConfig& cfg
     if (cfg.fix)
         return launch_apply_fix(full, g->cubic, g->matkind, params_at(g, g->P64, X, Y, Z, slot), items, item_ph, nitems,
                                 cfg.tz, dot_partials, dot_stride, s);
+    if (cfg.cell)
+        return launch_apply_cell(full, g->cubic, g->matkind, params_at(g, g->P32, X, Y, Z, slot), items, item_ph, nitems,
+                                 cfg.tz, dot_partials, dot_stride, g->d_err, s);
     if (cfg.split) {
         const size_t need = split_scratch_bytes(X, Y, Z, nitems, dtype);
         if (g->split_bytes < need) {
@@ -567,7 +582,7 @@ int grid_apply(pc_grid* g, int dtype, bool full, const ApplyItem* items, int nit
     }
     void* th = timing_enabled() ? timing_begin(s) : nullptr;
     int rc = PC_OK;
-    const bool per_item = cfg.split || cfg.fix || (dtype == PC_C64 && cfg.pipe);
+    const bool per_item = cfg.split || cfg.fix || cfg.cell || (dtype == PC_C64 && cfg.pipe);
     if (uniform || per_item) {
         rc = apply_launch(g, dtype, full, cfg, items, iph.data(), nitems, nitems ? items[0].kslot : 0, dot_partials,
                           dot_stride, s);

@@ -1,5 +1,6 @@
 // Integer-pipe complex128 stencil apply (see pc_apply_int.cuh): kernel and launcher.
 #include <algorithm>
+#include <type_traits>
 
 #include "pc_apply_int.cuh"
 
@@ -17,8 +18,8 @@ struct FixBatch {
 
 // blockIdx.x = (tile, chunk of planes), blockIdx.y = item (full space: item * 4 + parity block).
 template <bool CUBIC, int MATK>
-__global__ void __launch_bounds__(kFixCells, 2)
-    fix_apply(const __grid_constant__ FixParams F, const __grid_constant__ FixBatch B, const __grid_constant__ FixGeom G,
+__global__ void __launch_bounds__(kCells, 2)
+    fix_apply(const __grid_constant__ FixParams F, const __grid_constant__ FixBatch B, const __grid_constant__ CellGeom G,
               double* __restrict__ dot_partials, int dot_stride) {
     using T = FixApply<CUBIC, MATK>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -26,7 +27,7 @@ __global__ void __launch_bounds__(kFixCells, 2)
     const ApplyItem& it = B.it[item];
     if (it.skip != nullptr && *it.skip) return;
     typename T::Shared sh;
-    T::carve(sh, smem_raw, G);
+    T::carve(sh, smem_raw);
     const int tid = threadIdx.x, n = G.ncell;
     const bool live = tid < n;
     typename T::Ctx c;
@@ -52,41 +53,40 @@ __global__ void __launch_bounds__(kFixCells, 2)
     T::init(c, min(tid, n - 1), r);
     if (!live) r.flags = 0;
     const int klast = c.k0 + c.tz + 1;  // last plane of x
-    if (live) {
-        // the first three planes go through the flux cells, which nothing uses yet
+    // the first three planes go through the flux cells, which nothing uses yet; k0 is even, so planes
+    // k0 - 2 .. k0 + 1 have parities 0, 1, 0, 1
+    typename T::Shared pre[3] = {sh, sh, sh};
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            typename T::Shared t = sh;
-            t.raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * n;
-            T::stage(c, t, r, tid, c.k0 - 2 + i);
-        }
-        T::stage(c, sh, r, tid, c.k0 + 1);
-        r.mcur = T::read_mat(c, r, c.k0 - 1);
+    for (int i = 0; i < 3; ++i) pre[i].raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * kCells;
+    if (live) {
+        T::template stage<0>(c, pre[0], r, tid, c.k0 - 2);
+        T::template stage<1>(c, pre[1], r, tid, c.k0 - 1);
+        T::template stage<0>(c, pre[2], r, tid, c.k0);
+        T::template stage<1>(c, sh, r, tid, c.k0 + 1);
+        r.mcur = T::template read_mat<1>(c, r, c.k0 - 1);
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();  // phase table
     if (live) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            typename T::Shared t = sh;
-            t.raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * n;
-            T::convert(c, t, r, tid, c.k0 - 2 + i, i);
-        }
+        T::template convert<0>(c, pre[0], r, tid, c.k0 - 2, 0);
+        T::template convert<1>(c, pre[1], r, tid, c.k0 - 1, 1);
+        T::template convert<0>(c, pre[2], r, tid, c.k0, 2);
     }
     __syncthreads();
     int sm = 0, sc = 1, sp = 2;
-    for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; ++kf) {
+    auto step = [&](auto parity, int kf) {
+        constexpr int Q = decltype(parity)::value;
         if (live) {
-            if (kf < c.k0 + c.tz) r.mnext = T::read_mat(c, r, kf + 1);
-            T::flux(c, sh, r, tid, kf, sm, sc, sp);
-            T::load_own(c, r, kf);
+            if (kf < c.k0 + c.tz) r.mnext = T::template read_mat<1 - Q>(c, r, kf + 1);
+            T::template flux<Q>(c, sh, r, kf, sm, sc, sp);
+            T::template load_own<Q>(c, r, kf);
         }
         __syncthreads();
-        T::gather(c, sh, r, kf);
+        T::template gather<Q>(c, sh, r, kf);
         if (kf + 2 <= klast && live) {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
-            T::convert(c, sh, r, tid, kf + 2, sm);
-            if (kf + 3 <= klast) T::stage(c, sh, r, tid, kf + 3);
+            T::template convert<Q>(c, sh, r, tid, kf + 2, sm);
+            if (kf + 3 <= klast) T::template stage<1 - Q>(c, sh, r, tid, kf + 3);
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
         T::next_mat(r);
@@ -95,6 +95,10 @@ __global__ void __launch_bounds__(kFixCells, 2)
         sm = sc;
         sc = sp;
         sp = t;
+    };
+    for (int kf = c.k0 - 1; kf <= c.k0 + c.tz; kf += 2) {
+        step(std::integral_constant<int, 1>(), kf);
+        step(std::integral_constant<int, 0>(), kf + 1);
     }
     if (r.ks < c.k0 + c.tz) r.dot += T::slow_column(c, r.ks, r.off[0], r.off[1]);
     if (c.dot) {
@@ -113,10 +117,10 @@ __global__ void __launch_bounds__(kFixCells, 2)
 }
 
 template <bool CUBIC, int MATK>
-int launch_fix_t(const FixParams& F, const FixBatch& B, const FixGeom& G, double* dp, int ds, cudaStream_t s) {
+int launch_fix_t(const FixParams& F, const FixBatch& B, const CellGeom& G, double* dp, int ds, cudaStream_t s) {
     using T = FixApply<CUBIC, MATK>;
     auto kern = fix_apply<CUBIC, MATK>;
-    const size_t smem = T::shared_bytes(G);
+    const size_t smem = T::shared_bytes();
     // the largest tile's need, set on every launch: an attribute of the kernel on the current device
     PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 << 10));
     const dim3 grid(G.ntx * G.nty * G.nch, B.n * (G.full ? 4 : 1));
@@ -127,35 +131,16 @@ int launch_fix_t(const FixParams& F, const FixBatch& B, const FixGeom& G, double
     return PC_OK;
 }
 
-// Chunks of planes per tile.  A chunk repeats two flux planes and loads three more of x, so few
-// chunks are best once every SM has work; below that more CTAs shorten the march.
-void fix_chunks(FixGeom& G, int nitems) {
-    const long base = (long)G.ntx * G.nty * (G.full ? 4 : 1) * std::max(nitems, 1);
-    const int sm = device_sm_count();
-    double best = -1;
-    for (int nch = 1; nch <= std::max(1, G.Z / 2); ++nch) {
-        const int tz = (G.Z + nch - 1) / nch;
-        if ((G.Z + tz - 1) / tz != nch) continue;
-        const long per = (base * nch + sm - 1) / sm;  // CTAs of the fullest SM
-        const double cost = (per == 1 ? 1.0 : 0.75 * per) * (tz + 4);
-        if (best < 0 || cost < best) {
-            best = cost;
-            G.tz = tz;
-            G.nch = nch;
-        }
-    }
-}
-
 }  // namespace
 
 int fix_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz) {
-    FixGeom G;
-    make_fix_geom(G, N, full);
+    CellGeom G;
+    make_cell_geom(G, N, full, false);
     if (tz_in > 0) {
-        G.tz = std::min(tz_in, G.Z);
-        G.nch = (G.Z + G.tz - 1) / G.tz;
+        cell_planes(G, tz_in);
     } else {
-        fix_chunks(G, std::min(nitems, kFixMaxItems));
+        const double rate[2] = {1.0, 1.8};
+        cell_chunks(G, std::min(nitems, kFixMaxItems), device_sm_count(), rate, 2);
     }
     if (tz) *tz = G.tz;
     return G.ntx * G.nty * G.nch * (full ? 4 : 1);
@@ -168,10 +153,9 @@ bool fix_apply_ok(const StencilParams<double>& P, bool cubic, int matkind) {
 
 int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<double>& P, const ApplyItem* items,
                      const double* item_ph, int nitems, int tz, double* dp, int ds, cudaStream_t s) {
-    FixGeom G;
-    make_fix_geom(G, P.N, full);
-    G.tz = std::max(1, std::min(tz, G.Z));
-    G.nch = (G.Z + G.tz - 1) / G.tz;
+    CellGeom G;
+    make_cell_geom(G, P.N, full, false);
+    cell_planes(G, tz);
     if (dp != nullptr && G.ntx * G.nty * G.nch * (full ? 4 : 1) > ds)
         return fail(PC_EINVAL, "apply: launch has more CTAs than partial-sum slots");
     FixParams F;

@@ -19,12 +19,9 @@
 // vector is treated as its four parity blocks with strided addresses (the blocks do not couple), so
 // one geometry serves both layouts.
 //
-// Tile.  A CTA owns TX x TY columns of the quarter grid and marches through tz planes.  Thread
-// cells: the TX x TY output columns first, then the column at a0 + TX or a0 - 1 (by the plane's
-// parity), the row b0 + TY and the row b0 - 1.  Each cell is one thread: it stages x of its column
-// (asynchronous copy, Bloch phase if wrapped, conversion), forms the fluxes of its column when the
-// plane's parity needs them, and the first TX x TY finish the outputs.  Whatever wraps around the
-// cell sits in the last warps, so the FP64 phase products are not spread over all of them.
+// The tile and its march are pc_apply_cells.cuh's: each cell is one thread, which stages x of its
+// column (asynchronous copy, Bloch phase if wrapped, conversion), forms the fluxes of its column when
+// the plane's parity needs them, and, among the first TX x TY, finishes the outputs.
 //
 // Measured (one GB300, N = 48, 64 block vectors, shift on): 0.205 ms against 0.667 ms of the two-pass
 // FP64 kernels; N = 60 FCC sub-pixel material, four blocks: 0.084 against 0.195 ms; N = 64 nodewise
@@ -39,6 +36,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "pc_apply_cells.cuh"
 #include "pc_apply_tile.cuh"  // PC_IDX
 #include "pc_complex.cuh"
 #include "pc_internal.h"
@@ -51,17 +49,8 @@
 
 namespace pc {
 
-constexpr int kFixCells = 256;       // most cells (threads) of a CTA
 constexpr int kFixSpecial = 1 << 14;  // exponent of a node that FP64 has to handle
 constexpr int kFixLow = 200, kFixHigh = 1900;  // biased exponents the integer path takes
-
-struct FixGeom {
-    int X, Y, Z;   // quarter-grid extents (N/2, N/2, N)
-    int N, full;   // full-space layout: addresses of the full grid
-    int TX, TY, ntx, nty, ncell;
-    int tz, nch;
-    int plane, vstr;  // nodes per plane and per component of the vector layout (N <= 1024: below 2^31)
-};
 
 struct FixHalf {
     int hi, lo;  // c = hi 2^32 + lo, lo signed
@@ -133,39 +122,6 @@ inline bool make_fix_params(FixParams& F, const StencilParams<double>& P, bool c
     for (int p = 0; p < 2; ++p)
         if (F.coff[p] + F.moff > 100 || F.coff[p] + F.moff < -100) return false;
     return true;
-}
-
-// Tile extents: least warps over the whole plane with at most kFixCells cells per CTA (ties: the
-// larger tile).  CTAs and planes per CTA: see fix_chunks.
-inline void make_fix_geom(FixGeom& G, int N, bool full) {
-    G.N = N;
-    G.full = full ? 1 : 0;
-    G.X = N / 2;
-    G.Y = N / 2;
-    G.Z = N;
-    G.plane = full ? N * N : G.X * G.Y;
-    G.vstr = G.plane * N;
-    long best = -1;
-    for (int nx = 1; nx <= G.X; ++nx) {
-        const int tx = (G.X + nx - 1) / nx, most = kFixCells / (tx + 1) - 2;
-        if (most < 1) continue;
-        const int ny0 = (G.Y + most - 1) / most;
-        for (int ny = ny0; ny <= G.Y && ny < ny0 + 3; ++ny) {
-            const int ty = (G.Y + ny - 1) / ny;
-            const int cells = (tx + 1) * (ty + 2);
-            const long cost = (long)nx * ny * ((cells + 31) / 32);
-            if (best < 0 || cost < best) {
-                best = cost;
-                G.TX = tx;
-                G.TY = ty;
-                G.ntx = (G.X + tx - 1) / tx;
-                G.nty = (G.Y + ty - 1) / ty;
-                G.ncell = cells;
-            }
-        }
-    }
-    G.tz = G.Z;
-    G.nch = 1;
 }
 
 PC_HD longlong2 fix_ashr2(longlong2 v, int s) {
@@ -273,19 +229,19 @@ PC_HD int64_t fix_theta(float t) {
 template <bool CUBIC, int MATK>
 struct FixApply {
     struct Shared {
-        longlong2* xs;  // [3 slots][3][ncell]
-        longlong2* fs;  // [12][ncell]: F_l of component c at l * 3 + c
-        double2* raw;   // [3][ncell]: the next plane of x, as read
+        longlong2* xs;  // [3 slots][3][kCells]
+        longlong2* fs;  // [12][kCells]: F_l of component c at l * 3 + c
+        double2* raw;   // [3][kCells]: the next plane of x, as read
         double2* ph;    // [27] Bloch phases of the wraps (wa, wb, wk)
         FixHalf* c;     // [2][21]
-        int* xe;        // [3][ncell]
-        int* fe;        // [ncell]
+        int* xe;        // [3][kCells]
+        int* fe;        // [kCells]
     };
-    static inline size_t shared_bytes(const FixGeom& G) {
-        return (size_t)G.ncell * (16 * (9 + 12 + 3) + 4 * 4) + 16 * 27 + sizeof(FixHalf) * 42;
+    static constexpr size_t shared_bytes() {
+        return (size_t)kCells * (16 * (9 + 12 + 3) + 4 * 4) + 16 * 27 + sizeof(FixHalf) * 42;
     }
-    static PC_HD void carve(Shared& sh, unsigned char* p, const FixGeom& G) {
-        const int n = G.ncell;
+    static PC_HD void carve(Shared& sh, unsigned char* p) {
+        constexpr int n = kCells;
         sh.xs = reinterpret_cast<longlong2*>(p);
         sh.fs = sh.xs + 9 * n;
         sh.raw = reinterpret_cast<double2*>(sh.fs + 12 * n);
@@ -297,7 +253,7 @@ struct FixApply {
 
     struct Ctx {
         const FixParams* F;
-        const FixGeom* G;
+        const CellGeom* G;
         const double (*kph)[2];
         const double2* x;
         double2* y;
@@ -306,12 +262,7 @@ struct FixApply {
         bool dot;
         int a0, b0, k0, tz, p12, p13;
     };
-    struct Regs {
-        int off[2];  // in-plane offset of the cell's node, by plane parity
-        int wab[2];  // (wa + 1) + 3 (wb + 1) of that node
-        int nb[2];   // backward neighbour cells, s2 = +1 low half, -1 high half (flux)
-        int gn[2];   // forward flux cells, s2 = +1 low half, -1 high half (gather)
-        int flags;   // bit 0, 1: flux on even, odd planes; bit 2: output
+    struct Regs : CellMap {
         int mprev, mcur, mnext;  // material of planes kf - 1, kf, kf + 1 (id, or the float's bits)
         longlong2 pv[3], cv[3];  // y(kf - 1) and y(kf) so far
         int pe, ce;
@@ -320,53 +271,10 @@ struct FixApply {
         double dot;
     };
 
-    static PC_HD int wrap1(int v, int n, int& w) {
-        w = v < 0 ? -1 : (v >= n ? 1 : 0);
-        return v - w * n;
-    }
-    // cell of tile coordinates (cx in [0, TX], row r in [-1, TY])
-    static PC_HD int cell_of(const FixGeom& G, int cx, int r) {
-        const int main = G.TX * G.TY;
-        if (r >= 0 && r < G.TY) return cx < G.TX ? r * G.TX + cx : main + r;
-        return main + G.TY + (r < 0 ? G.TX + 1 : 0) + cx;
-    }
+    static PC_HD int wrap1(int v, int n, int& w) { return cell_wrap(v, n, w); }
 
     static PC_HD void init(const Ctx& c, int tid, Regs& r) {
-        const FixGeom& G = *c.G;
-        const int main = G.TX * G.TY;
-        int cx, row;
-        if (tid < main) {
-            row = tid / G.TX;
-            cx = tid - row * G.TX;
-        } else if (tid < main + G.TY) {
-            cx = G.TX;
-            row = tid - main;
-        } else {
-            const int e = tid - main - G.TY;
-            row = e > G.TX ? -1 : G.TY;
-            cx = e > G.TX ? e - (G.TX + 1) : e;
-        }
-        r.flags = 0;
-        if (tid < main && c.a0 + cx < G.X && c.b0 + row < G.Y) r.flags |= 4;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int i0 = (q + c.p13) & 1, j0 = (q + c.p12 + c.p13) & 1;
-            int wa, wb;
-            const int a = wrap1(c.a0 + ((cx == G.TX && i0) ? -1 : cx), G.X, wa);
-            const int b = wrap1(c.b0 + row, G.Y, wb);
-            r.off[q] = G.full ? (2 * a + i0) + G.N * (2 * b + j0) : a + G.X * b;
-            r.wab[q] = (wa + 1) + 3 * (wb + 1);
-            // fluxes: columns a0 .. a0 + TX - i0, rows b0 - j0 .. b0 + TY - j0
-            const bool f = (cx < G.TX || !i0) && row >= -j0 && row <= G.TY - j0;
-            if (f) r.flags |= 1 << q;
-            r.nb[q] = 0;
-            if (f) {
-                const int ncx = i0 ? cx : (cx > 0 ? cx - 1 : G.TX);
-                r.nb[q] = cell_of(G, ncx, row + j0 - 1) | (cell_of(G, ncx, row + j0) << 16);
-            }
-            r.gn[q] = 0;
-            if (tid < main) r.gn[q] = cell_of(G, cx + i0, row + j0) | (cell_of(G, cx + i0, row + j0 - 1) << 16);
-        }
+        cell_init(*c.G, c.a0, c.b0, c.p12, c.p13, tid, r);
         r.pe = r.ce = 0;
         r.ks = 1 << 30;
 #pragma unroll
@@ -389,17 +297,18 @@ struct FixApply {
         }
     }
 
-    // Start the copy of plane kp of x into the staging cells (a cell is read by its own thread only).
+    // Start the copy of plane kp (parity Q) of x into the staging cells (a cell is read by its own thread only).
+    template <int Q>
     static PC_HD void stage(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp) {
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         int wk;
         const int k = wrap1(kp, G.Z, wk);
-        const int at = k * G.plane + ((kp & 1) ? r.off[1] : r.off[0]);
+        const int at = k * G.plane + r.off[Q];
         PC_IDX(at, G.vstr);
         PC_IDX(tid, G.ncell);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            double2* d = sh.raw + a * G.ncell + tid;
+            double2* d = sh.raw + a * kCells + tid;
             const double2* s = c.x + at + (int64_t)a * G.vstr;
 #if defined(__CUDA_ARCH__)
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(s)
@@ -411,14 +320,15 @@ struct FixApply {
     }
 
     // Plane kp from the staging cells into slot sl: phase, exponent, integers.
+    template <int Q>
     static PC_HD void convert(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp, int sl) {
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         int wk;
         wrap1(kp, G.Z, wk);
-        const int w = ((kp & 1) ? r.wab[1] : r.wab[0]) + 9 * (wk + 1);
+        const int w = r.wab[Q] + 9 * (wk + 1);
         double2 v[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) v[a] = sh.raw[a * G.ncell + tid];
+        for (int a = 0; a < 3; ++a) v[a] = sh.raw[a * kCells + tid];
         if (w != 13) {
             const double2 ph = sh.ph[w];
 #pragma unroll
@@ -433,23 +343,24 @@ struct FixApply {
             base = 64;
             E = any ? kFixSpecial : 0;
         }
-        longlong2* xs = sh.xs + (int64_t)sl * 3 * G.ncell + tid;
+        longlong2* xs = sh.xs + sl * 3 * kCells + r.own[Q];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             longlong2 o;
             o.x = E == 0 ? 0 : fix_from_double(v[a].x, base, 3);
             o.y = E == 0 ? 0 : fix_from_double(v[a].y, base, 3);
-            xs[a * G.ncell] = o;
+            xs[a * kCells] = o;
         }
-        sh.xe[sl * G.ncell + tid] = E;
+        sh.xe[sl * kCells + r.own[Q]] = E;
     }
 
+    template <int Q>
     static PC_HD int read_mat(const Ctx& c, const Regs& r, int kp) {
         if (MATK == 2) return 0;
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         int wk;
         const int k = wrap1(kp, G.Z, wk);
-        const int at = k * G.plane + ((kp & 1) ? r.off[1] : r.off[0]);
+        const int at = k * G.plane + r.off[Q];
         PC_IDX(at, G.vstr);
         if (MATK == 0) return static_cast<const uint8_t*>(c.mat)[at];
 #if defined(__CUDA_ARCH__)
@@ -487,32 +398,34 @@ struct FixApply {
         }
     }
 
-    // Fluxes of plane kf at the thread's column; -4 P_0 into y(kf).  sm, sc, sp: slots of planes
+    // Fluxes of plane kf (parity Q) at the thread's column; -4 P_0 into y(kf).  sm, sc, sp: slots of planes
     // kf - 1, kf, kf + 1.
-    static PC_HD void flux(const Ctx& c, Shared& sh, Regs& r, int tid, int kf, int sm, int sc, int sp) {
-        const FixGeom& G = *c.G;
-        const int q = kf & 1, n = G.ncell;
-        if (!((r.flags >> q) & 1)) return;
-        const int nb = q ? r.nb[1] : r.nb[0];
-        const int n0 = nb & 0xffff, n1 = nb >> 16;
-        PC_IDX(n0, n);
-        PC_IDX(n1, n);
-        const int eo = sh.xe[sc * n + tid];
+    template <int Q>
+    static PC_HD void flux(const Ctx& c, Shared& sh, Regs& r, int kf, int sm, int sc, int sp) {
+        const CellGeom& G = *c.G;
+        constexpr int n = kCells;
+        if (!((r.flags >> Q) & 1)) return;
+        const int n0 = r.nb[Q] & 0xffff, n1 = r.nb[Q] >> 16, own = r.own[Q];
+        PC_IDX(n0, G.ncell);
+        PC_IDX(n1, G.ncell);
+        const int eo = sh.xe[sc * n + own];
         const int e0 = sh.xe[sm * n + n0], e1 = sh.xe[sp * n + n0], e2 = sh.xe[sm * n + n1], e3 = sh.xe[sp * n + n1];
         const int E = imax(imax(imax(e0, e1), imax(e2, e3)), eo);
         if (E >= kFixSpecial) {
-            sh.fe[tid] = kFixSpecial;
+            sh.fe[own] = kFixSpecial;
             r.ce = kFixSpecial;
             return;
         }
         const int s0 = imin(E - e0, 63), s1 = imin(E - e1, 63), s2 = imin(E - e2, 63), s3 = imin(E - e3, 63),
                   so = imin(E - eo, 63);
+        const longlong2 *p0 = sh.xs + sm * 3 * n + n0, *p1 = sh.xs + sp * 3 * n + n0, *p2 = sh.xs + sm * 3 * n + n1,
+                        *p3 = sh.xs + sp * 3 * n + n1, *po = sh.xs + sc * 3 * n + own;
         longlong2 H[3][3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const longlong2 v0 = fix_ashr2(sh.xs[(sm * 3 + a) * n + n0], s0), v1 = fix_ashr2(sh.xs[(sp * 3 + a) * n + n0], s1);
-            const longlong2 v2 = fix_ashr2(sh.xs[(sm * 3 + a) * n + n1], s2), v3 = fix_ashr2(sh.xs[(sp * 3 + a) * n + n1], s3);
-            const longlong2 vo = fix_ashr2(sh.xs[(sc * 3 + a) * n + tid], so);
+            const longlong2 v0 = fix_ashr2(p0[a * n], s0), v1 = fix_ashr2(p1[a * n], s1);
+            const longlong2 v2 = fix_ashr2(p2[a * n], s2), v3 = fix_ashr2(p3[a * n], s3);
+            const longlong2 vo = fix_ashr2(po[a * n], so);
             const int64_t ux = v0.x + v1.x, uy = v0.y + v1.y, vx = v2.x + v3.x, vy = v2.y + v3.y;
             H[0][a].x = ux + vx - 4 * vo.x;
             H[0][a].y = uy + vy - 4 * vo.y;
@@ -575,7 +488,7 @@ struct FixApply {
                 fe += c.F->coff[0];
             } else {
                 int wk;
-                const int at = wrap1(kf, G.Z, wk) * G.plane + (q ? r.off[1] : r.off[0]);
+                const int at = wrap1(kf, G.Z, wk) * G.plane + r.off[Q];
                 md = static_cast<const double*>(c.mat) + at;
                 int top = 0;
 #pragma unroll
@@ -583,7 +496,7 @@ struct FixApply {
                 base = top >> 20;  // entries below 2^59: row sums below 2^62
                 fe += base - 1017;
                 if (base < 950 || base > 1100) {  // tables far outside hat units
-                    sh.fe[tid] = kFixSpecial;
+                    sh.fe[own] = kFixSpecial;
                     r.ce = kFixSpecial;
                     return;
                 }
@@ -624,41 +537,41 @@ struct FixApply {
             }
         }
         if (E == 0) fe = 0;  // zero fluxes
-        sh.fe[tid] = fe;
+        sh.fe[own] = fe;
         // P_s (s, component)
-        longlong2 Q[3][3];
-        Q[0][0] = t[0];
-        Q[1][1] = t[1];
-        Q[2][2] = t[2];
-        Q[0][1] = Q[1][0] = t[5];
-        Q[0][2] = Q[2][0] = t[4];
-        Q[1][2] = Q[2][1] = t[3];
-        if (!CUBIC) mix3(c, Q, true);
+        longlong2 Ps[3][3];
+        Ps[0][0] = t[0];
+        Ps[1][1] = t[1];
+        Ps[2][2] = t[2];
+        Ps[0][1] = Ps[1][0] = t[5];
+        Ps[0][2] = Ps[2][0] = t[4];
+        Ps[1][2] = Ps[2][1] = t[3];
+        if (!CUBIC) mix3(c, Ps, true);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             longlong2 f;
-            const int64_t ux = Q[0][a].x + Q[1][a].x, uy = Q[0][a].y + Q[1][a].y;
-            const int64_t vx = Q[0][a].x - Q[1][a].x, vy = Q[0][a].y - Q[1][a].y;
-            f.x = ux + Q[2][a].x;
-            f.y = uy + Q[2][a].y;
-            sh.fs[(0 + a) * n + tid] = f;
-            f.x = ux - Q[2][a].x;
-            f.y = uy - Q[2][a].y;
-            sh.fs[(3 + a) * n + tid] = f;
-            f.x = vx + Q[2][a].x;
-            f.y = vy + Q[2][a].y;
-            sh.fs[(6 + a) * n + tid] = f;
-            f.x = vx - Q[2][a].x;
-            f.y = vy - Q[2][a].y;
-            sh.fs[(9 + a) * n + tid] = f;
+            const int64_t ux = Ps[0][a].x + Ps[1][a].x, uy = Ps[0][a].y + Ps[1][a].y;
+            const int64_t vx = Ps[0][a].x - Ps[1][a].x, vy = Ps[0][a].y - Ps[1][a].y;
+            f.x = ux + Ps[2][a].x;
+            f.y = uy + Ps[2][a].y;
+            sh.fs[(0 + a) * n + own] = f;
+            f.x = ux - Ps[2][a].x;
+            f.y = uy - Ps[2][a].y;
+            sh.fs[(3 + a) * n + own] = f;
+            f.x = vx + Ps[2][a].x;
+            f.y = vy + Ps[2][a].y;
+            sh.fs[(6 + a) * n + own] = f;
+            f.x = vx - Ps[2][a].x;
+            f.y = vy - Ps[2][a].y;
+            sh.fs[(9 + a) * n + own] = f;
         }
         if (r.flags & 4) {
             const int m = imax(r.ce, fe);
             const int sa = imin(m - r.ce, 63), sf = imin(m - fe, 63);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                r.cv[a].x = (r.cv[a].x >> sa) - 4 * (Q[0][a].x >> sf);
-                r.cv[a].y = (r.cv[a].y >> sa) - 4 * (Q[0][a].y >> sf);
+                r.cv[a].x = (r.cv[a].x >> sa) - 4 * (Ps[0][a].x >> sf);
+                r.cv[a].y = (r.cv[a].y >> sa) - 4 * (Ps[0][a].y >> sf);
             }
             r.ce = m;
         }
@@ -691,27 +604,29 @@ struct FixApply {
     }
 
     // The node's own x of plane kf - 1, for the shift term and the inner product.
+    template <int Q>
     static PC_HD void load_own(const Ctx& c, Regs& r, int kf) {
         const int k = kf - 1;
         if (!(r.flags & 4) || k < c.k0) return;
-        const int at = k * c.G->plane + ((k & 1) ? r.off[1] : r.off[0]);
+        const int at = k * c.G->plane + r.off[1 - Q];
         PC_IDX(at, c.G->vstr);
 #pragma unroll
         for (int a = 0; a < 3; ++a) r.xo[a] = (c.x + at)[(int64_t)a * c.G->vstr];
     }
 
     // Outputs y(kf - 1); y(kf) moves on; y(kf + 1) starts with F_1, F_3 of plane kf.
+    template <int Q>
     static PC_HD void gather(const Ctx& c, Shared& sh, Regs& r, int kf) {
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         if (!(r.flags & 4)) return;
-        const int n = G.ncell, k = kf - 1, q = k & 1;  // planes kf - 1 and kf + 1 share the offsets
-        const int gn = q ? r.gn[1] : r.gn[0];
-        const int c0 = gn & 0xffff, c1 = gn >> 16;
-        PC_IDX(c0, n);
-        PC_IDX(c1, n);
+        constexpr int n = kCells;
+        const int k = kf - 1;  // planes kf - 1 and kf + 1 share the offsets
+        const int c0 = r.gn[1 - Q] & 0xffff, c1 = r.gn[1 - Q] >> 16;
+        PC_IDX(c0, G.ncell);
+        PC_IDX(c1, G.ncell);
         const int f0 = sh.fe[c0], f1 = sh.fe[c1];
         if (k >= c.k0) {
-            const int at = k * G.plane + (q ? r.off[1] : r.off[0]);
+            const int at = k * G.plane + r.off[1 - Q];
             const int E = imax(r.pe, imax(f0, f1));
             if (E >= kFixSpecial && r.ks > k) r.ks = k;
             if (k < r.ks) {
@@ -756,7 +671,7 @@ struct FixApply {
 
     // Fluxes at node (a, b, k) of the block in FP64 (coordinates inside the grid).
     static __host__ __device__ void slow_flux(const Ctx& c, int a, int b, int k, double2 (*Fo)[3]) {
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         const StencilParams<double>& P = c.F->P;
         auto addr = [&](int aa, int bb, int kk) -> int64_t {
             const int i0 = (kk + c.p13) & 1, j0 = (kk + c.p12 + c.p13) & 1;
@@ -847,7 +762,7 @@ struct FixApply {
     // its speed does not matter; after the march and not inlined, so that it costs the march no
     // registers.  Returns the column's part of Re<x, y>.
     static __host__ __device__ PC_FIX_COLD double slow_column(const Ctx& c, int k, int off0, int off1) {
-        const FixGeom& G = *c.G;
+        const CellGeom& G = *c.G;
         double dot = 0.0;
         for (; k < c.k0 + c.tz; ++k) {
             const int off = (k & 1) ? off1 : off0;

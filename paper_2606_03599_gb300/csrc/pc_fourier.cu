@@ -377,7 +377,6 @@ Precond::~Precond() {
     cudaFree(d_wn);
     cudaFree(d_wn32);
     cudaFree(d_blockids);
-    cudaFree(d_part);
 }
 
 namespace pc {
@@ -393,7 +392,6 @@ int precond_create(pc_grid* g) {
     // roots of the own quarter-grid DFT (Bloch-independent) and the block ids
     P->own_dft = g->X == g->Y && g->Z == 2 * g->X && bloch_dft_supported(g->X, nullptr, nullptr);
     P->fused = P->own_dft && fused::supported(g->X);
-    PC_CUDA_TRY(cudaMalloc(&P->d_part, sizeof(double) * 4 * precond_partials(g)));
     {
         const int n = g->X;
         std::vector<double2> w(n);
@@ -409,7 +407,9 @@ int precond_create(pc_grid* g) {
         P->wn = P->d_wn;
         P->wn32 = P->d_wn32;
         const int ids[4] = {0, 1, 2, 3};
-        PC_CUDA_TRY(cudaMalloc(&P->d_blockids, sizeof(ids)));
+        // one allocation: the ids, then the partial sums of pc_block_precond
+        PC_CUDA_TRY(cudaMalloc(&P->d_blockids, 256 + sizeof(double) * 4 * precond_partials(g)));
+        P->d_part = reinterpret_cast<double*>(P->d_blockids + 64);
         PC_CUDA_TRY(cudaMemcpy(P->d_blockids, ids, sizeof(ids), cudaMemcpyHostToDevice));
     }
     // reference medium: volume averages of rho and C over the grid

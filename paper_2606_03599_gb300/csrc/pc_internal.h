@@ -101,6 +101,10 @@ int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<dou
                      const double* item_ph, int nitems, int tz, double* dp, int ds, cudaStream_t s);
 int fix_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz);
 bool fix_apply_ok(const StencilParams<double>& P, bool cubic, int matkind);
+// Complex64 cell apply (blocks and full space; every item its own Bloch phases); as fix_apply_ctas.
+int launch_apply_cell(bool full, bool cubic, int matkind, const StencilParams<float>& P, const ApplyItem* items,
+                      const double* item_ph, int nitems, int tz, double* dp, int ds, int* err, cudaStream_t s);
+int cell_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz);
 size_t split_scratch_bytes(int X, int Y, int Z, int nitems, int dtype);
 int split_apply_ctas(int64_t m);
 
@@ -113,8 +117,9 @@ struct ApplyConfig {
     bool split = false;  // two-pass complex128 kernels (flux, then gather)
     bool pipe = false;   // plane-pipelined kernel (complex64 parity blocks, even X)
     bool fix = false;    // integer-pipe complex128 kernel (shape code kFixShape)
+    bool cell = false;   // complex64 cell kernel (shape code kCellShape)
 };
-constexpr int kFixShape = 8;
+constexpr int kFixShape = 8, kCellShape = 9;
 // Kind code of a configuration as pc_tuned_config reports it.
 inline int config_kind(const ApplyConfig& c) {
     return c.pipe ? 4 : (c.split ? 3 : (c.row ? 2 : (c.tma ? 1 : 0)));
@@ -122,7 +127,7 @@ inline int config_kind(const ApplyConfig& c) {
 // scratch_ok = false: only kernels that need no scratch memory of their own (no two-pass apply);
 // int_ok: the integer-pipe complex128 kernel may be chosen.
 ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks = false, int matkind = 0,
-                                bool scratch_ok = true, bool int_ok = false);
+                                bool scratch_ok = true, bool int_ok = false, bool cubic = true);
 // Launch configuration for a grid layout: the autotuned one when present, else the heuristic.
 ApplyConfig apply_config_for(const pc_grid* g, bool full, int nitems, int dtype);
 bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool cubic, int nitems, ApplyConfig* out);

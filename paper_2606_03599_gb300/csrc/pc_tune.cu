@@ -78,6 +78,7 @@ void load_locked() {
         c.split = kind == 3;
         c.pipe = kind == 4;
         c.fix = kind == 0 && shape == kFixShape;
+        c.cell = kind == 0 && shape == kCellShape;
         g_tuned[key] = c;
     }
 }
@@ -102,6 +103,8 @@ bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool c
     // a tuned chunking for a bucket is reused for every batch size in it: recount the CTAs
     if (out->fix) {
         out->ctas = fix_apply_ctas(Z, full, nitems, out->tz, nullptr);
+    } else if (out->cell) {
+        out->ctas = cell_apply_ctas(Z, full, nitems, out->tz, nullptr);
     } else if (out->split) {
         out->ctas = split_apply_ctas((int64_t)X * Y * Z);
     } else if (out->pipe) {
@@ -121,7 +124,7 @@ ApplyConfig apply_config_for(const pc_grid* g, bool full, int nitems, int dtype)
     ApplyConfig c;
     if (tuned_config(X, Y, Z, dtype, full, g->matkind, g->cubic, nitems, &c) && !(c.fix && !g->int_ok)) return c;
     c = ApplyConfig();
-    return choose_apply_config(X, Y, Z, nitems, dtype, !full, g->matkind, true, g->int_ok);
+    return choose_apply_config(X, Y, Z, nitems, dtype, !full, g->matkind, true, g->int_ok, g->cubic);
 }
 
 // Time one candidate on scratch vectors: after two warm-up launches, the best of three
@@ -153,6 +156,13 @@ static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool 
         c.fix = true;
         c.shape = kFixShape;
         c.ctas = fix_apply_ctas(Z, full, nitems, 0, &c.tz);
+        out.push_back(c);
+    }
+    if (dtype == PC_C64 && matkind != 2) {  // cell kernel: the default chunking
+        ApplyConfig c;
+        c.cell = true;
+        c.shape = kCellShape;
+        c.ctas = cell_apply_ctas(Z, full, nitems, 0, &c.tz);
         out.push_back(c);
     }
     const int sm = device_sm_count();
@@ -187,7 +197,7 @@ static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool 
         base.tz = (int)((Z + nch - 1) / nch);
         base.ctas = tiles * ((Z + base.tz - 1) / base.tz);
         for (auto& o : out)
-            if (!o.pipe && !o.fix && o.row == base.row && o.tma == base.tma && o.shape == base.shape && o.tz == base.tz) return;
+            if (!o.pipe && !o.fix && !o.cell && o.row == base.row && o.tma == base.tma && o.shape == base.shape && o.tz == base.tz) return;
         out.push_back(base);
     };
     if (!full && dtype == PC_C64 && pipe_geom_ok(X, Y, Z, matkind)) {
@@ -279,7 +289,7 @@ int autotune_layout(pc_grid* g, int dtype, bool full, int nitems, cudaStream_t s
         if (rc != PC_OK) break;
         if (verbose)
             std::fprintf(stderr, "[pcband tune] %s kind=%s shape=%d tz=%d ctas=%d: %.1f us\n", key.c_str(),
-                         c.fix ? "int" : c.pipe ? "pipe" : (c.split ? "split" : (c.row ? "row" : (c.tma ? "tma" : "regs"))), c.shape,
+                         c.fix ? "int" : c.cell ? "cell" : c.pipe ? "pipe" : (c.split ? "split" : (c.row ? "row" : (c.tma ? "tma" : "regs"))), c.shape,
                          c.tz, c.ctas, us);
         if (us < best_us) {
             best_us = us;

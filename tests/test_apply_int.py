@@ -1,5 +1,5 @@
-"""The integer-pipe complex128 apply (host emulation of its per-thread functions) against the
-two-pass FP64 apply, over the forms both accept (CPU only).
+"""The integer-pipe complex128 apply and the complex64 cell apply (host emulation of their per-thread
+functions) against the two-pass apply, over the forms both accept (CPU only).
 
 Tolerance: both sides round at most about 60 times in a chain, and a unit roundoff is 2^-53, so
 two correct results differ by at most 2 * 60 * 2^-53 = 1.4e-14 of the output's norm on broad-band
@@ -67,7 +67,7 @@ def both(lib, N, block, lattice, matkind, x, tilings, kappa=(0.21, -0.33, 0.4), 
     out = []
     for shape, tz in [(TWO_PASS, 0)] + list(tilings):
         y = np.full_like(x, np.nan)
-        assert lib.pc_emu_apply(N, block, 2, shape, tz, C72.ctypes.data_as(dp), rho.ctypes.data_as(dp),
+        assert lib.pc_emu_apply(N, block, 1 if x.dtype == np.complex64 else 2, shape, tz, C72.ctypes.data_as(dp), rho.ctypes.data_as(dp),
                                 ainv.ctypes.data_as(dp), int(lattice == "cubic"), phi.ctypes.data_as(dp),
                                 mat.ctypes.data, matkind, x.ctypes.data, y.ctypes.data, shift) == 0
         out.append(y)
@@ -89,6 +89,22 @@ def test_integer_apply_equals_two_pass(emu, N, lattice, matkind, block):
     for y in got:
         assert np.linalg.norm(y - ref) <= TOL * np.linalg.norm(ref)
         assert np.array_equal(y, got[0])  # a node's arithmetic does not depend on the tile
+
+
+@pytest.mark.parametrize("N", [4, 6, 8, 14, 34])
+@pytest.mark.parametrize("lattice", ["cubic", "skew"])
+@pytest.mark.parametrize("matkind", [0, 1])
+@pytest.mark.parametrize("block", [-1, 1, 2])
+def test_cell_apply_equals_two_pass_in_complex64(emu, N, lattice, matkind, block):
+    """The complex64 cell kernel against the two-pass kernels in complex64: the same operations in
+    nearly the same order, so at most 2 * 60 roundings of 2^-24 apart."""
+    if N == 34 and (block != 2 or lattice == "skew"):
+        pytest.skip("one block and one lattice at the largest size")
+    x = complex_gaussian((3, N ** 3), 7).astype(np.complex64)
+    ref, *got = both(emu, N, block, lattice, matkind, x, TILINGS)
+    for y in got:
+        assert np.linalg.norm(y - ref) <= 120 * 2.0 ** -24 * np.linalg.norm(ref)
+        assert np.array_equal(y, got[0])
 
 
 @pytest.mark.parametrize("lattice,matkind", [("cubic", 0), ("fcc", 1), ("cubic", 2)])
