@@ -362,7 +362,7 @@ static void emu_run_split(const StencilParams<R>& P, int block, const void* x, v
 template <bool CUBIC, int MATK>
 static int emu_run_fix(const StencilParams<double>& P, int block, const void* x, void* y, const void* mat,
                        double shift, int tz, int tx, int ty) {
-    using T = FixApply<CUBIC, MATK>;
+    using T = FixApply<CUBIC, MATK, 2>;
     CellGeom G;
     make_cell_geom(G, P.N, block < 0, false);
     if (tx > 0) {
@@ -403,7 +403,7 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
             c.p12 = pb >> 1;
             c.p13 = pb & 1;
             for (int t = 0; t < n; ++t) T::load_tables(c, sh, t, n);
-            for (int t = 0; t < n; ++t) T::init(c, t, regs[t]);
+            for (int t = 0; t < n; ++t) T::init(c, t, 0, regs[t]);
             for (int t = 0; t < n; ++t) {
                 auto& r = regs[t];
                 T::template stage<0>(c, sh, r, t, c.k0 - 2);

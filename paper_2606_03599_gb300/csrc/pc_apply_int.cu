@@ -17,19 +17,20 @@ struct FixBatch {
 };
 
 // blockIdx.x = (tile, chunk of planes), blockIdx.y = item (full space: item * 4 + parity block).
-template <bool CUBIC, int MATK>
-__global__ void __launch_bounds__(kCells, 2)
+// NP parts of a cell per thread: 2 / NP threads per cell.
+template <bool CUBIC, int MATK, int NP>
+__global__ void __launch_bounds__(2 / NP * kCells, NP)
     fix_apply(const __grid_constant__ FixParams F, const __grid_constant__ FixBatch B, const __grid_constant__ CellGeom G,
               double* __restrict__ dot_partials, int dot_stride) {
-    using T = FixApply<CUBIC, MATK>;
+    using T = FixApply<CUBIC, MATK, NP>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int item = G.full ? (int)blockIdx.y >> 2 : (int)blockIdx.y;
     const ApplyItem& it = B.it[item];
     if (it.skip != nullptr && *it.skip) return;
     typename T::Shared sh;
     T::carve(sh, smem_raw);
-    const int tid = threadIdx.x, n = G.ncell;
-    const bool live = tid < n;
+    const int tid = threadIdx.x, cell = tid / (2 / NP), n = G.ncell;
+    const bool live = cell < n;
     typename T::Ctx c;
     c.F = &F;
     c.G = &G;
@@ -50,27 +51,27 @@ __global__ void __launch_bounds__(kCells, 2)
     c.p13 = blk & 1;
     typename T::Regs r;
     T::load_tables(c, sh, tid, blockDim.x);
-    T::init(c, min(tid, n - 1), r);
+    T::init(c, min(cell, n - 1), NP == 1 ? tid & 1 : 0, r);
     if (!live) r.flags = 0;
     const int klast = c.k0 + c.tz + 1;  // last plane of x
     // the first three planes go through the flux cells, which nothing uses yet; k0 is even, so planes
     // k0 - 2 .. k0 + 1 have parities 0, 1, 0, 1
     typename T::Shared pre[3] = {sh, sh, sh};
 #pragma unroll
-    for (int i = 0; i < 3; ++i) pre[i].raw = reinterpret_cast<double2*>(sh.fs) + 3 * i * kCells;
+    for (int i = 0; i < 3; ++i) pre[i].raw = reinterpret_cast<double*>(sh.fs) + 3 * i * T::kRow;
     if (live) {
-        T::template stage<0>(c, pre[0], r, tid, c.k0 - 2);
-        T::template stage<1>(c, pre[1], r, tid, c.k0 - 1);
-        T::template stage<0>(c, pre[2], r, tid, c.k0);
-        T::template stage<1>(c, sh, r, tid, c.k0 + 1);
+        T::template stage<0>(c, pre[0], r, cell, c.k0 - 2);
+        T::template stage<1>(c, pre[1], r, cell, c.k0 - 1);
+        T::template stage<0>(c, pre[2], r, cell, c.k0);
+        T::template stage<1>(c, sh, r, cell, c.k0 + 1);
         r.mcur = T::template read_mat<1>(c, r, c.k0 - 1);
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();  // phase table
     if (live) {
-        T::template convert<0>(c, pre[0], r, tid, c.k0 - 2, 0);
-        T::template convert<1>(c, pre[1], r, tid, c.k0 - 1, 1);
-        T::template convert<0>(c, pre[2], r, tid, c.k0, 2);
+        T::template convert<0>(c, pre[0], r, cell, c.k0 - 2, 0);
+        T::template convert<1>(c, pre[1], r, cell, c.k0 - 1, 1);
+        T::template convert<0>(c, pre[2], r, cell, c.k0, 2);
     }
     __syncthreads();
     int sm = 0, sc = 1, sp = 2;
@@ -85,8 +86,8 @@ __global__ void __launch_bounds__(kCells, 2)
         T::template gather<Q>(c, sh, r, kf);
         if (kf + 2 <= klast && live) {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
-            T::template convert<Q>(c, sh, r, tid, kf + 2, sm);
-            if (kf + 3 <= klast) T::template stage<1 - Q>(c, sh, r, tid, kf + 3);
+            T::template convert<Q>(c, sh, r, cell, kf + 2, sm);
+            if (kf + 3 <= klast) T::template stage<1 - Q>(c, sh, r, cell, kf + 3);
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
         T::next_mat(r);
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kCells, 2)
         step(std::integral_constant<int, 1>(), kf);
         step(std::integral_constant<int, 0>(), kf + 1);
     }
-    if (r.ks < c.k0 + c.tz) r.dot += T::slow_column(c, r.ks, r.off[0], r.off[1]);
+    if (r.ks < c.k0 + c.tz && r.part() == 0) r.dot += T::slow_column(c, r.ks, r.off[0], r.off[1]);  // both parts
     if (c.dot) {
         double v = r.dot;
         double* red = reinterpret_cast<double*>(sh.fs);
@@ -116,19 +117,26 @@ __global__ void __launch_bounds__(kCells, 2)
     }
 }
 
-template <bool CUBIC, int MATK>
-int launch_fix_t(const FixParams& F, const FixBatch& B, const CellGeom& G, double* dp, int ds, cudaStream_t s) {
-    using T = FixApply<CUBIC, MATK>;
-    auto kern = fix_apply<CUBIC, MATK>;
-    const size_t smem = T::shared_bytes();
-    // the largest tile's need, set on every launch: an attribute of the kernel on the current device
-    PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 << 10));
+template <bool CUBIC, int MATK, int NP>
+int launch_fix_np(const FixParams& F, const FixBatch& B, const CellGeom& G, double* dp, int ds, cudaStream_t s) {
+    using T = FixApply<CUBIC, MATK, NP>;
+    auto kern = fix_apply<CUBIC, MATK, NP>;
+    // set on every launch: an attribute of the kernel on the current device
+    PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::shared_bytes()));
     const dim3 grid(G.ntx * G.nty * G.nch, B.n * (G.full ? 4 : 1));
-    kern<<<grid, (G.ncell + 31) / 32 * 32, smem, s>>>(F, B, G, dp, ds);
+    kern<<<grid, (2 / NP * G.ncell + 31) / 32 * 32, T::shared_bytes(), s>>>(F, B, G, dp, ds);
     note_launch();
     note_apply_launch();
     PC_CUDA_TRY(cudaGetLastError());
     return PC_OK;
+}
+
+template <bool CUBIC, int MATK>
+int launch_fix_t(const FixParams& F, const FixBatch& B, const CellGeom& G, double* dp, int ds, cudaStream_t s) {
+    // one CTA per SM at most: two threads per cell (see FixApply)
+    const long ctas = (long)G.ntx * G.nty * G.nch * B.n * (G.full ? 4 : 1);
+    return ctas <= device_sm_count() ? launch_fix_np<CUBIC, MATK, 1>(F, B, G, dp, ds, s)
+                                     : launch_fix_np<CUBIC, MATK, 2>(F, B, G, dp, ds, s);
 }
 
 }  // namespace

@@ -226,29 +226,34 @@ PC_HD int64_t fix_theta(float t) {
 }
 
 // MATK: 0 = phase ids, 1 = inclusion fraction, 2 = nodewise material (as SplitApply).
-template <bool CUBIC, int MATK>
+// NP: parts (real, imaginary) of a cell in one thread; they meet in the Bloch phase and in the shared
+// exponent only.  NP = 2 runs fewer instructions and is the form of launches that fill the GPU (N = 48, 64
+// block vectors: 212 us, 267 us with NP = 1).  NP = 1, two adjacent lanes per cell, halves a thread's chain
+// of dependent instructions: the form of launches with at most one CTA per SM, which wait for that chain
+// (N = 8, one block vector: 14.3 us, 18.4 us with NP = 2).  The results are the same.
+template <bool CUBIC, int MATK, int NP>
 struct FixApply {
     struct Shared {
-        longlong2* xs;  // [3 slots][3][kCells]
-        longlong2* fs;  // [12][kCells]: F_l of component c at l * 3 + c
-        double2* raw;   // [3][kCells]: the next plane of x, as read
-        double2* ph;    // [27] Bloch phases of the wraps (wa, wb, wk)
-        FixHalf* c;     // [2][21]
-        int* xe;        // [3][kCells]
-        int* fe;        // [kCells]
+        int64_t* xs;  // [3 slots][3][kCells][2]
+        int64_t* fs;  // [12][kCells][2]: F_l of component c at l * 3 + c
+        double* raw;  // [3][kCells][2]: the next plane of x, as read
+        double2* ph;  // [27] Bloch phases of the wraps (wa, wb, wk)
+        FixHalf* c;   // [2][21]
+        int* xe;      // [3][kCells]
+        int* fe;      // [kCells]
     };
+    static constexpr int kRow = 2 * kCells;  // stride of one component's array
     static constexpr size_t shared_bytes() {
         return (size_t)kCells * (16 * (9 + 12 + 3) + 4 * 4) + 16 * 27 + sizeof(FixHalf) * 42;
     }
     static PC_HD void carve(Shared& sh, unsigned char* p) {
-        constexpr int n = kCells;
-        sh.xs = reinterpret_cast<longlong2*>(p);
-        sh.fs = sh.xs + 9 * n;
-        sh.raw = reinterpret_cast<double2*>(sh.fs + 12 * n);
-        sh.ph = sh.raw + 3 * n;
+        sh.xs = reinterpret_cast<int64_t*>(p);
+        sh.fs = sh.xs + 9 * kRow;
+        sh.raw = reinterpret_cast<double*>(sh.fs + 12 * kRow);
+        sh.ph = reinterpret_cast<double2*>(sh.raw + 3 * kRow);
         sh.c = reinterpret_cast<FixHalf*>(sh.ph + 27);
         sh.xe = reinterpret_cast<int*>(sh.c + 42);
-        sh.fe = sh.xe + 3 * n;
+        sh.fe = sh.xe + 3 * kCells;
     }
 
     struct Ctx {
@@ -263,25 +268,77 @@ struct FixApply {
         int a0, b0, k0, tz, p12, p13;
     };
     struct Regs : CellMap {
+        int half;                // NP = 1: 0 real, 1 imaginary
+        PC_HD int part() const { return NP == 1 ? half : 0; }
         int mprev, mcur, mnext;  // material of planes kf - 1, kf, kf + 1 (id, or the float's bits)
-        longlong2 pv[3], cv[3];  // y(kf - 1) and y(kf) so far
+        int64_t pv[3][NP], cv[3][NP];  // y(kf - 1) and y(kf) so far
         int pe, ce;
         int ks;  // first output plane left to slow_column
-        double2 xo[3];
+        double xo[3][NP];
         double dot;
     };
 
     static PC_HD int wrap1(int v, int n, int& w) { return cell_wrap(v, n, w); }
 
-    static PC_HD void init(const Ctx& c, int tid, Regs& r) {
-        cell_init(*c.G, c.a0, c.b0, c.p12, c.p13, tid, r);
+    // Combine over the two parts of a cell (NP = 1: the neighbouring lane's, which takes every branch alike).
+#if defined(__CUDA_ARCH__)
+    static __device__ unsigned pair() { return 3u << (threadIdx.x & 30); }
+#endif
+    static PC_HD int pair_max(int v) {
+#if defined(__CUDA_ARCH__)
+        if (NP == 1) v = imax(v, __shfl_xor_sync(pair(), v, 1));
+#endif
+        return v;
+    }
+    static PC_HD int pair_or(int v) {
+#if defined(__CUDA_ARCH__)
+        if (NP == 1) v |= __shfl_xor_sync(pair(), v, 1);
+#endif
+        return v;
+    }
+
+    // a cell's parts: one 16-byte access, or 8 bytes of it
+    static PC_HD void get(const int64_t* p, int64_t* v) {
+        if (NP == 2) {
+            const longlong2 t = *reinterpret_cast<const longlong2*>(p);
+            v[0] = t.x;
+            v[NP - 1] = t.y;
+        } else {
+            v[0] = *p;
+        }
+    }
+    static PC_HD void put(int64_t* p, const int64_t* v) {
+        if (NP == 2) {
+            longlong2 t;
+            t.x = v[0];
+            t.y = v[NP - 1];
+            *reinterpret_cast<longlong2*>(p) = t;
+        } else {
+            *p = v[0];
+        }
+    }
+    static PC_HD void get(const double* p, double* v) {
+        if (NP == 2) {
+            const double2 t = *reinterpret_cast<const double2*>(p);
+            v[0] = t.x;
+            v[NP - 1] = t.y;
+        } else {
+            v[0] = *p;
+        }
+    }
+
+    static PC_HD void init(const Ctx& c, int cell, int part, Regs& r) {
+        cell_init(*c.G, c.a0, c.b0, c.p12, c.p13, cell, r);
+        if (NP == 1) r.half = part;
         r.pe = r.ce = 0;
         r.ks = 1 << 30;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            r.pv[a].x = r.pv[a].y = r.cv[a].x = r.cv[a].y = 0;
-            r.xo[a] = czero(0.0);
-        }
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                r.pv[a][i] = r.cv[a][i] = 0;
+                r.xo[a][i] = 0.0;
+            }
         r.dot = 0.0;
         r.mprev = r.mcur = r.mnext = 0;
     }
@@ -297,59 +354,81 @@ struct FixApply {
         }
     }
 
-    // Start the copy of plane kp (parity Q) of x into the staging cells (a cell is read by its own thread only).
+    // Start the copy of plane kp (parity Q) of x into the staging cells (one read by its own threads only).
     template <int Q>
-    static PC_HD void stage(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp) {
+    static PC_HD void stage(const Ctx& c, Shared& sh, const Regs& r, int cell, int kp) {
         const CellGeom& G = *c.G;
         int wk;
         const int k = wrap1(kp, G.Z, wk);
         const int at = k * G.plane + r.off[Q];
         PC_IDX(at, G.vstr);
-        PC_IDX(tid, G.ncell);
+        PC_IDX(cell, G.ncell);
+        const double2* s = c.x + at;
+        double* d = sh.raw + 2 * cell + r.part();
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            double2* d = sh.raw + a * kCells + tid;
-            const double2* s = c.x + at + (int64_t)a * G.vstr;
 #if defined(__CUDA_ARCH__)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(s)
-                         : "memory");
+            const uint32_t to = (uint32_t)__cvta_generic_to_shared(d + a * kRow);
+            const double* from = reinterpret_cast<const double*>(s + (int64_t)a * G.vstr) + r.part();
+            if (NP == 2) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(from) : "memory");
+            else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to), "l"(from) : "memory");
 #else
-            *d = *s;
+            const double* from = reinterpret_cast<const double*>(s + (int64_t)a * G.vstr);
+            for (int i = 0; i < NP; ++i) d[a * kRow + i] = from[i];
 #endif
         }
     }
 
     // Plane kp from the staging cells into slot sl: phase, exponent, integers.
     template <int Q>
-    static PC_HD void convert(const Ctx& c, Shared& sh, const Regs& r, int tid, int kp, int sl) {
+    static PC_HD void convert(const Ctx& c, Shared& sh, const Regs& r, int cell, int kp, int sl) {
         const CellGeom& G = *c.G;
         int wk;
         wrap1(kp, G.Z, wk);
         const int w = r.wab[Q] + 9 * (wk + 1);
-        double2 v[3];
+        double v[3][NP];
+        const double* d = sh.raw + 2 * cell + r.part();
 #pragma unroll
-        for (int a = 0; a < 3; ++a) v[a] = sh.raw[a * kCells + tid];
+        for (int a = 0; a < 3; ++a) get(d + a * kRow, v[a]);
         if (w != 13) {
             const double2 ph = sh.ph[w];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) v[a] = cmul(v[a], ph);
+            for (int a = 0; a < 3; ++a) {
+                if (NP == 2) {
+                    const double2 z = cmul(cmk(v[a][0], v[a][NP - 1]), ph);
+                    v[a][0] = z.x;
+                    v[a][NP - 1] = z.y;
+                } else {
+#if defined(__CUDA_ARCH__)
+                    const double o = __shfl_xor_sync(pair(), v[a][0], 1);
+                    const double m = r.part() ? o * ph.y : v[a][0] * ph.x;  // as cmul rounds
+                    v[a][0] = fma(r.part() ? v[a][0] : -o, r.part() ? ph.x : ph.y, m);
+#endif
+                }
+            }
         }
-        const int top = fix_high(v[2], fix_high(v[1], fix_high(v[0], 0)));
-        int E = top >> 20, base = E;
+        int top = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int i = 0; i < NP; ++i) top = imax(top, (int)(fix_bits(v[a][i]) >> 32) & 0x7fffffff);
+        int E = pair_max(top) >> 20, base = E;
         if (E < kFixLow || E > kFixHigh) {
             int64_t any = 0;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) any |= (fix_bits(v[a].x) | fix_bits(v[a].y)) & 0x7fffffffffffffffLL;
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int i = 0; i < NP; ++i) any |= fix_bits(v[a][i]) & 0x7fffffffffffffffLL;
             base = 64;
-            E = any ? kFixSpecial : 0;
+            E = pair_or(any != 0) ? kFixSpecial : 0;
         }
-        longlong2* xs = sh.xs + sl * 3 * kCells + r.own[Q];
+        int64_t* xs = sh.xs + sl * 3 * kRow + 2 * r.own[Q] + r.part();
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            longlong2 o;
-            o.x = E == 0 ? 0 : fix_from_double(v[a].x, base, 3);
-            o.y = E == 0 ? 0 : fix_from_double(v[a].y, base, 3);
-            xs[a * kCells] = o;
+            int64_t o[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) o[i] = E == 0 ? 0 : fix_from_double(v[a][i], base, 3);
+            put(xs + a * kRow, o);
         }
         sh.xe[sl * kCells + r.own[Q]] = E;
     }
@@ -382,19 +461,21 @@ struct FixApply {
     }
 
     template <bool ORTHO>
-    static PC_HD void stress(const FixHalf* C, const FixHalf* ex, const FixHalf* ey, longlong2* t) {
+    static PC_HD void stress(const FixHalf* C, const FixHalf (*e)[NP], int64_t (*t)[NP]) {
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
-            int64_t hx = 0, hy = 0, mx = 0, my = 0;
+            int64_t h[NP], m[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) h[i] = m[i] = 0;
 #pragma unroll
             for (int u = 0; u < 6; ++u) {
                 if (ORTHO && !((p < 3 && u < 3) || p == u)) continue;
                 const FixHalf cc = C[fix_upper(p, u)];
-                fix_mac(hx, mx, ex[u], cc);
-                fix_mac(hy, my, ey[u], cc);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) fix_mac(h[i], m[i], e[u][i], cc);
             }
-            t[p].x = fix_sum(hx, mx, CUBIC ? 0 : 2);
-            t[p].y = fix_sum(hy, my, CUBIC ? 0 : 2);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) t[p][i] = fix_sum(h[i], m[i], CUBIC ? 0 : 2);
         }
     }
 
@@ -418,21 +499,41 @@ struct FixApply {
         }
         const int s0 = imin(E - e0, 63), s1 = imin(E - e1, 63), s2 = imin(E - e2, 63), s3 = imin(E - e3, 63),
                   so = imin(E - eo, 63);
-        const longlong2 *p0 = sh.xs + sm * 3 * n + n0, *p1 = sh.xs + sp * 3 * n + n0, *p2 = sh.xs + sm * 3 * n + n1,
-                        *p3 = sh.xs + sp * 3 * n + n1, *po = sh.xs + sc * 3 * n + own;
-        longlong2 H[3][3];
+        const int64_t *p0 = sh.xs + sm * 3 * kRow + 2 * n0 + r.part(), *p1 = sh.xs + sp * 3 * kRow + 2 * n0 + r.part(),
+                      *p2 = sh.xs + sm * 3 * kRow + 2 * n1 + r.part(), *p3 = sh.xs + sp * 3 * kRow + 2 * n1 + r.part(),
+                      *po = sh.xs + sc * 3 * kRow + 2 * own + r.part();
+        int64_t H[3][3][NP];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const longlong2 v0 = fix_ashr2(p0[a * n], s0), v1 = fix_ashr2(p1[a * n], s1);
-            const longlong2 v2 = fix_ashr2(p2[a * n], s2), v3 = fix_ashr2(p3[a * n], s3);
-            const longlong2 vo = fix_ashr2(po[a * n], so);
-            const int64_t ux = v0.x + v1.x, uy = v0.y + v1.y, vx = v2.x + v3.x, vy = v2.y + v3.y;
-            H[0][a].x = ux + vx - 4 * vo.x;
-            H[0][a].y = uy + vy - 4 * vo.y;
-            H[1][a].x = ux - vx;
-            H[1][a].y = uy - vy;
-            H[2][a].x = (v0.x - v1.x) + (v2.x - v3.x);
-            H[2][a].y = (v0.y - v1.y) + (v2.y - v3.y);
+            int64_t x0[NP], x1[NP], x2[NP], x3[NP], xo[NP];
+            get(p0 + a * kRow, x0);
+            get(p1 + a * kRow, x1);
+            get(p2 + a * kRow, x2);
+            get(p3 + a * kRow, x3);
+            get(po + a * kRow, xo);
+            int64_t u[NP], v[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                x0[i] >>= s0;
+                x1[i] >>= s1;
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                x2[i] >>= s2;
+                x3[i] >>= s3;
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                xo[i] >>= so;
+                u[i] = x0[i] + x1[i];
+                v[i] = x2[i] + x3[i];
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) H[0][a][i] = u[i] + v[i] - 4 * xo[i];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) H[1][a][i] = u[i] - v[i];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) H[2][a][i] = (x0[i] - x1[i]) + (x2[i] - x3[i]);
         }
         int up = 0;
         if (!CUBIC || MATK != 0) {
@@ -442,43 +543,42 @@ struct FixApply {
             for (int m = 0; m < 3; ++m)
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
-                    top |= (int)((H[m][a].x ^ (H[m][a].x >> 63)) >> 32) | (int)((H[m][a].y ^ (H[m][a].y >> 63)) >> 32);
-            up = fix_clz64((uint64_t)(uint32_t)top | 1) - 32 - 5;
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) top |= (int)((H[m][a][i] ^ (H[m][a][i] >> 63)) >> 32);
+            up = fix_clz64((uint64_t)(uint32_t)pair_or(top) | 1) - 32 - 5;
 #pragma unroll
             for (int m = 0; m < 3; ++m)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    H[m][a].x <<= up;
-                    H[m][a].y <<= up;
-                }
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) H[m][a][i] <<= up;
         }
         if (!CUBIC) mix3(c, H, false);
-        // strain halves: xx, yy, zz, yz, xz, xy (real and imaginary parts)
-        FixHalf ex[6], ey[6];
+        // strain halves: xx, yy, zz, yz, xz, xy
+        FixHalf e[6][NP];
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
-            ex[p] = fix_split(H[p][p].x);
-            ey[p] = fix_split(H[p][p].y);
             const int u = p == 0 ? 1 : 0, v = p == 2 ? 1 : 2;
-            ex[3 + p] = fix_split(H[v][u].x + H[u][v].x);
-            ey[3 + p] = fix_split(H[v][u].y + H[u][v].y);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) e[p][i] = fix_split(H[p][p][i]);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) e[3 + p][i] = fix_split(H[v][u][i] + H[u][v][i]);
         }
-        longlong2 t[6];
+        int64_t t[6][NP];
         int fe = E - up + c.F->moff;
         if (MATK == 0) {
             const int ph = r.mcur != 0 ? 1 : 0;
             const FixHalf* C = sh.c + 21 * ph;
             fe += ph ? c.F->coff[1] : c.F->coff[0];
             // every node of the warp orthotropic: normal block and shear diagonal only
-            if (warp_all(c.F->P.ortho[ph] != 0)) stress<true>(C, ex, ey, t);
-            else stress<false>(C, ex, ey, t);
+            if (warp_all(c.F->P.ortho[ph] != 0)) stress<true>(C, e, t);
+            else stress<false>(C, e, t);
         } else {
-            int64_t hx[6], hy[6], mx[6], my[6];
+            int64_t h[6][NP], m[6][NP];
 #pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                hx[p] = hy[p] = 0;
-                mx[p] = my[p] = 0;
-            }
+            for (int p = 0; p < 6; ++p)
+#pragma unroll
+                for (int i = 0; i < NP; ++i) h[p][i] = m[p][i] = 0;
             int row[6] = {0, 0, 0, 0, 0, 0};  // row sums of |c| / 2^32
             FixHalf th = {0, 0};
             const double* md = nullptr;
@@ -507,21 +607,20 @@ struct FixApply {
                 for (int u = p; u < 6; ++u) {
                     FixHalf cc;
                     if (MATK == 1) {  // c = C_0 + theta (C_1 - C_0)
-                        int64_t h = 0, m = 1LL << 29;
+                        int64_t hh = 0, mm = 1LL << 29;
                         const FixHalf d = sh.c[21 + fix_upper(p, u)], z = sh.c[fix_upper(p, u)];
-                        fix_mac(h, m, th, d);
-                        cc = fix_split((int64_t)z.hi * 0x100000000LL + z.lo + h * 4 + (m >> 30));
+                        fix_mac(hh, mm, th, d);
+                        cc = fix_split((int64_t)z.hi * 0x100000000LL + z.lo + hh * 4 + (mm >> 30));
                     } else {
                         cc = fix_split(fix_from_double(md[(int64_t)fix_upper(p, u) * G.vstr], base, 6));
                     }
                     const int ab = cc.hi < 0 ? -cc.hi : cc.hi;
                     row[p] += ab;
-                    fix_mac(hx[p], mx[p], ex[u], cc);
-                    fix_mac(hy[p], my[p], ey[u], cc);
-                    if (u != p) {
-                        row[u] += ab;
-                        fix_mac(hx[u], mx[u], ex[p], cc);
-                        fix_mac(hy[u], my[u], ey[p], cc);
+                    if (u != p) row[u] += ab;
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) {
+                        fix_mac(h[p][i], m[p][i], e[u][i], cc);
+                        if (u != p) fix_mac(h[u][i], m[u][i], e[p][i], cc);
                     }
                 }
             // the node's own row sums are below the bound the scale allows for: keep that many more bits
@@ -531,76 +630,69 @@ struct FixApply {
             fe -= sh2;
             sh2 += CUBIC ? 0 : 2;
 #pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                t[p].x = fix_sum(hx[p], mx[p], sh2);
-                t[p].y = fix_sum(hy[p], my[p], sh2);
-            }
+            for (int p = 0; p < 6; ++p)
+#pragma unroll
+                for (int i = 0; i < NP; ++i) t[p][i] = fix_sum(h[p][i], m[p][i], sh2);
         }
         if (E == 0) fe = 0;  // zero fluxes
         sh.fe[own] = fe;
         // P_s (s, component)
-        longlong2 Ps[3][3];
-        Ps[0][0] = t[0];
-        Ps[1][1] = t[1];
-        Ps[2][2] = t[2];
-        Ps[0][1] = Ps[1][0] = t[5];
-        Ps[0][2] = Ps[2][0] = t[4];
-        Ps[1][2] = Ps[2][1] = t[3];
+        int64_t Ps[3][3][NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            Ps[0][0][i] = t[0][i];
+            Ps[1][1][i] = t[1][i];
+            Ps[2][2][i] = t[2][i];
+            Ps[0][1][i] = Ps[1][0][i] = t[5][i];
+            Ps[0][2][i] = Ps[2][0][i] = t[4][i];
+            Ps[1][2][i] = Ps[2][1][i] = t[3][i];
+        }
         if (!CUBIC) mix3(c, Ps, true);
+        int64_t* f = sh.fs + 2 * own + r.part();
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            longlong2 f;
-            const int64_t ux = Ps[0][a].x + Ps[1][a].x, uy = Ps[0][a].y + Ps[1][a].y;
-            const int64_t vx = Ps[0][a].x - Ps[1][a].x, vy = Ps[0][a].y - Ps[1][a].y;
-            f.x = ux + Ps[2][a].x;
-            f.y = uy + Ps[2][a].y;
-            sh.fs[(0 + a) * n + own] = f;
-            f.x = ux - Ps[2][a].x;
-            f.y = uy - Ps[2][a].y;
-            sh.fs[(3 + a) * n + own] = f;
-            f.x = vx + Ps[2][a].x;
-            f.y = vy + Ps[2][a].y;
-            sh.fs[(6 + a) * n + own] = f;
-            f.x = vx - Ps[2][a].x;
-            f.y = vy - Ps[2][a].y;
-            sh.fs[(9 + a) * n + own] = f;
+            int64_t u[NP], v[NP], g[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                u[i] = Ps[0][a][i] + Ps[1][a][i];
+                v[i] = Ps[0][a][i] - Ps[1][a][i];
+            }
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) g[i] = (l < 2 ? u[i] : v[i]) + (l & 1 ? -Ps[2][a][i] : Ps[2][a][i]);
+                put(f + (l * 3 + a) * kRow, g);
+            }
         }
         if (r.flags & 4) {
             const int m = imax(r.ce, fe);
             const int sa = imin(m - r.ce, 63), sf = imin(m - fe, 63);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                r.cv[a].x = (r.cv[a].x >> sa) - 4 * (Ps[0][a].x >> sf);
-                r.cv[a].y = (r.cv[a].y >> sa) - 4 * (Ps[0][a].y >> sf);
-            }
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int i = 0; i < NP; ++i) r.cv[a][i] = (r.cv[a][i] >> sa) - 4 * (Ps[0][a][i] >> sf);
             r.ce = m;
         }
     }
 
-    // Rows of a 3 x 3 complex table through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or
-    // (transposed) out[s] = sum_m Mmix[s][m] in[m].
-    static PC_HD void mix3(const Ctx& c, longlong2 (*V)[3], bool rows) {
+    // Rows of a 3 x 3 table through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or (rows)
+    // out[s] = sum_m Mmix[s][m] in[m].
+    static PC_HD void mix3(const Ctx& c, int64_t (*V)[3][NP], bool rows) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            FixHalf vx[3], vy[3];
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int s = 0; s < 3; ++s) {
-                vx[s] = fix_split(V[s][a].x);
-                vy[s] = fix_split(V[s][a].y);
-            }
+            for (int i = 0; i < NP; ++i) {
+                FixHalf v[3];
 #pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                int64_t hx = 0, hy = 0, mx = 0, my = 0;
+                for (int s = 0; s < 3; ++s) v[s] = fix_split(V[s][a][i]);
 #pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    const FixHalf w = c.F->mix[rows ? m * 3 + s : s * 3 + m];
-                    fix_mac(hx, mx, vx[s], w);
-                    fix_mac(hy, my, vy[s], w);
+                for (int m = 0; m < 3; ++m) {
+                    int64_t h = 0, md = 0;
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) fix_mac(h, md, v[s], c.F->mix[rows ? m * 3 + s : s * 3 + m]);
+                    V[m][a][i] = fix_sum(h, md, rows ? 1 : 2);
                 }
-                V[m][a].x = fix_sum(hx, mx, rows ? 1 : 2);
-                V[m][a].y = fix_sum(hy, my, rows ? 1 : 2);
             }
-        }
     }
 
     // The node's own x of plane kf - 1, for the shift term and the inner product.
@@ -610,8 +702,9 @@ struct FixApply {
         if (!(r.flags & 4) || k < c.k0) return;
         const int at = k * c.G->plane + r.off[1 - Q];
         PC_IDX(at, c.G->vstr);
+        const double2* s = c.x + at;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) r.xo[a] = (c.x + at)[(int64_t)a * c.G->vstr];
+        for (int a = 0; a < 3; ++a) get(reinterpret_cast<const double*>(s + (int64_t)a * c.G->vstr) + r.part(), r.xo[a]);
     }
 
     // Outputs y(kf - 1); y(kf) moves on; y(kf + 1) starts with F_1, F_3 of plane kf.
@@ -619,12 +712,12 @@ struct FixApply {
     static PC_HD void gather(const Ctx& c, Shared& sh, Regs& r, int kf) {
         const CellGeom& G = *c.G;
         if (!(r.flags & 4)) return;
-        constexpr int n = kCells;
         const int k = kf - 1;  // planes kf - 1 and kf + 1 share the offsets
         const int c0 = r.gn[1 - Q] & 0xffff, c1 = r.gn[1 - Q] >> 16;
         PC_IDX(c0, G.ncell);
         PC_IDX(c1, G.ncell);
         const int f0 = sh.fe[c0], f1 = sh.fe[c1];
+        const int64_t *a0 = sh.fs + 2 * c0 + r.part(), *a1 = sh.fs + 2 * c1 + r.part();
         if (k >= c.k0) {
             const int at = k * G.plane + r.off[1 - Q];
             const int E = imax(r.pe, imax(f0, f1));
@@ -634,13 +727,22 @@ struct FixApply {
                 const int sa = imin(E - r.pe, 63), s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    const longlong2 g0 = sh.fs[a * n + c0], g1 = sh.fs[(6 + a) * n + c1];
-                    double2 w;
-                    w.x = fix_to_double((r.pv[a].x >> sa) + (g0.x >> s0) + (g1.x >> s1), E);
-                    w.y = fix_to_double((r.pv[a].y >> sa) + (g0.y >> s0) + (g1.y >> s1), E);
-                    w = cfma(-sr, r.xo[a], w);
-                    (c.y + at)[(int64_t)a * G.vstr] = w;
-                    if (c.dot) r.dot = cdotre(r.xo[a], w, r.dot);
+                    int64_t g0[NP], g1[NP];
+                    double w[NP];
+                    get(a0 + a * kRow, g0);
+                    get(a1 + (6 + a) * kRow, g1);
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) {
+                        w[i] = fix_to_double((r.pv[a][i] >> sa) + (g0[i] >> s0) + (g1[i] >> s1), E);
+                        w[i] = fma(-sr, r.xo[a][i], w[i]);
+                    }
+                    double2* y = c.y + at + (int64_t)a * G.vstr;
+                    if (NP == 2) *y = cmk(w[0], w[NP - 1]);
+                    else reinterpret_cast<double*>(y)[r.part()] = w[0];
+                    if (c.dot) {
+#pragma unroll
+                        for (int i = 0; i < NP; ++i) r.dot = fma(r.xo[a][i], w[i], r.dot);
+                    }
                 }
             }
         }
@@ -650,10 +752,14 @@ struct FixApply {
         const int s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            r.pv[a] = r.cv[a];
-            const longlong2 g0 = sh.fs[(3 + a) * n + c0], g1 = sh.fs[(9 + a) * n + c1];
-            r.cv[a].x = (g0.x >> s0) + (g1.x >> s1);
-            r.cv[a].y = (g0.y >> s0) + (g1.y >> s1);
+            int64_t g0[NP], g1[NP];
+            get(a0 + (3 + a) * kRow, g0);
+            get(a1 + (9 + a) * kRow, g1);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                r.pv[a][i] = r.cv[a][i];
+                r.cv[a][i] = (g0[i] >> s0) + (g1[i] >> s1);
+            }
         }
     }
 
