@@ -7,7 +7,8 @@
 // One iteration: q = (A - sigma M) p with fused partials of Re<p, q> (stencil
 // kernel) -> alpha -> x += alpha p, r -= alpha q with partials of ||r||^2 ->
 // z = P r (block Fourier preconditioner) with partials of Re<r, z> -> beta and
-// the convergence test ||r|| <= tol ||b|| -> p = z + beta p.
+// the convergence test ||r|| <= tol ||b|| -> p = z + beta p.  While the vector
+// kernels are a few CTAs per SM, they compute alpha and beta themselves (sum_in_place).
 #include <cstdlib>
 #include <string>
 #include <cmath>
@@ -38,6 +39,29 @@ __device__ __forceinline__ double reduce_partials(const double* p, int n) {
     return block_sum_pcg(v);
 }
 
+// The sums of up to three lists of partials in every thread of the CTA, each in the order of reduce_partials.
+template <int NS>
+__device__ __forceinline__ void reduce_partials_all(const double* const (&p)[NS], const int (&n)[NS], double (&sum)[NS]) {
+    __shared__ double red[NS][32];
+    double v[NS];
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        v[l] = 0.0;
+        for (int i = threadIdx.x; i < n[l]; i += blockDim.x) v[l] += p[l][i];
+    }
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        for (int o = 16; o > 0; o >>= 1) v[l] += __shfl_down_sync(0xffffffffu, v[l], o);
+        if ((threadIdx.x & 31) == 0) red[l][threadIdx.x >> 5] = v[l];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        sum[l] = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum[l] += red[l][w];
+    }
+}
+
 template <typename C>
 __global__ void pcg_start(const C* __restrict__ b, C* __restrict__ x, C* __restrict__ r, int64_t vs,
                           double* __restrict__ part, int npart) {
@@ -63,8 +87,7 @@ __global__ void pcg_start_bb(PcgScal* sc, int* done, const double* part_bb, int 
     double bb = reduce_partials(part_bb + (int64_t)s * sbb, nbb);
     if (threadIdx.x == 0) {
         PcgScal v;
-        v.rz = 0;
-        v.pq = 0;
+        v.rz[0] = v.rz[1] = 0;
         v.alpha = 0;
         v.beta = 0;
         v.rr = bb;
@@ -92,7 +115,7 @@ __global__ void pcg_start_rz(PcgScal* sc, int* done, const double* part_rz, int 
     double rz = reduce_partials(part_rz + (int64_t)s * nrz, nrz);
     if (threadIdx.x == 0) {
         PcgScal v = sc[s];
-        v.rz = rz;
+        v.rz[0] = rz;
         if (!isfinite(rz)) {
             v.status = PC_ENAN;
             v.done = 1;
@@ -113,37 +136,86 @@ __global__ void pcg_copy(const C* __restrict__ z, C* __restrict__ p, int64_t vs,
         p[s * vs + e] = z[s * vs + e];
 }
 
-__global__ void pcg_alpha(PcgScal* sc, int* done, const double* part_pq, int spq, int npq) {
-    const int s = blockIdx.x;
-    if (done[s]) return;
-    double pq = reduce_partials(part_pq + (int64_t)s * spq, npq);
-    if (threadIdx.x == 0) {
-        sc[s].pq = pq;
-        if (!isfinite(pq)) {
-            sc[s].status = PC_ENAN;
-            sc[s].done = 1;
-            done[s] = 1;
-        } else if (!(pq > 0.0)) {
-            sc[s].status = PC_EBREAKDOWN;
-            sc[s].done = 1;
-            done[s] = 1;
-        } else {
-            sc[s].alpha = sc[s].rz / pq;
-        }
+// The scalars of a step.  alpha = rz / pq; beta = rz_new / rz_old (Fletcher-Reeves form) or, flexible, the
+// Polak-Ribiere form (rz_new - Re<r_new, z_old>) / rz_old (rzd = 0 otherwise).  Each also retires a system.
+__device__ __forceinline__ bool step_ok(double pq) { return isfinite(pq) && pq > 0.0; }
+__device__ __forceinline__ void end_half_step(PcgScal* sc, int* done, double pq, int parity) {
+    if (step_ok(pq)) {
+        sc->alpha = sc->rz[parity] / pq;
+    } else {
+        sc->status = isfinite(pq) ? PC_EBREAKDOWN : PC_ENAN;
+        sc->done = 1;
+        *done = 1;
     }
 }
+// rz_new goes to the other parity's slot: CTAs that sum in place may still read rz_old.
+__device__ __forceinline__ void end_step(PcgScal* sc, int* done, double rr, double rz, double rzd, int maxit, int parity) {
+    const int iters = sc->iters + 1;
+    int status = PC_OK, end = 1;
+    if (!isfinite(rr) || !isfinite(rz)) status = PC_ENAN;
+    else if (rr <= sc->thr) status = PC_OK;
+    else if (iters >= maxit) status = PC_ENOCONV;
+    else if (!(rz > 0.0)) status = PC_EBREAKDOWN;
+    else end = 0;
+    sc->beta = (rz - rzd) / sc->rz[parity];
+    sc->rz[parity ^ 1] = rz;
+    sc->rr = rr;
+    sc->iters = iters;
+    sc->status = status;
+    sc->done = end;
+    *done = end;
+}
 
-// x += alpha p, r -= alpha q with partials of ||r||^2; with zold non-null also partials of
-// Re<r_new, z_old> (flexible CG: the preconditioner is applied in lower precision).
-template <typename C>
+__global__ void pcg_alpha(PcgScal* sc, int* done, const double* part_pq, int spq, int npq, int parity) {
+    const int s = blockIdx.x;
+    if (done[s]) return;
+    const double pq = reduce_partials(part_pq + (int64_t)s * spq, npq);
+    if (threadIdx.x == 0) end_half_step(sc + s, done + s, pq, parity);
+}
+
+__global__ void pcg_beta(PcgScal* sc, int* done, const double* part_rr, int srr, int nrr, const double* part_rz,
+                         int nrz, int maxit, const double* part_d, int parity) {
+    const int s = blockIdx.x;
+    if (done[s]) return;
+    double v[3];
+    reduce_partials_all<3>({part_rr + (int64_t)s * srr, part_rz + (int64_t)s * nrz, part_d + (int64_t)s * srr},
+                           {nrr, nrz, part_d != nullptr ? nrr : 0}, v);
+    if (threadIdx.x == 0) end_step(sc + s, done + s, v[0], v[1], v[2], maxit, parity);
+}
+
+// Whether the vector kernels sum the partials in every CTA of a system (OWN below) instead of waiting for a
+// kernel of one CTA per system.  It saves two of some nine launches per iteration and costs every CTA a
+// latency of about 2 us, which more CTAs per SM pay one after the other.  Measured on one GB300, two kernels
+// against none: N = 48, one system (81 CTAs) 3.08 and 2.91 ms per solve; N = 64 (192 CTAs) 4.63 and 4.43 ms;
+// bands at N = 8 31.2 and 28.4 ms; even at N = 24, 20 bands (about 260 CTAs, 41.5 ms); lost at N = 32
+// (about 580 CTAs, 48.1 and 49.8 ms) and N = 48 with four Bloch vectors (220 and 263 ms).  The line lies at
+// two CTAs per SM.
+static bool sum_in_place(int vc, int nsys) { return (long)vc * nsys <= 2L * device_sm_count(); }
+
+// x += alpha p, r -= alpha q with partials of ||r||^2; with zold non-null also partials of Re<r_new, z_old>
+// (flexible CG: the preconditioner is applied in lower precision).
+//
+// OWN: every CTA of a system sums the partials of Re<p, q> itself, in the same order, and CTA 0 alone
+// writes the system's state.  A CTA that starts after CTA 0 has retired the system (a breakdown) returns
+// at once, an earlier one finds the same breakdown: neither changes x.
+template <typename C, bool OWN>
 __global__ void pcg_update_xr(C* __restrict__ x, C* __restrict__ r, const C* __restrict__ p, const C* __restrict__ q,
-                              const PcgScal* __restrict__ sc, const int* __restrict__ done, int64_t vs,
-                              double* __restrict__ part, int npart, const C* __restrict__ zold,
-                              double* __restrict__ part_d) {
+                              PcgScal* sc, int* done, int64_t vs, double* __restrict__ part, int npart,
+                              const C* __restrict__ zold, double* __restrict__ part_d,
+                              const double* __restrict__ part_pq, int npq, int parity) {
     const int s = blockIdx.y;
     if (done[s]) return;
     using R = decltype(x[0].x);
-    const R a = (R)sc[s].alpha;
+    R a;
+    if (OWN) {
+        double pq[1];
+        reduce_partials_all<1>({part_pq + (int64_t)s * npart}, {npq}, pq);
+        if (blockIdx.x == 0 && threadIdx.x == 0) end_half_step(sc + s, done + s, pq[0], parity);
+        if (!step_ok(pq[0])) return;
+        a = (R)(sc[s].rz[parity] / pq[0]);
+    } else {
+        a = (R)sc[s].alpha;
+    }
     // per-thread sums in the working precision (complex64: FP32 accumulation), FP64 across threads
     R acc = 0, accd = 0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
@@ -162,51 +234,29 @@ __global__ void pcg_update_xr(C* __restrict__ x, C* __restrict__ r, const C* __r
     }
 }
 
-// beta = rz_new / rz_old (Fletcher-Reeves form), or with part_d non-null the flexible
-// (Polak-Ribiere) form beta = (rz_new - Re<r_new, z_old>) / rz_old.
-__global__ void pcg_beta(PcgScal* sc, int* done, const double* part_rr, int srr, int nrr, const double* part_rz,
-                         int nrz, int maxit, const double* part_d) {
-    const int s = blockIdx.x;
-    if (done[s]) return;
-    double rr = reduce_partials(part_rr + (int64_t)s * srr, nrr);
-    double rz = reduce_partials(part_rz + (int64_t)s * nrz, nrz);
-    double rzd = part_d != nullptr ? reduce_partials(part_d + (int64_t)s * srr, nrr) : 0.0;
-    if (threadIdx.x == 0) {
-        PcgScal v = sc[s];
-        v.iters += 1;
-        v.rr = rr;
-        if (!isfinite(rr) || !isfinite(rz)) {
-            v.status = PC_ENAN;
-            v.done = 1;
-        } else if (rr <= v.thr) {
-            v.status = PC_OK;
-            v.done = 1;
-        } else if (v.iters >= maxit) {
-            v.status = PC_ENOCONV;
-            v.done = 1;
-        } else if (!(rz > 0.0)) {
-            v.status = PC_EBREAKDOWN;
-            v.done = 1;
-        } else {
-            v.beta = (rz - rzd) / v.rz;
-            v.rz = rz;
-        }
-        sc[s] = v;
-        done[s] = v.done;
-    }
-}
-
-template <typename C>
-__global__ void pcg_update_p(C* __restrict__ p, const C* __restrict__ z, const PcgScal* __restrict__ sc,
-                             const int* __restrict__ done, int64_t vs) {
+// p = z + beta p.  OWN: every CTA sums the partials itself, as in pcg_update_xr; CTA 0 alone decides whether
+// the system is done, the others update p in any case (a retired system's p is not read again).
+template <typename C, bool OWN>
+__global__ void pcg_update_p(C* __restrict__ p, const C* __restrict__ z, PcgScal* sc, int* done, int64_t vs,
+                             const double* __restrict__ part_rr, int srr, int nrr, const double* __restrict__ part_rz,
+                             int nrz, int maxit, const double* __restrict__ part_d, int parity) {
     const int s = blockIdx.y;
     if (done[s]) return;
     using R = decltype(p[0].x);
-    const R b = (R)sc[s].beta;
+    double v[3];  // ||r||^2 (CTA 0), Re<r, z>, Re<r, z_old>
+    R b;
+    if (OWN) {
+        reduce_partials_all<3>({part_rr + (int64_t)s * srr, part_rz + (int64_t)s * nrz, part_d + (int64_t)s * srr},
+                               {blockIdx.x == 0 ? nrr : 0, nrz, part_d != nullptr ? nrr : 0}, v);
+        b = (R)((v[1] - v[2]) / sc[s].rz[parity]);
+    } else {
+        b = (R)sc[s].beta;
+    }
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = s * vs + e;
         p[i] = cfma(b, p[i], z[i]);
     }
+    if (OWN && blockIdx.x == 0 && threadIdx.x == 0) end_step(sc + s, done + s, v[0], v[1], v[2], maxit, parity);
 }
 
 // Gather/scatter between a full-space vector and its four block vectors (stacked).
@@ -422,19 +472,26 @@ static int pcg_solve_t(pc_grid* g, int dtype, int nsys, const int* blocks, const
     }
     const ApplyConfig cfg = apply_config_for(g, full, nsys, dtype);
     const int napc = cfg.ctas;
-    const int chunk = 4;
-    auto iterate = [&]() -> int {
+    const int chunk = 4;  // even: an iteration's parity is its place in the chunk
+    const bool own = sum_in_place(vc, nsys);
+    auto iterate = [&](int c) -> int {
         PC_TRY(grid_apply(g, dtype, full, items.data(), nsys, part_a, npm, s, &cfg));
-        pcg_alpha<<<nsys, 256, 0, s>>>(w->sc, w->done, part_a, npm, napc);
-        note_launch();
-        pcg_update_xr<C><<<vgrid, 256, 0, s>>>(X, R, P, Q, w->sc, w->done, vs, part_b, npm, flex ? Z : nullptr,
-                                                part_d);
+        if (!own) {
+            pcg_alpha<<<nsys, 256, 0, s>>>(w->sc, w->done, part_a, npm, napc, c & 1);
+            note_launch();
+        }
+        auto xr = own ? pcg_update_xr<C, true> : pcg_update_xr<C, false>;
+        xr<<<vgrid, 256, 0, s>>>(X, R, P, Q, w->sc, w->done, vs, part_b, npm, flex ? Z : nullptr, part_d, part_a, napc,
+                                 c & 1);
         note_launch();
         PC_CUDA_TRY(cudaGetLastError());
         PC_TRY(precondition(full ? nullptr : w->done));
-        pcg_beta<<<nsys, 256, 0, s>>>(w->sc, w->done, part_b, npm, vc, part_c, nrz, maxit, part_d);
-        note_launch();
-        pcg_update_p<C><<<vgrid, 256, 0, s>>>(P, Z, w->sc, w->done, vs);
+        if (!own) {
+            pcg_beta<<<nsys, 256, 0, s>>>(w->sc, w->done, part_b, npm, vc, part_c, nrz, maxit, part_d, c & 1);
+            note_launch();
+        }
+        auto up = own ? pcg_update_p<C, true> : pcg_update_p<C, false>;
+        up<<<vgrid, 256, 0, s>>>(P, Z, w->sc, w->done, vs, part_b, npm, vc, part_c, nrz, maxit, part_d, c & 1);
         note_launch();
         PC_CUDA_TRY(cudaGetLastError());
         return PC_OK;
@@ -459,7 +516,7 @@ static int pcg_solve_t(pc_grid* g, int dtype, int nsys, const int* blocks, const
             const long long n0 = launch_count(), a0 = apply_launch_count();
             TimedSet* ts = timing_enabled() ? timing_capture_begin() : nullptr;
             int rc = PC_OK;
-            for (int c = 0; c < chunk && rc == PC_OK; ++c) rc = iterate();
+            for (int c = 0; c < chunk && rc == PC_OK; ++c) rc = iterate(c);
             cudaError_t e = cudaStreamEndCapture(s, &graph);
             if (ts) timing_capture_end(ts);
             if (rc != PC_OK || e != cudaSuccess) {
@@ -492,7 +549,7 @@ static int pcg_solve_t(pc_grid* g, int dtype, int nsys, const int* blocks, const
         if (graphs && it >= chunk) {
             PC_TRY(chunk_graph());
         } else {
-            for (int c = 0; c < chunk; ++c) PC_TRY(iterate());
+            for (int c = 0; c < chunk; ++c) PC_TRY(iterate(c));
         }
         it += chunk;
         PC_CUDA_TRY(cudaMemcpyAsync(w->h_sc, w->sc, sizeof(PcgScal) * nsys, cudaMemcpyDeviceToHost, s));

@@ -10,10 +10,9 @@ namespace pc {
 
 // Per-system PCG scalars (device).
 struct PcgScal {
-    double rz;     // Re <r, z>
-    double pq;     // Re <p, (A - sigma M) p>
-    double alpha;  // rz / pq
-    double beta;   // rz_new / rz
+    double rz[2];  // Re <r, z> of the running iteration and of the next, by iteration parity
+    double alpha;  // step of the solution, where a kernel of its own computes it
+    double beta;   // and of the search direction
     double rr;     // ||r||^2
     double bb;     // ||b||^2
     double thr;    // tol^2 ||b||^2: converged once ||r||^2 <= thr (set per solve, outside the graphs)
