@@ -381,8 +381,9 @@ int pc_eigs_batch(pc_batch_job* jobs, int njobs, const pc_options* opt, int work
 /* ---- launch tuning ----------------------------------------------------- */
 
 /* Autotuner of the stencil apply (no counterpart in the paper: an implementation choice).
- * Times every applicable kernel and launch shape (row-tile kernel with several persistent CTA
- * counts, TMA tile kernel, register-staged kernel, two-pass kernels; several k-chunkings) on scratch vectors for
+ * Times every applicable kernel and launch shape (integer-pipe, cell and two-pass kernels, row-tile and
+ * plane-pipelined kernels with several persistent CTA counts, TMA tile kernel, register-staged kernel;
+ * several k-chunkings) on scratch vectors for
  * batches of `nitems` (rounded up to a power of two, 1..64) vectors of precision `dtype` in the
  * parity-block layout (layout 0), the full-space layout (1) or both (2), and keeps the fastest
  * for every later apply, PCG and eigen-solve on grids of the same size, material kind and lattice

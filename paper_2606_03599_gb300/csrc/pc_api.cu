@@ -94,7 +94,7 @@ ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool
         return c;
     }
     if (scratch_ok && ((dtype == PC_C128 && (apply_kernel_mode() == 0 || apply_kernel_mode() == 5 || matkind == 2)) || apply_kernel_mode() == 3)) {
-        // complex128 is bound by GB300's FP64 pipe: fluxes once per node (two-pass kernels)
+        // out of the integer kernel's range, bound by the FP64 pipe: fluxes once per node (two-pass kernels)
         c.split = true;
         c.shape = 0;
         c.tz = Z;
@@ -510,8 +510,8 @@ static StencilParams<R> params_at(const pc_grid* g, const StencilParams<R>& base
     return P;
 }
 
-// One launch of items whose kernel takes grid-uniform Bloch phases (all items in `slot`), or, for
-// the two-pass and plane-pipelined kernels, each item's own phases from item_ph.
+// One launch of items whose kernel takes grid-uniform Bloch phases (all items in `slot`), or, for the
+// integer-pipe, cell, two-pass and plane-pipelined kernels, each item's own phases from item_ph.
 static int apply_launch(pc_grid* g, int dtype, bool full, const ApplyConfig& cfg, const ApplyItem* items,
                         const double* item_ph, int nitems, int slot, double* dot_partials, int dot_stride,
                         cudaStream_t s) {
@@ -564,8 +564,8 @@ static int apply_launch(pc_grid* g, int dtype, bool full, const ApplyConfig& cfg
 }
 
 // Launch one batch of stencil applies on grid g (items share the layout kind; each item at the
-// Bloch vector of its slot).  The two-pass and plane-pipelined kernels take every item's phases,
-// so one launch serves several Bloch vectors; the other kernels run once per run of equal slots.
+// Bloch vector of its slot).  The integer-pipe, cell, two-pass and plane-pipelined kernels take every
+// item's phases, so one launch serves several Bloch vectors; the other kernels run once per run of equal slots.
 int grid_apply(pc_grid* g, int dtype, bool full, const ApplyItem* items, int nitems, double* dot_partials,
                int dot_stride, cudaStream_t s, const ApplyConfig* cfg_in) {
     const int X = full ? g->N : g->X, Y = full ? g->N : g->Y, Z = g->Z;

@@ -19,13 +19,14 @@
 // vector is treated as its four parity blocks with strided addresses (the blocks do not couple), so
 // one geometry serves both layouts.
 //
-// The tile and its march are pc_apply_cells.cuh's: each cell is one thread, which stages x of its
-// column (asynchronous copy, Bloch phase if wrapped, conversion), forms the fluxes of its column when
-// the plane's parity needs them, and, among the first TX x TY, finishes the outputs.
+// The tile and its march are pc_apply_cells.cuh's: each cell is one thread (two in small launches, see
+// FixApply), which stages x of its column (asynchronous copy, Bloch phase if wrapped, conversion), forms
+// the fluxes of its column when the plane's parity needs them, and, among the first TX x TY, finishes the
+// outputs.
 //
-// Measured (one GB300, N = 48, 64 block vectors, shift on): 0.205 ms against 0.667 ms of the two-pass
-// FP64 kernels; N = 60 FCC sub-pixel material, four blocks: 0.084 against 0.195 ms; N = 64 nodewise
-// material, full space: 0.102 against 0.146 ms.  Bound by the instruction stream (half the issue slots
+// Measured (one GB300, N = 48, 64 block vectors, shift on): 0.212 ms against 0.667 ms of the two-pass
+// FP64 kernels; N = 60 FCC sub-pixel material, four blocks: 0.086 against 0.195 ms; N = 64 nodewise
+// material, full space: 0.090 against 0.146 ms.  Bound by the instruction stream (half the issue slots
 // at 16 warps per SM); DRAM moves 143 MB per launch at N = 48, close to the 170 MB of x and y.
 //
 // Values outside the exponent range (infinities, NaN, below 2^-823 or above 2^877) mark their node;

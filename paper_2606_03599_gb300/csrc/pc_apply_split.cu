@@ -1,5 +1,6 @@
-// Two-pass stencil apply (see pc_apply_split.cuh): kernels and launchers.  Complex128 by default
-// (bound by the FP64 pipe); complex64 as an autotuner candidate for grids whose fluxes stay in L2.
+// Two-pass stencil apply (see pc_apply_split.cuh): kernels and launchers.  Complex128 (bound by
+// the FP64 pipe) where the integer-pipe kernel does not apply; complex64 as an autotuner candidate for
+// grids whose fluxes stay in L2.
 #include <algorithm>
 
 #include "pc_apply_split.cuh"

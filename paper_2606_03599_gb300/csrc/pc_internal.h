@@ -114,7 +114,7 @@ struct ApplyConfig {
     int ctas = 1;      // CTAs per item (row kernel: CTAs of the persistent launch)
     bool tma = false;  // TMA-staged kernel (quarter grids of even width >= 8)
     bool row = false;  // row-tile kernel (complex64 parity blocks, X even)
-    bool split = false;  // two-pass complex128 kernels (flux, then gather)
+    bool split = false;  // two-pass kernels (flux, then gather)
     bool pipe = false;   // plane-pipelined kernel (complex64 parity blocks, even X)
     bool fix = false;    // integer-pipe complex128 kernel (shape code kFixShape)
     bool cell = false;   // complex64 cell kernel (shape code kCellShape)
@@ -254,7 +254,7 @@ struct pc_grid {
     int items_cap = 0;
     double* d_dot = nullptr;
     int dot_cap = 0;
-    void* d_split = nullptr;  // scratch of the two-pass complex128 apply (extended x and fluxes)
+    void* d_split = nullptr;  // scratch of the two-pass apply (ghost cells of x and fluxes)
     size_t split_bytes = 0;
     // preconditioner / solver workspaces are attached by their modules
     struct Precond* pre = nullptr;

@@ -2,10 +2,10 @@
 // or full space, material kind, lattice) and one batch size, time every applicable kernel and
 // launch shape on the GPU and keep the fastest.
 //
-// Candidates: the plane-pipelined and row-tile kernels (complex64 blocks) with several persistent
-// CTA counts, the
-// TMA tile kernel (16-wide and 8-wide tiles) and the register-staged kernel (four tile shapes),
-// each with k-chunkings that target one, two or four resident CTAs per SM.  Results live in a
+// Candidates: the integer-pipe kernel (complex128) and the cell kernel (complex64) with their own
+// chunking, the two-pass kernels, the plane-pipelined and row-tile kernels (complex64 blocks) with several
+// persistent CTA counts, the TMA tile kernel (16-wide and 8-wide tiles) and the register-staged kernel
+// (four tile shapes), each with k-chunkings that target one, two or four resident CTAs per SM.  Results live in a
 // process-wide table keyed by (X, Y, Z, dtype, layout, material kind, lattice, batch-size
 // bucket, SM count) and, when PC_TUNE_CACHE names a file, are read from and appended to it
 // (one JSON object per key), so a later process starts tuned.
@@ -166,11 +166,10 @@ static std::vector<ApplyConfig> candidates(int X, int Y, int Z, int dtype, bool 
         out.push_back(c);
     }
     const int sm = device_sm_count();
-    // two-pass kernels: the default for complex128; for complex64 a candidate while the batch's
-    // scratch (15 complex64 flux arrays per extended cell plus x's ghost cells) fits in L2
-    // (126 MB on GB300)
+    // two-pass kernels: a candidate for complex128; for complex64 while the batch's scratch (15 complex64
+    // flux arrays per extended cell plus x's ghost cells) fits in L2 (126 MB on GB300)
     const double split_mb = (double)split_scratch_bytes(X, Y, Z, nitems, dtype) / (1 << 20);
-    if (matkind == 2) {  // a nodewise material: the complex128 two-pass kernels only
+    if (matkind == 2) {  // a nodewise material: the integer-pipe (above) and two-pass kernels only
         if (dtype == PC_C128) {
             ApplyConfig c;
             c.split = true;
