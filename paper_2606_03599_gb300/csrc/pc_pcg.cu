@@ -192,6 +192,14 @@ __global__ void pcg_beta(PcgScal* sc, int* done, const double* part_rr, int srr,
 // two CTAs per SM.
 static bool sum_in_place(int vc, int nsys) { return (long)vc * nsys <= 2L * device_sm_count(); }
 
+// Whether the system is done, the same answer for the whole CTA: with OWN, CTA 0 of the running launch may be
+// about to write the flag, and threads that read it one by one could part before a barrier.
+template <bool OWN>
+__device__ __forceinline__ bool retired(const int* done) {
+    if (!OWN) return *done != 0;
+    return __syncthreads_or(threadIdx.x == 0 && *reinterpret_cast<const volatile int*>(done)) != 0;
+}
+
 // x += alpha p, r -= alpha q with partials of ||r||^2; with zold non-null also partials of Re<r_new, z_old>
 // (flexible CG: the preconditioner is applied in lower precision).
 //
@@ -204,7 +212,7 @@ __global__ void pcg_update_xr(C* __restrict__ x, C* __restrict__ r, const C* __r
                               const C* __restrict__ zold, double* __restrict__ part_d,
                               const double* __restrict__ part_pq, int npq, int parity) {
     const int s = blockIdx.y;
-    if (done[s]) return;
+    if (retired<OWN>(done + s)) return;
     using R = decltype(x[0].x);
     R a;
     if (OWN) {
@@ -241,7 +249,7 @@ __global__ void pcg_update_p(C* __restrict__ p, const C* __restrict__ z, PcgScal
                              const double* __restrict__ part_rr, int srr, int nrr, const double* __restrict__ part_rz,
                              int nrz, int maxit, const double* __restrict__ part_d, int parity) {
     const int s = blockIdx.y;
-    if (done[s]) return;
+    if (retired<OWN>(done + s)) return;
     using R = decltype(p[0].x);
     double v[3];  // ||r||^2 (CTA 0), Re<r, z>, Re<r, z_old>
     R b;
