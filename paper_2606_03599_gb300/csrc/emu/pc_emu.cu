@@ -357,6 +357,9 @@ static void emu_run_split(const StencilParams<R>& P, int block, const void* x, v
         T::gather_node(P, G, p12, p13, fe.data(), xv, static_cast<C*>(y), mat, (R)shift, t, true);
 }
 
+static int emu_slow_columns = 0;  // columns of the last integer-pipe apply that were handed to FP64
+extern "C" int pc_emu_slow_columns() { return emu_slow_columns; }
+
 // Same step sequence as fix_apply (tz planes per CTA; tx, ty > 0 force the tile extents); shared
 // memory poisoned first.
 template <bool CUBIC, int MATK>
@@ -376,6 +379,7 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
     FixParams F;
     if (!make_fix_params(F, P, CUBIC, MATK)) return -2;
     const int n = G.ncell;
+    emu_slow_columns = 0;
     std::vector<unsigned char> mem(T::shared_bytes() + 64);
     std::vector<typename T::Regs> regs(n);
     for (int sub = 0; sub < (G.full ? 4 : 1); ++sub)
@@ -440,7 +444,10 @@ static int emu_run_fix(const StencilParams<double>& P, int block, const void* x,
                 step(std::integral_constant<int, 0>(), kf + 1);
             }
             for (int t = 0; t < n; ++t)
-                if (regs[t].ks < c.k0 + c.tz) T::slow_column(c, regs[t].ks, regs[t].off[0], regs[t].off[1]);
+                if (regs[t].ks < c.k0 + c.tz) {
+                    T::slow_column(c, regs[t].ks, regs[t].off[0], regs[t].off[1]);
+                    ++emu_slow_columns;
+                }
         }
     return 0;
 }

@@ -584,6 +584,7 @@ struct FixApply {
             FixHalf th = {0, 0};
             const double* md = nullptr;
             int base = 64;
+            bool empty = false;  // a void: zero fluxes, whatever x is
             if (MATK == 1) {
                 th = fix_split(fix_theta(mat_theta(r.mcur)));
                 fe += c.F->coff[0];
@@ -596,6 +597,13 @@ struct FixApply {
                 for (int u = 0; u < 21; ++u) top = imax(top, (int)(fix_bits(md[(int64_t)u * G.vstr]) >> 32) & 0x7fffffff);
                 base = top >> 20;  // entries below 2^59: row sums below 2^62
                 fe += base - 1017;
+                if (base == 0) {
+                    int64_t any = 0;
+#pragma unroll
+                    for (int u = 0; u < 21; ++u) any |= fix_bits(md[(int64_t)u * G.vstr]);
+                    empty = (any & 0x7fffffffffffffffLL) == 0;
+                    base = empty ? 1000 : 0;
+                }
                 if (base < 950 || base > 1100) {  // tables far outside hat units
                     sh.fe[own] = kFixSpecial;
                     r.ce = kFixSpecial;
@@ -628,7 +636,7 @@ struct FixApply {
             const int top = imax(imax(imax(row[0], row[1]), imax(row[2], row[3])), imax(row[4], row[5])) + 6;
             int sh2 = (top < (1 << 24) ? 6 : top < (1 << 25) ? 5 : top < (1 << 26) ? 4 : top < (1 << 27) ? 3
                        : top < (1 << 28) ? 2 : top < (1 << 29) ? 1 : 0);
-            fe -= sh2;
+            fe = empty ? 0 : fe - sh2;
             sh2 += CUBIC ? 0 : 2;
 #pragma unroll
             for (int p = 0; p < 6; ++p)
