@@ -46,8 +46,8 @@
  * Environment (read once per process; results do not depend on them):
  *            PC_APPLY_KERNEL = legacy | tma | split | row | pipe forces one
  *            stencil-kernel family for A/B comparisons (default: the cell kernel
- *            for complex64, the integer-pipe kernel for complex128, or the
- *            autotuner's choice); PC_PCG_GRAPHS = 0 turns off CUDA-graph replay of PCG
+ *            for complex64, the integer-pipe or two-pass kernels for complex128 by
+ *            material and size, or the autotuner's choice); PC_PCG_GRAPHS = 0 turns off CUDA-graph replay of PCG
  *            iterations; PC_TUNE_CACHE names the autotuner's cache file
  *            (pc_autotune); PC_WAIT_LIMIT = n sets how many polls a kernel's
  *            wait on its own shared-memory copies makes before it gives up
@@ -164,7 +164,7 @@ int pc_grid_create(int N, const pc_material* m, pc_grid** out);
  * Voigt stiffness in row order ([11,22,33,23,13,12], engineering shear, Pa); rho: host [N^3],
  * kg/m^3, positive; a_lat as in pc_material.  Both arrays are copied (caller keeps ownership).
  * The device holds 22 FP64 values per node in each layout (about 0.35 KB per node in all).
- * Supported paths: complex128 applies (integer-pipe or two-pass kernels), PC_PREC_FP64 eigen-solves, PCG,
+ * Supported paths: complex128 applies (two-pass kernels, or the integer-pipe kernel where tuned), PC_PREC_FP64 eigen-solves, PCG,
  * mass, gradients (pc_eig_grad); complex64 applies and PC_PREC_MIXED return PC_EINVAL.  The
  * preconditioner's reference medium and the default shift use the nodes' volume averages and
  * largest entries.  PC_EINVAL for a non-finite entry or a non-positive density. */
@@ -394,9 +394,9 @@ int pc_autotune(pc_grid* g, int dtype, int layout, int nitems, void* stream);
 
 /* The launch configuration the library will use for a batch of `nitems` vectors of `dtype` in
  * layout 0 (blocks) or 1 (full): kind 0 = fused tile (shapes 0-3 register-staged; shape 8 the
- * integer-pipe kernel, the default for complex128; shape 9 the cell kernel, the default for
+ * integer-pipe kernel, the default for complex128 with phase ids and for larger batches of fractions; shape 9 the cell kernel, the default for
  * complex64), 1 = TMA tile, 2 = row tile, 3 = two-pass
- * (fluxes once per node, then gather), 4 = plane-pipelined (producer
+ * (fluxes once per node, then gather; the default for complex128 otherwise), 4 = plane-pipelined (producer
  * warp + consumer warps); tile shape code; planes per CTA
  * (tz; row and plane-pipelined kernels: least planes per CTA); CTAs of the launch (two-pass: of
  * its gather). */

@@ -85,7 +85,14 @@ int device_sm_count() {
 ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool blocks, int matkind, bool scratch_ok,
                                 bool int_ok, bool cubic) {
     ApplyConfig c;
-    if (int_ok && dtype == PC_C128 && (apply_kernel_mode() == 0 || apply_kernel_mode() == 5)) {
+    // Nodes from which the integer-pipe kernel is the faster one.  With phase ids it always is (a few percent
+    // either way on general lattices between 40k and 130k nodes); a stiffness per node costs it 36 products and their
+    // alignments, chains that a small launch waits for, where the two-pass kernels take a constant 31 to 35 us.
+    // Measured, integer / two-pass: fractions on a cubic lattice 16k nodes 41 / 33, 28k 39 / 43 us; on FCC
+    // 186k 164 / 162, 221k 129 / 208 us.  Nodewise tables read once from memory: 262k nodes 157 / 146 us.
+    const int64_t int_from = matkind == 0 ? 0 : matkind == 2 ? INT64_MAX : cubic ? 20000 : 200000;
+    if (int_ok && (int64_t)X * Y * Z * nitems >= int_from && dtype == PC_C128 &&
+        (apply_kernel_mode() == 0 || apply_kernel_mode() == 5)) {
         // the FP64 pipe of GB300 (2 lanes per clock and SM) is left to the integer units; see
         // pc_apply_int.cuh
         c.fix = true;
@@ -94,7 +101,7 @@ ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool
         return c;
     }
     if (scratch_ok && ((dtype == PC_C128 && (apply_kernel_mode() == 0 || apply_kernel_mode() == 5 || matkind == 2)) || apply_kernel_mode() == 3)) {
-        // out of the integer kernel's range, bound by the FP64 pipe: fluxes once per node (two-pass kernels)
+        // nodewise materials and small launches of fractions: fluxes once per node (two-pass kernels)
         c.split = true;
         c.shape = 0;
         c.tz = Z;

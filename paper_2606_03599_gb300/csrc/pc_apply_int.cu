@@ -133,9 +133,11 @@ int launch_fix_np(const FixParams& F, const FixBatch& B, const CellGeom& G, doub
 
 template <bool CUBIC, int MATK>
 int launch_fix_t(const FixParams& F, const FixBatch& B, const CellGeom& G, double* dp, int ds, cudaStream_t s) {
-    // one CTA per SM at most: two threads per cell (see FixApply)
+    // Two threads per cell (see FixApply) in launches of one CTA per SM at most, and where a tile has so few cells
+    // that its CTA has half the threads and two still share an SM (N = 16, 64 items: 28.9 us, 44.9 us with one
+    // thread per cell; N = 10 26.8 / 39.1, N = 18 43.9 / 67.3 us).
     const long ctas = (long)G.ntx * G.nty * G.nch * B.n * (G.full ? 4 : 1);
-    return ctas <= device_sm_count() ? launch_fix_np<CUBIC, MATK, 1>(F, B, G, dp, ds, s)
+    return ctas <= device_sm_count() || G.ncell <= kCells / 2 ? launch_fix_np<CUBIC, MATK, 1>(F, B, G, dp, ds, s)
                                      : launch_fix_np<CUBIC, MATK, 2>(F, B, G, dp, ds, s);
 }
 
@@ -167,7 +169,7 @@ int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<dou
     if (dp != nullptr && G.ntx * G.nty * G.nch * (full ? 4 : 1) > ds)
         return fail(PC_EINVAL, "apply: launch has more CTAs than partial-sum slots");
     FixParams F;
-    if (!make_fix_params(F, P, cubic, matkind)) return fail(PC_EINVAL, "apply: material scale outside the integer kernel's range");
+    if (!make_fix_params(F, P, cubic, matkind)) return fail(PC_EINVAL, "apply: a stiffness entry is not finite");
     for (int base = 0; base < nitems; base += kFixMaxItems) {
         FixBatch B;
         B.n = std::min(nitems - base, kFixMaxItems);

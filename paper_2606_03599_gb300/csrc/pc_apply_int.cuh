@@ -1,19 +1,23 @@
-// Complex128 stencil apply on the integer pipe: y = (A - shift M) x with every FP64 operand of the
-// stencil held as a 64-bit integer and one binary exponent per node.
+// Complex128 stencil apply on the integer pipe: y = (A - shift M) x with the FP64 operations of the stencil
+// done on 64-bit integers with an exponent each (pc_wide.cuh).
 //
-// GB300 issues 2 FP64 lanes per clock and SM, but 64 lanes of 64-bit integer addition and 64 of
-// 32 x 32 + 64 bit multiply-add (measured: add.s64 63.9, mad.wide.s32 63.7, fma.f64 2.0).  The
-// stencil is additions and products with constants, so it is done in block floating point: a node's
-// six reals are integers below 2^56 in units of 2^(E - 1078), E the largest biased exponent among
-// them (FP64 values with an exponent within 3 of E keep every bit).  Sums are exact; a product with
-// a stiffness entry is 3 multiply-adds of 32-bit halves (the low x low part, below 2^-2 units, is
-// left out) and rounds once per output.  The rounding of a flux is a few units of 2^-57 of the
-// largest strain its node's values allow, where FP64 rounds the same sums at 2^-53 of them.
-//
-// Bounds (units of the node's exponent): x < 2^56, the sums H < 2^59 and strain < 2^60, stiffness
-// rows sum to less than 2^62 so that a stress is below 2^58 after the division by 2^64 (general
-// lattice: mixed sums < 2^59, stresses < 2^60 and their mixing < 0.98 2^59), fluxes < 2^59.6 and an output
-// below 2^62.2 (2^60.6 and 0.98 2^63).  Accumulated products: high parts < 2^58, middle parts < 2^62.4.
+// GB300 issues 2 FP64 lanes per clock and SM and 64 of 64-bit integer additions, so even written out as
+// alignment, addition and normalisation an FP64 operation costs a fraction of its instruction.  Real and
+// imaginary parts, components, strains, stresses and stiffness entries all keep exponents of their own: what
+// is not added never shares a unit, so a small part, a small component or a soft phase is as accurate next to
+// a large one as in FP64.  Errors, against FP64's 2^-53 of the result of every operation:
+//   x           53 bits and 6 below them; the five values of a difference sum (one component, one part) are cut
+//               at 2^-59 of the largest, and the sums themselves are exact
+//   strain      normal exact, shear cut at 2^-59 of the larger component's x; a difference that vanishes
+//               does not count (a uniform component leaves the other's bits alone)
+//   stress      products at 2^-57, their sums cut at 2^-58 of the largest product
+//   flux        stresses cut at 2^-54 to 2^-57 of the largest, their sums exact
+//   output      sums of fluxes of one unit exact (others cut at that of the largest), one rounding to FP64, the
+//               shift term by an FMA
+// Against extended precision the result is 5e-17 off on broad-band vectors (FP64: 1.1e-16) and 3e-16 on long
+// waves at N = 48 (FP64: 2e-15).  One exponent shared by a node's six reals took two thirds of the time and left
+// 1e-13 of a transverse wave along an axis in steel, 1e-9 in a gel, 2e-8 of a strain next to a uniform
+// displacement 1e8 times as large.
 //
 // The operator, the layouts and the flux regions are those of pc_apply_tile.cuh.  A full-space
 // vector is treated as its four parity blocks with strided addresses (the blocks do not couple), so
@@ -24,13 +28,17 @@
 // the fluxes of its column when the plane's parity needs them, and, among the first TX x TY, finishes the
 // outputs.
 //
-// Measured (one GB300, N = 48, 64 block vectors, shift on): 0.212 ms against 0.667 ms of the two-pass
-// FP64 kernels; N = 60 FCC sub-pixel material, four blocks: 0.086 against 0.195 ms; N = 64 nodewise
-// material, full space: 0.090 against 0.146 ms.  Bound by the instruction stream (half the issue slots
-// at 16 warps per SM); DRAM moves 143 MB per launch at N = 48, close to the 170 MB of x and y.
+// Measured (one GB300, shift on, against the two-pass FP64 kernels): N = 48, 64 block vectors, one phase fully
+// anisotropic 0.353 / 0.667 ms; N = 60 FCC sub-pixel material, four blocks 0.137 / 0.195 ms; N = 64 nodewise
+// material, full space 0.157 / 0.146 ms, which is why nodewise materials take it only where the autotuner finds
+// it faster.  Bound by the integer instruction stream (16 warps per SM): a product and its place in a sum are ten
+// instructions, half of them at half rate.  (Nine products instead of 36 in warps whose nodes are orthotropic pay
+// for phase ids; for fractions and nodewise tables the second copy of the loop cost more than it saved: 169 and
+// 144 us.)
 //
-// Values outside the exponent range (infinities, NaN, below 2^-823 or above 2^877) mark their node;
-// a column is handed to FP64 (slow_column) from the first output that depends on a marked node.
+// Infinities, NaN and nodes whose values are all below 2^-943 (their products with the Bloch phase round as
+// subnormals, and FP64's order of operations counts) mark their node; a column is handed to FP64 (slow_column)
+// from the first output that depends on a marked node.
 #pragma once
 
 #include <math.h>
@@ -41,6 +49,7 @@
 #include "pc_apply_tile.cuh"  // PC_IDX
 #include "pc_complex.cuh"
 #include "pc_internal.h"
+#include "pc_wide.cuh"
 
 #if defined(__CUDACC__)
 #define PC_FIX_COLD __noinline__
@@ -50,211 +59,69 @@
 
 namespace pc {
 
-constexpr int kFixSpecial = 1 << 14;  // exponent of a node that FP64 has to handle
-constexpr int kFixLow = 200, kFixHigh = 1900;  // biased exponents the integer path takes
-
-struct FixHalf {
-    int hi, lo;  // c = hi 2^32 + lo, lo signed
-};
-
 struct FixParams {
     StencilParams<double> P;  // FP64 tables: density, slow_column
-    FixHalf c[2][21];         // phase tables; MATK 1: C_0 and C_1 - C_0
-    FixHalf mix[9];           // lattice mixing (general lattices)
-    int coff[2];              // exponent a product with c[p] adds
-    int moff;                 // and the two lattice mixings together
-    int nthr;
+    WideEntry c[2][21];       // MATK 0: phase tables
+    double c0[21], dc[21];    // MATK 1: C_0 and C_1 - C_0
+    WideEntry mix[9];         // lattice mixing (general lattices)
 };
 
-PC_HD FixHalf fix_split(int64_t v) {
-    FixHalf h;
-    h.hi = (int)((v + 0x80000000LL) >> 32);
-    h.lo = (int)(uint32_t)v;
-    return h;
-}
 PC_HD int fix_upper(int p, int r) { return p <= r ? p * 6 - p * (p - 1) / 2 + (r - p) : r * 6 - r * (r - 1) / 2 + (p - r); }
 
-// Tables of one launch; false when a scale is out of the exponent range the kernel allows for.
+// Tables of one launch; false when an entry is not finite.
 inline bool make_fix_params(FixParams& F, const StencilParams<double>& P, bool cubic, int matkind) {
+    memset(&F, 0, sizeof(F));
     F.P = P;
-    memset(F.c, 0, sizeof(F.c));
-    memset(F.mix, 0, sizeof(F.mix));
-    F.coff[0] = F.coff[1] = F.moff = 0;
-    if (matkind != 2) {
-        double rs[2];
-        for (int p = 0; p < 2; ++p) {
-            rs[p] = 0.0;
-            for (int i = 0; i < 6; ++i) {
-                double s = 0.0;
-                for (int j = 0; j < 6; ++j) s += fabs(P.C[p][i * 6 + j]);
-                rs[p] = fmax(rs[p], s);
-            }
-        }
-        if (matkind == 1) rs[0] = rs[1] = fmax(rs[0], rs[1]);
-        int k[2];
-        for (int p = 0; p < 2; ++p) {
-            int ex = 0;
-            if (!isfinite(rs[p])) return false;
-            if (rs[p] > 0) frexp(rs[p], &ex);
-            k[p] = (matkind == 1 ? 61 : 62) - ex;  // row sums of |c| below 2^62 (2^61: C_1 - C_0)
-            F.coff[p] = 64 - k[p];
-        }
+    bool ok = true;
+    if (matkind != 2)
         for (int i = 0; i < 6; ++i)
             for (int j = i; j < 6; ++j) {
-                const int64_t a = llrint(ldexp(P.C[0][i * 6 + j], k[0]));
-                const int64_t b = llrint(ldexp(P.C[1][i * 6 + j], k[1]));
-                F.c[0][fix_upper(i, j)] = fix_split(a);
-                F.c[1][fix_upper(i, j)] = fix_split(matkind == 1 ? b - a : b);
+                const int q = fix_upper(i, j);
+                for (int p = 0; p < 2; ++p) {
+                    ok = ok && isfinite(P.C[p][i * 6 + j]);
+                    F.c[p][q] = wide_entry(P.C[p][i * 6 + j]);
+                }
+                F.c0[q] = P.C[0][i * 6 + j];
+                F.dc[q] = P.C[1][i * 6 + j] - P.C[0][i * 6 + j];
+                ok = ok && isfinite(F.dc[q]);
             }
-    }
-    if (!cubic) {
-        double ms = 0.0;
-        for (int i = 0; i < 3; ++i) {
-            ms = fmax(ms, fabs(P.Mmix[i]) + fabs(P.Mmix[3 + i]) + fabs(P.Mmix[6 + i]));
-            ms = fmax(ms, fabs(P.Mmix[3 * i]) + fabs(P.Mmix[3 * i + 1]) + fabs(P.Mmix[3 * i + 2]));
+    if (!cubic)
+        for (int e = 0; e < 9; ++e) {
+            ok = ok && isfinite(P.Mmix[e]);
+            F.mix[e] = wide_entry(P.Mmix[e]);
         }
-        int ex = 0;
-        if (!isfinite(ms)) return false;
-        // sums below 0.98 2^62: the outputs, below 16 x 0.98 2^59, stay clear of the sign bit
-        if (ms > 0 && frexp(ms, &ex) > 0.98) ++ex;
-        F.moff = 2 * (64 - (62 - ex)) - 5;  // both mixings, less the bits their shifts keep
-        for (int e = 0; e < 9; ++e) F.mix[e] = fix_split(llrint(ldexp(P.Mmix[e], 62 - ex)));
-    }
-    for (int p = 0; p < 2; ++p)
-        if (F.coff[p] + F.moff > 100 || F.coff[p] + F.moff < -100) return false;
-    return true;
-}
-
-PC_HD longlong2 fix_ashr2(longlong2 v, int s) {
-    longlong2 r;
-    r.x = v.x >> s;
-    r.y = v.y >> s;
-    return r;
-}
-PC_HD int imax(int a, int b) { return a > b ? a : b; }
-PC_HD int imin(int a, int b) { return a < b ? a : b; }
-
-PC_HD int64_t fix_bits(double v) {
-#if defined(__CUDA_ARCH__)
-    return __double_as_longlong(v);
-#else
-    int64_t b;
-    memcpy(&b, &v, 8);
-    return b;
-#endif
-}
-PC_HD double fix_from_bits(int64_t b) {
-#if defined(__CUDA_ARCH__)
-    return __longlong_as_double(b);
-#else
-    double v;
-    memcpy(&v, &b, 8);
-    return v;
-#endif
-}
-PC_HD int fix_clz64(uint64_t v) {
-#if defined(__CUDA_ARCH__)
-    return __clzll((long long)v);
-#else
-    return __builtin_clzll(v);
-#endif
-}
-
-// v as an integer below 2^up (up in 53..63) in units of 2^(E - 1022 - up); base = E, or 64 for E = 0
-// (all values of the node zero).  Bits below the unit are dropped.
-PC_HD int64_t fix_from_double(double v, int base, int lead) {
-    const int64_t b = fix_bits(v);
-    const int hi = (int)(b >> 32);
-    const int e = (hi >> 20) & 0x7ff;
-    const uint64_t m = (((uint64_t)b & 0xfffffffffffffULL) | 0x10000000000000ULL) << lead;
-    const int64_t s = hi >> 31;
-    return ((int64_t)(m >> imin(base - e, 63)) ^ s) - s;
-}
-// largest |high word| of a complex number
-PC_HD int fix_high(double2 v, int m) {
-    m = imax(m, (int)(fix_bits(v.x) >> 32) & 0x7fffffff);
-    return imax(m, (int)(fix_bits(v.y) >> 32) & 0x7fffffff);
-}
-// v 2^(E - 1078), rounded to nearest
-PC_HD double fix_to_double(int64_t v, int E) {
-#if defined(__CUDA_ARCH__)
-    // one conversion on the FP64 pipe, which has room, instead of twenty integer instructions; the
-    // scale goes into the exponent field
-    const double d = __ll2double_rn(v);
-    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (E - 1078) * (1 << 20), __double2loint(d));
-#else
-    const int64_t s = v >> 63;
-    const uint64_t mag = (uint64_t)((v ^ s) - s);
-    if (mag == 0) return 0.0;
-    const int lz = fix_clz64(mag);
-    const uint64_t n = mag << lz;
-    const uint64_t r = (n >> 11) + ((n >> 10) & 1);
-    const uint64_t bits = ((uint64_t)(E + 7 - lz) << 52) + r;
-    return fix_from_bits((int64_t)(bits | ((uint64_t)s & 0x8000000000000000ULL)));
-#endif
-}
-
-// acc + a b.  In PTX on the device: written in C++ the compiler loses sight of the operands being
-// 32 bits wide and multiplies 64 x 64.
-PC_HD void fix_mad(int64_t& acc, int a, int b) {
-#if defined(__CUDA_ARCH__)
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
-#else
-    acc += (int64_t)a * b;
-#endif
-}
-// hi 2^64 + mid 2^32 accumulates e c for signed halves
-PC_HD void fix_mac(int64_t& hi, int64_t& mid, FixHalf e, FixHalf c) {
-    fix_mad(hi, e.hi, c.hi);
-    fix_mad(mid, e.hi, c.lo);
-    fix_mad(mid, e.lo, c.hi);
-}
-// the accumulated product over 2^(64 - s), rounded (s in 0..8)
-PC_HD int64_t fix_sum(int64_t hi, int64_t mid, int s) { return (hi << s) + ((mid + (0x80000000LL >> s)) >> (32 - s)); }
-
-// theta in [0, 1] as an integer in units of 2^-62
-PC_HD int64_t fix_theta(float t) {
-#if defined(__CUDA_ARCH__)
-    const uint32_t b = __float_as_uint(t);
-#else
-    uint32_t b;
-    memcpy(&b, &t, 4);
-#endif
-    const int e = (int)(b >> 23);
-    if (e == 0) return 0;
-    const uint64_t m = (uint64_t)((b & 0x7fffffu) | 0x800000u) << 39;
-    return (int64_t)(m >> imin(127 - e, 63));
+    return ok;
 }
 
 // MATK: 0 = phase ids, 1 = inclusion fraction, 2 = nodewise material (as SplitApply).
-// NP: parts (real, imaginary) of a cell in one thread; they meet in the Bloch phase and in the shared
-// exponent only.  NP = 2 runs fewer instructions and is the form of launches that fill the GPU (N = 48, 64
-// block vectors: 212 us, 267 us with NP = 1).  NP = 1, two adjacent lanes per cell, halves a thread's chain
-// of dependent instructions: the form of launches with at most one CTA per SM, which wait for that chain
-// (N = 8, one block vector: 14.3 us, 18.4 us with NP = 2).  The results are the same.
+// NP: parts (real, imaginary) of a cell in one thread; they meet in the Bloch phase only.  NP = 2 computes
+// addresses and node-dependent stiffness once for both and is the form of launches that fill the GPU (N = 48, 64
+// block vectors: 340 us, 379 us with NP = 1 in the same run).  NP = 1, two adjacent lanes per cell, halves a thread's chain of
+// dependent instructions: the form of small launches, which wait for that chain (N = 8, one block vector:
+// 16.6 us, 24.8 us with NP = 2).  The results are the same.
 template <bool CUBIC, int MATK, int NP>
 struct FixApply {
     struct Shared {
-        int64_t* xs;  // [3 slots][3][kCells][2]
-        int64_t* fs;  // [12][kCells][2]: F_l of component c at l * 3 + c
-        double* raw;  // [3][kCells][2]: the next plane of x, as read
-        double2* ph;  // [27] Bloch phases of the wraps (wa, wb, wk)
-        FixHalf* c;   // [2][21]
-        int* xe;      // [3][kCells]
-        int* fe;      // [kCells]
+        int64_t* xs;   // [2 parts][3 slots][3][kCells]
+        int64_t* fs;   // [12][2][kCells]: F_l of component c at l * 3 + c, in units of 2^fe
+        double* raw;   // [3][kCells][2]: the next plane of x, as read
+        double2* ph;   // [27] Bloch phases of the wraps (wa, wb, wk)
+        WideEntry* c;  // [2][21]
+        int* xe;       // [3 slots][3][kCells]: units of the two parts, 16 bits each
+        int* fe;       // [3][kCells]
     };
-    static constexpr int kRow = 2 * kCells;  // stride of one component's array
+    static constexpr int kRow = 2 * kCells;  // stride of one component's two arrays
     static constexpr size_t shared_bytes() {
-        return (size_t)kCells * (16 * (9 + 12 + 3) + 4 * 4) + 16 * 27 + sizeof(FixHalf) * 42;
+        return (size_t)kCells * (16 * (9 + 12 + 3) + 4 * (9 + 3)) + 16 * 27 + sizeof(WideEntry) * 42;
     }
     static PC_HD void carve(Shared& sh, unsigned char* p) {
         sh.xs = reinterpret_cast<int64_t*>(p);
         sh.fs = sh.xs + 9 * kRow;
         sh.raw = reinterpret_cast<double*>(sh.fs + 12 * kRow);
         sh.ph = reinterpret_cast<double2*>(sh.raw + 3 * kRow);
-        sh.c = reinterpret_cast<FixHalf*>(sh.ph + 27);
+        sh.c = reinterpret_cast<WideEntry*>(sh.ph + 27);
         sh.xe = reinterpret_cast<int*>(sh.c + 42);
-        sh.fe = sh.xe + 3 * kCells;
+        sh.fe = sh.xe + 9 * kCells;
     }
 
     struct Ctx {
@@ -272,8 +139,8 @@ struct FixApply {
         int half;                // NP = 1: 0 real, 1 imaginary
         PC_HD int part() const { return NP == 1 ? half : 0; }
         int mprev, mcur, mnext;  // material of planes kf - 1, kf, kf + 1 (id, or the float's bits)
-        int64_t pv[3][NP], cv[3][NP];  // y(kf - 1) and y(kf) so far
-        int pe, ce;
+        int64_t pv[3][NP], cv[3][NP];  // y(kf - 1) and y(kf) so far, with their units
+        int pe[3][NP], ce[3][NP];
         int ks;  // first output plane left to slow_column
         double xo[3][NP];
         double dot;
@@ -281,16 +148,10 @@ struct FixApply {
 
     static PC_HD int wrap1(int v, int n, int& w) { return cell_wrap(v, n, w); }
 
-    // Combine over the two parts of a cell (NP = 1: the neighbouring lane's, which takes every branch alike).
+    // OR over the two parts of a cell (NP = 1: the neighbouring lane's, which takes every branch alike).
 #if defined(__CUDA_ARCH__)
     static __device__ unsigned pair() { return 3u << (threadIdx.x & 30); }
 #endif
-    static PC_HD int pair_max(int v) {
-#if defined(__CUDA_ARCH__)
-        if (NP == 1) v = imax(v, __shfl_xor_sync(pair(), v, 1));
-#endif
-        return v;
-    }
     static PC_HD int pair_or(int v) {
 #if defined(__CUDA_ARCH__)
         if (NP == 1) v |= __shfl_xor_sync(pair(), v, 1);
@@ -298,26 +159,7 @@ struct FixApply {
         return v;
     }
 
-    // a cell's parts: one 16-byte access, or 8 bytes of it
-    static PC_HD void get(const int64_t* p, int64_t* v) {
-        if (NP == 2) {
-            const longlong2 t = *reinterpret_cast<const longlong2*>(p);
-            v[0] = t.x;
-            v[NP - 1] = t.y;
-        } else {
-            v[0] = *p;
-        }
-    }
-    static PC_HD void put(int64_t* p, const int64_t* v) {
-        if (NP == 2) {
-            longlong2 t;
-            t.x = v[0];
-            t.y = v[NP - 1];
-            *reinterpret_cast<longlong2*>(p) = t;
-        } else {
-            *p = v[0];
-        }
-    }
+    // a cell's parts of x as read: one 16-byte access, or 8 bytes of it
     static PC_HD void get(const double* p, double* v) {
         if (NP == 2) {
             const double2 t = *reinterpret_cast<const double2*>(p);
@@ -327,17 +169,33 @@ struct FixApply {
             v[0] = *p;
         }
     }
+    static PC_HD int unit_of(const int* p, int part) { return reinterpret_cast<const int16_t*>(p)[part]; }
+
+    // a cell's units: both, or the part's own 16 bits
+    static PC_HD void get_units(const int* p, int part, int* u) {
+        if (NP == 2) {
+            const int w = *p;
+            u[0] = (int16_t)w;
+            u[NP - 1] = w >> 16;
+        } else {
+            u[0] = reinterpret_cast<const int16_t*>(p)[part];
+        }
+    }
+    static PC_HD void put_units(int* p, int part, const int* u) {
+        if (NP == 2) *p = (int)((uint32_t)u[NP - 1] << 16 | ((uint32_t)u[0] & 0xffffu));
+        else reinterpret_cast<int16_t*>(p)[part] = (int16_t)u[0];
+    }
 
     static PC_HD void init(const Ctx& c, int cell, int part, Regs& r) {
         cell_init(*c.G, c.a0, c.b0, c.p12, c.p13, cell, r);
         if (NP == 1) r.half = part;
-        r.pe = r.ce = 0;
         r.ks = 1 << 30;
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
                 r.pv[a][i] = r.cv[a][i] = 0;
+                r.pe[a][i] = r.ce[a][i] = kWideZero;
                 r.xo[a][i] = 0.0;
             }
         r.dot = 0.0;
@@ -408,30 +266,31 @@ struct FixApply {
                 }
             }
         }
-        int top = 0;
+        int64_t o[3][NP];
+        int u[3][NP];
+        int has = 0;  // 1: infinities or NaN, 2: values of 2^-943 or more, 4: values other than zero
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int i = 0; i < NP; ++i) top = imax(top, (int)(fix_bits(v[a][i]) >> 32) & 0x7fffffff);
-        int E = pair_max(top) >> 20, base = E;
-        if (E < kFixLow || E > kFixHigh) {
-            int64_t any = 0;
+            for (int i = 0; i < NP; ++i) {
+                o[a][i] = wide_from_double(v[a][i], 6, u[a][i]);
+                has |= u[a][i] == kWideSpecial ? 1 : u[a][i] >= 80 - 1075 - 6 ? 2 : u[a][i] == kWideZero ? 0 : 4;
+            }
+        has = pair_or(has);
+        if (has == 4 || (has & 1)) {  // all of the node's units: its readers look at one component
 #pragma unroll
             for (int a = 0; a < 3; ++a)
 #pragma unroll
-                for (int i = 0; i < NP; ++i) any |= fix_bits(v[a][i]) & 0x7fffffffffffffffLL;
-            base = 64;
-            E = pair_or(any != 0) ? kFixSpecial : 0;
+                for (int i = 0; i < NP; ++i) u[a][i] = kWideSpecial;
         }
-        int64_t* xs = sh.xs + sl * 3 * kRow + 2 * r.own[Q] + r.part();
+        int64_t* xs = sh.xs + (r.part() * 9 + sl * 3) * kCells + r.own[Q];
+        int* xe = sh.xe + sl * 3 * kCells + r.own[Q];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            int64_t o[NP];
 #pragma unroll
-            for (int i = 0; i < NP; ++i) o[i] = E == 0 ? 0 : fix_from_double(v[a][i], base, 3);
-            put(xs + a * kRow, o);
+            for (int i = 0; i < NP; ++i) xs[(a + 9 * i) * kCells] = o[a][i];
+            put_units(xe + a * kCells, r.part(), u[a]);
         }
-        sh.xe[sl * kCells + r.own[Q]] = E;
     }
 
     template <int Q>
@@ -461,247 +320,238 @@ struct FixApply {
 #endif
     }
 
+    // t = C e of one part with the phase table C; t in units of 2^tu, a product below 2^60.
     template <bool ORTHO>
-    static PC_HD void stress(const FixHalf* C, const FixHalf (*e)[NP], int64_t (*t)[NP]) {
+    static PC_HD void stress(const WideEntry* C, const WideHalf* e, const int* eu, int64_t* t, int* tu) {
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
-            int64_t h[NP], m[NP];
-#pragma unroll
-            for (int i = 0; i < NP; ++i) h[i] = m[i] = 0;
-#pragma unroll
-            for (int u = 0; u < 6; ++u) {
-                if (ORTHO && !((p < 3 && u < 3) || p == u)) continue;
-                const FixHalf cc = C[fix_upper(p, u)];
-#pragma unroll
-                for (int i = 0; i < NP; ++i) fix_mac(h[i], m[i], e[u][i], cc);
+            if (ORTHO && p >= 3) {
+                const WideEntry cc = C[fix_upper(p, p)];
+                t[p] = wide_mul(e[p], cc);
+                tu[p] = eu[p] + cc.u + 64;
+                continue;
             }
+            constexpr int n = ORTHO ? 3 : 6;
+            int64_t m[n];
+            int u[n], U = 2 * kWideZero;
 #pragma unroll
-            for (int i = 0; i < NP; ++i) t[p][i] = fix_sum(h[i], m[i], CUBIC ? 0 : 2);
+            for (int v = 0; v < n; ++v) {
+                const WideEntry cc = C[fix_upper(p, v)];
+                m[v] = wide_mul(e[v], cc);
+                u[v] = eu[v] + cc.u;
+                U = imax(U, u[v]);
+            }
+            t[p] = 0;
+#pragma unroll
+            for (int v = 0; v < n; ++v) t[p] += wide_shr(m[v], U - u[v]);
+            tu[p] = U + 64;
         }
     }
 
-    // Fluxes of plane kf (parity Q) at the thread's column; -4 P_0 into y(kf).  sm, sc, sp: slots of planes
-    // kf - 1, kf, kf + 1.
+    // Rows of a 3 x 3 table of normalised numbers through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or
+    // (rows) out[s] = sum_m Mmix[s][m] in[m]; one column of the table, below 3 2^60.
+    static PC_HD void mix3(const Ctx& c, int64_t* V, int* U, bool rows) {
+        WideHalf v[3];
+        int u[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            v[s] = wide_split(V[s]);
+            u[s] = U[s];
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            int64_t p[3];
+            int pu[3], top = 2 * kWideZero;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const WideEntry& w = c.F->mix[rows ? m * 3 + s : s * 3 + m];
+                p[s] = wide_mul(v[s], w);
+                pu[s] = u[s] + w.u;
+                top = imax(top, pu[s]);
+            }
+            U[m] = top + 64;
+            V[m] = wide_shr(p[0], top - pu[0]) + wide_shr(p[1], top - pu[1]) + wide_shr(p[2], top - pu[2]);
+        }
+    }
+
+    // Strain (xx, yy, zz, yz, xz, xy) of one part from the five x: normalised halves and units.  at: the cells
+    // of the four neighbours and of the node itself, slot * 3 * kCells + cell.
+    static PC_HD void strain(const Ctx& c, const Shared& sh, const int (&at)[5], int part, WideHalf* e, int* eu) {
+        int64_t H[3][3];
+        int hu[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            int u[5];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) u[l] = unit_of(sh.xe + at[l] + a * kCells, part);
+            const int U = imax(imax(imax(u[0], u[1]), imax(u[2], u[3])), u[4]);
+            int64_t x[5];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) x[l] = wide_shr(sh.xs[at[l] + (a + 9 * part) * kCells], U - u[l]);
+            const int64_t p = x[0] + x[1], q = x[2] + x[3];
+            H[0][a] = p + q - 4 * x[4];  // below 8 2^59
+            H[1][a] = p - q;
+            H[2][a] = (x[0] - x[1]) + (x[2] - x[3]);
+#pragma unroll
+            for (int s = 0; s < 3; ++s) hu[s][a] = U;
+            if (!CUBIC) {
+                int64_t V[3] = {H[0][a], H[1][a], H[2][a]};
+                int W[3] = {U, U, U};
+#pragma unroll
+                for (int s = 0; s < 3; ++s) V[s] = wide_norm(V[s], W[s]);
+                mix3(c, V, W, false);
+#pragma unroll
+                for (int s = 0; s < 3; ++s) {
+                    H[s][a] = V[s];
+                    hu[s][a] = W[s];
+                }
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            const int a = p == 0 ? 1 : 0, b = p == 2 ? 1 : 2;
+            eu[p] = hu[p][p];
+            e[p] = wide_split(wide_norm(H[p][p], eu[p]));
+            // a difference that vanishes (a uniform component) leaves the other's bits alone
+            const int ua = H[b][a] == 0 ? kWideZero : hu[b][a], ub = H[a][b] == 0 ? kWideZero : hu[a][b];
+            eu[3 + p] = imax(ua, ub);
+            const int64_t sum = wide_shr(H[b][a], eu[3 + p] - ua) + wide_shr(H[a][b], eu[3 + p] - ub);
+            e[3 + p] = wide_split(wide_norm(sum, eu[3 + p]));
+        }
+    }
+
+    // Fluxes of one part from its stresses; -4 P_0 into y(kf).  Stresses are cut `pad` bits below their unit, so that
+    // four fluxes and 4 P_0 sum to less than 2^63: rows of one product and of three (cubic lattice, orthotropic: 32
+    // products, pad 3), of six (96, pad 4), or mixed (48, pad 3).
+    static PC_HD void spread(const Ctx& c, Shared& sh, Regs& r, int own, int i, int part, int64_t* t, int* tu, int pad) {
+        if (!CUBIC) {
+#pragma unroll
+            for (int p = 0; p < 6; ++p) t[p] = wide_norm(t[p], tu[p]);
+            pad = 3;
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            constexpr int voigt[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};
+            int64_t P[3] = {t[voigt[a][0]], t[voigt[a][1]], t[voigt[a][2]]};
+            int u[3] = {tu[voigt[a][0]], tu[voigt[a][1]], tu[voigt[a][2]]};
+            if (!CUBIC) mix3(c, P, u, true);
+            const int fu = imax(imax(u[0], u[1]), u[2]) + pad;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) P[s] = wide_shr(P[s], fu - u[s]);
+            const int64_t g = P[0] + P[1], h = P[0] - P[1];
+            int64_t* f = sh.fs + a * kRow + part * kCells + own;
+            f[0] = g + P[2];
+            f[3 * kRow] = g - P[2];
+            f[6 * kRow] = h + P[2];
+            f[9 * kRow] = h - P[2];
+            reinterpret_cast<int16_t*>(sh.fe + a * kCells + own)[part] = (int16_t)fu;
+            if (r.flags & 4) {
+                const int m = imax(r.ce[a][i], fu);
+                r.cv[a][i] = wide_shr(r.cv[a][i], m - r.ce[a][i]) - 4 * wide_shr(P[0], m - fu);
+                r.ce[a][i] = m;
+            }
+        }
+    }
+
+    // Stiffness entry (p, v) of a node with its own: blended in FP64 as the FP64 kernels do, or its table's.
+    static PC_HD WideEntry node_entry(const Ctx& c, float theta, const double* md, int q) {
+        if (MATK == 1) return wide_entry(fma((double)theta, c.F->dc[q], c.F->c0[q]));
+        return wide_entry(md[(int64_t)q * c.G->vstr]);
+    }
+
+    // Fluxes of plane kf (parity Q) at the thread's column.  sm, sc, sp: slots of planes kf - 1, kf, kf + 1.
+    // The parts one after the other: together they spill.
     template <int Q>
     static PC_HD void flux(const Ctx& c, Shared& sh, Regs& r, int kf, int sm, int sc, int sp) {
         const CellGeom& G = *c.G;
         constexpr int n = kCells;
         if (!((r.flags >> Q) & 1)) return;
-        const int n0 = r.nb[Q] & 0xffff, n1 = r.nb[Q] >> 16, own = r.own[Q];
+        const int own = r.own[Q], part = r.part(), n0 = r.nb[Q] & 0xffff, n1 = r.nb[Q] >> 16;
         PC_IDX(n0, G.ncell);
         PC_IDX(n1, G.ncell);
-        const int eo = sh.xe[sc * n + own];
-        const int e0 = sh.xe[sm * n + n0], e1 = sh.xe[sp * n + n0], e2 = sh.xe[sm * n + n1], e3 = sh.xe[sp * n + n1];
-        const int E = imax(imax(imax(e0, e1), imax(e2, e3)), eo);
-        if (E >= kFixSpecial) {
-            sh.fe[own] = kFixSpecial;
-            r.ce = kFixSpecial;
-            return;
-        }
-        const int s0 = imin(E - e0, 63), s1 = imin(E - e1, 63), s2 = imin(E - e2, 63), s3 = imin(E - e3, 63),
-                  so = imin(E - eo, 63);
-        const int64_t *p0 = sh.xs + sm * 3 * kRow + 2 * n0 + r.part(), *p1 = sh.xs + sp * 3 * kRow + 2 * n0 + r.part(),
-                      *p2 = sh.xs + sm * 3 * kRow + 2 * n1 + r.part(), *p3 = sh.xs + sp * 3 * kRow + 2 * n1 + r.part(),
-                      *po = sh.xs + sc * 3 * kRow + 2 * own + r.part();
-        int64_t H[3][3][NP];
+        const int at[5] = {sm * 3 * n + n0, sp * 3 * n + n0, sm * 3 * n + n1, sp * 3 * n + n1, sc * 3 * n + own};
+        {
+            int U = 0;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int64_t x0[NP], x1[NP], x2[NP], x3[NP], xo[NP];
-            get(p0 + a * kRow, x0);
-            get(p1 + a * kRow, x1);
-            get(p2 + a * kRow, x2);
-            get(p3 + a * kRow, x3);
-            get(po + a * kRow, xo);
-            int64_t u[NP], v[NP];
+            for (int l = 0; l < 5; ++l) U = imax(U, unit_of(sh.xe + at[l], part));
+            if (U >= kWideSpecial) {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                x0[i] >>= s0;
-                x1[i] >>= s1;
+                for (int i = 0; i < NP; ++i) reinterpret_cast<int16_t*>(sh.fe + own)[part + i] = kWideSpecial;
+                r.ce[0][0] = kWideSpecial;
+                return;
             }
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                x2[i] >>= s2;
-                x3[i] >>= s3;
-            }
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                xo[i] >>= so;
-                u[i] = x0[i] + x1[i];
-                v[i] = x2[i] + x3[i];
-            }
-#pragma unroll
-            for (int i = 0; i < NP; ++i) H[0][a][i] = u[i] + v[i] - 4 * xo[i];
-#pragma unroll
-            for (int i = 0; i < NP; ++i) H[1][a][i] = u[i] - v[i];
-#pragma unroll
-            for (int i = 0; i < NP; ++i) H[2][a][i] = (x0[i] - x1[i]) + (x2[i] - x3[i]);
         }
-        int up = 0;
-        if (!CUBIC || MATK != 0) {
-            // more roundings follow than in the plain case: scale the sums up to their bound first
-            int top = 0;
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) top |= (int)((H[m][a][i] ^ (H[m][a][i] >> 63)) >> 32);
-            up = fix_clz64((uint64_t)(uint32_t)pair_or(top) | 1) - 32 - 5;
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) H[m][a][i] <<= up;
-        }
-        if (!CUBIC) mix3(c, H, false);
-        // strain halves: xx, yy, zz, yz, xz, xy
-        FixHalf e[6][NP];
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const int u = p == 0 ? 1 : 0, v = p == 2 ? 1 : 2;
-#pragma unroll
-            for (int i = 0; i < NP; ++i) e[p][i] = fix_split(H[p][p][i]);
-#pragma unroll
-            for (int i = 0; i < NP; ++i) e[3 + p][i] = fix_split(H[v][u][i] + H[u][v][i]);
-        }
-        int64_t t[6][NP];
-        int fe = E - up + c.F->moff;
         if (MATK == 0) {
             const int ph = r.mcur != 0 ? 1 : 0;
-            const FixHalf* C = sh.c + 21 * ph;
-            fe += ph ? c.F->coff[1] : c.F->coff[0];
-            // every node of the warp orthotropic: normal block and shear diagonal only
-            if (warp_all(c.F->P.ortho[ph] != 0)) stress<true>(C, e, t);
-            else stress<false>(C, e, t);
-        } else {
-            int64_t h[6][NP], m[6][NP];
+            const WideEntry* C = sh.c + 21 * ph;
+            // every node of the warp orthotropic: normal block and shear diagonal only (the same bits as with the zeros)
+            const bool ortho = warp_all(c.F->P.ortho[ph] != 0);
+            const int pad = c.F->P.ortho[ph] != 0 ? 3 : 4;
+            // a loop, with y(kf) of the part at hand in the first place: unrolled, the parts' instructions are
+            // interleaved and their registers spill
+#pragma unroll 1
+            for (int i = 0; i < NP; ++i) {
+                WideHalf e[6];
+                int64_t t[6];
+                int eu[6], tu[6];
+                strain(c, sh, at, part + i, e, eu);
+                if (ortho) stress<true>(C, e, eu, t, tu);
+                else stress<false>(C, e, eu, t, tu);
+                spread(c, sh, r, own, 0, part + i, t, tu, pad);
+                if (NP == 2) {
 #pragma unroll
-            for (int p = 0; p < 6; ++p)
-#pragma unroll
-                for (int i = 0; i < NP; ++i) h[p][i] = m[p][i] = 0;
-            int row[6] = {0, 0, 0, 0, 0, 0};  // row sums of |c| / 2^32
-            FixHalf th = {0, 0};
-            const double* md = nullptr;
-            int base = 64;
-            bool empty = false;  // a void: zero fluxes, whatever x is
-            if (MATK == 1) {
-                th = fix_split(fix_theta(mat_theta(r.mcur)));
-                fe += c.F->coff[0];
-            } else {
-                int wk;
-                const int at = wrap1(kf, G.Z, wk) * G.plane + r.off[Q];
-                md = static_cast<const double*>(c.mat) + at;
-                int top = 0;
-#pragma unroll
-                for (int u = 0; u < 21; ++u) top = imax(top, (int)(fix_bits(md[(int64_t)u * G.vstr]) >> 32) & 0x7fffffff);
-                base = top >> 20;  // entries below 2^59: row sums below 2^62
-                fe += base - 1017;
-                if (base == 0) {
-                    int64_t any = 0;
-#pragma unroll
-                    for (int u = 0; u < 21; ++u) any |= fix_bits(md[(int64_t)u * G.vstr]);
-                    empty = (any & 0x7fffffffffffffffLL) == 0;
-                    base = empty ? 1000 : 0;
-                }
-                if (base < 950 || base > 1100) {  // tables far outside hat units
-                    sh.fe[own] = kFixSpecial;
-                    r.ce = kFixSpecial;
-                    return;
+                    for (int a = 0; a < 3; ++a) {
+                        const int64_t v = r.cv[a][0];
+                        const int u = r.ce[a][0];
+                        r.cv[a][0] = r.cv[a][NP - 1];
+                        r.ce[a][0] = r.ce[a][NP - 1];
+                        r.cv[a][NP - 1] = v;
+                        r.ce[a][NP - 1] = u;
+                    }
                 }
             }
-#pragma unroll
-            for (int p = 0; p < 6; ++p)
-#pragma unroll
-                for (int u = p; u < 6; ++u) {
-                    FixHalf cc;
-                    if (MATK == 1) {  // c = C_0 + theta (C_1 - C_0)
-                        int64_t hh = 0, mm = 1LL << 29;
-                        const FixHalf d = sh.c[21 + fix_upper(p, u)], z = sh.c[fix_upper(p, u)];
-                        fix_mac(hh, mm, th, d);
-                        cc = fix_split((int64_t)z.hi * 0x100000000LL + z.lo + hh * 4 + (mm >> 30));
-                    } else {
-                        cc = fix_split(fix_from_double(md[(int64_t)fix_upper(p, u) * G.vstr], base, 6));
-                    }
-                    const int ab = cc.hi < 0 ? -cc.hi : cc.hi;
-                    row[p] += ab;
-                    if (u != p) row[u] += ab;
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) {
-                        fix_mac(h[p][i], m[p][i], e[u][i], cc);
-                        if (u != p) fix_mac(h[u][i], m[u][i], e[p][i], cc);
-                    }
-                }
-            // the node's own row sums are below the bound the scale allows for: keep that many more bits
-            const int top = imax(imax(imax(row[0], row[1]), imax(row[2], row[3])), imax(row[4], row[5])) + 6;
-            int sh2 = (top < (1 << 24) ? 6 : top < (1 << 25) ? 5 : top < (1 << 26) ? 4 : top < (1 << 27) ? 3
-                       : top < (1 << 28) ? 2 : top < (1 << 29) ? 1 : 0);
-            fe = empty ? 0 : fe - sh2;
-            sh2 += CUBIC ? 0 : 2;
-#pragma unroll
-            for (int p = 0; p < 6; ++p)
-#pragma unroll
-                for (int i = 0; i < NP; ++i) t[p][i] = fix_sum(h[p][i], m[p][i], sh2);
+            return;
         }
-        if (E == 0) fe = 0;  // zero fluxes
-        sh.fe[own] = fe;
-        // P_s (s, component)
-        int64_t Ps[3][3][NP];
+        WideHalf e[NP][6];
+        int64_t t[NP][6];
+        int eu[NP][6], tu[NP][6];
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            Ps[0][0][i] = t[0][i];
-            Ps[1][1][i] = t[1][i];
-            Ps[2][2][i] = t[2][i];
-            Ps[0][1][i] = Ps[1][0][i] = t[5][i];
-            Ps[0][2][i] = Ps[2][0][i] = t[4][i];
-            Ps[1][2][i] = Ps[2][1][i] = t[3][i];
-        }
-        if (!CUBIC) mix3(c, Ps, true);
-        int64_t* f = sh.fs + 2 * own + r.part();
+            strain(c, sh, at, part + i, e[i], eu[i]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int64_t u[NP], v[NP], g[NP];
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                u[i] = Ps[0][a][i] + Ps[1][a][i];
-                v[i] = Ps[0][a][i] - Ps[1][a][i];
-            }
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-#pragma unroll
-                for (int i = 0; i < NP; ++i) g[i] = (l < 2 ? u[i] : v[i]) + (l & 1 ? -Ps[2][a][i] : Ps[2][a][i]);
-                put(f + (l * 3 + a) * kRow, g);
+            for (int p = 0; p < 6; ++p) {
+                t[i][p] = 0;
+                tu[i][p] = 2 * kWideZero;
             }
         }
-        if (r.flags & 4) {
-            const int m = imax(r.ce, fe);
-            const int sa = imin(m - r.ce, 63), sf = imin(m - fe, 63);
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int i = 0; i < NP; ++i) r.cv[a][i] = (r.cv[a][i] >> sa) - 4 * (Ps[0][a][i] >> sf);
-            r.ce = m;
+        const double* md = nullptr;
+        if (MATK == 2) {
+            int wk;
+            md = static_cast<const double*>(c.mat) + wrap1(kf, G.Z, wk) * G.plane + r.off[Q];
         }
-    }
-
-    // Rows of a 3 x 3 table through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or (rows)
-    // out[s] = sum_m Mmix[s][m] in[m].
-    static PC_HD void mix3(const Ctx& c, int64_t (*V)[3][NP], bool rows) {
+        const float theta = MATK == 1 ? mat_theta(r.mcur) : 0.f;
+        auto add = [&](int i, int p, int64_t m, int u) {
+            const int U = imax(tu[i][p], u);
+            t[i][p] = wide_shr(t[i][p], U - tu[i][p]) + wide_shr(m, U - u);
+            tu[i][p] = U;
+        };
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+        for (int p = 0; p < 6; ++p)
 #pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                FixHalf v[3];
+            for (int v = p; v < 6; ++v) {
+                const WideEntry cc = node_entry(c, theta, md, fix_upper(p, v));
 #pragma unroll
-                for (int s = 0; s < 3; ++s) v[s] = fix_split(V[s][a][i]);
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    int64_t h = 0, md = 0;
-#pragma unroll
-                    for (int s = 0; s < 3; ++s) fix_mac(h, md, v[s], c.F->mix[rows ? m * 3 + s : s * 3 + m]);
-                    V[m][a][i] = fix_sum(h, md, rows ? 1 : 2);
+                for (int i = 0; i < NP; ++i) {
+                    add(i, p, wide_mul(e[i][v], cc), eu[i][v] + cc.u);
+                    if (v != p) add(i, v, wide_mul(e[i][p], cc), eu[i][p] + cc.u);
                 }
             }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+#pragma unroll
+            for (int p = 0; p < 6; ++p) tu[i][p] += 64;
+            spread(c, sh, r, own, i, part + i, t[i], tu[i], 4);
+        }
     }
 
     // The node's own x of plane kf - 1, for the shift term and the inner product.
@@ -725,24 +575,28 @@ struct FixApply {
         const int c0 = r.gn[1 - Q] & 0xffff, c1 = r.gn[1 - Q] >> 16;
         PC_IDX(c0, G.ncell);
         PC_IDX(c1, G.ncell);
-        const int f0 = sh.fe[c0], f1 = sh.fe[c1];
-        const int64_t *a0 = sh.fs + 2 * c0 + r.part(), *a1 = sh.fs + 2 * c1 + r.part();
+        const int64_t *a0 = sh.fs + r.part() * kCells + c0, *a1 = sh.fs + r.part() * kCells + c1;
+        int f0[3][NP], f1[3][NP];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            get_units(sh.fe + a * kCells + c0, r.part(), f0[a]);
+            get_units(sh.fe + a * kCells + c1, r.part(), f1[a]);
+        }
         if (k >= c.k0) {
             const int at = k * G.plane + r.off[1 - Q];
-            const int E = imax(r.pe, imax(f0, f1));
-            if (E >= kFixSpecial && r.ks > k) r.ks = k;
+            if (imax(r.pe[0][0], imax(f0[0][0], f1[0][0])) >= kWideSpecial && r.ks > k) r.ks = k;
             if (k < r.ks) {
                 const double sr = c.shift * density(c, r.mprev, at);
-                const int sa = imin(E - r.pe, 63), s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    int64_t g0[NP], g1[NP];
                     double w[NP];
-                    get(a0 + a * kRow, g0);
-                    get(a1 + (6 + a) * kRow, g1);
 #pragma unroll
                     for (int i = 0; i < NP; ++i) {
-                        w[i] = fix_to_double((r.pv[a][i] >> sa) + (g0[i] >> s0) + (g1[i] >> s1), E);
+                        const int E = imax(r.pe[a][i], imax(f0[a][i], f1[a][i]));
+                        w[i] = wide_to_double(wide_shr(r.pv[a][i], E - r.pe[a][i]) + 
+                                                  wide_shr(a0[a * kRow + i * kCells], E - f0[a][i]) +
+                                                  wide_shr(a1[(6 + a) * kRow + i * kCells], E - f1[a][i]),
+                                              E);
                         w[i] = fma(-sr, r.xo[a][i], w[i]);
                     }
                     double2* y = c.y + at + (int64_t)a * G.vstr;
@@ -755,19 +609,16 @@ struct FixApply {
                 }
             }
         }
-        const int E = imax(f0, f1);
-        r.pe = r.ce;
-        r.ce = E;
-        const int s0 = imin(E - f0, 63), s1 = imin(E - f1, 63);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            int64_t g0[NP], g1[NP];
-            get(a0 + (3 + a) * kRow, g0);
-            get(a1 + (9 + a) * kRow, g1);
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
+                const int E = imax(f0[a][i], f1[a][i]);
                 r.pv[a][i] = r.cv[a][i];
-                r.cv[a][i] = (g0[i] >> s0) + (g1[i] >> s1);
+                r.pe[a][i] = r.ce[a][i];
+                r.cv[a][i] = wide_shr(a0[(3 + a) * kRow + i * kCells], E - f0[a][i]) +
+                             wide_shr(a1[(9 + a) * kRow + i * kCells], E - f1[a][i]);
+                r.ce[a][i] = E;
             }
         }
     }

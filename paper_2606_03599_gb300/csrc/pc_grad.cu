@@ -34,6 +34,64 @@ namespace pc {
 
 namespace {
 
+struct FixHalf {
+    int hi, lo;  // c = hi 2^32 + lo, lo signed
+};
+
+PC_HD FixHalf fix_split(int64_t v) {
+    FixHalf h;
+    h.hi = (int)((v + 0x80000000LL) >> 32);
+    h.lo = (int)(uint32_t)v;
+    return h;
+}
+PC_HD longlong2 fix_ashr2(longlong2 v, int s) {
+    longlong2 r;
+    r.x = v.x >> s;
+    r.y = v.y >> s;
+    return r;
+}
+PC_HD int64_t fix_bits(double v) {
+#if defined(__CUDA_ARCH__)
+    return __double_as_longlong(v);
+#else
+    int64_t b;
+    memcpy(&b, &v, 8);
+    return b;
+#endif
+}
+// v as an integer below 2^up (up in 53..63) in units of 2^(E - 1022 - up); base = E, or 64 for E = 0
+// (all values of the node zero).  Bits below the unit are dropped.
+PC_HD int64_t fix_from_double(double v, int base, int lead) {
+    const int64_t b = fix_bits(v);
+    const int hi = (int)(b >> 32);
+    const int e = (hi >> 20) & 0x7ff;
+    const uint64_t m = (((uint64_t)b & 0xfffffffffffffULL) | 0x10000000000000ULL) << lead;
+    const int64_t s = hi >> 31;
+    return ((int64_t)(m >> imin(base - e, 63)) ^ s) - s;
+}
+// largest |high word| of a complex number
+PC_HD int fix_high(double2 v, int m) {
+    m = imax(m, (int)(fix_bits(v.x) >> 32) & 0x7fffffff);
+    return imax(m, (int)(fix_bits(v.y) >> 32) & 0x7fffffff);
+}
+// acc + a b.  In PTX on the device: written in C++ the compiler loses sight of the operands being
+// 32 bits wide and multiplies 64 x 64.
+PC_HD void fix_mad(int64_t& acc, int a, int b) {
+#if defined(__CUDA_ARCH__)
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+#else
+    acc += (int64_t)a * b;
+#endif
+}
+// hi 2^64 + mid 2^32 accumulates e c for signed halves
+PC_HD void fix_mac(int64_t& hi, int64_t& mid, FixHalf e, FixHalf c) {
+    fix_mad(hi, e.hi, c.hi);
+    fix_mad(mid, e.hi, c.lo);
+    fix_mad(mid, e.lo, c.hi);
+}
+// the accumulated product over 2^(64 - s), rounded (s in 0..8)
+PC_HD int64_t fix_sum(int64_t hi, int64_t mid, int s) { return (hi << s) + ((mid + (0x80000000LL >> s)) >> (32 - s)); }
+
 constexpr int kGradVecs = 32;  // vectors per launch: their limb products sum to less than 2^62
 constexpr int kGradThreads = 128;
 constexpr int kGradLow = 720;  // least biased exponent of the integer path: squares stay above FP64's smallest
