@@ -15,7 +15,6 @@
 #include "../pc_apply_split.cuh"
 #include "../pc_apply_int.cuh"
 #include "../pc_apply_cell.cuh"
-#include "../pc_limb.cuh"
 #include "../pc_small_dft.cuh"
 
 using namespace pc;
@@ -660,28 +659,27 @@ extern "C" int pc_emu_small_dft(int L, int inv, const double* in, double* out) {
     }
 }
 
-// sum of a b over n <= 8 complex pairs, one limb group, as the outer-loop products form it.
-// Returns 0, or 1 when the group's exponents leave the integer path's range.
+// sum of a b over n <= 8 complex pairs, one group, as the outer-loop products form it.  Returns 0, or 1 when
+// the group's exponents leave the integer path's range.
 extern "C" int pc_emu_limb_dot(int n, const double* a, const double* b, double* out) {
     const double2* x = reinterpret_cast<const double2*>(a);
     const double2* y = reinterpret_cast<const double2*>(b);
     int ta = 0, tb = 0;
     for (int q = 0; q < n; ++q) {
-        ta = limb_top(x[q], ta);
-        tb = limb_top(y[q], tb);
+        ta = wide_top(x[q], ta);
+        tb = wide_top(y[q], tb);
     }
     const int Ea = ta >> 20, Eb = tb >> 20;
-    if (Ea < kLimbLow || Ea > kLimbHigh || Eb < kLimbLow || Eb > kLimbHigh) return 1;
-    LimbAcc re = {0, 0}, im = {0, 0};
+    if (Ea < kWideLow || Ea > kWideHigh || Eb < kWideLow || Eb > kWideHigh) return 1;
+    WideSum re = wide_sum0(), im = wide_sum0();
     for (int q = 0; q < n; ++q) {
-        const LimbC u = limb_of(x[q], Ea), v = limb_of(y[q], Eb);
-        limb_mac(re, u.re, v.re);
-        limb_mac(re, limb_neg(u.im), v.im);
-        limb_mac(im, u.re, v.im);
-        limb_mac(im, u.im, v.re);
+        int ur, ui, vr, vi;
+        const WideC u = wide_factor(x[q], ur, ui), v = wide_factor(y[q], vr, vi);
+        wide_mac2(re, u.re, ur, v.re, vr, u.im, ui, v.im, vi);
+        wide_mac2(im, u.re, ur, v.im, vi, wide_neg(u.im), ui, v.re, vr);
     }
-    out[0] = limb_sum(re, Ea, Eb);
-    out[1] = limb_sum(im, Ea, Eb);
+    out[0] = wide_to_double(re);
+    out[1] = wide_to_double(im);
     return 0;
 }
 

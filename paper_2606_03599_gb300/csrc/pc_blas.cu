@@ -7,18 +7,22 @@
 // so the work is a sum over a long index with a small dense result.  In FP64 arithmetic they are
 // bound by GB300's FP64 pipe (2 lanes per clock and SM, 8 FMAs for every 16-byte operand), 4 to 6
 // times above their memory time.  So products run on the integer pipe in groups of eight
-// (pc_limb.cuh): the group's operands are split into limbs once, a real product is three 32 x 32 + 64
-// bit multiply-adds, and the FP64 pipe sees two instructions per group and result.  Operands are
+// (pc_wide.cuh): every value keeps its own exponent, a real product is four 32 x 32 + 64 bit
+// multiply-adds and its place in the group's sum a shift and an addition, and the FP64 pipe sees two
+// instructions per group and result.  Operands are
 // read once per register block with coalesced 16-byte loads, the mass weight is applied once per
 // element of W (not per product), and Gram partial sums are reduced in a fixed order (per CTA, then
 // across CTAs) so results are deterministic.
 //
-// Measured in a mixed-precision solve at N = 128 (four blocks, 2 columns, up to 26 rows; vectors of
-// 25 MB): Gram products 1.16 -> 0.49 ms and updates 1.40 -> 0.62 ms per launch on average.
+// Measured in an FP64 solve at N = 48 (sixteen spaces, vectors of 1.3 MB), FP64 / integer form: Gram products of
+// more than four rows 0.56 / 0.29 ms, updates of 2 columns 0.21 / 0.13 ms, of 4 columns 1.20 / 0.74 ms; at N = 128
+// (four spaces, vectors of 25 MB) 1.23, 0.55 and 3.6 ms in the integer form.  (Eight values cut into limbs of one shared
+// exponent took 0.19, 0.11 and 0.42 ms at N = 48, but lost small values next to large ones and made every
+// squared norm 5e-17 too small.)
 #include <algorithm>
 
-#include "pc_limb.cuh"
 #include "pc_solver.h"
+#include "pc_wide.cuh"
 
 namespace pc {
 
@@ -110,12 +114,10 @@ __device__ __forceinline__ void gram_chunk(const double2* __restrict__ A, int ro
 }
 
 // Integer form, rows i0 .. i0 + 8 RW - 1 (warp w has rows i0 + w, i0 + w + 8, ...): a tile of 1024
-// elements of the two columns is weighted and split into limbs once, eight elements of a lane to a
-// group with one exponent, and every warp runs its rows over the tile; a group whose exponents are
-// out of range runs in FP64.  Splitting a row's elements costs about what their products do, so two
-// columns go together and the columns' own splitting is shared by all rows through shared memory (kept
-// in registers for eight rows of one thread it took 244 of them, and 8 warps per SM ran no faster than
-// the FP64 form).
+// elements of the two columns is weighted and made factors once, and every warp runs its rows over the
+// tile, eight elements of a lane to a group; a group whose largest value is out of range runs in FP64.
+// Making a row's elements factors costs a third of their products, so two columns go together and the columns'
+// own factors are shared by all rows through shared memory.
 constexpr int kGramTile = 1024;
 
 template <int RW, int MATK>
@@ -123,8 +125,9 @@ __device__ __forceinline__ void gram_tile(const double2* __restrict__ A, int row
                                           int cols, int64_t m, const void* __restrict__ mat, double rho0, double drho,
                                           int i0, int j0, int nchunk, double* __restrict__ part, int64_t base) {
     constexpr int CB = kGramCB, NB = 8;
-    __shared__ LimbC lb[CB][kGramTile];
-    __shared__ int Eb[CB][kGramTile / NB];  // -1: FP64
+    __shared__ WideC lb[CB][kGramTile];
+    __shared__ short2 ub[CB][kGramTile];  // units of the two parts
+    __shared__ bool okb[CB][kGramTile / NB];
     const int64_t vs = 3 * m;
     const int64_t t0 = (int64_t)blockIdx.x * m / nchunk, t1 = (int64_t)(blockIdx.x + 1) * m / nchunk;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -157,20 +160,23 @@ __device__ __forceinline__ void gram_tile(const double2* __restrict__ A, int row
             for (int q = 0; q < NB; ++q) {
                 const int x = x0 + g * 256 + q * 32 + lane;
                 b[q] = x < total ? weighted(j, x) : make_double2(0.0, 0.0);
-                top = limb_top(b[q], top);
+                top = wide_top(b[q], top);
             }
-            const int E = top == 0 ? 1000 : top >> 20;  // zeros, or values too small to count
+            const int E = top == 0 ? kWideLow : top >> 20;  // zeros, or values too small to count
 #pragma unroll
-            for (int q = 0; q < NB; ++q) lb[j][g * 256 + q * 32 + lane] = limb_of(b[q], E);
-            Eb[j][g * 32 + lane] = (E >= kLimbLow && E <= kLimbHigh) ? E : -1;
+            for (int q = 0; q < NB; ++q) {
+                int ur, ui;
+                lb[j][g * 256 + q * 32 + lane] = wide_factor(b[q], ur, ui);
+                ub[j][g * 256 + q * 32 + lane] = make_short2((short)ur, (short)ui);
+            }
+            okb[j][g * 32 + lane] = E >= kWideLow && E <= kWideHigh;
         }
         __syncthreads();
 #pragma unroll 1
         for (int g = 0; g < kGramTile / 256; ++g) {
             const int xg = x0 + g * 256 + lane;
             if (xg - lane >= total) break;
-            const int E0 = Eb[0][g * 32 + lane], E1 = Eb[1][g * 32 + lane];
-            const bool ok = (E0 | E1) >= 0;
+            const bool ok = okb[0][g * 32 + lane] && okb[1][g * 32 + lane];
 #pragma unroll
             for (int r = 0; r < RW; ++r) {
                 const int i = i0 + warp + 8 * r;
@@ -184,29 +190,30 @@ __device__ __forceinline__ void gram_tile(const double2* __restrict__ A, int row
                     a[q] = x < total ? Ai[element(x)] : make_double2(0.0, 0.0);
                 }
 #pragma unroll
-                for (int q = 0; q < NB; ++q) top = limb_top(a[q], top);
+                for (int q = 0; q < NB; ++q) top = wide_top(a[q], top);
                 const int E = top >> 20;
-                if (ok && E >= kLimbLow && E <= kLimbHigh) {
-                    LimbAcc re[CB], im[CB];
+                if (ok && E >= kWideLow && E <= kWideHigh) {
+                    WideSum re[CB], im[CB];
 #pragma unroll
-                    for (int j = 0; j < CB; ++j) re[j].hi = re[j].mid = im[j].hi = im[j].mid = 0;
+                    for (int j = 0; j < CB; ++j) re[j] = im[j] = wide_sum0();
 #pragma unroll
                     for (int q = 0; q < NB; ++q) {
-                        const LimbC la = limb_of(a[q], E);
-                        const Limb ni = limb_neg(la.im);
+                        int ur, ui;
+                        const WideC la = wide_factor(a[q], ur, ui);
+                        const WideHalf ni = wide_neg(la.im);
 #pragma unroll
                         for (int j = 0; j < CB; ++j) {  // conj(a) b
-                            const LimbC lv = lb[j][g * 256 + q * 32 + lane];
-                            limb_mac(re[j], la.re, lv.re);
-                            limb_mac(re[j], la.im, lv.im);
-                            limb_mac(im[j], la.re, lv.im);
-                            limb_mac(im[j], ni, lv.re);
+                            const WideC lv = lb[j][g * 256 + q * 32 + lane];
+                            const short2 uv = ub[j][g * 256 + q * 32 + lane];
+                            wide_mac2(re[j], la.re, ur, lv.re, uv.x, ni, ui, lv.im, uv.y);
+                            wide_mac2(im[j], la.re, ur, lv.im, uv.y, la.im, ui, lv.re, uv.x);
                         }
                     }
-                    ar[r][0] += limb_sum(re[0], E, E0);
-                    ai[r][0] += limb_sum(im[0], E, E0);
-                    ar[r][1] += limb_sum(re[1], E, E1);
-                    ai[r][1] += limb_sum(im[1], E, E1);
+#pragma unroll
+                    for (int j = 0; j < CB; ++j) {
+                        ar[r][j] += wide_to_double(re[j]);
+                        ai[r][j] += wide_to_double(im[j]);
+                    }
                 } else if (top != 0 || !ok) {
 #pragma unroll 1
                     for (int q = 0; q < NB; ++q) {
@@ -294,40 +301,40 @@ __global__ void ts_gram_reduce(const double* __restrict__ part, int nentries, in
 }
 
 // cr + i ci += sum over NB columns kk .. kk + NB - 1 of A of a(e) h(., j): a group of columns on the
-// integer pipe, or in FP64 where its exponents (or those of h: hok) are out of range.
+// integer pipe, or in FP64 where its largest value (or that of a column of h: hok) is out of range.
 template <int CB, int NB>
-__device__ __forceinline__ void update_group(const double2* __restrict__ Ae, int64_t vs, const LimbC* hs,
-                                             const int* Eh, bool hok, const double2* __restrict__ h, int64_t hstr,
+__device__ __forceinline__ void update_group(const double2* __restrict__ Ae, int64_t vs, const WideC* hs, const short2* hu,
+                                             bool hok, const double2* __restrict__ h, int64_t hstr,
                                              int jn, double* cr, double* ci) {
     double2 a[NB];
     int top = 0;
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
         a[q] = Ae[(int64_t)q * vs];
-        top = limb_top(a[q], top);
+        top = wide_top(a[q], top);
     }
     const int E = top >> 20;
-    if (hok && E >= kLimbLow && E <= kLimbHigh) {
-        LimbAcc re[CB], im[CB];
+    if (hok && E >= kWideLow && E <= kWideHigh) {
+        WideSum re[CB], im[CB];
 #pragma unroll
-        for (int j = 0; j < CB; ++j) re[j].hi = re[j].mid = im[j].hi = im[j].mid = 0;
+        for (int j = 0; j < CB; ++j) re[j] = im[j] = wide_sum0();
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
-            const LimbC la = limb_of(a[q], E);
-            const Limb ni = limb_neg(la.im);
+            int ur, ui;
+            const WideC la = wide_factor(a[q], ur, ui);
+            const WideHalf ni = wide_neg(la.im);
 #pragma unroll
             for (int j = 0; j < CB; ++j) {
-                const LimbC hv = hs[q * CB + j];
-                limb_mac(re[j], la.re, hv.re);
-                limb_mac(re[j], ni, hv.im);
-                limb_mac(im[j], la.re, hv.im);
-                limb_mac(im[j], la.im, hv.re);
+                const WideC hv = hs[q * CB + j];
+                const short2 uv = hu[q * CB + j];
+                wide_mac2(re[j], la.re, ur, hv.re, uv.x, la.im, ui, hv.im, uv.y);
+                wide_mac2(im[j], la.re, ur, hv.im, uv.y, ni, ui, hv.re, uv.x);
             }
         }
 #pragma unroll
         for (int j = 0; j < CB; ++j) {
-            cr[j] += limb_sum(re[j], E, Eh[j]);
-            ci[j] += limb_sum(im[j], E, Eh[j]);
+            cr[j] += wide_to_double(re[j]);
+            ci[j] += wide_to_double(im[j]);
         }
     } else if (top != 0 || !hok) {
 #pragma unroll 1
@@ -344,34 +351,31 @@ __device__ __forceinline__ void update_group(const double2* __restrict__ Ae, int
 }
 
 // C[:, j] = beta C[:, j] + alpha sum_k A[:, k] h(k, j) for the CB columns j0 .. j0 + CB - 1 of
-// column group blockIdx.y; the limbs of h (k x cols, column-major, one exponent per column) are
-// staged in shared memory.  With beta == 0, C is not read (it may hold anything).
+// column group blockIdx.y; the factors of h (k x cols, column-major) are staged in shared memory.  With beta == 0, C is not read (it may hold anything).
 template <int CB>
 __device__ __forceinline__ void update_columns(const double2* __restrict__ A, int k, const double2* __restrict__ h,
                                                int cols, double2* __restrict__ C, int64_t vs, double alpha,
                                                double beta, int j0) {
-    extern __shared__ LimbC hs[];  // [k][CB]
+    extern __shared__ WideC hs[];  // [k][CB], then their units
+    short2* hu = reinterpret_cast<short2*>(hs + (size_t)k * CB);
     __shared__ int tops[CB];
     if (threadIdx.x < CB) tops[threadIdx.x] = 0;
     __syncthreads();
     for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
         const int kk = q / CB, j = q % CB;
-        if (j0 + j < cols) atomicMax(&tops[j], limb_top(h[kk + (int64_t)(j0 + j) * k], 0));
+        const double2 hv = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
+        int ur, ui;
+        hs[q] = wide_factor(hv, ur, ui);
+        hu[q] = make_short2((short)ur, (short)ui);
+        atomicMax(&tops[j], wide_top(hv, 0));
     }
     __syncthreads();
-    int Eh[CB];
     bool hok = true;
 #pragma unroll
     for (int j = 0; j < CB; ++j) {
-        Eh[j] = tops[j] == 0 ? 1000 : tops[j] >> 20;
-        hok = hok && Eh[j] >= kLimbLow && Eh[j] <= kLimbHigh;
+        const int E = tops[j] >> 20;
+        hok = hok && (tops[j] == 0 || (E >= kWideLow && E <= kWideHigh));
     }
-    for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
-        const int kk = q / CB, j = q % CB;
-        const double2 hv = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
-        hs[q] = limb_of(hv, tops[j] == 0 ? 1000 : tops[j] >> 20);
-    }
-    __syncthreads();
     const double2* __restrict__ hj = h + (int64_t)j0 * k;
     const int jn = cols - j0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
@@ -380,13 +384,13 @@ __device__ __forceinline__ void update_columns(const double2* __restrict__ A, in
         for (int j = 0; j < CB; ++j) cr[j] = ci[j] = 0.0;
         int kk = 0;
         for (; kk + 8 <= k; kk += 8)
-            update_group<CB, 8>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
+            update_group<CB, 8>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
         if (k & 4) {
-            update_group<CB, 4>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
+            update_group<CB, 4>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
             kk += 4;
         }
         for (; kk < k; ++kk)
-            update_group<CB, 1>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, Eh, hok, hj + kk, k, jn, cr, ci);
+            update_group<CB, 1>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
 #pragma unroll
         for (int j = 0; j < CB; ++j) {
             if (j0 + j >= cols) continue;
@@ -484,6 +488,15 @@ __global__ void __launch_bounds__(256)
     update_columns<CB>(J.A, J.k, J.h, J.cols, J.C, vs, J.alpha, J.beta, j0);
 }
 
+// Shared memory of an update of k basis columns, granted beyond the default 48 KB where it takes more.
+template <typename K>
+int update_smem(K kern, int k, int CB, size_t* smem) {
+    if ((size_t)k * CB > 3072) return fail(PC_EINVAL, "ts_update: too many basis columns");
+    *smem = (sizeof(WideC) + sizeof(short2)) * (size_t)k * CB;
+    if (*smem > 47 * 1024) PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
+    return PC_OK;
+}
+
 }  // namespace
 
 int ts_gram(const double2* A, int rows, const double2* B, int cols, int64_t m, const void* mat, int matkind,
@@ -532,8 +545,8 @@ int ts_update(const double2* A, int k, const double2* d_h, int cols, double2* C,
     // column blocks of 2 when cols <= 2 (the Gram-Schmidt updates of a 2-wide Krylov block:
     // no FMAs on padding columns), else of 4
     const int CB = cols <= 2 ? 2 : 4;
-    const size_t smem = sizeof(LimbC) * (size_t)k * CB;
-    if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update: too many basis columns");
+    size_t smem;
+    PC_TRY(CB == 2 ? update_smem(ts_update_kernel<2>, k, CB, &smem) : update_smem(ts_update_kernel<4>, k, CB, &smem));
     const int ngc = (cols + CB - 1) / CB;
     int64_t gx = (vs + 255) / 256;
     gx = std::min<int64_t>(gx, std::max<int64_t>(1, 8LL * device_sm_count() / ngc));
@@ -605,8 +618,9 @@ int ts_update_batch(const UpdateJob* jobs, int njobs, int64_t vs, cudaStream_t s
         }
         if (U.n == 0) continue;
         const int CB = maxc <= 2 ? 2 : 4;
-        const size_t smem = sizeof(LimbC) * (size_t)maxk * CB;
-        if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update_batch: too many basis columns");
+        size_t smem;
+        PC_TRY(CB == 2 ? update_smem(ts_update_batch_kernel<2>, maxk, CB, &smem)
+                       : update_smem(ts_update_batch_kernel<4>, maxk, CB, &smem));
         const int ngc = (maxc + CB - 1) / CB;
         int64_t gx = (vs + 255) / 256;
         gx = std::min<int64_t>(gx, std::max<int64_t>(1, 8LL * device_sm_count() / ((int64_t)ngc * U.n)));

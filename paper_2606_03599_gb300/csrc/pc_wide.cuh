@@ -142,6 +142,62 @@ PC_HD WideEntry wide_entry(double v) {
     return e;
 }
 
+// Factors of sums of complex products (pc_blas.cu).
+struct WideC {
+    WideHalf re, im;
+};
+constexpr int kWideLow = 600, kWideHigh = 1450;  // biased exponents of a group's largest value: its sum stays in
+                                                 // FP64's normal range; all others go to FP64
+// the larger of m and the magnitude bits of v's high words
+PC_HD int wide_top(double2 v, int m) {
+    m = imax(m, (int)(wide_bits(v.x) >> 32) & 0x7fffffff);
+    return imax(m, (int)(wide_bits(v.y) >> 32) & 0x7fffffff);
+}
+// A double of such a group as a factor; subnormal values count as zero.
+PC_HD WideHalf wide_factor(double v, int& u) {
+    const int64_t b = wide_bits(v);
+    const int hi = (int)(b >> 32), e = (hi >> 20) & 0x7ff;
+    const int64_t m = (int64_t)(((uint64_t)b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9;
+    const int64_t s = hi >> 31;
+    WideHalf h = wide_split((m ^ s) - s);
+    u = e - 1084;
+    if (e == 0) {
+        h.hi = h.lo = 0;
+        u = kWideZero;
+    }
+    return h;
+}
+PC_HD WideC wide_factor(double2 v, int& ur, int& ui) {
+    WideC r;
+    r.re = wide_factor(v.x, ur);
+    r.im = wide_factor(v.y, ui);
+    return r;
+}
+PC_HD WideHalf wide_neg(WideHalf a) {
+    a.hi = -a.hi;
+    a.lo = -a.lo;
+    return a;
+}
+// A running sum of up to 16 products (eight complex ones): m 2^(u + 64).
+struct WideSum {
+    int64_t m;
+    int u;
+};
+PC_HD WideSum wide_sum0() {
+    WideSum s;
+    s.m = 0;
+    s.u = 2 * kWideZero;
+    return s;
+}
+// s + a b - c d, in units of the largest product and two bits up, so that 16 products stay below 2^62.  A shift
+// rounds down: taking one of the products away rather than adding its negative, the two roundings cancel in the mean
+// (all added, a squared norm came out 2e-16 too small).
+PC_HD void wide_mac2(WideSum& s, WideHalf a, int ua, WideHalf b, int ub, WideHalf c, int uc, WideHalf d, int ud) {
+    const int u1 = ua + ub, u2 = uc + ud, U = imax(s.u, imax(u1, u2) + 2);
+    s.m = wide_shr(s.m, U - s.u) + wide_shr(wide_mul(a, b), U - u1) - wide_shr(wide_mul(c, d), U - u2);
+    s.u = U;
+}
+
 // m 2^u to the nearest double (results below the normal range round twice).
 PC_HD double wide_to_double(int64_t m, int u) {
     const double d = (double)m;
@@ -152,5 +208,7 @@ PC_HD double wide_to_double(int64_t m, int u) {
 #endif
     return m == 0 ? 0.0 : ldexp(d, u);
 }
+
+PC_HD double wide_to_double(WideSum s) { return wide_to_double(s.m, s.u + 64); }
 
 }  // namespace pc
