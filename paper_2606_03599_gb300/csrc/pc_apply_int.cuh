@@ -348,76 +348,19 @@ struct FixApply {
         }
     }
 
-    // Rows of a 3 x 3 table of normalised numbers through the lattice mixing: out[m] = sum_s Mmix[s][m] in[s], or
-    // (rows) out[s] = sum_m Mmix[s][m] in[m]; one column of the table, below 3 2^60.
-    static PC_HD void mix3(const Ctx& c, int64_t* V, int* U, bool rows) {
-        WideHalf v[3];
-        int u[3];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            v[s] = wide_split(V[s]);
-            u[s] = U[s];
-        }
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            int64_t p[3];
-            int pu[3], top = 2 * kWideZero;
-#pragma unroll
-            for (int s = 0; s < 3; ++s) {
-                const WideEntry& w = c.F->mix[rows ? m * 3 + s : s * 3 + m];
-                p[s] = wide_mul(v[s], w);
-                pu[s] = u[s] + w.u;
-                top = imax(top, pu[s]);
-            }
-            U[m] = top + 64;
-            V[m] = wide_shr(p[0], top - pu[0]) + wide_shr(p[1], top - pu[1]) + wide_shr(p[2], top - pu[2]);
-        }
-    }
-
-    // Strain (xx, yy, zz, yz, xz, xy) of one part from the five x: normalised halves and units.  at: the cells
-    // of the four neighbours and of the node itself, slot * 3 * kCells + cell.
+    // Strain of one part from the staged planes.  at: the cells of the four neighbours and of the node itself,
+    // slot * 3 * kCells + cell.
     static PC_HD void strain(const Ctx& c, const Shared& sh, const int (&at)[5], int part, WideHalf* e, int* eu) {
-        int64_t H[3][3];
-        int hu[3][3];
+        wide_strain<CUBIC>(
+            c.F->mix,
+            [&](int a, int64_t* x, int* u) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int u[5];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) u[l] = unit_of(sh.xe + at[l] + a * kCells, part);
-            const int U = imax(imax(imax(u[0], u[1]), imax(u[2], u[3])), u[4]);
-            int64_t x[5];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) x[l] = wide_shr(sh.xs[at[l] + (a + 9 * part) * kCells], U - u[l]);
-            const int64_t p = x[0] + x[1], q = x[2] + x[3];
-            H[0][a] = p + q - 4 * x[4];  // below 8 2^59
-            H[1][a] = p - q;
-            H[2][a] = (x[0] - x[1]) + (x[2] - x[3]);
-#pragma unroll
-            for (int s = 0; s < 3; ++s) hu[s][a] = U;
-            if (!CUBIC) {
-                int64_t V[3] = {H[0][a], H[1][a], H[2][a]};
-                int W[3] = {U, U, U};
-#pragma unroll
-                for (int s = 0; s < 3; ++s) V[s] = wide_norm(V[s], W[s]);
-                mix3(c, V, W, false);
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    H[s][a] = V[s];
-                    hu[s][a] = W[s];
+                for (int l = 0; l < 5; ++l) {
+                    u[l] = unit_of(sh.xe + at[l] + a * kCells, part);
+                    x[l] = sh.xs[at[l] + (a + 9 * part) * kCells];
                 }
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const int a = p == 0 ? 1 : 0, b = p == 2 ? 1 : 2;
-            eu[p] = hu[p][p];
-            e[p] = wide_split(wide_norm(H[p][p], eu[p]));
-            // a difference that vanishes (a uniform component) leaves the other's bits alone
-            const int ua = H[b][a] == 0 ? kWideZero : hu[b][a], ub = H[a][b] == 0 ? kWideZero : hu[a][b];
-            eu[3 + p] = imax(ua, ub);
-            const int64_t sum = wide_shr(H[b][a], eu[3 + p] - ua) + wide_shr(H[a][b], eu[3 + p] - ub);
-            e[3 + p] = wide_split(wide_norm(sum, eu[3 + p]));
-        }
+            },
+            e, eu);
     }
 
     // Fluxes of one part from its stresses; -4 P_0 into y(kf).  Stresses are cut `pad` bits below their unit, so that
@@ -434,7 +377,7 @@ struct FixApply {
             constexpr int voigt[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};
             int64_t P[3] = {t[voigt[a][0]], t[voigt[a][1]], t[voigt[a][2]]};
             int u[3] = {tu[voigt[a][0]], tu[voigt[a][1]], tu[voigt[a][2]]};
-            if (!CUBIC) mix3(c, P, u, true);
+            if (!CUBIC) wide_mix3(c.F->mix, P, u, true);
             const int fu = imax(imax(u[0], u[1]), u[2]) + pad;
 #pragma unroll
             for (int s = 0; s < 3; ++s) P[s] = wide_shr(P[s], fu - u[s]);

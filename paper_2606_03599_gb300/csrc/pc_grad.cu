@@ -14,102 +14,43 @@
 //
 // The work is FP64 arithmetic in form (about 220 operations per node and vector, 1.63 ms for 12
 // vectors on 64^3 nodes when done so) against 48 bytes read, so it runs on the integer pipe like the
-// apply (pc_apply_int.cuh): the five values a component's differences need become integers
-// with one exponent, sums are exact, and the strain, scaled by sqrt(|w|), is split into limbs
-// (pc_limb.cuh) whose products are summed over the vectors in integers; the running sums carry one
-// exponent per node and turn into doubles once, after up to 32 vectors.  A node with values outside the exponent range is left to FP64.
+// apply (pc_wide.cuh): real and imaginary parts, components, strains and each of the 21 sums have exponents of
+// their own, so that a small strain's products are as accurate next to a large one's as in FP64.  The strain is
+// scaled by sqrt(|w|) and normalised, its products are summed over up to 32 vectors in integers and turn into
+// doubles once.  A node with infinities or NaN is left to FP64.
 //
-// Measured (one GB300, N = 64 full space, 12 vectors): 0.44 ms, where the FP64 form took 1.63 ms; bound by
-// the integer instructions, half of them the conversion of a node's 15 values (196 MB of DRAM traffic
-// would take 0.03 ms).
+// Measured (one GB300, FP64 form / this one): N = 64 full space, 12 vectors 1.63 / 0.95 ms, one vector 0.183 / 0.143
+// ms; N = 8, 12 vectors 138 / 85 us.  Bound by the integer instructions, about 1700 per node, vector and part (196 MB
+// of DRAM traffic would take 0.03 ms).  (One exponent for a node's strains and sums took 0.44 ms and left nothing
+// of a strain's square 1e-8 below another's.)
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
 
-#include "pc_apply_int.cuh"
-#include "pc_limb.cuh"
+#include "pc_complex.cuh"
 #include "pc_solver.h"
+#include "pc_wide.cuh"
 
 namespace pc {
 
 namespace {
 
-struct FixHalf {
-    int hi, lo;  // c = hi 2^32 + lo, lo signed
-};
-
-PC_HD FixHalf fix_split(int64_t v) {
-    FixHalf h;
-    h.hi = (int)((v + 0x80000000LL) >> 32);
-    h.lo = (int)(uint32_t)v;
-    return h;
-}
-PC_HD longlong2 fix_ashr2(longlong2 v, int s) {
-    longlong2 r;
-    r.x = v.x >> s;
-    r.y = v.y >> s;
-    return r;
-}
-PC_HD int64_t fix_bits(double v) {
-#if defined(__CUDA_ARCH__)
-    return __double_as_longlong(v);
-#else
-    int64_t b;
-    memcpy(&b, &v, 8);
-    return b;
-#endif
-}
-// v as an integer below 2^up (up in 53..63) in units of 2^(E - 1022 - up); base = E, or 64 for E = 0
-// (all values of the node zero).  Bits below the unit are dropped.
-PC_HD int64_t fix_from_double(double v, int base, int lead) {
-    const int64_t b = fix_bits(v);
-    const int hi = (int)(b >> 32);
-    const int e = (hi >> 20) & 0x7ff;
-    const uint64_t m = (((uint64_t)b & 0xfffffffffffffULL) | 0x10000000000000ULL) << lead;
-    const int64_t s = hi >> 31;
-    return ((int64_t)(m >> imin(base - e, 63)) ^ s) - s;
-}
-// largest |high word| of a complex number
-PC_HD int fix_high(double2 v, int m) {
-    m = imax(m, (int)(fix_bits(v.x) >> 32) & 0x7fffffff);
-    return imax(m, (int)(fix_bits(v.y) >> 32) & 0x7fffffff);
-}
-// acc + a b.  In PTX on the device: written in C++ the compiler loses sight of the operands being
-// 32 bits wide and multiplies 64 x 64.
-PC_HD void fix_mad(int64_t& acc, int a, int b) {
-#if defined(__CUDA_ARCH__)
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
-#else
-    acc += (int64_t)a * b;
-#endif
-}
-// hi 2^64 + mid 2^32 accumulates e c for signed halves
-PC_HD void fix_mac(int64_t& hi, int64_t& mid, FixHalf e, FixHalf c) {
-    fix_mad(hi, e.hi, c.hi);
-    fix_mad(mid, e.hi, c.lo);
-    fix_mad(mid, e.lo, c.hi);
-}
-// the accumulated product over 2^(64 - s), rounded (s in 0..8)
-PC_HD int64_t fix_sum(int64_t hi, int64_t mid, int s) { return (hi << s) + ((mid + (0x80000000LL >> s)) >> (32 - s)); }
-
-constexpr int kGradVecs = 32;  // vectors per launch: their limb products sum to less than 2^62
+constexpr int kGradVecs = 32;  // vectors per launch: the 64 products of their parts, four bits down, sum to 2^62 at most
 constexpr int kGradThreads = 128;
-constexpr int kGradLow = 720;  // least biased exponent of the integer path: squares stay above FP64's smallest
 
 struct GradVec {
-    FixHalf s;     // sqrt(|w| scaleC) (times the lattice factor on a cubic lattice) = s 2^(ex - 62)
-    int ex, neg;   // neg: w < 0
-    double wC, wR; // w scaleC, -w lambda scaleR
+    WideEntry s;    // sqrt(|w| scaleC) (times the lattice factor on a cubic lattice)
+    int neg;        // w < 0
+    double wC, wR;  // w scaleC, -w lambda scaleR
 };
 struct GradParams {
     double Mmix[9];  // (A_hat^-1)_{s m} / (4 h_s)
     double ph[3][2];
-    FixHalf mix[9], pi[3][2];  // the same in units of 2^(mex - 62) and 2^-62
-    int mex;
-    int X, Y, Z, N;  // quarter-grid extents
+    WideEntry mix[9], phase[27][2];  // the same; cos and sin of every wrap's phase
+    int X, Y, Z, N;                  // quarter-grid extents
     int full, block;
     int plane, vstr;  // nodes per plane and component of the layout
-    int nvec, all_slow;  // all_slow: a weight's scale is outside the exponents the sums allow for
+    int nvec;
     GradVec v[kGradVecs];
 };
 
@@ -142,7 +83,7 @@ __device__ __forceinline__ GradNode grad_node(const GradParams& P, int blk, int 
     return r;
 }
 
-__device__ __forceinline__ double2 grad_phase(const GradParams& P, int wrap) {
+__host__ __device__ __forceinline__ double2 grad_phase(const GradParams& P, int wrap) {
     double2 e = make_double2(1.0, 0.0);
     const int w[3] = {wrap % 3 - 1, (wrap / 3) % 3 - 1, wrap / 9 - 1};
     for (int s = 0; s < 3; ++s)
@@ -196,18 +137,21 @@ __device__ __noinline__ void grad_slow(const GradParams& P, const double2* __res
     drho[l] += gr;
 }
 
-// One thread per node; loops over the vectors, so that each output entry has a single writer (no
-// atomics, deterministic).  blockIdx.y: parity block of a full-space layout.
-// Bounds: x < 2^57, phased values below sqrt(2) of it, sums H scaled up to 2^61, strain < 2^62 and as
-// much after the products with s; limbs of 28 and 29 bits, so a vector adds at most 2^57 to a high sum
-// and 2^58 to a middle one.
+// Two adjacent lanes per node, one for the real parts and one for the imaginary ones, which meet in the wraps'
+// phases only (one lane for both: N = 24, 12 vectors 165 us instead of 121, N = 64 0.84 ms).  They loop over the vectors and
+// their sums are added at the end, so that each output entry has a single writer (no atomics, deterministic).
+// blockIdx.y: parity block of a full-space layout.
 template <bool CUBIC>
-__global__ void __launch_bounds__(kGradThreads, 3)
+__global__ void __launch_bounds__(kGradThreads, 4)
     eig_grad_kernel(const __grid_constant__ GradParams P, const double2* __restrict__ X, double* __restrict__ dC,
                     double* __restrict__ drho, int64_t n_full) {
+    __shared__ WideEntry phase[27][2];
+    for (int i = threadIdx.x; i < 54; i += kGradThreads) phase[i >> 1][i & 1] = P.phase[i >> 1][i & 1];
+    __syncthreads();
     const int blk = P.full ? (int)blockIdx.y : P.block;
     const uint32_t nodes = (uint32_t)P.X * P.Y * P.Z;
-    const uint32_t t = blockIdx.x * kGradThreads + threadIdx.x;
+    const uint32_t t = (blockIdx.x * kGradThreads + threadIdx.x) >> 1;
+    const int part = threadIdx.x & 1;
     if (t >= nodes) return;
     int a, b, k;
     split3(t, P.X, P.Y, a, b, k);
@@ -217,196 +161,87 @@ __global__ void __launch_bounds__(kGradThreads, 3)
         const int p12 = blk >> 1, p13 = blk & 1;
         l = (2 * a + ((k + p13) & 1)) + (int64_t)P.N * ((2 * b + ((k + p12 + p13) & 1)) + (int64_t)P.N * k);
     }
-    bool slow = P.all_slow != 0;
+    bool slow = false;
     double gr = 0.0;
-    int64_t hi[21], mid[21];
+    int64_t g[21];
+    int gu[21];
 #pragma unroll
-    for (int q = 0; q < 21; ++q) hi[q] = mid[q] = 0;
-    int A = -100000;  // exponent of the limbs' unit
+    for (int q = 0; q < 21; ++q) {
+        g[q] = 0;
+        gu[q] = 2 * kWideZero;
+    }
     for (int v = 0; v < P.nvec; ++v) {
         const GradVec& V = P.v[v];
         const double2* __restrict__ x = X + (int64_t)v * 3 * P.vstr;
-        longlong2 H[3][3];
-        int E[3], any = 0;
         double xx = 0.0;
-        bool bad = false;
 #pragma unroll
         for (int al = 0; al < 3; ++al) {
-            const double2* xc = x + (int64_t)al * P.vstr;
-            double2 xv[5];
-#pragma unroll
-            for (int ll = 0; ll < 4; ++ll) xv[ll] = xc[nd.nb[ll]];
-            xv[4] = xc[nd.at];
-            int top = 0;
-#pragma unroll
-            for (int ll = 0; ll < 5; ++ll) top = fix_high(xv[ll], top);
-            xx = cdotre(xv[4], xv[4], xx);
-            E[al] = top >> 20;
-            if (E[al] < kGradLow || E[al] > kLimbHigh) {
-                // a component of zeros counts as such; anything else goes to FP64
-                int64_t low = 0;
-#pragma unroll
-                for (int ll = 0; ll < 5; ++ll) low |= fix_bits(xv[ll].x) | fix_bits(xv[ll].y);
-                bad = bad || (low & 0x7fffffffffffffffLL) != 0;
-                E[al] = kGradLow;
-            }
-            longlong2 n[5];
-#pragma unroll
-            for (int ll = 0; ll < 5; ++ll) {
-                n[ll].x = fix_from_double(xv[ll].x, E[al], 4);
-                n[ll].y = fix_from_double(xv[ll].y, E[al], 4);
-            }
-#pragma unroll
-            for (int ll = 0; ll < 4; ++ll) {
-                int w = nd.wrap[ll];
-                if (w != 13) {
-#pragma unroll 1
-                    for (int d = 0; d < 3; ++d) {
-                        const int wd = w % 3 - 1;
-                        w /= 3;
-                        if (wd == 0) continue;
-                        const FixHalf c = P.pi[d][0], sn = P.pi[d][1];
-                        FixHalf sp, sm;
-                        sp.hi = wd < 0 ? -sn.hi : sn.hi;
-                        sp.lo = wd < 0 ? -sn.lo : sn.lo;
-                        sm.hi = -sp.hi;
-                        sm.lo = -sp.lo;
-                        const FixHalf zx = fix_split(n[ll].x), zy = fix_split(n[ll].y);
-                        int64_t hx = 0, mx = 0, hy = 0, my = 0;
-                        fix_mac(hx, mx, zx, c);
-                        fix_mac(hx, mx, zy, sm);
-                        fix_mac(hy, my, zy, c);
-                        fix_mac(hy, my, zx, sp);
-                        n[ll].x = fix_sum(hx, mx, 2);
-                        n[ll].y = fix_sum(hy, my, 2);
-                    }
-                }
-            }
-            const int64_t ux = n[0].x + n[1].x, uy = n[0].y + n[1].y, vx = n[2].x + n[3].x, vy = n[2].y + n[3].y;
-            H[0][al].x = ux + vx - 4 * n[4].x;
-            H[0][al].y = uy + vy - 4 * n[4].y;
-            H[1][al].x = ux - vx;
-            H[1][al].y = uy - vy;
-            H[2][al].x = (n[0].x - n[1].x) + (n[2].x - n[3].x);
-            H[2][al].y = (n[0].y - n[1].y) + (n[2].y - n[3].y);
-            any |= top;
+            const double2 z = x[(int64_t)al * P.vstr + nd.at];
+            const double xo = part ? z.y : z.x;
+            xx = fma(xo, xo, xx);
         }
         gr = fma(V.wR, xx, gr);
-        slow = slow || bad;
-        if (!bad && any != 0 && V.wC != 0.0) {
-            const int Em = imax(imax(E[0], E[1]), E[2]);
-            int bits = 0;
+        WideHalf f[6];
+        int fu[6];
+        wide_strain<CUBIC>(
+            P.mix,
+            [&](int al, int64_t* m, int* u) {
+                const double2* xc = x + (int64_t)al * P.vstr;
 #pragma unroll
-            for (int al = 0; al < 3; ++al) {
-                const int d = imin(Em - E[al], 63);
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    H[s][al] = fix_ashr2(H[s][al], d);
-                    bits |= (int)((H[s][al].x ^ (H[s][al].x >> 63)) >> 32) | (int)((H[s][al].y ^ (H[s][al].y >> 63)) >> 32);
-                }
-            }
-            const int up = __clz(bits | 1) - 3;
-#pragma unroll
-            for (int s = 0; s < 3; ++s)
-#pragma unroll
-                for (int al = 0; al < 3; ++al) {
-                    H[s][al].x <<= up;
-                    H[s][al].y <<= up;
-                }
-            int u = Em - 1079 - up + V.ex;  // exponent of the strain's unit
-            if (!CUBIC) {
-                u += P.mex;
-#pragma unroll
-                for (int al = 0; al < 3; ++al) {
-                    FixHalf hx[3], hy[3];
-#pragma unroll
-                    for (int s = 0; s < 3; ++s) {
-                        hx[s] = fix_split(H[s][al].x);
-                        hy[s] = fix_split(H[s][al].y);
-                    }
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) {
-                        int64_t px = 0, qx = 0, py = 0, qy = 0;
-#pragma unroll
-                        for (int s = 0; s < 3; ++s) {
-                            fix_mac(px, qx, hx[s], P.mix[s * 3 + m]);
-                            fix_mac(py, qy, hy[s], P.mix[s * 3 + m]);
-                        }
-                        H[m][al].x = fix_sum(px, qx, 2);
-                        H[m][al].y = fix_sum(py, qy, 2);
+                for (int ll = 0; ll < 5; ++ll) {
+                    const double2 z = xc[ll < 4 ? nd.nb[ll] : nd.at];
+                    m[ll] = wide_from_double(part ? z.y : z.x, 6, u[ll]);
+                    slow = slow || u[ll] == kWideSpecial;
+                    if (ll < 4 && nd.wrap[ll] != 13) {  // times the phase, the other part's share included
+                        const WideEntry p = wide_entry(part ? z.y : z.x), o = wide_entry(part ? z.x : z.y);
+                        const WideEntry c = phase[nd.wrap[ll]][0], sn = phase[nd.wrap[ll]][1];
+                        const WideHalf ph = {p.hi, p.lo}, oh = {o.hi, o.lo};
+                        const int u1 = p.u + c.u, u2 = o.u + sn.u, U = imax(u1, u2) + 2;
+                        const int64_t m1 = wide_shr(wide_mul(ph, c), U - u1), m2 = wide_shr(wide_mul(oh, sn), U - u2);
+                        slow = slow || o.u == kWideSpecial;
+                        m[ll] = part ? m1 + m2 : m1 - m2;
+                        u[ll] = U + 64;
                     }
                 }
+            },
+            f, fu);
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+            fu[p] += V.s.u + 64;
+            f[p] = wide_split(wide_norm(wide_mul(f[p], V.s), fu[p]));
+        }
+        // a shift rounds down: the real parts' products are added, the imaginary parts' taken away with the
+        // sign turned, so that the roundings of a square cancel in the mean
+        const bool turn = (V.neg != 0) != (part != 0);
+        int q = 0;
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+            WideHalf h = f[p];
+            if (turn) {
+                h.hi = -h.hi;
+                h.lo = -h.lo;
             }
-            longlong2 e[6];
-            e[0] = H[0][0];
-            e[1] = H[1][1];
-            e[2] = H[2][2];
-            e[3] = make_longlong2(H[2][1].x + H[1][2].x, H[2][1].y + H[1][2].y);
-            e[4] = make_longlong2(H[2][0].x + H[0][2].x, H[2][0].y + H[0][2].y);
-            e[5] = make_longlong2(H[1][0].x + H[0][1].x, H[1][0].y + H[0][1].y);
-            bits = 0;
 #pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                const FixHalf ex = fix_split(e[p].x), ey = fix_split(e[p].y);
-                int64_t h = 0, m = 0;
-                fix_mac(h, m, ex, V.s);
-                e[p].x = fix_sum(h, m, 2);
-                h = m = 0;
-                fix_mac(h, m, ey, V.s);
-                e[p].y = fix_sum(h, m, 2);
-                bits |= (int)((e[p].x ^ (e[p].x >> 63)) >> 32) | (int)((e[p].y ^ (e[p].y >> 63)) >> 32);
-            }
-            // common unit of the running sums: a larger strain scales them down
-            const int need = u + imax(0, 7 - __clz(bits | 1));  // 57 bits: seven leading bits clear
-            if (need > A) {
-                const int d = imin(2 * (need - A), 63);
-                if (d > 0 && A > -100000) {
-#pragma unroll
-                    for (int q = 0; q < 21; ++q) {
-                        hi[q] >>= d;
-                        mid[q] >>= d;
-                    }
-                }
-                A = need;
-            }
-            const int sh = imin(A - u, 63);
-            Limb lx[6], ly[6];
-#pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                const int64_t px = e[p].x >> sh, py = e[p].y >> sh;
-                lx[p].hi = (int)((px + (1 << 28)) >> 29);
-                lx[p].lo = ((int)px << 3) >> 3;
-                ly[p].hi = (int)((py + (1 << 28)) >> 29);
-                ly[p].lo = ((int)py << 3) >> 3;
-            }
-            const int sg = V.neg ? -1 : 0;
-            int q = 0;
-#pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                Limb fx, fy;
-                fx.hi = (lx[p].hi ^ sg) - sg;
-                fx.lo = (lx[p].lo ^ sg) - sg;
-                fy.hi = (ly[p].hi ^ sg) - sg;
-                fy.lo = (ly[p].lo ^ sg) - sg;
-#pragma unroll
-                for (int r = p; r < 6; ++r, ++q) {
-                    limb_mad(hi[q], fx.hi, lx[r].hi);
-                    limb_mad(hi[q], fy.hi, ly[r].hi);
-                    limb_mad(mid[q], fx.hi, lx[r].lo);
-                    limb_mad(mid[q], fx.lo, lx[r].hi);
-                    limb_mad(mid[q], fy.hi, ly[r].lo);
-                    limb_mad(mid[q], fy.lo, ly[r].hi);
-                }
+            for (int r = p; r < 6; ++r, ++q) {
+                const int u = fu[p] + fu[r] + 4, U = imax(gu[q], u);
+                const int64_t m = wide_shr(wide_mul(h, f[r]), U - u + 4), s = wide_shr(g[q], U - gu[q]);
+                g[q] = part ? s - m : s + m;
+                gu[q] = U;
             }
         }
-        // the middle sums hold eight vectors: their upper part moves on
-        if ((v & 7) == 7)
-#pragma unroll
-            for (int q = 0; q < 21; ++q) {
-                hi[q] += mid[q] >> 29;
-                mid[q] &= (1 << 29) - 1;
-            }
     }
+    // the two lanes of a node take every branch alike
+    const unsigned pair = 3u << (threadIdx.x & 30);
+    slow = __shfl_xor_sync(pair, (int)slow, 1) != 0 || slow;
+    gr += __shfl_xor_sync(pair, gr, 1);
+#pragma unroll
+    for (int q = 0; q < 21; ++q) {
+        const int64_t o = __shfl_xor_sync(pair, g[q], 1);
+        const int ou = __shfl_xor_sync(pair, gu[q], 1), U = imax(gu[q], ou);
+        g[q] = wide_shr(g[q], U - gu[q]) + wide_shr(o, U - ou);
+        gu[q] = U;
+    }
+    if (part != 0) return;
     if (slow) {
         grad_slow(P, X, nd, l, dC, drho, n_full);
         return;
@@ -415,13 +250,8 @@ __global__ void __launch_bounds__(kGradThreads, 3)
 #pragma unroll
     for (int p = 0; p < 6; ++p)
 #pragma unroll
-        for (int r = p; r < 6; ++r, ++q) {
-            const int64_t tt = hi[q] + ((mid[q] + (1 << 28)) >> 29);  // units of 2^(2 A + 58)
-            const double d = __ll2double_rn(tt);
-            if (tt != 0)
-                dC[(int64_t)q * n_full + l] += __hiloint2double(
-                    __double2hiint(d) + (2 * A + 58 + (p == r ? 0 : 1)) * (1 << 20), __double2loint(d));
-        }
+        for (int r = p; r < 6; ++r, ++q)
+            if (g[q] != 0) dC[(int64_t)q * n_full + l] += wide_to_double(g[q], gu[q] + 64 + (p == r ? 0 : 1));
     drho[l] += gr;
 }
 
@@ -448,17 +278,18 @@ extern "C" int pc_eig_grad(pc_grid* g, int block, int nvec, const void* X, const
     for (int base = 0; base < nvec; base += kGradVecs) {
         GradParams P;
         P.nvec = std::min(nvec - base, kGradVecs);
-        P.all_slow = 0;
-        double ms = 0.0;
-        for (int e = 0; e < 9; ++e) P.Mmix[e] = g->Ainv[e] * q;
-        for (int i = 0; i < 3; ++i)
-            ms = std::fmax(ms, std::fabs(P.Mmix[i]) + std::fabs(P.Mmix[3 + i]) + std::fabs(P.Mmix[6 + i]));
-        std::frexp(ms, &P.mex);
-        for (int e = 0; e < 9; ++e) P.mix[e] = fix_split(std::llrint(std::ldexp(P.Mmix[e], 62 - P.mex)));
+        for (int e = 0; e < 9; ++e) {
+            P.Mmix[e] = g->Ainv[e] * q;
+            P.mix[e] = wide_entry(P.Mmix[e]);
+        }
         for (int l = 0; l < 3; ++l) {
             P.ph[l][0] = std::cos(g->k.phi[l]);
             P.ph[l][1] = std::sin(g->k.phi[l]);
-            for (int c = 0; c < 2; ++c) P.pi[l][c] = fix_split(std::llrint(std::ldexp(P.ph[l][c], 62)));
+        }
+        for (int w = 0; w < 27; ++w) {
+            const double2 e = grad_phase(P, w);
+            P.phase[w][0] = wide_entry(e.x);
+            P.phase[w][1] = wide_entry(e.y);
         }
         P.N = g->N;
         P.full = block < 0 ? 1 : 0;
@@ -475,15 +306,18 @@ extern "C" int pc_eig_grad(pc_grid* g, int block, int nvec, const void* X, const
             const long double sq = sqrtl((long double)std::fabs(w) / ((long double)g->rho0 * g->L * g->L)) *
                                    (g->cubic ? (long double)q : 1.0L);
             V.neg = w < 0 ? 1 : 0;
-            V.ex = 0;
-            if (sq > 0) frexpl(sq, &V.ex);
-            if (std::abs(V.ex) + std::abs(P.mex) > 60) P.all_slow = 1;
-            V.s = fix_split(llrintl(ldexpl(sq, 62 - V.ex)));
+            int ex = 0;
+            if (sq > 0) frexpl(sq, &ex);
+            const WideHalf h = wide_split(llrintl(ldexpl(sq, 62 - ex)));
+            V.s.hi = h.hi;
+            V.s.lo = h.lo;
+            V.s.u = sq > 0 ? ex - 62 : kWideZero;
+            V.s.pad = 0;
             V.wC = w * scaleC;
             V.wR = -w * lambdas[base + v] * scaleR;
         }
         const int64_t nodes = (int64_t)P.X * P.Y * P.Z;
-        const dim3 grid((unsigned)((nodes + kGradThreads - 1) / kGradThreads), P.full ? 4 : 1);
+        const dim3 grid((unsigned)((2 * nodes + kGradThreads - 1) / kGradThreads), P.full ? 4 : 1);
         const double2* Xb = static_cast<const double2*>(X) + (int64_t)base * 3 * P.vstr;
         if (g->cubic) eig_grad_kernel<true><<<grid, kGradThreads, 0, s>>>(P, Xb, dC, drho, g->n);
         else eig_grad_kernel<false><<<grid, kGradThreads, 0, s>>>(P, Xb, dC, drho, g->n);

@@ -142,6 +142,78 @@ PC_HD WideEntry wide_entry(double v) {
     return e;
 }
 
+// Rows of a 3 x 3 table of normalised numbers through the lattice mixing M: out[m] = sum_s M[s][m] in[s], or
+// (rows) out[s] = sum_m M[s][m] in[m]; one column of the table, below 3 2^60.
+PC_HD void wide_mix3(const WideEntry* M, int64_t* V, int* U, bool rows) {
+    WideHalf v[3];
+    int u[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        v[s] = wide_split(V[s]);
+        u[s] = U[s];
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        int64_t p[3];
+        int pu[3], top = 2 * kWideZero;
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            const WideEntry& w = M[rows ? m * 3 + s : s * 3 + m];
+            p[s] = wide_mul(v[s], w);
+            pu[s] = u[s] + w.u;
+            top = imax(top, pu[s]);
+        }
+        U[m] = top + 64;
+        V[m] = wide_shr(p[0], top - pu[0]) + wide_shr(p[1], top - pu[1]) + wide_shr(p[2], top - pu[2]);
+    }
+}
+
+// Strain (xx, yy, zz, yz, xz, xy) of one part of a node: normalised halves and units.  load(a, x, u) gives component
+// a's values, 2^59 at most, at the four backward neighbours and at the node itself, and their units.
+template <bool CUBIC, typename Load>
+PC_HD void wide_strain(const WideEntry* mix, const Load& load, WideHalf* e, int* eu) {
+    int64_t H[3][3];
+    int hu[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        int64_t x[5];
+        int u[5];
+        load(a, x, u);
+        const int U = imax(imax(imax(u[0], u[1]), imax(u[2], u[3])), u[4]);
+#pragma unroll
+        for (int l = 0; l < 5; ++l) x[l] = wide_shr(x[l], U - u[l]);
+        const int64_t p = x[0] + x[1], q = x[2] + x[3];
+        H[0][a] = p + q - 4 * x[4];  // 8 2^59 at most
+        H[1][a] = p - q;
+        H[2][a] = (x[0] - x[1]) + (x[2] - x[3]);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) hu[s][a] = U;
+        if (!CUBIC) {
+            int64_t V[3] = {H[0][a], H[1][a], H[2][a]};
+            int W[3] = {U, U, U};
+#pragma unroll
+            for (int s = 0; s < 3; ++s) V[s] = wide_norm(V[s], W[s]);
+            wide_mix3(mix, V, W, false);
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                H[s][a] = V[s];
+                hu[s][a] = W[s];
+            }
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const int a = p == 0 ? 1 : 0, b = p == 2 ? 1 : 2;
+        eu[p] = hu[p][p];
+        e[p] = wide_split(wide_norm(H[p][p], eu[p]));
+        // a difference that vanishes (a uniform component) leaves the other's bits alone
+        const int ua = H[b][a] == 0 ? kWideZero : hu[b][a], ub = H[a][b] == 0 ? kWideZero : hu[a][b];
+        eu[3 + p] = imax(ua, ub);
+        const int64_t sum = wide_shr(H[b][a], eu[3 + p] - ua) + wide_shr(H[a][b], eu[3 + p] - ub);
+        e[3 + p] = wide_split(wide_norm(sum, eu[3 + p]));
+    }
+}
+
 // Factors of sums of complex products (pc_blas.cu).
 struct WideC {
     WideHalf re, im;
