@@ -51,12 +51,10 @@ template <int N1, int N2>
 constexpr int plane_nt() { return N1 > 0 && N1 * N2 >= 40 ? 512 : kPlaneThreads; }
 template <int N1, int N2, typename C>
 constexpr int pencil_nt() {
-    return sizeof(C) == 16 ? 128 : N1 > 0 && N1 * N2 >= 40 ? 512 : kPencilThreads;
+    return N1 > 0 && sizeof(C) == 16 ? 128 : N1 > 0 && N1 * N2 >= 40 ? 512 : kPencilThreads;
 }
-// p positions per pencil CTA: the largest divisor of n up to this.  complex64: 128-byte rows.  complex128
-// is bound by the FP64 pipe, so it takes small tiles (64-byte rows) that reach every SM also for one
-// system: N = 48, one system, 144 CTAs instead of 48.
-template <typename C> constexpr int pencil_tile_max() { return sizeof(C) == 16 ? 4 : 16; }
+constexpr int kPencilTileMax = 16;   // p positions per pencil CTA: the largest divisor of n up to this,
+constexpr int kPencilTileSmall = 4;  // complex128 up to this (pencil_shape)
 
 template <typename C> struct RTy;
 template <> struct RTy<float2> { using R = float; };
@@ -170,13 +168,33 @@ __device__ __forceinline__ void dft_inv(C* buf, const Lines ln, int n1, int n2, 
 // Planes per CTA of the plane kernels (one: many small CTAs keep every SM busy at the solver's sizes).
 __host__ __device__ __forceinline__ int planes_per_cta(int) { return 1; }
 
-// p positions per pencil CTA: the largest divisor of n that is at most the precision's bound (no ragged tile).
-template <typename C>
-__host__ __device__ constexpr int pencil_tile(int n) {
+// The largest divisor of n that is at most `most` (no ragged tile).
+__host__ __device__ constexpr int largest_divisor(int n, int most) {
     int t = 1;
-    for (int d = 1; d <= pencil_tile_max<C>() && d <= n; ++d)
+    for (int d = 1; d <= most && d <= n; ++d)
         if (n % d == 0) t = d;
     return t;
+}
+// Tile of the sizes whose factors are compiled in.
+template <typename C>
+__host__ __device__ constexpr int pencil_tile_ct(int n) {
+    return largest_divisor(n, sizeof(C) == 16 ? kPencilTileSmall : kPencilTileMax);
+}
+
+// Tile and threads of a pencil CTA.  complex64: 128-byte rows.  complex128 is bound by the FP64 pipe, so it takes
+// small tiles (64-byte rows) that reach every SM also for one system: n = 24, one system, 144 CTAs instead of 48, 80
+// to 53 us for the three kernels, four systems 166 to 139 us.  Sizes without compiled factors lose by them once the
+// large tiles have more than 2.5 CTAs per SM (n = 36, four systems: 461 us with tiles of 12, 477 us with 4; n = 27,
+// 324 CTAs: 268 and 252 us), and where the only divisor up to four is one, a row of 16 bytes (n = 13, four systems:
+// 91 us with tiles of 13, 112 us with 1; n = 25, one system: 64 and 78 us).
+template <int N1, typename C>
+void pencil_shape(int n, int nsys, int nt, int* tile, int* threads) {
+    *threads = nt;
+    *tile = pencil_tile_ct<C>(n);
+    if (N1 > 0 || sizeof(C) != 16) return;
+    const int large = largest_divisor(n, kPencilTileMax);
+    if (*tile == 1 || 2L * nsys * n * (n / large) > 5L * device_sm_count()) *tile = large;
+    else *threads = 128;
 }
 
 // position of mode m = k1 + n1 k2 in the digit-permuted order
@@ -314,7 +332,7 @@ __global__ void __launch_bounds__(plane_nt<N1, N2>())
     }
 }
 
-// K2: per (system, q, tile of pencil_tile(n) p positions): DFT over k' of the six (component, parity)
+// K2: per (system, q, tile of pt p positions; N1 > 0: pencil_tile_ct): DFT over k' of the six (component, parity)
 // pencils, then by `mode`: 0 = preconditioner (butterfly, (A_ref - sigma rho_ref)^-1 scaled, inverse
 // butterfly, inverse DFT over k'); 1 = forward block transform (butterfly, scaled, written to `out` in
 // mode order [comp][r < 2n][q][p]); 2 = inverse block transform (reads `out`'s layout from W, inverse
@@ -323,7 +341,7 @@ template <int N1, int N2, typename C, typename R, typename TT>
 __global__ void __launch_bounds__(pencil_nt<N1, N2, C>())
     bdft_pencil(C* __restrict__ W, C* __restrict__ out, const C* __restrict__ wn_g, const R* __restrict__ Aref,
                 const TT* __restrict__ ea, const TT* __restrict__ eb, const TT* __restrict__ eg,
-                const int* __restrict__ sys_block, const int* __restrict__ skip, int n_rt, int n1, int n2,
+                const int* __restrict__ sys_block, const int* __restrict__ skip, int n_rt, int n1, int n2, int pt,
                 int64_t sys_stride, double shift_rho_d, double scale_d, int mode, const int* __restrict__ sys_k,
                 int64_t tab_stride, int64_t aref_stride) {
     const int n = N1 > 0 ? N1 * N2 : n_rt;
@@ -332,8 +350,8 @@ __global__ void __launch_bounds__(pencil_nt<N1, N2, C>())
         n2 = N2;
     }
     extern __shared__ __align__(16) unsigned char smem_bdft[];
-    constexpr int PTc = N1 > 0 ? pencil_tile<C>(N1 * N2) : 1;
-    const int PT = N1 > 0 ? PTc : pencil_tile<C>(n);
+    constexpr int PTc = N1 > 0 ? pencil_tile_ct<C>(N1 * N2) : 1;
+    const int PT = N1 > 0 ? PTc : pt;
     C* buf = reinterpret_cast<C*>(smem_bdft);  // [pencil = comp * 2 + par][k'][pl]
     C* wn = buf + 6 * n * PT;
     const int tiles = n / PT;
@@ -460,7 +478,7 @@ __global__ void __launch_bounds__(pencil_nt<N1, N2, C>())
 template <typename C>
 size_t plane_smem(int n) { return sizeof(C) * ((size_t)planes_per_cta(n) * n * n + n); }
 template <typename C>
-size_t pencil_smem(int n) { return sizeof(C) * ((size_t)6 * n * pencil_tile<C>(n) + n); }
+size_t pencil_smem(int n, int tile) { return sizeof(C) * ((size_t)6 * n * tile + n); }
 
 // Dynamic shared memory beyond 48 KB is granted once per kernel (the largest size asked so far).
 template <typename K>
@@ -488,7 +506,9 @@ static int precond_launch(int n, int n1, int n2, int nsys, const V* r, V* z, C* 
     using R = typename RTy<C>::R;
     const int64_t vs = (int64_t)6 * n * n * n;
     const int64_t aref_stride = (int64_t)9 * 2 * n * n * n;
-    const size_t sp = plane_smem<C>(n), sq = pencil_smem<C>(n);
+    int tile, nt;
+    pencil_shape<N1, C>(n, nsys, pencil_nt<N1, N2, C>(), &tile, &nt);
+    const size_t sp = plane_smem<C>(n), sq = pencil_smem<C>(n, tile);
     PC_TRY(allow_smem(bdft_plane_fwd<N1, N2, C, V>, sp));
     PC_TRY(allow_smem(bdft_pencil<N1, N2, C, R, TT>, sq));
     PC_TRY(allow_smem(bdft_plane_inv<N1, N2, C, V>, sp));
@@ -496,9 +516,9 @@ static int precond_launch(int n, int n1, int n2, int nsys, const V* r, V* z, C* 
     bdft_plane_fwd<N1, N2, C, V><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(r, W, wn, twa, twb, twk, n, n1, n2, planes, vs, vs,
                                                                skip, 0, sys_k, tab_stride);
     note_launch();
-    const int tiles = n / pencil_tile<C>(n);
-    bdft_pencil<N1, N2, C, R, TT><<<nsys * n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
-        W, nullptr, wn, Aref, ea, eb, eg, sys_block, skip, n, n1, n2, vs, shift_rho, scale, 0, sys_k, tab_stride,
+    const int tiles = n / tile;
+    bdft_pencil<N1, N2, C, R, TT><<<nsys * n * tiles, nt, sq, s>>>(
+        W, nullptr, wn, Aref, ea, eb, eg, sys_block, skip, n, n1, n2, tile, vs, shift_rho, scale, 0, sys_k, tab_stride,
         aref_stride);
     note_launch();
     bdft_plane_inv<N1, N2, C, V><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(W, z, r, wn, twa, twb, twk, n, n1, n2, planes, vs,
@@ -515,22 +535,24 @@ static int fourier_launch(int n, int n1, int n2, int inverse, const C* in, C* ou
                           double scale, cudaStream_t s) {
     using R = typename RTy<C>::R;
     const int64_t vs = (int64_t)6 * n * n * n;
-    const size_t sp = plane_smem<C>(n), sq = pencil_smem<C>(n);
+    int tile, nt;
+    pencil_shape<N1, C>(n, 1, pencil_nt<N1, N2, C>(), &tile, &nt);
+    const size_t sp = plane_smem<C>(n), sq = pencil_smem<C>(n, tile);
     PC_TRY(allow_smem(bdft_plane_fwd<N1, N2, C, C>, sp));
     PC_TRY(allow_smem(bdft_pencil<N1, N2, C, R, C>, sq));
     PC_TRY(allow_smem(bdft_plane_inv<N1, N2, C, C>, sp));
     const int planes = 6 * n, pctas = (planes + planes_per_cta(n) - 1) / planes_per_cta(n);
-    const int tiles = n / pencil_tile<C>(n);
+    const int tiles = n / tile;
     if (!inverse) {
         bdft_plane_fwd<N1, N2, C, C><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(in, W, wn, twa, twb, twk, n, n1, n2, planes, vs,
                                                                    vs, nullptr, 0, nullptr, 0);
         note_launch();
-        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
-            W, out, wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, vs, 0.0, scale, 1, nullptr, 0, 0);
+        bdft_pencil<N1, N2, C, R, C><<<n * tiles, nt, sq, s>>>(
+            W, out, wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, tile, vs, 0.0, scale, 1, nullptr, 0, 0);
         note_launch();
     } else {
-        bdft_pencil<N1, N2, C, R, C><<<n * tiles, (pencil_nt<N1, N2, C>()), sq, s>>>(
-            W, const_cast<C*>(in), wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, vs, 0.0, 1.0, 2, nullptr, 0, 0);
+        bdft_pencil<N1, N2, C, R, C><<<n * tiles, nt, sq, s>>>(
+            W, const_cast<C*>(in), wn, nullptr, ea, eb, eg, d_block, nullptr, n, n1, n2, tile, vs, 0.0, 1.0, 2, nullptr, 0, 0);
         note_launch();
         bdft_plane_inv<N1, N2, C, C><<<pctas, (plane_nt<N1, N2>()), sp, s>>>(W, out, nullptr, wn, twa, twb, twk, n, n1, n2,
                                                                    planes, vs, vs, scale, nullptr, nullptr, 0, nullptr,
