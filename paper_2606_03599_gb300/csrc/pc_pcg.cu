@@ -184,9 +184,10 @@ __global__ void pcg_beta(PcgScal* sc, int* done, const double* part_rr, int srr,
 }
 
 // Whether the vector kernels sum the partials in every CTA of a system (OWN below) instead of waiting for a
-// kernel of one CTA per system.  It saves two of some nine launches per iteration and costs every CTA a
-// latency of about 2 us, which more CTAs per SM pay one after the other.  Measured on one GB300, two kernels
-// against none: N = 48, one system (81 CTAs) 3.08 and 2.91 ms per solve; N = 64 (192 CTAs) 4.63 and 4.43 ms;
+// kernel of one CTA per system.  It saves two of some nine launches per iteration and costs every CTA the sums:
+// each of its 8 warps adds 5 shuffle steps and 8 warps' sums per list, with three lists some 300 FP64 instructions of 16
+// clocks (2 lanes per clock and SM), 2.6 us of a pipe that the CTAs of an SM share.  Measured on one GB300, two
+// kernels against none: N = 48, one system (81 CTAs) 3.08 and 2.91 ms per solve; N = 64 (192 CTAs) 4.63 and 4.43 ms;
 // bands at N = 8 31.2 and 28.4 ms; even at N = 24, 20 bands (about 260 CTAs, 41.5 ms); lost at N = 32
 // (about 580 CTAs, 48.1 and 49.8 ms) and N = 48 with four Bloch vectors (220 and 263 ms).  The line lies at
 // two CTAs per SM.
