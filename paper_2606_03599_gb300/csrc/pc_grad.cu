@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kGradThreads, 4)
             xx = fma(xo, xo, xx);
         }
         gr = fma(V.wR, xx, gr);
-        WideHalf f[6];
+        WideHalf f[6], h[6];
         int fu[6];
         wide_strain<CUBIC>(
             P.mix,
@@ -205,26 +205,23 @@ __global__ void __launch_bounds__(kGradThreads, 4)
                 }
             },
             f, fu);
+        // a shift rounds down: the real parts' products are added, the imaginary parts' taken away with the
+        // sign turned (as 64 bits: a low half of -2^31 has no negative), so that the roundings of a square cancel
+        const int64_t turn = (V.neg != 0) != (part != 0) ? -1 : 0;
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
             fu[p] += V.s.u + 64;
-            f[p] = wide_split(wide_norm(wide_mul(f[p], V.s), fu[p]));
+            const int64_t m = wide_norm(wide_mul(f[p], V.s), fu[p]);
+            f[p] = wide_split(m);
+            h[p] = wide_split((m ^ turn) - turn);
         }
-        // a shift rounds down: the real parts' products are added, the imaginary parts' taken away with the
-        // sign turned, so that the roundings of a square cancel in the mean
-        const bool turn = (V.neg != 0) != (part != 0);
         int q = 0;
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
-            WideHalf h = f[p];
-            if (turn) {
-                h.hi = -h.hi;
-                h.lo = -h.lo;
-            }
 #pragma unroll
             for (int r = p; r < 6; ++r, ++q) {
                 const int u = fu[p] + fu[r] + 4, U = imax(gu[q], u);
-                const int64_t m = wide_shr(wide_mul(h, f[r]), U - u + 4), s = wide_shr(g[q], U - gu[q]);
+                const int64_t m = wide_shr(wide_mul(h[p], f[r]), U - u + 4), s = wide_shr(g[q], U - gu[q]);
                 g[q] = part ? s - m : s + m;
                 gu[q] = U;
             }
