@@ -659,8 +659,8 @@ extern "C" int pc_emu_small_dft(int L, int inv, const double* in, double* out) {
     }
 }
 
-// sum of a b over n <= 8 complex pairs, one group, as the outer-loop products form it.  Returns 0, or 1 when
-// the group's exponents leave the integer path's range.
+// sum of a b over n <= 8 complex pairs, one group, as the Gram products form it.  Returns 0, or 1 when the group's
+// exponents leave the integer path's range.
 extern "C" int pc_emu_limb_dot(int n, const double* a, const double* b, double* out) {
     const double2* x = reinterpret_cast<const double2*>(a);
     const double2* y = reinterpret_cast<const double2*>(b);
@@ -673,10 +673,14 @@ extern "C" int pc_emu_limb_dot(int n, const double* a, const double* b, double* 
     if (Ea < kWideLow || Ea > kWideHigh || Eb < kWideLow || Eb > kWideHigh) return 1;
     WideSum re = wide_sum0(), im = wide_sum0();
     for (int q = 0; q < n; ++q) {
+        wide_reach(re, wide_unit(x[q].x), wide_unit(y[q].x), wide_unit(x[q].y), wide_unit(y[q].y));
+        wide_reach(im, wide_unit(x[q].x), wide_unit(y[q].y), wide_unit(x[q].y), wide_unit(y[q].x));
+    }
+    for (int q = 0; q < n; ++q) {
         int ur, ui, vr, vi;
         const WideC u = wide_factor(x[q], ur, ui), v = wide_factor(y[q], vr, vi);
-        wide_mac2(re, u.re, ur, v.re, vr, u.im, ui, v.im, vi);
-        wide_mac2(im, u.re, ur, v.im, vi, wide_neg(u.im), ui, v.re, vr);
+        wide_mac2<true>(re, u.re, ur, v.re, vr, u.im, ui, v.im, vi);
+        wide_mac2<false>(im, u.re, ur, v.im, vi, u.im, ui, v.re, vr);
     }
     out[0] = wide_to_double(re);
     out[1] = wide_to_double(im);

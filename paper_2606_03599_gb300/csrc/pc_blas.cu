@@ -6,19 +6,20 @@
 // The shapes are a few to a few dozen columns of length 3 n_b (83k at N = 48, 3.1M at N = 160),
 // so the work is a sum over a long index with a small dense result.  In FP64 arithmetic they are
 // bound by GB300's FP64 pipe (2 lanes per clock and SM, 8 FMAs for every 16-byte operand), 4 to 6
-// times above their memory time.  So products run on the integer pipe in groups of eight
-// (pc_wide.cuh): every value keeps its own exponent, a real product is four 32 x 32 + 64 bit
-// multiply-adds and its place in the group's sum a shift and an addition, and the FP64 pipe sees two
+// times above their memory time.  Gram products of more than four rows therefore run on the integer pipe in
+// groups of eight (pc_wide.cuh): every value keeps its own exponent, a real product is four 32 x 32 + 64 bit
+// multiply-adds and its place in the group's sum a rounding shift and an addition, and the FP64 pipe sees two
 // instructions per group and result.  Operands are
 // read once per register block with coalesced 16-byte loads, the mass weight is applied once per
 // element of W (not per product), and Gram partial sums are reduced in a fixed order (per CTA, then
 // across CTAs) so results are deterministic.
 //
 // Measured in an FP64 solve at N = 48 (sixteen spaces, vectors of 1.3 MB), FP64 / integer form: Gram products of
-// more than four rows 0.56 / 0.29 ms, updates of 2 columns 0.21 / 0.13 ms, of 4 columns 1.20 / 0.74 ms; at N = 128
-// (four spaces, vectors of 25 MB) 1.23, 0.55 and 3.6 ms in the integer form.  (Eight values cut into limbs of one shared
-// exponent took 0.19, 0.11 and 0.42 ms at N = 48, but lost small values next to large ones and made every
-// squared norm 5e-17 too small.)
+// more than four rows 0.56 / 0.34 ms.  Updates stay in FP64 (0.21 ms for 2 columns, 1.20 ms for 4): their rounding has
+// to be free of any common offset, a long wave of the lattice that the shift-invert iteration would amplify, and with
+// that the integer form took 0.18 and 1.11 ms.  (Eight values cut into limbs of one shared exponent took 0.19 ms for
+// Gram products and 0.11 and 0.42 ms for updates, but lost small values next to large ones and made every squared norm
+// 5e-17 too small.)
 #include <algorithm>
 
 #include "pc_solver.h"
@@ -198,15 +199,24 @@ __device__ __forceinline__ void gram_tile(const double2* __restrict__ A, int row
                     for (int j = 0; j < CB; ++j) re[j] = im[j] = wide_sum0();
 #pragma unroll
                     for (int q = 0; q < NB; ++q) {
+                        const int ur = wide_unit(a[q].x), ui = wide_unit(a[q].y);
+#pragma unroll
+                        for (int j = 0; j < CB; ++j) {
+                            const short2 uv = ub[j][g * 256 + q * 32 + lane];
+                            wide_reach(re[j], ur, uv.x, ui, uv.y);
+                            wide_reach(im[j], ur, uv.y, ui, uv.x);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) {
                         int ur, ui;
                         const WideC la = wide_factor(a[q], ur, ui);
-                        const WideHalf ni = wide_neg(la.im);
 #pragma unroll
                         for (int j = 0; j < CB; ++j) {  // conj(a) b
                             const WideC lv = lb[j][g * 256 + q * 32 + lane];
                             const short2 uv = ub[j][g * 256 + q * 32 + lane];
-                            wide_mac2(re[j], la.re, ur, lv.re, uv.x, ni, ui, lv.im, uv.y);
-                            wide_mac2(im[j], la.re, ur, lv.im, uv.y, la.im, ui, lv.re, uv.x);
+                            wide_mac2<false>(re[j], la.re, ur, lv.re, uv.x, la.im, ui, lv.im, uv.y);
+                            wide_mac2<true>(im[j], la.re, ur, lv.im, uv.y, la.im, ui, lv.re, uv.x);
                         }
                     }
 #pragma unroll
@@ -300,97 +310,32 @@ __global__ void ts_gram_reduce(const double* __restrict__ part, int nentries, in
     if (lane == 0) out[e] = make_double2(re, im);
 }
 
-// cr + i ci += sum over NB columns kk .. kk + NB - 1 of A of a(e) h(., j): a group of columns on the
-// integer pipe, or in FP64 where its largest value (or that of a column of h: hok) is out of range.
-template <int CB, int NB>
-__device__ __forceinline__ void update_group(const double2* __restrict__ Ae, int64_t vs, const WideC* hs, const short2* hu,
-                                             bool hok, const double2* __restrict__ h, int64_t hstr,
-                                             int jn, double* cr, double* ci) {
-    double2 a[NB];
-    int top = 0;
-#pragma unroll
-    for (int q = 0; q < NB; ++q) {
-        a[q] = Ae[(int64_t)q * vs];
-        top = wide_top(a[q], top);
-    }
-    const int E = top >> 20;
-    if (hok && E >= kWideLow && E <= kWideHigh) {
-        WideSum re[CB], im[CB];
-#pragma unroll
-        for (int j = 0; j < CB; ++j) re[j] = im[j] = wide_sum0();
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            int ur, ui;
-            const WideC la = wide_factor(a[q], ur, ui);
-            const WideHalf ni = wide_neg(la.im);
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                const WideC hv = hs[q * CB + j];
-                const short2 uv = hu[q * CB + j];
-                wide_mac2(re[j], la.re, ur, hv.re, uv.x, la.im, ui, hv.im, uv.y);
-                wide_mac2(im[j], la.re, ur, hv.im, uv.y, ni, ui, hv.re, uv.x);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-            cr[j] += wide_to_double(re[j]);
-            ci[j] += wide_to_double(im[j]);
-        }
-    } else if (top != 0 || !hok) {
-#pragma unroll 1
-        for (int q = 0; q < NB; ++q) {
-            const double2 av = Ae[(int64_t)q * vs];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                const double2 hv = j < jn ? h[q + (int64_t)j * hstr] : make_double2(0.0, 0.0);
-                cr[j] = fma(av.x, hv.x, fma(-av.y, hv.y, cr[j]));
-                ci[j] = fma(av.x, hv.y, fma(av.y, hv.x, ci[j]));
-            }
-        }
-    }
-}
-
 // C[:, j] = beta C[:, j] + alpha sum_k A[:, k] h(k, j) for the CB columns j0 .. j0 + CB - 1 of
-// column group blockIdx.y; the factors of h (k x cols, column-major) are staged in shared memory.  With beta == 0, C is not read (it may hold anything).
+// column group blockIdx.y, in FP64; h (k x cols, column-major) is staged in shared memory.  With
+// beta == 0, C is not read (it may hold anything).
 template <int CB>
 __device__ __forceinline__ void update_columns(const double2* __restrict__ A, int k, const double2* __restrict__ h,
                                                int cols, double2* __restrict__ C, int64_t vs, double alpha,
                                                double beta, int j0) {
-    extern __shared__ WideC hs[];  // [k][CB], then their units
-    short2* hu = reinterpret_cast<short2*>(hs + (size_t)k * CB);
-    __shared__ int tops[CB];
-    if (threadIdx.x < CB) tops[threadIdx.x] = 0;
-    __syncthreads();
+    extern __shared__ double2 hs[];  // [k][CB]
     for (int q = threadIdx.x; q < k * CB; q += blockDim.x) {
         const int kk = q / CB, j = q % CB;
-        const double2 hv = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
-        int ur, ui;
-        hs[q] = wide_factor(hv, ur, ui);
-        hu[q] = make_short2((short)ur, (short)ui);
-        atomicMax(&tops[j], wide_top(hv, 0));
+        hs[q] = (j0 + j < cols) ? h[kk + (int64_t)(j0 + j) * k] : make_double2(0.0, 0.0);
     }
     __syncthreads();
-    bool hok = true;
-#pragma unroll
-    for (int j = 0; j < CB; ++j) {
-        const int E = tops[j] >> 20;
-        hok = hok && (tops[j] == 0 || (E >= kWideLow && E <= kWideHigh));
-    }
-    const double2* __restrict__ hj = h + (int64_t)j0 * k;
-    const int jn = cols - j0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < vs; e += (int64_t)gridDim.x * blockDim.x) {
         double cr[CB], ci[CB];
 #pragma unroll
         for (int j = 0; j < CB; ++j) cr[j] = ci[j] = 0.0;
-        int kk = 0;
-        for (; kk + 8 <= k; kk += 8)
-            update_group<CB, 8>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
-        if (k & 4) {
-            update_group<CB, 4>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
-            kk += 4;
+        for (int kk = 0; kk < k; ++kk) {
+            const double2 a = A[(int64_t)kk * vs + e];
+#pragma unroll
+            for (int j = 0; j < CB; ++j) {  // a h
+                const double2 hv = hs[kk * CB + j];
+                cr[j] = fma(a.x, hv.x, fma(-a.y, hv.y, cr[j]));
+                ci[j] = fma(a.x, hv.y, fma(a.y, hv.x, ci[j]));
+            }
         }
-        for (; kk < k; ++kk)
-            update_group<CB, 1>(A + (int64_t)kk * vs + e, vs, hs + kk * CB, hu + kk * CB, hok, hj + kk, k, jn, cr, ci);
 #pragma unroll
         for (int j = 0; j < CB; ++j) {
             if (j0 + j >= cols) continue;
@@ -488,15 +433,6 @@ __global__ void __launch_bounds__(256)
     update_columns<CB>(J.A, J.k, J.h, J.cols, J.C, vs, J.alpha, J.beta, j0);
 }
 
-// Shared memory of an update of k basis columns, granted beyond the default 48 KB where it takes more.
-template <typename K>
-int update_smem(K kern, int k, int CB, size_t* smem) {
-    if ((size_t)k * CB > 3072) return fail(PC_EINVAL, "ts_update: too many basis columns");
-    *smem = (sizeof(WideC) + sizeof(short2)) * (size_t)k * CB;
-    if (*smem > 47 * 1024) PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
-    return PC_OK;
-}
-
 }  // namespace
 
 int ts_gram(const double2* A, int rows, const double2* B, int cols, int64_t m, const void* mat, int matkind,
@@ -545,8 +481,8 @@ int ts_update(const double2* A, int k, const double2* d_h, int cols, double2* C,
     // column blocks of 2 when cols <= 2 (the Gram-Schmidt updates of a 2-wide Krylov block:
     // no FMAs on padding columns), else of 4
     const int CB = cols <= 2 ? 2 : 4;
-    size_t smem;
-    PC_TRY(CB == 2 ? update_smem(ts_update_kernel<2>, k, CB, &smem) : update_smem(ts_update_kernel<4>, k, CB, &smem));
+    const size_t smem = sizeof(double2) * (size_t)k * CB;
+    if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update: too many basis columns");
     const int ngc = (cols + CB - 1) / CB;
     int64_t gx = (vs + 255) / 256;
     gx = std::min<int64_t>(gx, std::max<int64_t>(1, 8LL * device_sm_count() / ngc));
@@ -618,9 +554,8 @@ int ts_update_batch(const UpdateJob* jobs, int njobs, int64_t vs, cudaStream_t s
         }
         if (U.n == 0) continue;
         const int CB = maxc <= 2 ? 2 : 4;
-        size_t smem;
-        PC_TRY(CB == 2 ? update_smem(ts_update_batch_kernel<2>, maxk, CB, &smem)
-                       : update_smem(ts_update_batch_kernel<4>, maxk, CB, &smem));
+        const size_t smem = sizeof(double2) * (size_t)maxk * CB;
+        if (smem > 48 * 1024) return fail(PC_EINVAL, "ts_update_batch: too many basis columns");
         const int ngc = (maxc + CB - 1) / CB;
         int64_t gx = (vs + 255) / 256;
         gx = std::min<int64_t>(gx, std::max<int64_t>(1, 8LL * device_sm_count() / ((int64_t)ngc * U.n)));

@@ -214,7 +214,7 @@ PC_HD void wide_strain(const WideEntry* mix, const Load& load, WideHalf* e, int*
     }
 }
 
-// Factors of sums of complex products (pc_blas.cu).
+// Factors of sums of complex products (Gram products of pc_blas.cu).
 struct WideC {
     WideHalf re, im;
 };
@@ -245,12 +245,15 @@ PC_HD WideC wide_factor(double2 v, int& ur, int& ui) {
     r.im = wide_factor(v.y, ui);
     return r;
 }
-PC_HD WideHalf wide_neg(WideHalf a) {
-    a.hi = -a.hi;
-    a.lo = -a.lo;
-    return a;
+// p >> s to nearest, s >= 1.
+PC_HD int64_t wide_shr_near(int64_t p, int s) { return (wide_shr(p, s - 1) + 1) >> 1; }
+// The unit wide_factor gives a double.
+PC_HD int wide_unit(double v) {
+    const int e = (int)(wide_bits(v) >> 52) & 0x7ff;
+    return e == 0 ? kWideZero : e - 1084;
 }
-// A running sum of up to 16 products (eight complex ones): m 2^(u + 64).
+// A sum of up to 16 products (eight complex ones): m 2^(u + 64).  u is found from the products' units first
+// (wide_reach for each pair), three bits above the largest, so that the sum stays below 2^61.
 struct WideSum {
     int64_t m;
     int u;
@@ -261,13 +264,14 @@ PC_HD WideSum wide_sum0() {
     s.u = 2 * kWideZero;
     return s;
 }
-// s + a b - c d, in units of the largest product and two bits up, so that 16 products stay below 2^62.  A shift
-// rounds down: taking one of the products away rather than adding its negative, the two roundings cancel in the mean
-// (all added, a squared norm came out 2e-16 too small).
+PC_HD void wide_reach(WideSum& s, int ua, int ub, int uc, int ud) { s.u = imax(s.u, imax(ua + ub, uc + ud) + 3); }
+// s + a b + c d, or (SUB) s + a b - c d.  Shifts round to nearest, and one of the products is taken away, so that
+// halves rounded up cancel in the mean.  A product changes sign as 64 bits: a
+// factor's low half can be -2^31, whose negative has no 32 bits.
+template <bool SUB>
 PC_HD void wide_mac2(WideSum& s, WideHalf a, int ua, WideHalf b, int ub, WideHalf c, int uc, WideHalf d, int ud) {
-    const int u1 = ua + ub, u2 = uc + ud, U = imax(s.u, imax(u1, u2) + 2);
-    s.m = wide_shr(s.m, U - s.u) + wide_shr(wide_mul(a, b), U - u1) - wide_shr(wide_mul(c, d), U - u2);
-    s.u = U;
+    const int64_t p = wide_mul(c, d);
+    s.m += wide_shr_near(wide_mul(a, b), s.u - ua - ub) - wide_shr_near(SUB ? p : -p, s.u - uc - ud);
 }
 
 // m 2^u to the nearest double (results below the normal range round twice).
