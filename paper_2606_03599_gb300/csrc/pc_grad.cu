@@ -176,9 +176,8 @@ __global__ void __launch_bounds__(kGradThreads, 4)
         double xx = 0.0;
 #pragma unroll
         for (int al = 0; al < 3; ++al) {
-            const double2 z = x[(int64_t)al * P.vstr + nd.at];
-            const double xo = part ? z.y : z.x;
-            xx = fma(xo, xo, xx);
+            const double2 xo = x[(int64_t)al * P.vstr + nd.at];
+            xx = cdotre(xo, xo, xx);  // both parts in both lanes
         }
         gr = fma(V.wR, xx, gr);
         WideHalf f[6], h[6];
@@ -230,7 +229,6 @@ __global__ void __launch_bounds__(kGradThreads, 4)
     // the two lanes of a node take every branch alike
     const unsigned pair = 3u << (threadIdx.x & 30);
     slow = __shfl_xor_sync(pair, (int)slow, 1) != 0 || slow;
-    gr += __shfl_xor_sync(pair, gr, 1);
 #pragma unroll
     for (int q = 0; q < 21; ++q) {
         const int64_t o = __shfl_xor_sync(pair, g[q], 1);
@@ -299,9 +297,10 @@ extern "C" int pc_eig_grad(pc_grid* g, int block, int nvec, const void* X, const
         for (int v = 0; v < P.nvec; ++v) {
             const double w = weights[base + v];
             GradVec& V = P.v[v];
+            V.wC = w * scaleC;
+            V.wR = -w * lambdas[base + v] * scaleR;
             // extended precision: the root's rounding would enter every product twice
-            const long double sq = sqrtl((long double)std::fabs(w) / ((long double)g->rho0 * g->L * g->L)) *
-                                   (g->cubic ? (long double)q : 1.0L);
+            const long double sq = sqrtl((long double)std::fabs(V.wC)) * (g->cubic ? (long double)q : 1.0L);
             V.neg = w < 0 ? 1 : 0;
             int ex = 0;
             if (sq > 0) frexpl(sq, &ex);
@@ -310,8 +309,6 @@ extern "C" int pc_eig_grad(pc_grid* g, int block, int nvec, const void* X, const
             V.s.lo = h.lo;
             V.s.u = sq > 0 ? ex - 62 : kWideZero;
             V.s.pad = 0;
-            V.wC = w * scaleC;
-            V.wR = -w * lambdas[base + v] * scaleR;
         }
         const int64_t nodes = (int64_t)P.X * P.Y * P.Z;
         const dim3 grid((unsigned)((2 * nodes + kGradThreads - 1) / kGradThreads), P.full ? 4 : 1);
