@@ -122,7 +122,10 @@ bool tuned_config(int X, int Y, int Z, int dtype, bool full, int matkind, bool c
 ApplyConfig apply_config_for(const pc_grid* g, bool full, int nitems, int dtype) {
     const int X = full ? g->N : g->X, Y = full ? g->N : g->Y, Z = g->Z;
     ApplyConfig c;
-    if (tuned_config(X, Y, Z, dtype, full, g->matkind, g->cubic, nitems, &c) && !(c.fix && !g->int_ok)) return c;
+    // a cache file may name a kernel that is not one for this precision or material: the default then
+    if (tuned_config(X, Y, Z, dtype, full, g->matkind, g->cubic, nitems, &c) &&
+        !(c.fix && (dtype != PC_C128 || !g->int_ok)) && !(c.cell && (dtype != PC_C64 || g->matkind == 2)))
+        return c;
     c = ApplyConfig();
     return choose_apply_config(X, Y, Z, nitems, dtype, !full, g->matkind, true, g->int_ok, g->cubic);
 }
