@@ -112,7 +112,7 @@ ApplyConfig choose_apply_config(int X, int Y, int Z, int nitems, int dtype, bool
     // pipelined kernel has compiled in (N = 160, 4 items: 103 us against 107 us, 2 items 56.6 against 57.5;
     // one item: 35.8 against 32.9; N = 128, 4 items: 60.5 against 56.4; sizes without a compiled width take
     // it 1.6 to 5 times as long, e.g. N = 60, 64 items: 203 against 120 us)
-    const bool pipe_width = blocks && cubic && matkind == 0 && X == 80 && nitems >= 2 && pipe_geom_ok(X, Y, Z, matkind);
+    const bool pipe_width = blocks && cubic && matkind == 0 && X == kPipeWidest && nitems >= 2 && pipe_geom_ok(X, Y, Z, matkind);
     if (apply_kernel_mode() == 0 && scratch_ok && dtype == PC_C64 && matkind != 2 && !pipe_width) {
         c.cell = true;
         c.shape = kCellShape;

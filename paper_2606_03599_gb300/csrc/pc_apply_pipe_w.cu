@@ -25,7 +25,7 @@ int launch_pipe_widths(int X, const StencilParams<float>& P, const ApplyItem* it
     PC_PIPE_CASE(32)
     PC_PIPE_CASE(48)
     PC_PIPE_CASE(64)
-    PC_PIPE_CASE(80)
+    PC_PIPE_CASE(kPipeWidest)
 #undef PC_PIPE_CASE
     return PC_OK;
 }

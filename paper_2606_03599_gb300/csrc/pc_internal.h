@@ -76,6 +76,7 @@ int launch_apply_row_f32(bool cubic, int matkind, const StencilParams<float>& P,
                          const void* const* mats, int nitems, int ctas, double* dp, int ds, int* err, cudaStream_t s);
 int row_apply_ctas(int X, int Y, int Z, int matkind, int nitems, int minseg = 12);
 // Plane-pipelined kernel (complex64 parity blocks, even X): producer warp + consumer warps.
+constexpr int kPipeWidest = 80;  // widest quarter grid whose width is compiled in
 // item_ph: (cos, sin) of the three Bloch phases of each item ([nitems][3][2]).
 int launch_apply_pipe_f32(bool cubic, int matkind, const StencilParams<float>& P, const ApplyItem* items,
                           const double* item_ph, const void* const* mats, int nitems, int ctas, double* dp, int ds,
