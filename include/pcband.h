@@ -394,8 +394,8 @@ int pc_autotune(pc_grid* g, int dtype, int layout, int nitems, void* stream);
 
 /* The launch configuration the library will use for a batch of `nitems` vectors of `dtype` in
  * layout 0 (blocks) or 1 (full): kind 0 = fused tile (shapes 0-3 register-staged; shape 8 the
- * integer-pipe kernel, the default for complex128 with phase ids and for larger batches of fractions; shape 9 the cell kernel, the default for
- * complex64), 1 = TMA tile, 2 = row tile, 3 = two-pass
+ * integer-pipe kernel, the default for complex128 with phase ids and for larger batches of
+ * fractions; shape 9 the cell kernel, the default for complex64), 1 = TMA tile, 2 = row tile, 3 = two-pass
  * (fluxes once per node, then gather; the default for complex128 otherwise), 4 = plane-pipelined (producer
  * warp + consumer warps); tile shape code; planes per CTA
  * (tz; row and plane-pipelined kernels: least planes per CTA); CTAs of the launch (two-pass: of

@@ -29,7 +29,7 @@
 // outputs.
 //
 // Measured (one GB300, shift on, against the two-pass FP64 kernels): N = 48, 64 block vectors, one phase fully
-// anisotropic 0.353 / 0.667 ms; N = 60 FCC sub-pixel material, four blocks 0.137 / 0.195 ms; N = 64 nodewise
+// anisotropic 0.353 / 0.667 ms, both isotropic 0.286 ms; N = 60 FCC sub-pixel material, four blocks 0.137 / 0.195 ms; N = 64 nodewise
 // material, full space 0.157 / 0.146 ms, which is why nodewise materials take it only where the autotuner finds
 // it faster.  Bound by the integer instruction stream (16 warps per SM): a product and its place in a sum are ten
 // instructions, half of them at half rate.  (Nine products instead of 36 in warps whose nodes are orthotropic pay
@@ -96,9 +96,9 @@ inline bool make_fix_params(FixParams& F, const StencilParams<double>& P, bool c
 // MATK: 0 = phase ids, 1 = inclusion fraction, 2 = nodewise material (as SplitApply).
 // NP: parts (real, imaginary) of a cell in one thread; they meet in the Bloch phase only.  NP = 2 computes
 // addresses and node-dependent stiffness once for both and is the form of launches that fill the GPU (N = 48, 64
-// block vectors: 340 us, 379 us with NP = 1 in the same run).  NP = 1, two adjacent lanes per cell, halves a thread's chain of
-// dependent instructions: the form of small launches, which wait for that chain (N = 8, one block vector:
-// 16.6 us, 24.8 us with NP = 2).  The results are the same.
+// block vectors: 340 us, 379 us with NP = 1 in the same run).  NP = 1, two adjacent lanes per cell, halves a
+// thread's chain of dependent instructions: the form of small launches, which wait for that chain (N = 8, one block
+// vector: 16.6 us, 24.8 us with NP = 2).  The results are the same.
 template <bool CUBIC, int MATK, int NP>
 struct FixApply {
     struct Shared {

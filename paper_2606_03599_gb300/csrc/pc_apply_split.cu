@@ -1,5 +1,5 @@
 // Two-pass stencil apply (see pc_apply_split.cuh): kernels and launchers.  Complex128 (bound by
-// the FP64 pipe) where the integer-pipe kernel does not apply; complex64 as an autotuner candidate for
+// the FP64 pipe) for nodewise materials and small launches of fractions; complex64 as an autotuner candidate for
 // grids whose fluxes stay in L2.
 #include <algorithm>
 

@@ -1,7 +1,7 @@
 // Two-pass stencil apply in the vectors' own precision, written as per-node functions so that
-// the CUDA kernels and a host emulator share the index arithmetic.  Complex128 applies take it where
-// the material is out of the integer-pipe kernel's range (pc_apply_int.cuh, which is two to three times
-// as fast); for both precisions it is an autotuner candidate.
+// the CUDA kernels and a host emulator share the index arithmetic.  Complex128 applies take it for nodewise
+// materials and small launches of fractions (choose_apply_config; else pc_apply_int.cuh); for both precisions it is an
+// autotuner candidate.
 //
 // Operator and layouts as in pc_apply_tile.cuh (Sec. 3: y = (A - shift M) x with the
 // fluxes F_l of the adjoint differences).  On GB300 the FP64 pipe (2 lanes per cycle per

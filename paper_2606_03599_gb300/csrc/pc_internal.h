@@ -95,9 +95,9 @@ int launch_apply_split_f64(bool full, bool cubic, int matkind, const StencilPara
 int launch_apply_split_f32(bool full, bool cubic, int matkind, const StencilParams<float>& P, const ApplyItem* items,
                            const double* item_ph, int nitems, void* scratch, size_t scratch_bytes, double* dp, int ds,
                            cudaStream_t s);
-// Integer-pipe complex128 apply (block floating point, no scratch; every item its own Bloch phases):
+// Integer-pipe complex128 apply (FP64 operations on the integer units, no scratch; every item its own Bloch phases):
 // tz planes per CTA; fix_apply_ctas gives the CTAs per item of the default chunking (tz_in 0) or of
-// tz_in planes, and the planes in *tz.  fix_apply_ok: the material's scale is within its range.
+// tz_in planes, and the planes in *tz.  fix_apply_ok: the material's tables are finite.
 int launch_apply_fix(bool full, bool cubic, int matkind, const StencilParams<double>& P, const ApplyItem* items,
                      const double* item_ph, int nitems, int tz, double* dp, int ds, cudaStream_t s);
 int fix_apply_ctas(int N, bool full, int nitems, int tz_in, int* tz);
@@ -235,7 +235,7 @@ struct pc_grid {
     double rhohat[2];
     double Ainv[9];  // (A_hat^-1)_{s m}, row-major s*3+m
     bool cubic = true;
-    bool int_ok = false;  // the integer-pipe complex128 apply can take this material
+    bool int_ok = false;  // the integer-pipe complex128 apply can take this material (finite tables)
     int matkind = 0;  // 0 = uint8 phase ids, 1 = float theta, 2 = nodewise ([22][m] FP64)
     double sigma_cmax = 0.0, sigma_rmax = 0.0;  // largest |C| entry and density (hat units): default shift
     double mean_theta = 0.0;  // volume fraction of phase 1
